@@ -228,10 +228,8 @@ lbm_status lbm_get_owner(lbm_ctx *ctx, int *owner);
 
 /* Copy / replace the post-collision PDFs f_q (unshifted values), 19 x cells
  * doubles, direction-major (q = 0..18 in the order fixed by App. A). Solid
- * cells read as NaN: every PDF slot of a solid cell holds a NaN marker (with
- * the owning particle in its payload for f32 and f64 storage), by which the
- * dense kernel finds particle links; values given for solid cells are
- * replaced by that marker. Synchronises the stream. */
+ * cells read as NaN; values given for solid cells are not used. Synchronises
+ * the stream. */
 lbm_status lbm_get_pdfs(lbm_ctx *ctx, double *f);
 lbm_status lbm_set_pdfs(lbm_ctx *ctx, const double *f);
 

@@ -33,7 +33,7 @@ struct lbm_ctx {
     cudaStream_t stream = nullptr;
     bool own_memory = false;
     char* base = nullptr;
-    size_t bytes = 0;
+    size_t bytes = 0;              // of the simulation state (a checkpoint holds it)
     size_t elem = 4;
     void* f[2] = {nullptr, nullptr};
     int cur = 0;
@@ -51,6 +51,8 @@ struct lbm_ctx {
     int* status = nullptr;
     double* accel = nullptr;
     float* accel_f = nullptr;
+    uint32_t* solid = nullptr;     // one bit per cell (see launch.h)
+    uint32_t* shell = nullptr;
     unsigned int* miss_list = nullptr;
     int* miss_count = nullptr;
     int miss_cap = 0;
@@ -152,10 +154,11 @@ size_t elem_size(lbm_storage s) {
 
 // device memory layout: every piece 256-byte aligned, in a fixed order
 struct Layout {
-    size_t off[64];
-    size_t size[64];
+    size_t off[80];
+    size_t size[80];
     int n = 0;
     size_t total = 0;
+    size_t state = 0;   // bytes of the pieces a checkpoint holds (the first ones)
     int add(size_t bytes) {
         off[n] = total;
         size[n] = bytes;
@@ -255,7 +258,11 @@ void build_layout(const lbm_grid* g, lbm_storage st, int np, Layout& L, const Si
         L.add(4 * 3 * n);                        // 58/60 float32 u
         L.add(4 * 3 * n);                        // 59/61 float32 omega
     }
-    (void)g;
+    L.state = L.total;
+    // derived data, rebuilt after a restore: one bit per cell
+    const size_t words = (size_t)((g->nx + 31) / 32) * g->ny * g->nz;
+    L.add(4 * words);                            // 62 solid
+    L.add(4 * words);                            // 63 shell
 }
 
 lbm_status validate(const lbm_grid* g, const lbm_relax* r, const lbm_dem* d, lbm_storage st,
@@ -271,7 +278,7 @@ lbm_status validate(const lbm_grid* g, const lbm_relax* r, const lbm_dem* d, lbm
     if (!(r->magic > 0.0) || !(r->lambda_b_shell > 0.0) || !(r->lambda_b_bulk > 0.0) || !(r->shell_width >= 0.0))
         return fail(nullptr, LBM_ERR_INVALID, "magic, lambda_b must be > 0 and shell_width >= 0");
     if (st < LBM_STORE_F64 || st > LBM_STORE_BF16) return fail(nullptr, LBM_ERR_INVALID, "unknown storage format");
-    // the NaN marker of a solid cell carries particle + 1 in 22 bits
+    // a stated limit of the interface
     if (max_particles < 0 || max_particles > 4000000)
         return fail(nullptr, LBM_ERR_INVALID, "max_particles must be in [0, 4,000,000]");
     if (d->n_sub < 1) return fail(nullptr, LBM_ERR_INVALID, "n_sub must be >= 1");
@@ -304,14 +311,13 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
             ctx->num_sms = sms;
-        cudaError_t pe = prepare_stream_collide((int)st);
-        if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
+        cudaError_t pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
         if (pe != cudaSuccess) {
             destroy_handles(ctx);
             delete ctx;
-            return fail(nullptr, LBM_ERR_CUDA, std::string("kernel attributes: ") + cudaGetErrorString(pe));
+            return fail(nullptr, LBM_ERR_CUDA, std::string("streams and events: ") + cudaGetErrorString(pe));
         }
     }
     ctx->g.n[0] = g->nx; ctx->g.n[1] = g->ny; ctx->g.n[2] = g->nz;
@@ -327,7 +333,7 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
     Sizes s = compute_sizes(g, max_particles);
     Layout L;
     build_layout(g, st, max_particles, L, s);
-    ctx->bytes = L.total;
+    ctx->bytes = L.state;
     if (arena) {
         if (reinterpret_cast<uintptr_t>(arena) % 256 != 0) {
             destroy_handles(ctx);
@@ -374,6 +380,8 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
     ctx->accel_f = (float*)at(45);
     ctx->P.xf = (float*)at(46);
     ctx->miss_list = (unsigned int*)at(47);
+    ctx->solid = (uint32_t*)at(62);
+    ctx->shell = (uint32_t*)at(63);
     ctx->miss_cap = (int)s.ncells;
     ctx->P.acc_k = (long long*)at(49);
     ctx->P.xs[1] = (double*)at(50);
@@ -431,7 +439,7 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
     // the wall-adjacent cells need the NEAR flag even without particles
     MapParams mp{};
     mp.g = ctx->g; mp.P = ctx->P; mp.flags = ctx->flags; mp.owner = ctx->owner;
-    mp.pdf[0] = ctx->f[0]; mp.pdf[1] = ctx->f[1]; mp.elem = (int)ctx->elem;
+    mp.solid = ctx->solid; mp.shell = ctx->shell;
     for (int a = 0; a < 3; ++a) mp.ntile[a] = ctx->ntile[a];
     mp.tile_count = ctx->tile_count; mp.tile_list = ctx->tile_list;
     mp.shell_width = ctx->relax.shell_width;
@@ -463,7 +471,7 @@ MapParams map_params(lbm_ctx* ctx) {
     for (int a = 0; a < 3; ++a)
         mp.small[a] = ctx->g.per[a] && ctx->g.n[a] <= 2.0 * reach + ts[a] + 2.0;
     mp.g = ctx->g; mp.P = ctx->P; mp.flags = ctx->flags; mp.owner = ctx->owner;
-    mp.pdf[0] = ctx->f[0]; mp.pdf[1] = ctx->f[1]; mp.elem = (int)ctx->elem;
+    mp.solid = ctx->solid; mp.shell = ctx->shell;
     for (int a = 0; a < 3; ++a) mp.ntile[a] = ctx->ntile[a];
     mp.tile_count = ctx->tile_count; mp.tile_list = ctx->tile_list;
     mp.shell_width = ctx->relax.shell_width;
@@ -570,8 +578,6 @@ lbm_status check_status(lbm_ctx* ctx) {
         return fail(ctx, LBM_ERR_CAPACITY, buf);
     }
     if (st & ST_FAST_PARTICLE) return fail(ctx, LBM_ERR_UNSTABLE, "particle speed above 0.5 cells per step");
-    if (st & ST_TIMEOUT)
-        return fail(ctx, LBM_ERR_TIMEOUT, "a wait of the staged dense kernel on its copy pipeline ran out");
     return LBM_OK;
 }
 
@@ -809,6 +815,8 @@ void fill_step_params(const lbm_ctx* ctx, LbmStepParams& lp) {
     lp.src = ctx->f[ctx->cur];
     lp.dst = ctx->f[1 - ctx->cur];
     lp.flags = ctx->flags;
+    lp.solid = ctx->solid;
+    lp.shell = ctx->shell;
     lp.owner = ctx->owner;
     lp.g = ctx->g;
     lp.s_plus = s_nu;
@@ -824,11 +832,15 @@ void fill_step_params(const lbm_ctx* ctx, LbmStepParams& lp) {
     lp.counterforce = d.fluid_counterforce && ctx->P.n > 0;
     lp.P = ctx->P;
     lp.missing_links = d.missing_links && ctx->P.n > 0;
+    // float32 path: their constant parts stand in for those of the fluid links
+    lp.other_links = (d.missing_links || ctx->storage != LBM_STORE_F64) && ctx->P.n > 0;
     lp.status = ctx->status;
     lp.miss_list = ctx->miss_list;
     lp.miss_count = ctx->miss_count;
     lp.miss_cap = ctx->miss_cap;
     lp.num_sms = ctx->num_sms;
+    // a link cell lies within R + 2 cells of its particle's base cell on every axis
+    lp.margin = (int)std::ceil(ctx->r_max) + 3;
     lp.accel_d = ctx->accel;
     lp.accel_f = ctx->accel_f;
 }
@@ -870,12 +882,12 @@ lbm_status enqueue_pre(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepState& 
     // sums commute with the dense kernel's) and the DEM's neighbour lists,
     // which read only the positions the dense kernel reads too; finalize
     // waits for both streams
-    const bool side = lp.missing_links || dem;
+    const bool side = lp.other_links || dem;
     ss.side = side;
     if (side) {
         CK(cudaEventRecord(ctx->ev_fork, sm));
         CK(cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0));
-        if (lp.missing_links) {
+        if (lp.other_links) {
             launch_boundary(lp, ctx->side_stream, BC_LINKS);
             ctx->launches += 1;
         }
@@ -1246,6 +1258,10 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* buf, size_t bytes) {
     ctx->hx.assign(hd, hd + 3 * (size_t)h.np);
     ctx->hR.assign(hd + 3 * mp, hd + 3 * mp + (size_t)h.np);
     reset_graphs(ctx);
+    launch_cell_bits(map_params(ctx), ctx->stream);
+    ctx->launches += 1;
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(ctx->stream));
     return LBM_OK;
 }
 
@@ -1346,8 +1362,11 @@ lbm_status lbm_get_pdfs(lbm_ctx* ctx, double* f) {
     if (!ctx || !f) return fail(ctx, LBM_ERR_INVALID, "NULL argument");
     const size_t N = (size_t)ctx->g.ncells;
     std::vector<char> raw(19 * N * ctx->elem);
+    std::vector<uint8_t> flags(N);
     CK(cudaMemcpyAsync(raw.data(), ctx->f[ctx->cur], raw.size(), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(flags.data(), ctx->flags, N, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    const double nan = std::nan("");
     for (int q = 0; q < 19; ++q) {
         const double w = w_of(q);
         for (size_t k = 0; k < N; ++k) {
@@ -1359,7 +1378,7 @@ lbm_status lbm_get_pdfs(lbm_ctx* ctx, double* f) {
                 case LBM_STORE_F16: v = __half2float(reinterpret_cast<const __half*>(raw.data())[j]); break;
                 default: v = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(raw.data())[j]); break;
             }
-            f[j] = v + w;
+            f[j] = flags[k] & FL_SOLID ? nan : v + w;
         }
     }
     return LBM_OK;
@@ -1383,10 +1402,6 @@ lbm_status lbm_set_pdfs(lbm_ctx* ctx, const double* f) {
         }
     }
     CK(cudaMemcpyAsync(ctx->f[ctx->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice, ctx->stream));
-    // solid cells keep their NaN marker whatever was uploaded for them
-    launch_solid_markers(map_params(ctx), ctx->stream);
-    ctx->launches += 1;
-    CK(cudaGetLastError());
     CK(cudaStreamSynchronize(ctx->stream));
     return LBM_OK;
 }
@@ -1511,7 +1526,7 @@ std::vector<int4> batch_items(const lbm_batch* b) {
     for (size_t i = 0; i < b->ctx.size(); ++i) {
         if (!b->active[i]) continue;
         const Geom& g = b->ctx[i]->g;
-        const int bx = batch_tile_bx(b, (int)i), by = 256 / bx, zc = batch_zchunk(b, (int)i);
+        const int bx = batch_tile_bx(b, (int)i), by = sc_tile_rows((int)b->ctx[i]->elem, bx), zc = batch_zchunk(b, (int)i);
         for (int z0 = 0; z0 < g.n[2]; z0 += zc)
             for (int y0 = 0; y0 < g.n[1]; y0 += by)
                 for (int x0 = 0; x0 < g.n[0]; x0 += bx) per[i].push_back(make_int4((int)i, x0, y0, z0));
@@ -1584,7 +1599,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
         fill_bc_args(lp, bca.data());
         // the missing-link and refill lists grow with the particle count
         const int list_blocks = std::min(8 * b->num_sms, 1 + np / 8);
-        bc.add(bca.data(), lp.missing_links ? list_blocks : 1);
+        bc.add(bca.data(), lp.other_links ? list_blocks : 1);
         fill_batch_args(lp, batch_tile_bx(b, (int)i), batch_zchunk(b, (int)i), &host[ab * i]);
         DemParams dp = dem_params(c);
         if (dem) {

@@ -14,8 +14,7 @@
 // on the float64 path).
 //
 // The particle links themselves (CLI condition of Eq. (14), momentum exchange
-// of Eq. (15)) are handled inside the dense stream/collide kernel, which finds
-// them from the marker that solid cells hold in their PDF slots.
+// of Eq. (15)) are handled inside the dense stream/collide kernel.
 #include <cstring>
 
 #include "common.cuh"
@@ -41,7 +40,8 @@ struct BcArgs {
     double* acc_d;
     long long* acc_i;
     long long* acc_k;
-    int missing_links;
+    int missing_links;   // the correction is on
+    int other_links;     // the list is walked (float32 path: also without the correction)
     int* status;
     // fluid body force of the step: a_user - ext_total / N_fluid (counter force)
     double a_user[3];
@@ -52,8 +52,18 @@ struct BcArgs {
     float* accel_f;
 };
 
-// missing links of a solid cell s of particle i: links x -> s from cells x of
-// another body whose centre is not inside sphere i
+// Links x -> s into a solid cell s of particle i from cells x of another body.
+// Those whose centre is not inside sphere i are missing links: F = 2 w_q c_q
+// with its torque.
+//
+// Float32 path: the dense kernel leaves the constant part 2 w c of every fluid
+// link out. Over all links of the particle's cells to cells outside them the
+// constant parts and their torques cancel (a lattice line enters and leaves the
+// set with opposite c and the same n x c), so those of the fluid links are minus
+// those of the other links: a missing link then adds its term and takes it
+// away again, and what is left are minus the other links that are no missing
+// links (x inside sphere i, where spheres overlap) or, with the correction
+// off, minus all of them. All terms are integers (x 36).
 template <typename S, typename T>
 __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx, Acc<T>& acc, const Sinks& sk) {
     const int nx = a.g.n[0], ny = a.g.n[1];
@@ -61,6 +71,9 @@ __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx,
     const int x = (int)(idx % nx), y = (int)((idx / nx) % ny), z = (int)(idx / plane);
     const int cpos[3] = {x, y, z};
     const int i = a.owner[idx];
+    // float32 path with the correction on: only cells behind a wall or inside
+    // two spheres can be inside sphere i
+    const bool overlaps_only = sizeof(T) == 4 && a.missing_links;
     unsigned cand = 0, solidm = 0;
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
@@ -72,8 +85,12 @@ __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx,
             if (!a.g.per[d] && (v[d] < 0 || v[d] >= a.g.n[d])) outside = true;
             v[d] = wrap_idx(v[d], a.g.n[d]);
         }
-        if (outside) cand |= 1u << q;
-        else if (a.flags[(long long)v[2] * plane + (long long)v[1] * nx + v[0]] & FL_SOLID) solidm |= 1u << q;
+        if (outside) {
+            cand |= 1u << q;
+        } else {
+            const uint8_t f = a.flags[(long long)v[2] * plane + (long long)v[1] * nx + v[0]];
+            if (overlaps_only ? (f & FL_MULTI) : (f & FL_SOLID)) solidm |= 1u << q;
+        }
     }
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
@@ -93,7 +110,8 @@ __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx,
             dd[d] = min_image_d(((double)(cpos[d] - c[d]) + 0.5) - a.px[3 * i + d], a.g.n[d], a.g.per[d]);
         const double Ri = a.pR[i];
         const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dd[0], dd[0]), __dmul_rn(dd[1], dd[1])), __dmul_rn(dd[2], dd[2]));
-        if (!(d2 > __dmul_rn(Ri, Ri))) continue;
+        const bool missing = a.missing_links && d2 > __dmul_rn(Ri, Ri);
+        if (sizeof(T) == 4 ? missing : !missing) continue;
         T r[3], R, u[3], om[3];
         int n[3];
         PartOps<T>::load(a, i, x - c[0], y - c[1], z - c[2], r, n, R, u, om);
@@ -101,8 +119,8 @@ __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx,
         int K[6] = {0, 0, 0, 0, 0, 0};
         T F[3] = {T(0), T(0), T(0)}, Tq[3] = {T(0), T(0), T(0)};
         if (sizeof(T) == 4) {
-            // F = 2 w_q c_q and torque 2 w_q (r x c_q), r = n + g: exact integers (x 36)
-            const int kw = cc2 == 1 ? 4 : 2;
+            // minus 2 w_q c_q and 2 w_q (r x c_q), r = n + g (g common to all links)
+            const int kw = cc2 == 1 ? -4 : -2;
             K[0] = kw * c[0]; K[1] = kw * c[1]; K[2] = kw * c[2];
             K[3] = kw * (n[1] * c[2] - n[2] * c[1]);
             K[4] = kw * (n[2] * c[0] - n[0] * c[2]);
@@ -139,7 +157,7 @@ __device__ __forceinline__ void boundary_body(const BcArgs<S>& a, int mode, int 
             a.accel_f[d] = (float)acc3[d];
         }
     }
-    if (!(mode & BC_LINKS) || !a.missing_links) return;
+    if (!(mode & BC_LINKS) || !a.other_links) return;
     const Sinks sk{a.acc_d, a.acc_i, a.acc_k, a.status};
     const int mcount = min(*a.miss_count, a.miss_cap);
     const int stride = (int)(gx * blockDim.x);
@@ -182,6 +200,7 @@ void fill_bc_args_t(const LbmStepParams& p, BcArgs<S>& b) {
     b.acc_i = p.P.acc_i;
     b.acc_k = p.P.acc_k;
     b.missing_links = p.missing_links;
+    b.other_links = p.other_links;
     b.status = p.status;
     for (int d = 0; d < 3; ++d) {
         b.a_user[d] = p.a_user[d];
@@ -197,7 +216,7 @@ template <typename S>
 void launch_boundary_t(const LbmStepParams& p, cudaStream_t st, int mode) {
     BcArgs<S> b;
     fill_bc_args_t<S>(p, b);
-    const int blocks = (mode & BC_LINKS) && p.missing_links ? 8 * (p.num_sms > 0 ? p.num_sms : 1) : 1;
+    const int blocks = (mode & BC_LINKS) && p.other_links ? 8 * (p.num_sms > 0 ? p.num_sms : 1) : 1;
     boundary_kernel<S><<<blocks, 128, 0, st>>>(b, mode);
 }
 

@@ -12,6 +12,8 @@ struct LbmStepParams {
     const void* src;
     void* dst;
     const uint8_t* flags;
+    const uint32_t* solid;           // one bit per cell (x in the bits of a row's words): solid,
+    const uint32_t* shell;           // in the TRT+aB shell
     const int* owner;                // particle of a solid cell, -1 for fluid
     Geom g;
     double s_plus, s_minus, s_b_shell, s_b_bulk;
@@ -21,25 +23,24 @@ struct LbmStepParams {
     const unsigned long long* n_solid;
     int counterforce;
     Particles P;
-    int missing_links;
+    int missing_links;               // the missing-link correction is on
+    int other_links;                 // the missing-link list is walked
     int* status;
     const unsigned int* miss_list;   // solid cells with possible missing links
     const int* miss_count;
     int miss_cap;
+    int margin;                      // cells from a periodic face within which particle images matter
     int num_sms;                     // multiprocessors of the device (grid sizing)
     double* accel_d;                 // out: fluid body force of the step [3]
     float* accel_f;
-    int use_staged;                  // 1: the dense kernel with bulk-copy staging where it applies
-    int tile_bx;                     // x extent of the dense kernel's tile (0: automatic)
-    int zchunk;                      // z planes per block of the dense kernel (0: automatic)
-    int staged_zchunk;               // z planes per work item of the staged kernel (0: automatic)
 };
 // BC_ACCEL: the fluid body force of the step; BC_LINKS: the missing links
 constexpr int BC_ACCEL = 1, BC_LINKS = 2;
 void launch_boundary(const LbmStepParams& p, cudaStream_t st, int mode);
 void launch_stream_collide(const LbmStepParams& p, cudaStream_t st);
-// kernel attributes on the current device (before any launch or capture)
-cudaError_t prepare_stream_collide(int storage);
+// rows in y of the dense kernel's tile bx (32, 64 or 128) cells wide: 4 warps
+// of 32 x 2 cells (elem: bytes of a stored PDF), 32 x 1 for float64
+__host__ __device__ constexpr int sc_tile_rows(int elem, int bx) { return (elem == 8 ? 1 : 2) * 128 / bx; }
 // the dense kernels of many boxes in one persistent launch: per instance one
 // argument block (batch_args_bytes(storage) bytes, filled by fill_batch_args)
 // in device memory, and a table of work items (instance, x0, y0, z0)
@@ -48,18 +49,14 @@ void fill_batch_args(const LbmStepParams& p, int tile_bx, int zchunk, void* out)
 int default_tile_bx(int nx);
 void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, int grid,
                                  cudaStream_t st);
-// the dense kernel with bulk-copy staging of the pulls (4- and 2-byte formats)
-bool staged_applicable(const LbmStepParams& p);
-void launch_stream_collide_staged(const LbmStepParams& p, cudaStream_t st);
-cudaError_t prepare_stream_collide_staged(int storage);
 
 struct MapParams {
     Geom g;
     Particles P;
     uint8_t* flags;
     int* owner;
-    void* pdf[2];           // both PDF buffers (NaN markers into cells that turn solid), or NULL
-    int elem;               // bytes per stored PDF value (8, 4 or 2)
+    uint32_t* solid;        // one bit per cell: solid, in the shell (both or neither NULL)
+    uint32_t* shell;
     int ntile[3];
     int* tile_count;
     int* tile_list;
@@ -77,8 +74,8 @@ struct MapParams {
 };
 void launch_tile_scatter(const MapParams& p, cudaStream_t st);
 void launch_map(const MapParams& p, cudaStream_t st);
-// NaN markers into every PDF slot of every solid cell of both buffers
-void launch_solid_markers(const MapParams& p, cudaStream_t st);
+// the bits per cell from the flags (after a restore)
+void launch_cell_bits(const MapParams& p, cudaStream_t st);
 
 struct RefillParams {
     int storage;

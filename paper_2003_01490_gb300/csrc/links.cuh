@@ -95,6 +95,105 @@ __device__ __forceinline__ void commit(Acc<T>& a, const Sinks& s) {
     }
 }
 
+// Sums of one force and torque per lane over the warp, added to particle key: a
+// butterfly that halves the values each lane carries while it halves the lanes
+// (9 shuffles for 6 sums); the sums end in one lane each, which adds it.
+template <typename T>
+__device__ __forceinline__ void commit_warp(int key, const T (&v)[6], const Sinks& s, int lane) {
+    const unsigned full = 0xffffffffu;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    T t[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) t[c] = (h16 ? v[3 + c] : v[c]) + __shfl_xor_sync(full, h16 ? v[c] : v[3 + c], 16);
+    const T a = (h8 ? t[1] : t[0]) + __shfl_xor_sync(full, h8 ? t[0] : t[1], 8);
+    t[2] += __shfl_xor_sync(full, t[2], 8);
+    T b = (h4 ? t[2] : a) + __shfl_xor_sync(full, h4 ? a : t[2], 4);
+    b += __shfl_xor_sync(full, b, 2);
+    b += __shfl_xor_sync(full, b, 1);
+    if ((lane & 3) == 0 && !(h4 && h8)) add_float(s, key, (h16 ? 3 : 0) + (h4 ? 2 : (h8 ? 1 : 0)), b);
+}
+
+// The open particles of one warp: a few particles, each with its view
+// (float32 path) and, per lane, six partial force sums in shared memory
+// (lane-private, no conflicts). Links of a particle with a slot read the view
+// from there and cost a read-add-write; a further particle takes the place of
+// one that none of the present links needs, whose sums are committed. A warp
+// marching in z meets the same few spheres plane after plane.
+template <typename T>
+struct OpenParts {
+    static constexpr int SLOTS = sizeof(T) == 4 ? 4 : 3;
+    T f[SLOTS][6][32];
+    PartView view[sizeof(T) == 4 ? SLOTS : 1];
+};
+template <typename T>
+struct SlotKeys {
+    int k[OpenParts<T>::SLOTS];
+    int next;
+};
+
+template <typename T>
+__device__ __forceinline__ void commit_slot(OpenParts<T>& op, int slot, int key, const Sinks& s, int lane) {
+    T v[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) v[c] = op.f[slot][c][lane];
+    commit_warp<T>(key, v, s, lane);
+}
+
+// The slot of each lane's particle (key >= 0), opening slots for new ones.
+// Lanes whose particle finds no free slot (more particles than slots in the warp)
+// get -1 and have to come again. All lanes of the warp take part.
+template <typename T>
+__device__ __forceinline__ int find_slot(OpenParts<T>& op, SlotKeys<T>& sk, int key, const PartView* __restrict__ view,
+                                         const Sinks& s, int lane) {
+    constexpr int SUM_SLOTS = OpenParts<T>::SLOTS;
+    const unsigned full = 0xffffffffu;
+    int slot = -1;
+#pragma unroll
+    for (int j = 0; j < SUM_SLOTS; ++j)
+        if (key == sk.k[j]) slot = j;
+    if (key < 0) slot = -1;
+    unsigned miss = __ballot_sync(full, key >= 0 && slot < 0);
+    if (miss == 0u) return slot;
+    unsigned used = __reduce_or_sync(full, slot >= 0 ? 1u << slot : 0u);
+    while (miss && used != (1u << SUM_SLOTS) - 1u) {   // warp-uniform
+        const int kn = __shfl_sync(full, key, __ffs(miss) - 1);
+        const bool mine = key == kn;
+        miss &= ~__ballot_sync(full, mine);
+        int v = sk.next;
+        while ((used >> v) & 1u) v = (v + 1) % SUM_SLOTS;
+        sk.next = (v + 1) % SUM_SLOTS;
+        used |= 1u << v;
+        int old = -1;
+#pragma unroll
+        for (int j = 0; j < SUM_SLOTS; ++j)
+            if (j == v) {
+                old = sk.k[j];
+                sk.k[j] = kn;
+            }
+        if (old >= 0) commit_slot<T>(op, v, old, s, lane);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) op.f[v][c][lane] = T(0);
+        if (sizeof(T) == 4 && lane < (int)(sizeof(PartView) / 4))
+            reinterpret_cast<int*>(&op.view[v])[lane] = reinterpret_cast<const int*>(view + kn)[lane];
+        if (mine) slot = v;
+    }
+    __syncwarp();   // views written
+    return slot;
+}
+
+template <typename T>
+__device__ __forceinline__ void commit_open(OpenParts<T>& op, const SlotKeys<T>& sk, const Sinks& s, int lane) {
+    constexpr int SUM_SLOTS = OpenParts<T>::SLOTS;
+#pragma unroll 1
+    for (int j = 0; j < SUM_SLOTS; ++j) {
+        int key = -1;
+#pragma unroll
+        for (int i = 0; i < SUM_SLOTS; ++i)
+            if (i == j) key = sk.k[i];
+        if (key >= 0) commit_slot<T>(op, j, key, s, lane);   // warp-uniform
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ void accumulate(int i, const T (&F)[3], const T (&Tq)[3], const int (&K)[6], Acc<T>& a,
                                            const Sinks& s) {

@@ -14,8 +14,9 @@
 // refill list with their former particle. Fluid cells within R + sqrt(2) of a
 // particle get the NEAR flag; solid cells next to another body (candidates for
 // missing links) go to the missing-link list that the boundary kernel of the
-// next step reads. A cell that turns solid gets the NaN marker in all its PDF
-// slots of both buffers.
+// next step reads. The solid and shell cells are also written as one bit per
+// cell (a tile row of 32 cells is one word), from which the dense kernel finds
+// the particle links.
 #include <type_traits>
 
 #include "common.cuh"
@@ -123,22 +124,6 @@ void launch_tile_scatter(const MapParams& p, cudaStream_t st) {
 
 // ------------------------------------------------------------ mapping
 
-// The NaN marker of a solid cell (owner + 1 in the payload of the 4- and
-// 8-byte formats) into all its PDF slots of both buffers; the dense kernel
-// finds particle links and their particle by it.
-__device__ __forceinline__ void put_markers(void* const (&pdf)[2], int elem, long long ncells, long long idx,
-                                            int owner) {
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        for (int q = 0; q < Q; ++q) {
-            const long long k = (long long)q * ncells + idx;
-            if (elem == 8) reinterpret_cast<unsigned long long*>(pdf[b])[k] = marker_bits64(owner);
-            else if (elem == 4) reinterpret_cast<unsigned int*>(pdf[b])[k] = marker_bits32(owner);
-            else reinterpret_cast<unsigned short*>(pdf[b])[k] = (unsigned short)0x7fff;
-        }
-    }
-}
-
 // Exact float64 decision of the solid and shell tests for a cell centre whose
 // float32 distance lies within the tolerance of a threshold (kept out of line:
 // it runs for a tiny fraction of the tests). Returns bit 0 inside, bit 1 shell.
@@ -183,6 +168,7 @@ __device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int
     __shared__ unsigned int s_cnt[4];          // per warp: missing-link cells
     __shared__ unsigned int s_solid[4];
     __shared__ unsigned int s_base;
+    __shared__ unsigned char s_bits[2][TILE_Z * TILE_Y * 4];   // solid, shell: byte w of row (z, y) from warp w
     const long long t = ((long long)bz * p.ntile[1] + by) * p.ntile[0] + bx;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int lx = 8 * warp + (lane & 7), ly = lane >> 3;
@@ -313,7 +299,7 @@ __device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int
     bool wall_xy = false;
     if (!p.g.per[0] && (x == 0 || x == nx - 1)) wall_xy = true;
     if (!p.g.per[1] && (y == 0 || y == ny - 1)) wall_xy = true;
-    unsigned miss_bits = 0, solid_bits = 0;
+    unsigned miss_bits = 0, solid_bits = 0, shell_bits = 0;
 #pragma unroll
     for (int j = 0; j < TILE_Z; ++j) {
         const int z = org[2] + j;
@@ -330,16 +316,13 @@ __device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int
                 nf |= FL_MISS;
                 miss_bits |= 1u << j;
             }
-            // new solid cells get markers; the particle of a solid cell can only
-            // change where spheres overlap (now or at the last mapping), so
-            // those cells get them again
-            const bool multi = (multi4 >> j) & 1u;
-            if (multi) nf |= FL_MULTI;
+            if ((multi4 >> j) & 1u) nf |= FL_MULTI;
             p.owner[idx] = own[j];
-            if ((!(old & FL_SOLID) || multi || (old & FL_MULTI)) && p.pdf[0])
-                put_markers(p.pdf, p.elem, p.g.ncells, idx, own[j]);
         } else {
-            if (shell4 & (1u << j)) nf |= FL_SHELL;
+            if (shell4 & (1u << j)) {
+                nf |= FL_SHELL;
+                shell_bits |= 1u << j;
+            }
             if (nn >= 1u) nf |= FL_NEAR;
             if (old & FL_SOLID) {
                 // uncovered this step: refill with the former particle's velocity
@@ -367,7 +350,14 @@ __device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int
     for (int j = 0; j < TILE_Z; ++j) {
         mb[j] = __ballot_sync(FULL, (miss_bits >> j) & 1u);
         wm += __popc(mb[j]);
-        ws += __popc(__ballot_sync(FULL, (solid_bits >> j) & 1u));
+        const unsigned sb = __ballot_sync(FULL, (solid_bits >> j) & 1u);
+        const unsigned hb = __ballot_sync(FULL, (shell_bits >> j) & 1u);
+        ws += __popc(sb);
+        // lane l is column x = 8 warp + (l & 7), y = l >> 3: byte y of a ballot
+        if (lane < TILE_Y) {
+            s_bits[0][(j * TILE_Y + lane) * 4 + warp] = (unsigned char)(sb >> (8 * lane));
+            s_bits[1][(j * TILE_Y + lane) * 4 + warp] = (unsigned char)(hb >> (8 * lane));
+        }
     }
     if (lane == 0) {
         s_cnt[warp] = wm;
@@ -385,6 +375,15 @@ __device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int
         }
         s_base = tm ? (unsigned)atomicAdd(p.miss_count, (int)tm) : 0u;
         if (tsol) atomicAdd(p.n_solid, tsol);
+    }
+    if (p.solid && tid >= 32 && tid < 32 + 2 * TILE_Z * TILE_Y) {
+        const int k = tid - 32, kind = k / (TILE_Z * TILE_Y), row = k % (TILE_Z * TILE_Y);
+        const int yy = org[1] + row % TILE_Y, zz = org[2] + row / TILE_Y;
+        if (yy < ny && zz < nz) {
+            const unsigned char* b = s_bits[kind] + 4 * row;
+            const uint32_t word = b[0] | (uint32_t)b[1] << 8 | (uint32_t)b[2] << 16 | (uint32_t)b[3] << 24;
+            (kind ? p.shell : p.solid)[((long long)zz * ny + yy) * p.ntile[0] + bx] = word;
+        }
     }
     __syncthreads();
     if (miss_bits) {
@@ -421,15 +420,28 @@ void launch_map(const MapParams& p, cudaStream_t st) {
     map_kernel<<<grid, TILE_X * TILE_Y, 0, st>>>(p);
 }
 
-__global__ void solid_markers_kernel(const __grid_constant__ MapParams p) {
+// one thread per word of 32 cells
+__global__ void cell_bits_kernel(const __grid_constant__ MapParams p) {
+    const int nx = p.g.n[0], W = p.ntile[0];
+    const long long words = (long long)W * p.g.n[1] * p.g.n[2];
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < p.g.ncells; idx += stride)
-        if (p.flags[idx] & FL_SOLID) put_markers(p.pdf, p.elem, p.g.ncells, idx, p.owner[idx]);
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < words; k += stride) {
+        const long long row = k / W;
+        const int x0 = (int)(k % W) * 32;
+        uint32_t so = 0, sh = 0;
+        for (int b = 0; b < 32 && x0 + b < nx; ++b) {
+            const uint8_t f = p.flags[row * nx + x0 + b];
+            so |= (uint32_t)((f & FL_SOLID) != 0) << b;
+            sh |= (uint32_t)((f & FL_SHELL) != 0) << b;
+        }
+        p.solid[k] = so;
+        p.shell[k] = sh;
+    }
 }
 
-void launch_solid_markers(const MapParams& p, cudaStream_t st) {
-    if (!p.pdf[0]) return;
-    solid_markers_kernel<<<152 * 8, 256, 0, st>>>(p);
+void launch_cell_bits(const MapParams& p, cudaStream_t st) {
+    static_assert(TILE_X == 32, "a tile row is one word");
+    cell_bits_kernel<<<152 * 8, 128, 0, st>>>(p);
 }
 
 // ------------------------------------------------------------ refill

@@ -1,8 +1,7 @@
-// sc_common.cuh -- arithmetic shared by the dense stream/collide kernels:
-// the CLI moving no-slip value of one particle link with its momentum-exchange
-// force and torque (Eqs. (14)-(17)), and the TRT(+aB) collision with Guo
-// forcing of one fluid cell and the store of its PDFs (Eqs. (5), (10)-(12),
-// Sec. 2.3.2). See stream_collide.cu for the data layout.
+// sc_common.cuh -- arithmetic of the dense stream/collide kernel: the CLI
+// moving no-slip value of one particle link with its momentum-exchange force
+// and torque (Eqs. (14)-(17)), and the TRT(+aB) collision with Guo forcing
+// (Eqs. (5), (10)-(12), Sec. 2.3.2). See stream_collide.cu for the data layout.
 #pragma once
 
 #include "common.cuh"
@@ -11,21 +10,90 @@
 
 namespace lbmdem {
 
+// Two float32 values in one 64-bit register pair: one packed instruction
+// (add, sub, mul, fma .f32x2, each rounded like its scalar form) works on
+// both, which halves the instructions of the collision.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void split(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// a product that is rounded before it is added (the packed form is merged with
+// a following addition, which changes the collision's rounding)
+__device__ __forceinline__ F2 mul_rn(F2 a, F2 b) {
+    float a0, a1, b0, b1;
+    split(a, a0, a1);
+    split(b, b0, b1);
+    return f2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ double mul_rn(double a, double b) { return a * b; }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+
+// the cells a thread collides together: V holds ROWS values of type T
+template <typename T> struct Pack;
+template <> struct Pack<float> {
+    using V = F2;
+    static constexpr int ROWS = 2;
+    __device__ static V all(float a) { return f2(a, a); }
+    __device__ static V make(const float (&a)[2]) { return f2(a[0], a[1]); }
+    __device__ static void get(V v, float (&a)[2]) { split(v, a[0], a[1]); }
+};
+template <> struct Pack<double> {
+    using V = double;
+    static constexpr int ROWS = 1;
+    __device__ static V all(double a) { return a; }
+    __device__ static V make(const double (&a)[1]) { return a[0]; }
+    __device__ static void get(V v, double (&a)[1]) { a[0] = v; }
+};
+
 template <typename S, typename T>
 struct SCArgs {
-    const S* __restrict__ src;
-    S* __restrict__ dst;
-    const uint8_t* __restrict__ flags;
+    // the arrays of each direction: their addresses come from the argument
+    // block, so a load costs one 32-bit index and one multiply-add
+    const S* src[Q];
+    S* dst[Q];
     Geom g;
+    // one bit per cell, x in the bits of a row's words (bits past nx are 0)
+    const uint32_t* __restrict__ solid;
+    const uint32_t* __restrict__ shell;
+    int words;                       // 32-bit words per row
     T s_plus, s_minus, s_b_shell, s_b_bulk;
+    T ke, ko;                        // weights of the body force in the equilibrium (collide_core)
     T uw[2][3][3];                   // wall velocities [side][axis][component]
     int bulk_corr;
     const T* __restrict__ accel;     // [3]
     int* status;
     int zchunk;                      // z planes per block
-    int bx;                          // x extent of a block's tile (a multiple of 32; 256 / bx rows)
+    int bx;                          // x extent of a block's tile (32, 64 or 128)
     // particles (for the links)
     int np;
+    int margin;                      // cells from a periodic face within which images matter
     const int* __restrict__ owner;   // particle of a solid cell, -1 for fluid
     const double* __restrict__ px;
     const double* __restrict__ pu;
@@ -34,20 +102,25 @@ struct SCArgs {
     const PartView* __restrict__ view;
     double* acc_d;
     long long* acc_i;
-    long long* acc_k;
 };
 
 // kernel arguments from the step parameters
 template <typename S, typename T>
 void fill_sc_args(const LbmStepParams& p, SCArgs<S, T>& a) {
-    a.src = static_cast<const S*>(p.src);
-    a.dst = static_cast<S*>(p.dst);
-    a.flags = p.flags;
+    for (int q = 0; q < Q; ++q) {
+        a.src[q] = static_cast<const S*>(p.src) + q * p.g.ncells;
+        a.dst[q] = static_cast<S*>(p.dst) + q * p.g.ncells;
+    }
     a.g = p.g;
+    a.solid = p.solid;
+    a.shell = p.shell;
+    a.words = (p.g.n[0] + 31) / 32;
     a.s_plus = (T)p.s_plus;
     a.s_minus = (T)p.s_minus;
     a.s_b_shell = (T)p.s_b_shell;
     a.s_b_bulk = (T)p.s_b_bulk;
+    a.ke = (T)((2.0 - p.s_plus) / p.s_plus);
+    a.ko = (T)((1.0 - 0.5 * p.s_minus) / p.s_minus);
     for (int s = 0; s < 2; ++s)
         for (int ax = 0; ax < 3; ++ax)
             for (int c = 0; c < 3; ++c) a.uw[s][ax][c] = (T)p.g.wall_vel[s][ax][c];
@@ -57,6 +130,7 @@ void fill_sc_args(const LbmStepParams& p, SCArgs<S, T>& a) {
     a.zchunk = 0;
     a.bx = 128;
     a.np = p.P.n;
+    a.margin = p.margin;
     a.owner = p.owner;
     a.px = p.P.x;
     a.pu = p.P.u;
@@ -65,149 +139,177 @@ void fill_sc_args(const LbmStepParams& p, SCArgs<S, T>& a) {
     a.view = p.P.view;
     a.acc_d = p.P.acc_d;
     a.acc_i = p.P.acc_i;
-    a.acc_k = p.P.acc_k;
 }
 
-// NaN marker of a solid cell of particle owner, and a plain NaN
-template <typename T>
-__device__ __forceinline__ T solid_marker(int owner);
-template <> __device__ __forceinline__ float solid_marker<float>(int owner) { return __uint_as_float(marker_bits32(owner)); }
-template <> __device__ __forceinline__ double solid_marker<double>(int owner) {
-    return __longlong_as_double((long long)marker_bits64(owner));
-}
-template <typename T>
-__device__ __forceinline__ T plain_nan() { return solid_marker<T>(MARKER_PAYLOAD - 1); }
-
-// CLI value f_q(x, t+1) of the link of fluid cell (x, y, z) in pull direction
-// q into the solid cell x - c_q, and its force and torque into acc (float32
-// path: the remainder part in floats, the constant part as exact integers)
 // per-direction word of the link code: c_q + 1 in bits 0-1, 2-3, 4-5, the
 // opposite direction in bits 6-10 (read from shared memory: a warp's lanes
 // hold different directions)
 __host__ __device__ constexpr int qinfo(int q) { return (cx(q) + 1) | ((cy(q) + 1) << 2) | ((cz(q) + 1) << 4) | (opp(q) << 6); }
 
-template <typename S, typename T>
-__device__ __forceinline__ T link_value(const SCArgs<S, T>& a, int x, int y, int z, int q, int qi, int key1,
-                                        unsigned lm_src, T fdown_raw, Acc<T>& acc, const Sinks& sk) {
-    const int nx = a.g.n[0], ny = a.g.n[1];
-    const int plane = nx * ny;
-    const long long N = a.g.ncells;
-    const int c[3] = {(qi & 3) - 1, ((qi >> 2) & 3) - 1, ((qi >> 4) & 3) - 1};
-    const int p = (qi >> 6) & 31;
-    const int idx = z * plane + y * nx + x;
-    // the particle from the marker's payload (the owner array for 16-bit storage)
-    int i = key1 - 1;
-    if (key1 <= 0) {
-        const int uv[3] = {wrap_idx(x - c[0], nx), wrap_idx(y - c[1], ny), wrap_idx(z - c[2], a.g.n[2])};
-        i = a.owner[uv[2] * plane + uv[1] * nx + uv[0]];
-    }
-    if (i < 0 || i >= a.np) return plain_nan<T>();   // a NaN from a fluid cell: left for the stability check
-    const T fout = Store<S>::load(a.src + p * N + idx);
-    const T fin = Store<S>::load(a.src + q * N + idx);
-    // CLI needs x + c_q fluid and inside the box; its post-collision f_p is the
-    // cell's own pull in direction p (marker there: bounce-back coefficients)
-    bool cli = !((lm_src >> p) & 1u);
-    if (!a.g.per[0] && (x + c[0] < 0 || x + c[0] >= nx)) cli = false;
-    if (!a.g.per[1] && (y + c[1] < 0 || y + c[1] >= ny)) cli = false;
-    if (!a.g.per[2] && (z + c[2] < 0 || z + c[2] >= a.g.n[2])) cli = false;
-    const T fdown = cli ? fdown_raw : T(0);
-    T r[3], R, u[3], om[3];
+// link codes and (-c_q, |c_q|^2) of the directions, in shared memory
+template <typename S>
+struct DirTable {
+    float4 cf[Q];
+    const S* src[Q];
+    int qi[Q];
+    int dq[Q];   // cell index offset of c_q
+};
+
+// One particle link: cell (x, y, z) pulls direction q (velocity c) from a solid
+// cell of particle i. fout = f~_p(x), fin = f~_q(x), fdown = f~_p(x + c_q) (p
+// the opposite direction; cli: that cell is fluid and inside the box, else
+// bounce-back coefficients). Returns f_q(x, t+1) of Eq. (14) and the link's
+// force and torque (Eqs. (15)-(17)).
+template <typename S>
+__device__ __forceinline__ double link_value(const SCArgs<S, double>& a, int i, const PartView&, int x, int y, int z, int qi, float4,
+                                             bool cli, bool, double fout, double fin, double fdown, double (&F)[6]) {
+    double r[3], R, u[3], om[3];
     int n[3];
-    T cc;   // |r|^2 - R^2
-    if constexpr (sizeof(T) == 4) {
-        float g[3], C[2];
-        PartOps<T>::load(a, i, x, y, z, r, n, g, C, R, u, om);
-        cc = surface_cc_split(n, g, C);
-    } else {
-        PartOps<T>::load(a, i, x, y, z, r, n, R, u, om);
-        cc = surface_cc<T>(r, R);
-    }
-    const int cp[3] = {-c[0], -c[1], -c[2]};
-    const T cp0 = (T)cp[0], cp1 = (T)cp[1], cp2 = (T)cp[2];
+    const int c[3] = {(qi & 3) - 1, ((qi >> 2) & 3) - 1, ((qi >> 4) & 3) - 1};
+    PartOps<double>::load(a, i, x, y, z, r, n, R, u, om);
+    const double cp0 = -c[0], cp1 = -c[1], cp2 = -c[2];
     const int cc2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
-    const T w = cc2 == 1 ? T(1) / T(18) : T(1) / T(36);
-    const T delta = link_root<T>(r, cc, cp0, cp1, cp2, (T)cc2);
-    const T dbc = cli ? delta : T(0.5);
-    const T inv = fast_div(T(1), T(1) + T(2) * dbc);
-    const T kappa = (T(1) - T(2) * dbc) * inv;
-    const T rb[3] = {r[0] + delta * cp0, r[1] + delta * cp1, r[2] + delta * cp2};
-    const T ub[3] = {u[0] + (om[1] * rb[2] - om[2] * rb[1]), u[1] + (om[2] * rb[0] - om[0] * rb[2]),
-                     u[2] + (om[0] * rb[1] - om[1] * rb[0])};
-    const T ubc = ub[0] * cp0 + ub[1] * cp1 + ub[2] * cp2;
-    const T v = fout + kappa * (fdown - fin) - (T(12) * w * inv) * ubc;
+    const double w = cc2 == 1 ? 1.0 / 18.0 : 1.0 / 36.0;
+    const double delta = link_root<double>(r, surface_cc<double>(r, R), cp0, cp1, cp2, (double)cc2);
+    const double dbc = cli ? delta : 0.5;
+    const double inv = 1.0 / (1.0 + 2.0 * dbc);
+    const double kappa = (1.0 - 2.0 * dbc) * inv;
+    const double rb[3] = {r[0] + delta * cp0, r[1] + delta * cp1, r[2] + delta * cp2};
+    const double ub[3] = {u[0] + (om[1] * rb[2] - om[2] * rb[1]), u[1] + (om[2] * rb[0] - om[0] * rb[2]),
+                          u[2] + (om[0] * rb[1] - om[1] * rb[0])};
+    const double ubc = ub[0] * cp0 + ub[1] * cp1 + ub[2] * cp2;
+    const double v = fout + kappa * (fdown - fin) - (12.0 * w * inv) * ubc;
     // Eq. (15) on shifted PDFs: F = c_p (2 w + f~_p + f_q) - u_b (f~_p - f_q)
-    const T dif = fout - v;
-    int K[6] = {0, 0, 0, 0, 0, 0};
-    T sum;
-    if (sizeof(T) == 4) {
-        // 2 w_p c_p and its torque 2 w_p (n x c_p) as exact integers (x 36)
-        const int kw = cc2 == 1 ? 4 : 2;
-        sum = fout + v;
-        K[0] = kw * cp[0]; K[1] = kw * cp[1]; K[2] = kw * cp[2];
-        K[3] = kw * (n[1] * cp[2] - n[2] * cp[1]);
-        K[4] = kw * (n[2] * cp[0] - n[0] * cp[2]);
-        K[5] = kw * (n[0] * cp[1] - n[1] * cp[0]);
-    } else {
-        sum = T(2) * w + fout + v;
-    }
-    const T F[3] = {cp0 * sum - ub[0] * dif, cp1 * sum - ub[1] * dif, cp2 * sum - ub[2] * dif};
-    const T Tq[3] = {rb[1] * F[2] - rb[2] * F[1], rb[2] * F[0] - rb[0] * F[2], rb[0] * F[1] - rb[1] * F[0]};
-    accumulate<T>(i, F, Tq, K, acc, sk);
+    const double dif = fout - v, sum = 2.0 * w + fout + v;
+    F[0] = cp0 * sum - ub[0] * dif;
+    F[1] = cp1 * sum - ub[1] * dif;
+    F[2] = cp2 * sum - ub[2] * dif;
+    F[3] = rb[1] * F[2] - rb[2] * F[1];
+    F[4] = rb[2] * F[0] - rb[0] * F[2];
+    F[5] = rb[0] * F[1] - rb[1] * F[0];
     return v;
 }
 
-// TRT+aB collision of one fluid cell, in place, with the body force (ax, ay,
-// az); returns false when the density deviation of the streamed PDFs leaves
-// (-0.5, 0.5) or is NaN. The arithmetic is that of the moment-space update
-// with S of Eq. (12) written per pair of opposite directions (q, qbar): with
+// The same in float32, without the constant part 2 w_p c_p of the force and
+// its torque (boundary.cu adds their sum over the particle). wrap: the tile is
+// near a periodic face, where the particle's nearest image has to be chosen;
+// a link cell lies within R + 2 cells of the centre on every axis and a
+// periodic side is longer than 2 R + 4, so exactly one image has
+// |n_d| <= floor(n / 2). |n|^2 is a whole number below 2^24, exact in float32.
+// The link enters the sphere between t = 0 and 1, so |r + t c|^2 falls from
+// above R^2 to at most R^2: r.c < -|c|^2 / 2 and the smaller root is
+// cc / (sqrt(disc) - r.c) without cancellation.
+template <typename S>
+__device__ __forceinline__ float link_value(const SCArgs<S, float>& a, int, const PartView& v, int x, int y, int z, int, float4 cf,
+                                            bool cli, bool wrap, float fout, float fin, float fdown, float (&F)[6]) {
+    int nd[3] = {x - v.base[0], y - v.base[1], z - v.base[2]};
+    if (wrap) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int L = a.g.per[d] ? a.g.n[d] : 0x7fffffff, half = L >> 1;
+            if (nd[d] > half) nd[d] -= L;
+            if (nd[d] < -half) nd[d] += L;
+        }
+    }
+    const float n0 = (float)nd[0], n1 = (float)nd[1], n2 = (float)nd[2];
+    const float g0 = 0.5f - v.frac[0], g1 = 0.5f - v.frac[1], g2 = 0.5f - v.frac[2];
+    const float cp0 = cf.x, cp1 = cf.y, cp2 = cf.z;   // c_p
+    // |r|^2 - R^2 = (|n|^2 + C) + (2 n.g + C_lo): only the small terms round
+    const float nn = fmaf(n2, n2, fmaf(n1, n1, n0 * n0));
+    const float ng = fmaf(n2, g2, fmaf(n1, g1, n0 * g0));
+    const float cc = (nn + v.C) + fmaf(2.0f, ng, v.C_lo);
+    const float r0 = n0 + g0, r1 = n1 + g1, r2 = n2 + g2;
+    const float rc = fmaf(r2, cp2, fmaf(r1, cp1, r0 * cp0));
+    const float disc = fmaxf(fmaf(rc, rc, -cf.w * cc), 0.0f);
+    const float delta = __saturatef(fast_div(cc, fast_sqrt(disc) - rc));
+    const float dbc = cli ? delta : 0.5f;
+    const float inv = fast_div(1.0f, fmaf(2.0f, dbc, 1.0f));
+    const float kappa = fmaf(-2.0f, dbc, 1.0f) * inv;
+    const float b0 = fmaf(delta, cp0, r0), b1 = fmaf(delta, cp1, r1), b2 = fmaf(delta, cp2, r2);
+    const float u0 = v.u[0] + (v.om[1] * b2 - v.om[2] * b1), u1 = v.u[1] + (v.om[2] * b0 - v.om[0] * b2),
+                u2 = v.u[2] + (v.om[0] * b1 - v.om[1] * b0);
+    const float ubc = fmaf(u2, cp2, fmaf(u1, cp1, u0 * cp0));
+    const float w12 = cf.w == 1.0f ? 12.0f / 18.0f : 12.0f / 36.0f;
+    const float val = fmaf(kappa, fdown - fin, fout) - (w12 * inv) * ubc;
+    const float dif = fout - val, sum = fout + val;
+    F[0] = cp0 * sum - u0 * dif;
+    F[1] = cp1 * sum - u1 * dif;
+    F[2] = cp2 * sum - u2 * dif;
+    F[3] = b1 * F[2] - b2 * F[1];
+    F[4] = b2 * F[0] - b0 * F[2];
+    F[5] = b0 * F[1] - b1 * F[0];
+    return val;
+}
+
+// sign of the first non-zero component of c_q
+__host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? cy(q) : cz(q)); }
+
+// TRT+aB collision of the cells packed in f, in place, with the body force
+// (ax, ay, az); shell[r]: cell r lies in the shell. Returns the density
+// deviations. The arithmetic is that of the moment-space update with S of
+// Eq. (12) written per pair of opposite directions (q, qbar): with
 // s = f_q + f_qbar and d = f_q - f_qbar the even part relaxes with s_nu and
 // the odd part with s_nu^- (Eq. (10)),
 //   dp = -s_nu (s/2 - w X) + (1 - s_nu/2) w Y + corr,   X = drho - 3/2 u^2 + 9/2 (c.u)^2
 //   dm = -s_nu^- (d/2 - 3 w c.u) + (1 - s_nu^-/2) 3 w c.a, Y = -3 u.a + 9 (c.u)(c.a)
 //   f_q += dp + dm,  f_qbar += dp - dm,
 // the Guo source in Y and 3 w c.a; corr is the rank-2 bulk correction of the
-// shell cells. Each pair costs one chain of fused multiply-adds.
+// shell cells. The source is taken into the equilibrium's velocities:
+//   s_nu X + (1 - s_nu/2) 2 Y / 2 = s_nu [drho - 3/2 u^2 - 3/2 k u.a + 9/2 (c.u)(c.v)],  v = u + k a, k = (2 - s_nu)/s_nu
+//   s_nu^- 3 c.u + (1 - s_nu^-/2) 3 c.a = s_nu^- 3 c.t,                                  t = u + (k^-/2) a, k^- = (2 - s_nu^-)/s_nu^-
+// (ke = k, ko = k^-/2)
+// so a pair costs the same few multiply-adds with and without a body force.
 template <typename T>
-__device__ __forceinline__ bool collide_core(T (&f)[Q], uint8_t fl, T ax, T ay, T az, T sp, T sm, T s_b_shell,
-                                             T s_b_bulk, int bulk_corr) {
-    T sq[Q], dq[Q];   // pair sums and differences, entries q < opp(q) only
-    T drho = f[0], jx = T(0), jy = T(0), jz = T(0);
+__device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V (&f)[Q],
+                                                            const bool (&shell)[Pack<T>::ROWS], T ax, T ay, T az, T sp,
+                                                            T sm, T ke, T ko, T s_b_shell, T s_b_bulk,
+                                                            int bulk_corr) {
+    using P = Pack<T>;
+    using V = typename P::V;
+    // pair sums and differences are formed twice (here and in the update):
+    // keeping them takes 36 registers more than the cell's PDFs
+    V drho = f[0], jx = P::all(T(0)), jy = jx, jz = jx;
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
         const int qb = opp(q);
         if (qb < q) continue;
-        sq[q] = f[q] + f[qb];
-        dq[q] = f[q] - f[qb];
-        drho += sq[q];
-        if (cx(q)) jx += cx(q) > 0 ? dq[q] : -dq[q];
-        if (cy(q)) jy += cy(q) > 0 ? dq[q] : -dq[q];
-        if (cz(q)) jz += cz(q) > 0 ? dq[q] : -dq[q];
+        const int sg = lead(q);
+        const V d = sg > 0 ? f[q] - f[qb] : f[qb] - f[q];
+        drho = drho + (f[q] + f[qb]);
+        if (cx(q)) jx = cx(q) * sg > 0 ? jx + d : jx - d;
+        if (cy(q)) jy = cy(q) * sg > 0 ? jy + d : jy - d;
+        if (cz(q)) jz = cz(q) * sg > 0 ? jz + d : jz - d;
     }
-    const T ux = jx + T(0.5) * ax, uy = jy + T(0.5) * ay, uz = jz + T(0.5) * az;
-    const T usq = ux * ux + uy * uy + uz * uz;
-    const T ua = ux * ax + uy * ay + uz * az;
-    const T gp = T(1) - T(0.5) * sp, gm = T(1) - T(0.5) * sm;
+    const V ux = jx + P::all(T(0.5) * ax), uy = jy + P::all(T(0.5) * ay), uz = jz + P::all(T(0.5) * az);
+    const V usq = mad(uz, uz, mad(ux, ux, uy * uy));
+    const V ua = mad(ux, P::all(ax), mad(uy, P::all(ay), uz * P::all(az)));
+    const V vx = ux + P::all(ke * ax), vy = uy + P::all(ke * ay), vz = uz + P::all(ke * az);
+    const V tx = ux + P::all(ko * ax), ty = uy + P::all(ko * ay), tz = uz + P::all(ko * az);
     // bulk moments m4 = sum (c^2 - 1) f and m5 (row 6 of M) of the streamed
     // PDFs relax with s_b in shell cells (and everywhere when Lambda_b,bulk != 1)
-    const bool shell = (fl & FL_SHELL) != 0;
-    const bool bulk = shell || bulk_corr;
-    T k4 = T(0), k5 = T(0);
+    bool bulk = bulk_corr != 0;
+#pragma unroll
+    for (int r = 0; r < P::ROWS; ++r) bulk |= shell[r];
+    V k4 = P::all(T(0)), k5 = k4;
     if (bulk) {
-        const T ds = (shell ? s_b_shell : s_b_bulk) - sp;
-        T saxis = T(0), sdiag = T(0);
+        T dsr[P::ROWS];
+#pragma unroll
+        for (int r = 0; r < P::ROWS; ++r) dsr[r] = shell[r] ? s_b_shell - sp : (bulk_corr ? s_b_bulk - sp : T(0));
+        const V ds = P::make(dsr);
+        V saxis = P::all(T(0)), sdiag = saxis;
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
             if (opp(q) < q) continue;
-            if (c2(q) == 1) saxis += sq[q]; else sdiag += sq[q];
+            if (c2(q) == 1) saxis = saxis + (f[q] + f[opp(q)]); else sdiag = sdiag + (f[q] + f[opp(q)]);
         }
-        const T m4 = -f[0] + sdiag;
-        const T m5 = f[0] - T(2) * saxis + sdiag;
+        const V m4 = sdiag - f[0];
+        const V m5 = mad(P::all(T(-2)), saxis, f[0]) + sdiag;
         // M^-1 e_k = w_q M_kq / (sum_q w_q M_kq^2): norms 2/3 (row 4) and 2 (row 5)
-        k4 = T(1.5) * (ds * ((usq - m4) - ua));
-        k5 = T(0.5) * (ds * (-m5));
+        k4 = P::all(T(1.5)) * (ds * ((usq - m4) - ua));
+        k5 = P::all(T(-0.5)) * (ds * m5);
     }
-    const T drp = drho - T(1.5) * usq;
-    const T m3ua = T(-3) * ua;
+    // equilibrium part common to all directions, with the u.a term of the source
+    const V X0 = mad(P::all(T(-1.5)), mad(P::all(ke), ua, usq), drho);
     // Weights of the update: w2 = 2 w (even parts), w6 = 6 w (odd parts) per
     // class (axis, diagonal) and w0. In float32 they are chosen within 1.2e-7
     // of the exact fractions such that w0 + 3 w2_axis + 6 w2_diag = 1 and
@@ -220,51 +322,37 @@ __device__ __forceinline__ bool collide_core(T (&f)[Q], uint8_t fl, T ax, T ay, 
     const T w0 = T(1) - T(12) * w2d;
     const T w6d = T(1) / T(6);
     const T w6a = T(1) - T(4) * w6d;
-    {
-        f[0] = f[0] + sp * (w0 * drp - f[0]) + gp * (w0 * m3ua) + w0 * (k5 - k4);
-    }
-    const T hsp = T(-0.5) * sp, hsm = T(-0.5) * sm;
-    // per weight class (axis, diagonal); each part relaxes as rate x (value
-    // - its equilibrium)
-    const T w2[2] = {w2a, w2d}, w6[2] = {w6a, w6d};
-    const T gpw[2] = {T(0.5) * gp * w2a, T(0.5) * gp * w2d}, gmw3[2] = {T(0.5) * gm * w6a, T(0.5) * gm * w6d};
-    const T corr[2] = {-w2a * k5, T(0.5) * w2d * (k4 + k5)};
+    const V mw2[2] = {P::all(-w2a), P::all(-w2d)}, mw6[2] = {P::all(-w6a), P::all(-w6d)};
+    const V corr[2] = {mw2[0] * k5, P::all(T(0.5) * w2d) * (k4 + k5)};
+    f[0] = mad(P::all(w0), k5 - k4, mad(P::all(sp), mad(P::all(w0), X0, P::all(T(0)) - f[0]), f[0]));
+    const V hsp = P::all(T(-0.5) * sp), hsm = P::all(T(-0.5) * sm), c45 = P::all(T(4.5));
+    // each part relaxes as rate x (value - its equilibrium). The pair sums and
+    // differences as (exact) multiply-adds, which the compiler does not merge
+    // with the first ones
+    const V one = P::all(T(1)), mone = P::all(T(-1));
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
         const int qb = opp(q);
         if (qb < q) continue;
         const int k = c2(q) == 1 ? 0 : 1;
-        T cu = T(0), ca = T(0);
-        if (cx(q)) { cu += cx(q) > 0 ? ux : -ux; ca += cx(q) > 0 ? ax : -ax; }
-        if (cy(q)) { cu += cy(q) > 0 ? uy : -uy; ca += cy(q) > 0 ? ay : -ay; }
-        if (cz(q)) { cu += cz(q) > 0 ? uz : -uz; ca += cz(q) > 0 ? az : -az; }
-        const T X = fma_t<T>(T(4.5) * cu, cu, drp);
-        const T Y = fma_t<T>(T(9) * cu, ca, m3ua);
-        const T dp = fma_t<T>(hsp, fma_t<T>(-w2[k], X, sq[q]), fma_t<T>(gpw[k], Y, corr[k]));
-        const T dm = fma_t<T>(hsm, fma_t<T>(-w6[k], cu, dq[q]), gmw3[k] * ca);
-        f[q] = f[q] + (dp + dm);
-        f[qb] = f[qb] + (dp - dm);
+        const int sg = lead(q);
+        // c.u, c.v, c.t times lead(q), which their product and e share
+        const bool y_plus = cy(q) * sg > 0, z_plus = cz(q) * sg > 0;
+        V cu = cx(q) ? ux : (cy(q) ? uy : uz), cv = cx(q) ? vx : (cy(q) ? vy : vz), ct = cx(q) ? tx : (cy(q) ? ty : tz);
+        if (cx(q) && cy(q)) {
+            cu = y_plus ? cu + uy : cu - uy; cv = y_plus ? cv + vy : cv - vy; ct = y_plus ? ct + ty : ct - ty;
+        }
+        if ((cx(q) || cy(q)) && cz(q)) {
+            cu = z_plus ? cu + uz : cu - uz; cv = z_plus ? cv + vz : cv - vz; ct = z_plus ? ct + tz : ct - tz;
+        }
+        const V X = mad(c45 * cu, cv, X0);
+        const V dp = mad(hsp, mad(mw2[k], X, mad(one, f[q], f[qb])), corr[k]);
+        // lead(q) dm
+        const V dm = mul_rn(hsm, mad(mw6[k], ct, sg > 0 ? mad(mone, f[qb], f[q]) : mad(mone, f[q], f[qb])));
+        f[q] = f[q] + (sg > 0 ? dp + dm : dp - dm);
+        f[qb] = f[qb] + (sg > 0 ? dp - dm : dp + dm);
     }
-    return drho < T(0.5) && drho > T(-0.5);
+    return drho;
 }
-
-template <typename S, typename T>
-__device__ __forceinline__ bool collide_cell_a(const SCArgs<S, T>& a, T (&f)[Q], uint8_t fl, T ax, T ay, T az) {
-    return collide_core<T>(f, fl, ax, ay, az, a.s_plus, a.s_minus, a.s_b_shell, a.s_b_bulk, a.bulk_corr);
-}
-
-template <typename S, typename T>
-__device__ __forceinline__ bool collide_cell(const SCArgs<S, T>& a, T (&f)[Q], uint8_t fl) {
-    return collide_cell_a<S, T>(a, f, fl, a.accel[0], a.accel[1], a.accel[2]);
-}
-
-// collision of one fluid cell and the store of its PDFs
-template <typename S, typename T>
-__device__ __forceinline__ void collide_store(const SCArgs<S, T>& a, T (&f)[Q], uint8_t fl, long long N, int idx) {
-    if (!collide_cell<S, T>(a, f, fl)) atomicOr(a.status, ST_UNSTABLE);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) Store<S>::store(a.dst + q * N + idx, f[q]);
-}
-
 
 }  // namespace lbmdem

@@ -1,281 +1,452 @@
 // stream_collide.cu -- the dense kernel of one lattice Boltzmann step with
-// moving particles (Algorithm 1, lines 1-3): one thread per cell, pull
-// streaming (Eq. (2)), the particle links of the cell (CLI moving no-slip
-// condition, Eq. (14), and momentum exchange, Eqs. (15)-(17)), halfway
-// bounce-back on the walls of the box (Eq. (14), delta = 1/2, wall velocity),
-// then the two-relaxation-time collision (Eq. (10), magic parameter
-// Eq. (11)) with Guo forcing; in TRT+aB shell cells (Sec. 2.3.2) and for
-// Lambda_b,bulk != 1 the two bulk moments m4, m5 relax with s_b (Eq. (12))
-// through a rank-2 correction in moment space.
+// moving particles (Algorithm 1, lines 1-3): pull streaming (Eq. (2)), the
+// particle links (CLI moving no-slip condition, Eq. (14), and momentum
+// exchange, Eqs. (15)-(17)), halfway bounce-back on the walls of the box
+// (Eq. (14), delta = 1/2, wall velocity), then the two-relaxation-time
+// collision (Eq. (10), magic parameter Eq. (11)) with Guo forcing; in TRT+aB
+// shell cells (Sec. 2.3.2) and for Lambda_b,bulk != 1 the two bulk moments m4,
+// m5 relax with s_b (Eq. (12)) through a rank-2 correction in moment space.
 //
 // PDFs are stored shifted (f_q - w_q) in SoA layout f[q][z][y][x], read from
-// one buffer and written to the other (fluid cells only). Every PDF slot of a
-// solid cell holds a NaN marker written by the mapping (with the owning
-// particle in its payload for 4- and 8-byte storage), so the pull of a fluid
-// cell x finds its particle links for free: direction q is a link exactly
-// when the value pulled from y = x - c_q is a marker. The warp then spreads
-// its links evenly over its lanes; each link's CLI value f_q(x, t+1) (link
-// fraction delta_p from the ray-sphere intersection; bounce-back, delta = 1/2
-// in the coefficients, when x + c_q is not fluid) goes through shared memory
-// to the thread of x, and its force and torque are summed per lane while the
-// particle stays the same, then per warp by particle (lanes with the same
-// particle found with match_any) and added atomically.
+// one buffer and written to the other. What a solid cell's slots hold is
+// never used: which pulls are particle links is read from the mapping's bit
+// per cell (solid), so a warp finds the links of a row of 32 cells with a few
+// word operations per direction instead of testing 18 pulled values per cell.
 //
-// Per-particle sums. Float64 storage: float64 partial sums, float64 atomics.
-// Float32 compute: the link force splits into the constant part 2 w_p c_p,
-// an integer multiple of c_p / 36, and the small remainder
-// c_p (f~_p + f_q) - u_b (f~_p - f_q). The constant part and its torque
-// 2 w_p (n + g) x c_p (n the integer offset of the cell from the particle's
-// base cell, g the fractional offset common to all links) are summed exactly
-// in integers; the remainder is summed per warp in float32 and per particle
-// in 64-bit fixed point (scale 2^32) through integer atomics. No float64
-// arithmetic runs per cell or link on the float32 path.
+// A warp works alone (no block barriers) on 32 x 2 cells (32 x 1 in float64) of
+// one z plane after the other. For each plane it
+//   1. forms the link words of its cells, lane q for direction q: fluid(x) &
+//      solid(x - c_q), starts its pulls, and queues the links in shared memory,
+//      the left half of the cells first (links of one sphere then mostly share
+//      a chunk);
+//   2. takes the queue 32 links at a time, one per lane: CLI value into the
+//      cell's slot in shared memory, force and torque into the lane's open sums
+//      of the particle, kept in shared memory over the planes for the last few
+//      particles (added to a particle when its slot is needed and at the end);
+//   3. patches the linked values in, collides and stores. Float32 collides the
+//      two rows in packed arithmetic.
+// Sectors of 32 bytes with a fluid cell are written whole (solid cells get
+// whatever the arithmetic gives), so DRAM never has to merge part of one.
+//
+// What bounds it (256 x 256 x 512 cells, 10,000 spheres, 27 % solids, float32):
+// instruction issue and latency together, 930 warp instructions per row of 32
+// cells (1,310 with a test of every pulled value for a marker, one row per warp
+// and force sums flushed when a lane's particle changed) at 54 % issue; 1.36 ms
+// against 1.58 ms that way, 128 x 128 x 256 cells 214 us against 284 us, float16
+// 192^3 with 2,000 spheres 328 us against 466 us. Streaming alone takes the
+// memory's time (95 us of the 128 x 128 x 256 case at 6.7 TB/s).
+//
+// Per-particle sums. Float64 storage: float64 sums per lane and warp, float64
+// atomics. Float32 compute: the link force splits into the constant part
+// 2 w_p c_p and the small remainder c_p (f~_p + f_q) - u_b (f~_p - f_q). The
+// constant parts and their torques over a particle's fluid links are minus
+// those over its other links (the links of a set of cells to its outside
+// cancel), so boundary.cu adds them from the few cells that have others; the
+// remainder is summed per lane and warp in float32 and per particle in 64-bit
+// fixed point (scale 2^32) through integer atomics. The sums depend on the
+// chunk of planes a warp marches, not on the tile width.
 #include <cstring>
 
 #include "sc_common.cuh"
 
-// minimum resident blocks per SM requested for the kernel with 4-byte or
-// smaller storage (a register cap of 64 at 256 threads); tuned on GB300
+// resident blocks of 128 threads per SM (a register cap); tuned on GB300
 #ifndef LBM_SC_MIN_BLOCKS
 #define LBM_SC_MIN_BLOCKS 4
 #endif
 // the same for float64 storage
 #ifndef LBM_SC_MIN_BLOCKS_F64
-#define LBM_SC_MIN_BLOCKS_F64 2
+#define LBM_SC_MIN_BLOCKS_F64 4
 #endif
 // longest chunk of consecutive z planes marched by one block (shorter when
 // the box is too small to give every SM several blocks); tuned on GB300
 #ifndef LBM_SC_ZCHUNK
-#define LBM_SC_ZCHUNK 24
+#define LBM_SC_ZCHUNK 16
 #endif
-// x extent of a block (a multiple of 32; 256 / LBM_SC_BX rows in y)
-#ifndef LBM_SC_BX
-#define LBM_SC_BX 128
-#endif
+
 namespace lbmdem {
 
-// a lane's open force sums between rows: particle, float sums and the exact
-// integer sums (float32 path) as two 16-bit halves per word; sums that could
-// leave 16 bits are flushed to the particle first
+constexpr int SC_WARPS = 4;       // warps per block
+constexpr int QUEUE_CAP = 256;    // links queued at a time
+
+// Shared memory of one warp. A cell is numbered half (x < 16 or not) << 5 |
+// row << 4 | x & 15; a queue entry is q << 11 | p << 6 | cell, p opposite to q.
 template <typename T>
-__device__ __forceinline__ void load_sums(Acc<T>& acc, const int* s_key, T (*s_sum)[256], int (*s_int)[256], int tid) {
-    acc.key = s_key[tid];
+struct SCWarp {
+    static constexpr int ROWS = Pack<T>::ROWS;
+    T v[Q - 1][32 * ROWS];                   // CLI values
+    OpenParts<T> open;
+    uint32_t w[Q + 2][ROWS];                 // link words of directions 1 .. 18, fluid, shell
+    unsigned short queue[QUEUE_CAP];
+};
+// cell number of x = lane, row 0 (row 1: + 16)
+template <typename T>
+__device__ __forceinline__ int cell_of(int lane) {
+    return Pack<T>::ROWS == 1 ? lane : ((lane & 16) << 1) | (lane & 15);
+}
+
+// what one link reads: queue entry (bit 16: CLI), particle, PDFs
+template <typename T>
+struct LinkIn {
+    int e, key;
+    T fout, fin, fdown;
+};
+
+// a lane's words of one plane (see sc_warp)
+struct PlaneWords {
+    uint32_t at[2], side[2];
+};
+
+// g = *v where bit is set (a predicated load: no select, no load elsewhere)
+__device__ __forceinline__ void patch_link(float& g, uint32_t bit, const float* v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.f32 %0, [%2];\n\t}"
+                 : "+f"(g) : "r"(bit), "r"((uint32_t)__cvta_generic_to_shared(v)));
+}
+__device__ __forceinline__ void patch_link(double& g, uint32_t bit, const double* v) {
+    if (bit) g = *v;
+}
+
+// One warp's cells: x = 32 wx + lane, rows y0 .. y0 + ROWS - 1, planes
+// z_begin .. z_end - 1 marched in order.
+template <typename S, typename T>
+__device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, int z_begin, int z_end, SCWarp<T>& sm,
+                                        const DirTable<S>& dt) {
+    using P = Pack<T>;
+    constexpr int ROWS = P::ROWS;
+    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
+    const unsigned FULL = 0xffffffffu;
+    int lane;   // opaque, or the compiler reads the special register again and again
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+    const int plane = nx * ny;
+    const int W = a.words;
+    const int x = 32 * wx + lane;
+    const int xl = x < nx ? x : nx - 1;          // lanes past the row load its last cell
+    const bool last_word = wx == W - 1;
+    const uint32_t valid = last_word && (nx & 31) ? (1u << (nx & 31)) - 1u : FULL;
+    const bool rowB = ROWS > 1 && y0 + 1 < ny;   // the second row exists
+    // pull offsets in the plane: rows y0 - 1 .. y0 + ROWS, columns x - 1 .. x + 1
+    const int xo[3] = {xl == 0 ? nx - 1 : xl - 1, xl, xl == nx - 1 ? 0 : xl + 1};
+    int yo[ROWS + 2];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) acc.f[c] = s_sum[c][tid];
-    if (sizeof(T) == 4) {
+    for (int r = 0; r < ROWS + 2; ++r) {
+        int yy = y0 - 1 + r;
+        yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+        yo[r] = yy * nx;
+    }
+    const T ax = a.accel[0], ay = a.accel[1], az = a.accel[2];
+    const Sinks sk{a.acc_d, a.acc_i, nullptr, a.status};
+
+    SlotKeys<T> keys;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int v = s_int[c][tid];
-            acc.k[2 * c] = (int)(short)(v & 0xffff);
-            acc.k[2 * c + 1] = v >> 16;
+    for (int j = 0; j < OpenParts<T>::SLOTS; ++j) keys.k[j] = -1;
+    keys.next = 0;
+
+    // Words of a plane: lane q - 1 holds direction q's upstream words and the
+    // neighbouring ones whose bit shifts in (behind a wall there are no links),
+    // lane 18 the solid, lane 19 the shell words of the warp's own rows; loaded
+    // a plane ahead.
+    const int ql = lane < Q - 1 ? lane + 1 : 0;
+    int wz = 0;               // the words' plane: z - wz
+    int woff[ROWS], wside;    // word of each row, of the neighbouring word relative to it
+    uint32_t wcfg;            // rows on in bits 0-1, shift left / right 2-3, carry on 4, side bit 8-12, carry bit 16-20
+    {
+        const int qi = dt.qi[ql];
+        const int c0 = (qi & 3) - 1, c1 = ((qi >> 2) & 3) - 1;
+        wz = ((qi >> 4) & 3) - 1;
+        const bool carry = c0 != 0 && (a.g.per[0] || !((c0 > 0 && wx == 0) || (c0 < 0 && last_word)));
+        wcfg = (c0 > 0 ? 4u : 0u) | (c0 < 0 ? 8u : 0u) | (carry ? 16u : 0u) |
+               (c0 > 0 ? (uint32_t)(wx > 0 ? 31 : (nx - 1) & 31) << 8 : (uint32_t)(last_word ? (nx - 1) & 31 : 31) << 16);
+        wside = c0 > 0 ? (wx > 0 ? -1 : W - 1) : (c0 < 0 ? (last_word ? 1 - W : 1) : 0);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            int yu = y0 + r - c1;
+            if (ql ? a.g.per[1] || (yu >= 0 && yu < ny) : true) wcfg |= 1u << r;
+            yu = yu < 0 ? yu + ny : (yu >= ny ? yu - ny : yu);
+            woff[r] = yu * W + wx;
         }
     }
-}
-template <typename T>
-__device__ __forceinline__ void store_sums(Acc<T>& acc, int* s_key, T (*s_sum)[256], int (*s_int)[256], int tid,
-                                           const Sinks& sk) {
-    if (sizeof(T) == 4) {
-        bool big = false;
+    const uint32_t* const wbase = lane == Q ? a.shell : a.solid;
+    auto load_words = [&](int z) {
+        PlaneWords s;
+        int zu = z - wz;
+        const bool in = a.g.per[2] || (unsigned)zu < (unsigned)nz;
+        zu = zu < 0 ? zu + nz : (zu >= nz ? zu - nz : zu);
+        const uint32_t* p = wbase + zu * (ny * W);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) big |= acc.k[c] > 30000 || acc.k[c] < -30000;
-        if (big && acc.key >= 0) flush<T>(acc, sk);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) s_int[c][tid] = (acc.k[2 * c] & 0xffff) | (acc.k[2 * c + 1] << 16);
-    }
-    s_key[tid] = acc.key;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) s_sum[c][tid] = acc.f[c];
-}
-
-// One tile of bx x (256 / bx) cells in (x, y) from (x0, y0), planes z_begin
-// .. z_end - 1 marched in order: the links a warp meets in consecutive rows
-// mostly belong to the same spheres, so a lane's force sums (kept in shared
-// memory between rows) rarely change particle and the warp commits them once
-// per tile. Thread tid of the block's 256 handles column x0 + tid % bx, row
-// y0 + tid / bx (warps hold 32 consecutive tids). Cell indices are 32-bit
-// (the library limits boxes to 2^31 - 2^24 cells); each PDF array q starts at
-// src + q N. s_qi holds the link codes qinfo(q).
-// A single-box launch has blocks of (bx, 256 / bx) threads and takes its tile
-// from the block index (BATCH false: x0, y0 unused); the batched launch has
-// blocks of 256 threads and passes the tile.
-template <typename S, typename T, bool BATCH>
-__device__ __forceinline__ void sc_tile(const SCArgs<S, T>& a, int x0, int y0, int z_begin, int z_end, int bx,
-                                        unsigned char* sc_smem, const int* s_qi) {
-    const int nx = a.g.n[0], ny = a.g.n[1], nz = a.g.n[2];
-    // bx is 32, 64 or 128
-    const int tid = BATCH ? (int)threadIdx.x : (int)(threadIdx.x + blockDim.x * threadIdx.y);
-    const int x = BATCH ? x0 + (tid & (bx - 1)) : (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = BATCH ? y0 + (tid >> (bx == 128 ? 7 : (bx == 64 ? 6 : 5)))
-                        : (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const bool valid = x < nx && y < ny;
-    const int plane = nx * ny;
-    const long long N = a.g.ncells;
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    // dynamic shared memory (sc_smem_bytes): PDFs of the cells of warps with
-    // links [q][thread]; per lane the particle of its open force sums (-1:
-    // none), the open float sums (F, T) and the exact integer sums (float32
-    // path, two 16-bit halves per word); per warp the link entries q | lane << 8
-    T (*s_f)[256] = reinterpret_cast<T (*)[256]>(sc_smem);
-    T (*s_sum)[256] = reinterpret_cast<T (*)[256]>(sc_smem + Q * 256 * sizeof(T));
-    int (*s_int)[256] = reinterpret_cast<int (*)[256]>(sc_smem + (Q + 6) * 256 * sizeof(T));
-    int* s_key = reinterpret_cast<int*>(sc_smem + (Q + 6) * 256 * sizeof(T) + (sizeof(T) == 4 ? 3 * 256 * 4 : 0));
-    unsigned short (*s_queue)[32 * (Q - 1)] =
-        reinterpret_cast<unsigned short (*)[32 * (Q - 1)]>(reinterpret_cast<unsigned char*>(s_key) + 256 * 4);
-    const Sinks sk{a.acc_d, a.acc_i, a.acc_k, a.status};
-    s_key[tid] = -1;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        s_sum[c][tid] = T(0);
-        if (sizeof(T) == 4 && c < 3) s_int[c][tid] = 0;
-    }
-    bool open = false;   // warp-uniform: some lane of the warp holds sums
-
-    // the 19 pulls of cell (x, y, zz) with periodic wrap (walls are handled
-    // below), issued only for a fluid cell
-    auto pull_row = [&](int zz, bool fluid_zz, T (&g)[Q]) {
-        if (!fluid_zz) return;
-        const int idz = zz * plane + y * nx + x;
-        const int OX[3] = {x == 0 ? nx - 1 : -1, 0, x == nx - 1 ? 1 - nx : 1};
-        const int OY[3] = {y == 0 ? plane - nx : -nx, 0, y == ny - 1 ? nx - plane : nx};
-        const int OZ[3] = {zz == 0 ? (nz - 1) * plane : -plane, 0, zz == nz - 1 ? (1 - nz) * plane : plane};
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-            g[q] = Store<S>::load(a.src + q * N + (idz + OX[1 - cx(q)] + OY[1 - cy(q)] + OZ[1 - cz(q)]));
+        for (int r = 0; r < ROWS; ++r) {
+            s.at[r] = p[woff[r]];
+            s.side[r] = p[woff[r] + wside];
+            if (!in) s.at[r] = s.side[r] = 0u;
+        }
+        return s;
     };
-    for (int z = z_begin; z < z_end; ++z) {
-        const int idx = z * plane + y * nx + x;
-        T f[Q];
-        const uint8_t fl = valid ? a.flags[idx] : FL_SOLID;
-        pull_row(z, !(fl & FL_SOLID), f);
-        const bool fluid = !(fl & FL_SOLID);
-        unsigned lmask = 0;   // pull directions of this cell that are particle links
-        if (fluid) {
+    PlaneWords pw = load_words(z_begin);
+
+    // the gathers of queue entry k (the last one for lanes past the end) of a
+    // plane; edges: bit d, the warp's cells reach the box's faces on axis d
+    auto fetch = [&](int k, int n, int z, int edges) {
+        LinkIn<T> l;
+        const int e = sm.queue[min(k, n - 1)];
+        const int q = e >> 11, p = (e >> 6) & 31, row = (e >> 4) & (ROWS - 1);
+        const int xb = ROWS == 1 ? e & 31 : (e & 15) | ((e >> 1) & 16);
+        const int idx = z * plane + y0 * nx + 32 * wx + (row ? nx : 0) + xb, dq = dt.dq[q];
+        // x + c_q must be fluid and inside the box for CLI; its post-collision
+        // f_p is the cell's own pull in direction p
+        bool cli = !((sm.w[p][row] >> xb) & 1u);
+        int is = idx - dq, id = idx + dq;
+        if (edges) {
+            const int qi = dt.qi[q];
+            const int pos[3] = {32 * wx + xb, y0 + row, z};
+            const int step[3] = {nx, plane, (int)a.g.ncells};
 #pragma unroll
-            for (int q = 1; q < Q; ++q)
-                if (f[q] != f[q]) lmask |= 1u << q;   // marker of a solid upstream cell
-            // halfway bounce-back on the box walls (Eq. (14) with delta = 1/2)
-            const bool wx = !a.g.per[0] && (x == 0 || x == nx - 1);
-            const bool wy = !a.g.per[1] && (y == 0 || y == ny - 1);
-            const bool wz = !a.g.per[2] && (z == 0 || z == nz - 1);
-            if (wx || wy || wz) {
+            for (int d = 0; d < 3; ++d)
+                if ((edges >> d) & 1) {
+                    const int n_d = a.g.n[d], c = ((qi >> (2 * d)) & 3) - 1, us = pos[d] - c, ds = pos[d] + c;
+                    if (!a.g.per[d] && (unsigned)ds >= (unsigned)n_d) cli = false;
+                    is += us < 0 ? step[d] : (us >= n_d ? -step[d] : 0);
+                    id += ds < 0 ? step[d] : (ds >= n_d ? -step[d] : 0);
+                }
+        }
+        const S* const sp = dt.src[p];
+        l.key = a.owner[is];
+        l.fout = Store<S>::load(sp + idx);
+        l.fin = Store<S>::load(dt.src[q] + idx);
+        const T fd = Store<S>::load(sp + id);
+        l.fdown = cli ? fd : T(0);
+        l.e = e | (cli ? 0x10000 : 0);
+        return l;
+    };
+
+    // axes on which the warp's cells lie next to the box's faces, and z planes
+    // in which no image of a particle near the tile's links matters
+    const int wall_axes = (a.g.per[0] ? 0 : 1) | (a.g.per[1] ? 0 : 2) | (a.g.per[2] ? 0 : 4);
+    const int edges_xy = (wx == 0 || last_word ? 1 : 0) | (y0 == 0 || y0 + ROWS >= ny ? 2 : 0);
+    const int mx = a.g.per[0] ? a.margin : 1, my = a.g.per[1] ? a.margin : 1, mz = a.g.per[2] ? a.margin : 1;
+    const bool deep_xy = 32 * wx >= mx && 32 * wx + 31 < nx - mx && y0 >= my && y0 + ROWS <= ny - my;
+
+    for (int z = z_begin; z < z_end; ++z) {
+        // 1. link words and queue
+        __syncwarp();   // the last plane's words and values are read
+        uint32_t link[2] = {0u, 0u};
+        {
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const uint32_t u = pw.at[r];
+                const uint32_t carry = wcfg & 16u ? ((pw.side[r] >> ((wcfg >> 8) & 31)) & 1u) << ((wcfg >> 16) & 31) : 0u;
+                const uint32_t v = ((u << ((wcfg >> 2) & 1)) >> ((wcfg >> 3) & 1)) | carry;
+                link[r] = (wcfg >> r) & 1u ? v : 0u;
+                // the second row of the last pair may not exist
+                if (lane == Q - 1) link[r] = r == 0 || rowB ? ~v & valid : 0u;
+                if (lane < Q + 1) sm.w[lane + 1][r] = link[r];
+            }
+        }
+        if (z + 1 < z_end) pw = load_words(z + 1);
+        __syncwarp();
+        uint32_t fluid[2] = {sm.w[Q][0], ROWS > 1 ? sm.w[Q][ROWS - 1] : 0u};
+        if ((fluid[0] | fluid[1]) == 0u) continue;   // warp-uniform
+        link[0] = ql ? link[0] & fluid[0] : 0u;
+        link[1] = ql ? link[1] & fluid[1] : 0u;
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+            if (ql) sm.w[ql][r] = link[r];
+        // the pulls are under way while the links are worked on; lanes of a
+        // sector without fluid idle
+        constexpr int SECT = 32 / (int)sizeof(S) < 32 ? 32 / (int)sizeof(S) : 32;
+        const uint32_t sect = (uint32_t)((1ull << SECT) - 1ull) << (lane & ~(SECT - 1));
+        const bool actA = (fluid[0] & sect) != 0u, actB = ROWS > 1 && (fluid[1] & sect) != 0u;
+        const int zoff[3] = {(z == 0 ? nz - 1 : z - 1) * plane, z * plane, (z == nz - 1 ? 0 : z + 1) * plane};
+        typename P::V f[Q];
+        if (actA || actB) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                T g[ROWS];
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r)
+                    g[r] = Store<S>::load(a.src[q] + (zoff[1 - cz(q)] + yo[1 + r - cy(q)] + xo[1 - cx(q)]));
+                f[q] = P::make(g);
+            }
+        }
+        // links of the left half (low 16 bits) and of the right half (high); with
+        // one row all count as left, the order in which they are queued below
+        const int cl = ROWS == 1 ? __popc(link[0]) : __popc(link[0] & 0xffffu) + __popc(link[1] & 0xffffu);
+        const int cr = ROWS == 1 ? 0 : __popc(link[0] >> 16) + __popc(link[1] >> 16);
+        const int incl = warp_incl_scan(cl | (cr << 16), lane);
+        const int all = __shfl_sync(FULL, incl, 31);
+        const int left = all & 0xffff, total = left + (all >> 16);
+        const int edges = edges_xy | (z == 0 || z == nz - 1 ? 4 : 0);
+        if (total > 0) {   // warp-uniform
+            const bool deep = deep_xy && z >= mz && z < nz - mz;
+            const int pl = (incl & 0xffff) - cl, pr = left + (incl >> 16) - cr;
+            for (int base = 0; base < total; base += QUEUE_CAP) {
+                // this lane's links of direction ql with places in [base, base + QUEUE_CAP)
+                const bool all_fit = total <= QUEUE_CAP;
+#pragma unroll
+                for (int h = 0; h < (ROWS == 1 ? 1 : 2); ++h) {
+                    int pos = (h == 0 ? pl : pr) - base;
+                    const int e0 = (ql << 11) | (((dt.qi[ql] >> 6) & 31) << 6) | (h << 5);
+                    uint32_t m = ROWS == 1 ? link[0]
+                                           : (h == 0 ? __byte_perm(link[0], link[1], 0x5410)
+                                                     : __byte_perm(link[0], link[1], 0x7632));
+                    while (m) {
+                        const int b = 31 - __clz((int)m);
+                        m ^= 1u << b;
+                        if (all_fit || (unsigned)pos < (unsigned)QUEUE_CAP) sm.queue[pos] = (unsigned short)(e0 + b);
+                        ++pos;
+                    }
+                }
+                __syncwarp();
+                // 2. one link per lane; the gathers of the next 32 are under
+                // way while these are worked on
+                const int n = min(total - base, QUEUE_CAP);
+                LinkIn<T> l = fetch(lane, n, z, edges);
+                for (int k0 = 0; k0 < n; k0 += 32) {
+                    const LinkIn<T> cur = l;
+                    if (k0 + 32 < n) l = fetch(k0 + 32 + lane, n, z, edges);
+                    const int q = (cur.e >> 11) & 31, row = (cur.e >> 4) & (ROWS - 1);
+                    const int xb = ROWS == 1 ? cur.e & 31 : (cur.e & 15) | ((cur.e >> 1) & 16);
+                    // solid cells have an owner below np
+                    int key = k0 + lane < n && (unsigned)cur.key < (unsigned)a.np ? cur.key : -1;
+                    do {   // once, but where more particles meet than there are slots
+                        const int slot = find_slot<T>(sm.open, keys, key, a.view, sk, lane);
+                        if (slot >= 0) {
+                            T F[6];
+                            sm.v[q - 1][cur.e & (32 * ROWS - 1)] =
+                                link_value<S>(a, key, sm.open.view[sizeof(T) == 4 ? slot : 0], 32 * wx + xb, y0 + row, z,
+                                              dt.qi[q], dt.cf[q], (cur.e & 0x10000) != 0, !deep, cur.fout, cur.fin,
+                                              cur.fdown, F);
+                            T* p = &sm.open.f[slot][0][lane];
+#pragma unroll
+                            for (int d = 0; d < 6; ++d) p[32 * d] += F[d];
+                            key = -1;
+                        }
+                    } while (__any_sync(FULL, key >= 0));
+                }
+                __syncwarp();   // queue read, values written
+            }
+        }
+        // 3. patch, collide, store
+        if (actA || actB) {
+            const uint32_t me = 1u << lane;
+            const bool patch = total > 0;
+            const bool edge = (edges & wall_axes) != 0;
+            if (edge) {
+                // halfway bounce-back on the box walls (Eq. (14) with delta = 1/2)
 #pragma unroll
                 for (int q = 1; q < Q; ++q) {
-                    const int u0 = x - cx(q), u1 = y - cy(q), u2 = z - cz(q);
-                    int axis = -1, side = 0;
-                    if (wz && (u2 < 0 || u2 >= nz)) { axis = 2; side = u2 < 0 ? 0 : 1; }
-                    else if (wy && (u1 < 0 || u1 >= ny)) { axis = 1; side = u1 < 0 ? 0 : 1; }
-                    else if (wx && (u0 < 0 || u0 >= nx)) { axis = 0; side = u0 < 0 ? 0 : 1; }
-                    if (axis < 0) continue;
                     const int p = opp(q);
-                    const T ucp = a.uw[side][axis][0] * (T)(-cx(q)) + a.uw[side][axis][1] * (T)(-cy(q)) +
-                                  a.uw[side][axis][2] * (T)(-cz(q));
-                    f[q] = Store<S>::load(a.src + p * N + idx) - T(6) * wq<T>(p) * ucp;
-                    lmask &= ~(1u << q);
-                }
-            }
-        }
-        // particle links of the warp, spread evenly over its lanes: each lane
-        // with links queues (direction, lane) entries in shared memory at its
-        // prefix-sum offset
-        if (a.np > 0 && __any_sync(FULL, lmask != 0)) {
-            const int cnt = __popc(lmask);
-            const int incl = warp_incl_scan(cnt, lane);
-            const int total = __shfl_sync(FULL, incl, 31);
-            // the cell's PDFs wait in shared memory (freeing their registers for
-            // the link work); each link's CLI value lands in its cell's slot
+                    T g[ROWS];
+                    P::get(f[q], g);
 #pragma unroll
-            for (int q = 0; q < Q; ++q) s_f[q][tid] = f[q];
-            // entries q | lane << 8
-            unsigned short* queue = s_queue[tid >> 5];
-            {
-                unsigned mm = lmask;
-                int pos = incl - cnt;
-                while (mm) {
-                    const int q = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    queue[pos++] = (unsigned short)(q | (lane << 8));
-                }
-            }
-            __syncwarp();
-            Acc<T> acc;
-            load_sums<T>(acc, s_key, s_sum, s_int, tid);
-            // lane l takes the m consecutive entries l m .. l m + m - 1
-            const int m = (total + 31) >> 5;
-            for (int j = 0; j < m; ++j) {
-                const int k = lane * m + j;
-                const unsigned e = k < total ? queue[k] : 0u;
-                const int q = (int)(e & 31u), src = (int)(e >> 8);
-                const unsigned lm_src = __shfl_sync(FULL, lmask, src);
-                if (k < total) {
-                    const int st = tid - lane + src;
-                    const int qi = s_qi[q];
-                    // the particle from the marker's payload, still in the slot
-                    // (0: look it up in the owner array)
-                    int key1 = 0;
-                    if constexpr (sizeof(S) >= 4) key1 = marker_owner(s_f[q][st]) + 1;
-                    // f_p pulled by the same cell: f~_p(x + c_q) (read before any
-                    // link of direction p could overwrite it; such a link makes
-                    // x + c_q solid and its value unused)
-                    const T fdown_raw = s_f[(qi >> 6) & 31][st];
-                    s_f[q][st] = link_value<S, T>(a, x - lane + src, y, z, q, qi, key1, lm_src, fdown_raw, acc, sk);
-                }
-            }
-            store_sums<T>(acc, s_key, s_sum, s_int, tid, sk);
-            open = true;
-            __syncwarp();
+                    for (int r = 0; r < ROWS; ++r) {
+                        // upstream outside: direction +1 from the low face, -1 from the high one
+                        const bool oz = cz(q) && !a.g.per[2] && z == (cz(q) > 0 ? 0 : nz - 1);
+                        const bool oy = cy(q) && !a.g.per[1] && y0 + r == (cy(q) > 0 ? 0 : ny - 1);
+                        const bool ox = cx(q) && !a.g.per[0] && xl == (cx(q) > 0 ? 0 : nx - 1);
+                        if (!(oz || oy || ox)) continue;
+                        T ucp = T(0);   // c_p . u_wall, the z face before the y face before the x face
 #pragma unroll
-            for (int q = 0; q < Q; ++q) f[q] = s_f[q][tid];
+                        for (int d = 0; d < 3; ++d) {
+                            const int cd = d == 0 ? cx(q) : (d == 1 ? cy(q) : cz(q));
+                            const T uz = a.uw[cz(q) > 0 ? 0 : 1][2][d], uy = a.uw[cy(q) > 0 ? 0 : 1][1][d],
+                                    ux = a.uw[cx(q) > 0 ? 0 : 1][0][d];
+                            ucp += (oz ? uz : (oy ? uy : ux)) * (T)(-cd);
+                        }
+                        g[r] = Store<S>::load(a.src[p] + (zoff[1] + yo[1 + r] + xl)) - T(6) * wq<T>(p) * ucp;
+                    }
+                    f[q] = P::make(g);
+                }
+            }
+            if (patch) {
+#pragma unroll
+                for (int q = 1; q < Q; ++q) {
+                    T g[ROWS];
+                    P::get(f[q], g);
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r)
+                        patch_link(g[r], sm.w[q][r] & me, &sm.v[q - 1][cell_of<T>(lane) + 16 * r]);
+                    f[q] = P::make(g);
+                }
+            }
+            bool sh[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) sh[r] = (sm.w[Q + 1][r] & me) != 0u;
+            T dr[ROWS];
+            P::get(collide_core<T>(f, sh, ax, ay, az, a.s_plus, a.s_minus, a.ke, a.ko, a.s_b_shell, a.s_b_bulk,
+                                   a.bulk_corr),
+                   dr);
+            bool stable = true;
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                if ((fluid[r] & me) && !(dr[r] < T(0.5) && dr[r] > T(-0.5))) stable = false;
+            if (!stable) atomicOr(a.status, ST_UNSTABLE);
+            const int iA = zoff[1] + yo[1] + xl, iB = zoff[1] + yo[ROWS] + xl;
+            const bool stA = actA && x < nx, stB = actB && x < nx;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                T g[ROWS];
+                P::get(f[q], g);
+                if (stA) Store<S>::store(a.dst[q] + iA, g[0]);
+                if (ROWS > 1 && stB) Store<S>::store(a.dst[q] + iB, g[ROWS - 1]);
+            }
         }
-        // solid cells store nothing: their slots keep the marker of the mapping
-        if (fluid) {
-            collide_store<S, T>(a, f, fl, N, idx);
-        }
-
     }
-    if (open) {   // warp-uniform
-        Acc<T> acc;
-        load_sums<T>(acc, s_key, s_sum, s_int, tid);
-        commit<T>(acc, sk);
-    }
+    commit_open<T>(sm.open, keys, sk, lane);
 }
 
-
-// link codes of the directions into shared memory (before the first tile)
-__device__ __forceinline__ void load_qinfo(int* s_qi) {
-    const int t = threadIdx.x + blockDim.x * threadIdx.y;
-    if (t < Q) {
-        constexpr int QI[Q] = {qinfo(0), qinfo(1), qinfo(2), qinfo(3), qinfo(4), qinfo(5), qinfo(6),
+__constant__ int k_qinfo[Q] = {qinfo(0), qinfo(1), qinfo(2), qinfo(3), qinfo(4), qinfo(5), qinfo(6),
                                qinfo(7), qinfo(8), qinfo(9), qinfo(10), qinfo(11), qinfo(12), qinfo(13),
                                qinfo(14), qinfo(15), qinfo(16), qinfo(17), qinfo(18)};
-        s_qi[t] = QI[t];
+
+// the direction table into shared memory (before the first tile)
+template <typename S, typename T>
+__device__ __forceinline__ void load_dirs(DirTable<S>& dt, const SCArgs<S, T>& a) {
+    const int t = threadIdx.x;
+    if (t < Q) {
+        const int qi = k_qinfo[t];
+        const float c0 = (float)((qi & 3) - 1), c1 = (float)(((qi >> 2) & 3) - 1), c2_ = (float)(((qi >> 4) & 3) - 1);
+        dt.qi[t] = qi;
+        dt.dq[t] = (qi & 3) - 1 + (((qi >> 2) & 3) - 1) * a.g.n[0] + (((qi >> 4) & 3) - 1) * a.g.n[0] * a.g.n[1];
+        dt.src[t] = a.src[t];
+        dt.cf[t] = make_float4(-c0, -c1, -c2_, c0 * c0 + c1 * c1 + c2_ * c2_);
     }
 }
 
-// One box: block (bx, 256 / bx) tiles from blockIdx.x, blockIdx.y, a chunk of
-// a.zchunk planes from blockIdx.z.
+// the warp of a tile of bx x (SC_WARPS ROWS 32 / bx) cells at (x0, y0)
 template <typename S, typename T>
-__global__ void __launch_bounds__(256, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
-    stream_collide_kernel(const SCArgs<S, T> a) {
-    extern __shared__ __align__(16) unsigned char sc_smem[];
-    __shared__ int s_qi[Q];
-    load_qinfo(s_qi);
+__device__ __forceinline__ void sc_tile(const SCArgs<S, T>& a, int x0, int y0, int z_begin, SCWarp<T>* sm,
+                                        const DirTable<S>& dt) {
+    // opaque, or the compiler derives them from special registers again and again
+    int warp, wx, y;
+    asm volatile("mov.u32 %0, %1;" : "=r"(warp) : "r"((int)threadIdx.x >> 5));
+    const int across = a.bx >> 5;                       // 1, 2 or 4 warps along x
+    asm volatile("mov.u32 %0, %1;" : "=r"(wx) : "r"((x0 >> 5) + (warp & (across - 1))));
+    asm volatile("mov.u32 %0, %1;"
+                 : "=r"(y)
+                 : "r"(y0 + Pack<T>::ROWS * (across == 1 ? warp : (across == 2 ? warp >> 1 : 0))));
+    if (wx < a.words && y < a.g.n[1])
+        sc_warp<S, T>(a, wx, y, z_begin, min(a.g.n[2], z_begin + a.zchunk), sm[warp], dt);
+}
+
+// One box: block (x, y) tiles, a chunk of a.zchunk planes from blockIdx.z.
+template <typename S, typename T>
+__global__ void __launch_bounds__(32 * SC_WARPS, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
+    stream_collide_kernel(const __grid_constant__ SCArgs<S, T> a) {
+    __shared__ SCWarp<T> sm[SC_WARPS];
+    __shared__ DirTable<S> dt;
+    load_dirs<S, T>(dt, a);
     __syncthreads();
-    const int z_begin = blockIdx.z * a.zchunk;
-    sc_tile<S, T, false>(a, 0, 0, z_begin, min(a.g.n[2], z_begin + a.zchunk), (int)blockDim.x, sc_smem, s_qi);
+    sc_tile<S, T>(a, blockIdx.x * a.bx, blockIdx.y * sc_tile_rows(sizeof(S), a.bx), blockIdx.z * a.zchunk, sm, dt);
 }
 
 // Many boxes in one persistent launch: block b takes the work items b,
 // b + gridDim.x, ... of the table (instance, x0, y0, z0), copies the
 // arguments of the item's instance into shared memory and runs its tile
-// (a.bx x 256 / a.bx cells, a.zchunk planes from z0).
+// (a.zchunk planes from z0).
 template <typename S, typename T>
-__global__ void __launch_bounds__(256, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
+__global__ void __launch_bounds__(32 * SC_WARPS, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
     stream_collide_batch_kernel(const SCArgs<S, T>* __restrict__ args, const int4* __restrict__ items, int n_items) {
-    extern __shared__ __align__(16) unsigned char sc_smem[];
-    __shared__ int s_qi[Q];
+    __shared__ SCWarp<T> sm[SC_WARPS];
+    __shared__ DirTable<S> dt;
     __shared__ __align__(16) SCArgs<S, T> s_a;
-    load_qinfo(s_qi);
     constexpr int WORDS = (int)(sizeof(SCArgs<S, T>) / 4);
     static_assert(sizeof(SCArgs<S, T>) % 4 == 0, "argument block copied in words");
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -285,15 +456,33 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : 
         int* dst = reinterpret_cast<int*>(&s_a);
         for (int w = threadIdx.x; w < WORDS; w += blockDim.x) dst[w] = src[w];
         __syncthreads();
-        sc_tile<S, T, true>(s_a, item.y, item.z, item.w, min(s_a.g.n[2], item.w + s_a.zchunk), s_a.bx, sc_smem,
-                            s_qi);
+        load_dirs<S, T>(dt, s_a);
+        __syncthreads();
+        sc_tile<S, T>(s_a, item.y, item.z, item.w, sm, dt);
     }
 }
 
-// bytes of dynamic shared memory of the kernel (256 threads)
-template <typename T>
-constexpr size_t sc_smem_bytes() {
-    return (Q + 6) * 256 * sizeof(T) + (sizeof(T) == 4 ? 3 * 256 * 4 : 0) + 256 * 4 + 8 * 32 * (Q - 1) * 2;
+// Tile width of a box nx cells wide: 4, 2 or 1 words of 32 cells, the widest
+// that leaves at most an eighth of the warps idle at the end of a row
+// (neighbouring warps of a block share the sectors their shifted pulls overlap in).
+int default_tile_bx(int nx) {
+    const int W = (nx + 31) / 32;
+    int best = 1;
+    for (int b : {2, 4})
+        if (8 * ((W + b - 1) / b * b) <= 9 * W) best = b;
+    return 32 * best;
+}
+
+// Planes a warp marches: as many as leave about 4 blocks of 256 cells per SM,
+// beyond 8 only while 8 times as many blocks are left (longer marches commit
+// fewer force sums: 256 x 256 x 512 cells 1400 us with 8 planes, 1366 us with
+// 16; but 128 x 128 x 256 cells 216 and 226 us, the last wave being emptier).
+static int default_zchunk(int nx, int ny, int nz, int sms) {
+    const int bx = nx >= 128 ? 128 : (nx + 31) / 32 * 32, by = 256 / bx;
+    const long long bxy = (long long)((nx + bx - 1) / bx) * ((ny + by - 1) / by);
+    const long long zc = bxy * nz / (4LL * sms);
+    if (zc <= 8) return zc < 1 ? 1 : (int)zc;
+    return zc / 8 < 8 ? 8 : (zc / 8 > LBM_SC_ZCHUNK ? LBM_SC_ZCHUNK : (int)(zc / 8));
 }
 
 template <typename S>
@@ -302,20 +491,12 @@ void launch_stream_collide_t(const LbmStepParams& p, cudaStream_t st) {
     SCArgs<S, T> a;
     fill_sc_args<S, T>(p, a);
     const int nx = p.g.n[0];
-    int bx = nx >= LBM_SC_BX ? LBM_SC_BX : ((nx + 31) / 32) * 32;
-    if (p.tile_bx > 0) bx = p.tile_bx;
-    int by = 256 / bx;
-    a.bx = bx;
-    dim3 block(bx, by, 1);
-    const int bxy = ((nx + bx - 1) / bx) * ((p.g.n[1] + by - 1) / by);
-    // at least 4 blocks per SM where the box allows, else shorter chunks
-    const long long want = 4LL * (p.num_sms > 0 ? p.num_sms : 152);
-    int zc = (int)((long long)bxy * p.g.n[2] / want);
-    a.zchunk = zc < 1 ? 1 : (zc > LBM_SC_ZCHUNK ? LBM_SC_ZCHUNK : zc);
-    if (p.zchunk > 0) a.zchunk = p.zchunk;
-    dim3 grid((nx + bx - 1) / bx, (p.g.n[1] + by - 1) / by, (p.g.n[2] + a.zchunk - 1) / a.zchunk);
-    constexpr size_t smem = sc_smem_bytes<T>();
-    stream_collide_kernel<S, T><<<grid, block, smem, st>>>(a);
+    a.bx = default_tile_bx(nx);
+    while (p.g.n[1] > 65535 * sc_tile_rows(sizeof(S), a.bx)) a.bx /= 2;   // grid limit in y
+    const int by = sc_tile_rows(sizeof(S), a.bx);
+    a.zchunk = default_zchunk(nx, p.g.n[1], p.g.n[2], p.num_sms > 0 ? p.num_sms : 152);
+    dim3 grid((nx + a.bx - 1) / a.bx, (p.g.n[1] + by - 1) / by, (p.g.n[2] + a.zchunk - 1) / a.zchunk);
+    stream_collide_kernel<S, T><<<grid, 32 * SC_WARPS, 0, st>>>(a);
 }
 
 // ------------------------------------------------------------ batched launch
@@ -324,6 +505,7 @@ template <typename S>
 static void fill_batch_args_t(const LbmStepParams& p, int tile_bx, int zchunk, void* out) {
     using T = typename Store<S>::T;
     SCArgs<S, T> a;
+    std::memset(&a, 0, sizeof(a));
     fill_sc_args<S, T>(p, a);
     a.bx = tile_bx;
     a.zchunk = zchunk;
@@ -348,14 +530,11 @@ void fill_batch_args(const LbmStepParams& p, int tile_bx, int zchunk, void* out)
     }
 }
 
-int default_tile_bx(int nx) { return nx >= LBM_SC_BX ? LBM_SC_BX : ((nx + 31) / 32) * 32; }
-
 template <typename S>
 static void launch_batch_t(const void* d_args, const int4* d_items, int n_items, int grid, cudaStream_t st) {
     using T = typename Store<S>::T;
-    constexpr size_t smem = sc_smem_bytes<T>();
     stream_collide_batch_kernel<S, T>
-        <<<grid, 256, smem, st>>>(static_cast<const SCArgs<S, T>*>(d_args), d_items, n_items);
+        <<<grid, 32 * SC_WARPS, 0, st>>>(static_cast<const SCArgs<S, T>*>(d_args), d_items, n_items);
 }
 
 void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, int grid,
@@ -368,38 +547,7 @@ void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_
     }
 }
 
-template <typename S>
-cudaError_t prepare_t() {
-    using T = typename Store<S>::T;
-    constexpr size_t smem = sc_smem_bytes<T>();
-    if (smem <= 48 * 1024) return cudaSuccess;
-    // float64 storage: above the default dynamic shared memory limit
-    cudaError_t e =
-        cudaFuncSetAttribute(stream_collide_kernel<S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(stream_collide_batch_kernel<S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-}
-
-cudaError_t prepare_stream_collide(int storage) {
-    cudaError_t e;
-    switch (storage) {
-        case 0: e = prepare_t<double>(); break;
-        case 1: e = prepare_t<float>(); break;
-        case 2: e = prepare_t<__half>(); break;
-        default: e = prepare_t<__nv_bfloat16>(); break;
-    }
-    return e == cudaSuccess ? prepare_stream_collide_staged(storage) : e;
-}
-
 void launch_stream_collide(const LbmStepParams& p, cudaStream_t st) {
-    // on request, for 4- and 2-byte formats on boxes whose rows start on
-    // 16-byte boundaries: the kernel with bulk-copy staging
-    // (stream_collide_staged.cu)
-    if (p.use_staged && staged_applicable(p)) {
-        launch_stream_collide_staged(p, st);
-        return;
-    }
     switch (p.storage) {
         case 0: launch_stream_collide_t<double>(p, st); break;
         case 1: launch_stream_collide_t<float>(p, st); break;
@@ -407,6 +555,5 @@ void launch_stream_collide(const LbmStepParams& p, cudaStream_t st) {
         default: launch_stream_collide_t<__nv_bfloat16>(p, st); break;
     }
 }
-
 
 }  // namespace lbmdem
