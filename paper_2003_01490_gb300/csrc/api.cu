@@ -51,6 +51,8 @@ struct lbm_ctx {
     int* status = nullptr;
     double* accel = nullptr;
     float* accel_f = nullptr;
+    unsigned* barrier = nullptr;   // of the cooperative DEM launch
+    int grid_particles = 0;        // particles a cooperative DEM launch holds
     uint32_t* solid = nullptr;     // one bit per cell (see launch.h)
     uint32_t* shell = nullptr;
     unsigned int* miss_list = nullptr;
@@ -263,6 +265,7 @@ void build_layout(const lbm_grid* g, lbm_storage st, int np, Layout& L, const Si
     const size_t words = (size_t)((g->nx + 31) / 32) * g->ny * g->nz;
     L.add(4 * words);                            // 62 solid
     L.add(4 * words);                            // 63 shell
+    L.add(4);                                    // 64 barrier
 }
 
 lbm_status validate(const lbm_grid* g, const lbm_relax* r, const lbm_dem* d, lbm_storage st,
@@ -311,7 +314,8 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
             ctx->num_sms = sms;
-        cudaError_t pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
+        cudaError_t pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
+        if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
         if (pe != cudaSuccess) {
@@ -382,6 +386,7 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
     ctx->miss_list = (unsigned int*)at(47);
     ctx->solid = (uint32_t*)at(62);
     ctx->shell = (uint32_t*)at(63);
+    ctx->barrier = (unsigned*)at(64);
     ctx->miss_cap = (int)s.ncells;
     ctx->P.acc_k = (long long*)at(49);
     ctx->P.xs[1] = (double*)at(50);
@@ -483,13 +488,17 @@ MapParams map_params(lbm_ctx* ctx) {
 }
 
 // remap all particles: clear tile lists and counters, scatter, map
-lbm_status remap(lbm_ctx* ctx, cudaStream_t sm) {
-    // tile counts are zero here: the mapping kernel resets each one it reads
-    CK(cudaMemsetAsync(ctx->n_solid, 0, 16, sm));
+// (scattered: the first two are done)
+lbm_status remap(lbm_ctx* ctx, cudaStream_t sm, bool scattered) {
     MapParams mp = map_params(ctx);
-    launch_tile_scatter(mp, sm);
+    if (!scattered) {
+        // tile counts are zero here: the mapping kernel resets each one it reads
+        CK(cudaMemsetAsync(ctx->n_solid, 0, 16, sm));
+        launch_tile_scatter(mp, sm);
+        ctx->launches += ctx->P.n > 0 ? 1 : 0;
+    }
     launch_map(mp, sm);
-    ctx->launches += (ctx->P.n > 0 ? 1 : 0) + 1;
+    ctx->launches += 1;
     return LBM_OK;
 }
 
@@ -541,6 +550,7 @@ DemParams dem_params(lbm_ctx* ctx) {
     dp.tangential = d.tangential_lubrication;
     dp.dt = 1.0 / d.n_sub;
     dp.status = ctx->status;
+    dp.barrier = ctx->barrier;
     dp.pair_f32 = ctx->storage != LBM_STORE_F64;
     fill_consts(dp, dp.kd);
     fill_consts(dp, dp.kf);
@@ -577,6 +587,7 @@ lbm_status check_status(lbm_ctx* ctx) {
         std::snprintf(buf, sizeof buf, "device list capacity exceeded (status bits 0x%x)", st);
         return fail(ctx, LBM_ERR_CAPACITY, buf);
     }
+    if (st & ST_TIMEOUT) return fail(ctx, LBM_ERR_TIMEOUT, "a barrier of the DEM launch ran out");
     if (st & ST_FAST_PARTICLE) return fail(ctx, LBM_ERR_UNSTABLE, "particle speed above 0.5 cells per step");
     return LBM_OK;
 }
@@ -781,7 +792,7 @@ lbm_status lbm_add_spheres(lbm_ctx* ctx, int n, const double* pos, const double*
     ctx->hR.swap(hR);
     launch_view_update(P, sm);
     ctx->launches += 1;
-    lbm_status s = remap(ctx, ctx->stream);
+    lbm_status s = remap(ctx, ctx->stream, false);
     if (s != LBM_OK) return s;
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(sm));
@@ -803,6 +814,7 @@ struct StepState {
     bool first = false;
     bool move = false;
     bool dem = false;
+    bool one_launch = false;   // the DEM launch also finalises the forces and scatters the tiles
 };
 
 // parameters of the step's boundary and dense kernels from the context state
@@ -927,13 +939,19 @@ lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepStat
     fpp.use_fixed = ctx->storage != LBM_STORE_F64;
     fpp.first_step = first;
     fpp.averaging = d.force_averaging;
-    launch_finalize(fpp, sm);
-    ctx->launches += 2 + (ctx->P.n > 0 ? 1 : 0);
+    // the DEM step takes the finalisation and the mapping's tile scatter with
+    // it where its particles fit one launch
+    ss.one_launch = dem && (ctx->P.n <= DEM_ONE_BLOCK_MAX || ctx->P.n <= ctx->grid_particles);
+    ctx->launches += 2;
+    if (!ss.one_launch) {
+        launch_finalize(fpp, sm);
+        ctx->launches += ctx->P.n > 0 ? 1 : 0;
+    }
     CK(prof_mark(ctx));
     if (move) {
-        if (dem && ctx->P.n <= DEM_ONE_BLOCK_MAX) {
-            // Algorithm 1, lines 4-10, in one block: few particles
-            launch_dem_step_one_block(dp, ctx->hcur, d.n_sub, sm);
+        if (ss.one_launch) {
+            // Algorithm 1, lines 4-10, in one launch
+            CK(launch_dem_step(dp, fpp, map_params(ctx), ctx->hcur, d.n_sub, sm));
             ctx->launches += 1;
             if (d.n_sub & 1) ctx->hcur = 1 - ctx->hcur;
         } else if (dem) {
@@ -970,7 +988,7 @@ lbm_status enqueue_post_b(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, const St
     if (ss.move) {
         CK(prof_mark(ctx));
         // Algorithm 1, line 11: mapping update and refill
-        lbm_status st = remap(ctx, sm);
+        lbm_status st = remap(ctx, sm, ss.one_launch);
         if (st != LBM_OK) return st;
         CK(prof_mark(ctx));
         RefillParams rp{};
@@ -1637,7 +1655,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
                 ge.p.hout = 1 - hc;
                 ge.cur = cur;
                 ge.last = k == d.n_sub - 1;
-                sub[k].add(&ge, (np + DEM_ONE_BLOCK_MAX - 1) / DEM_ONE_BLOCK_MAX);
+                sub[k].add(&ge, (np + DEM_BLOCK_PARTICLES - 1) / DEM_BLOCK_PARTICLES);
                 hc = 1 - hc;
                 cur = 1 - cur;
             }

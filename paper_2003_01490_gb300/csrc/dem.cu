@@ -7,18 +7,18 @@
 // float64 PDF storage and in float32 (separations and overlaps from float64
 // positions) for the other formats.
 //
-// Each particle gathers every interaction of its own (its block evaluates
-// the queued pairs with all threads, then sums them per particle in slot
-// order), so no force atomics are needed; a pair is evaluated by both
-// partners with mirrored operands (n_ji = -n_ij, u_ji = -u_ij, ...). Each
-// particle keeps its own copy of the tangential spring of every active
-// contact (double buffered per subcycle). Up to 32 particles run a whole
-// step's subcycles in one block.
+// Each particle gathers every interaction of its own with eight lanes, so no
+// force atomics are needed; a pair is evaluated by both partners with mirrored
+// operands (n_ji = -n_ij, u_ji = -u_ij, ...). Each particle keeps its own copy of
+// the tangential spring of every active contact (double buffered per
+// subcycle). All subcycles of a step run in one launch: one block for up to 32
+// particles, a cooperative launch as long as its blocks fit the GPU at once.
 #include <cstring>
 
 #include "common.cuh"
 #include "gang.cuh"
 #include "launch.h"
+#include "scatter.cuh"
 
 namespace lbmdem {
 
@@ -36,13 +36,20 @@ template <typename T>
 __device__ __forceinline__ Vec3<T> operator-(Vec3<T> a, Vec3<T> b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 template <typename T>
 __device__ __forceinline__ Vec3<T> operator-(Vec3<T> a) { return {-a.x, -a.y, -a.z}; }
+// Products and multiply-adds of the interaction laws are written out, so that
+// every kernel they are compiled into rounds them alike (a batch then ends where
+// its instances end alone).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 template <typename T>
-__device__ __forceinline__ Vec3<T> operator*(T s, Vec3<T> a) { return {s * a.x, s * a.y, s * a.z}; }
+__device__ __forceinline__ Vec3<T> operator*(T s, Vec3<T> a) { return {mul_rn(s, a.x), mul_rn(s, a.y), mul_rn(s, a.z)}; }
 template <typename T>
-__device__ __forceinline__ T dot(Vec3<T> a, Vec3<T> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+__device__ __forceinline__ T dot(Vec3<T> a, Vec3<T> b) { return mad(a.z, b.z, mad(a.x, b.x, mul_rn(a.y, b.y))); }
 template <typename T>
 __device__ __forceinline__ Vec3<T> cross(Vec3<T> a, Vec3<T> b) {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+    return {mad(a.y, b.z, -mul_rn(a.z, b.y)), mad(a.z, b.x, -mul_rn(a.x, b.z)), mad(a.x, b.y, -mul_rn(a.y, b.x))};
 }
 __device__ __forceinline__ V3 ld3(const double* p, int i) { return {p[3 * i], p[3 * i + 1], p[3 * i + 2]}; }
 __device__ __forceinline__ Vec3<float> ld3(const float* p, int i) { return {p[3 * i], p[3 * i + 1], p[3 * i + 2]}; }
@@ -115,49 +122,64 @@ void launch_view_update(const Particles& P, cudaStream_t st) {
 // per particle: the step's hydrodynamic force and torque (Eqs. (16)-(17)) from
 // the float64 or fixed-point link sums and the exact integer missing-link
 // sums, their two-step average (Sec. 4.2), and the accumulators cleared
-__device__ __forceinline__ void finalize_body(const FinalizeParams& p, int bx) {
-    const int i = bx * blockDim.x + threadIdx.x;
-    if (i >= p.P.n) return;
-    double exact[6] = {0, 0, 0, 0, 0, 0};
+// (component c of particle i)
+__device__ __forceinline__ void finalize_component(const FinalizeParams& p, int i, int c) {
+    double v;
     if (p.use_fixed) {
-        // constant link parts summed exactly by the float32 boundary kernel:
+        // constant link parts, exact integers (see boundary.cu):
         // K = 36 sum 2 w c and 36 sum 2 w (n x c); torque adds g x (K / 36)
         // with g = 1/2 - (x - floor(x)) the common fractional cell offset
         // (two components per word: lo + hi 2^32)
-        double k[6], g[3];
-        for (int c2 = 0; c2 < 3; ++c2) {
-            const unsigned long long w = (unsigned long long)p.P.acc_k[3 * i + c2];
-            const long long lo = (long long)(int)(unsigned)(w & 0xffffffffull);
-            const long long hi = (long long)(w - (unsigned long long)lo) >> 32;
-            k[2 * c2] = (double)lo * (1.0 / 36.0);
-            k[2 * c2 + 1] = (double)hi * (1.0 / 36.0);
-            p.P.acc_k[3 * i + c2] = 0;
+        const unsigned long long w = (unsigned long long)p.P.acc_k[3 * i + (c >> 1)];
+        const long long lo = (long long)(int)(unsigned)(w & 0xffffffffull);
+        const long long k = c & 1 ? (long long)(w - (unsigned long long)lo) >> 32 : lo;
+        double exact = __dmul_rn((double)k, 1.0 / 36.0);
+        if (c >= 3) {
+            const int a = (c - 2) % 3, b = (c - 1) % 3;   // cross product axes
+            double kf[2], g[2];
+            for (int e = 0; e < 2; ++e) {
+                const int d = e == 0 ? a : b;
+                const unsigned long long wd = (unsigned long long)p.P.acc_k[3 * i + (d >> 1)];
+                const long long lod = (long long)(int)(unsigned)(wd & 0xffffffffull);
+                kf[e] = (double)(d & 1 ? (long long)(wd - (unsigned long long)lod) >> 32 : lod) * (1.0 / 36.0);
+                const double x = p.P.x[3 * i + d];
+                g[e] = 0.5 - (x - floor(x));
+            }
+            exact += fma(g[0], kf[1], -__dmul_rn(g[1], kf[0]));
         }
-        for (int d = 0; d < 3; ++d) {
-            const double x = p.P.x[3 * i + d];
-            g[d] = 0.5 - (x - floor(x));
-        }
-        exact[0] = k[0];
-        exact[1] = k[1];
-        exact[2] = k[2];
-        exact[3] = k[3] + (g[1] * k[2] - g[2] * k[1]);
-        exact[4] = k[4] + (g[2] * k[0] - g[0] * k[2]);
-        exact[5] = k[5] + (g[0] * k[1] - g[1] * k[0]);
+        v = fma((double)p.P.acc_i[6 * i + c], 1.0 / FIX_SCALE, exact);
+    } else {
+        v = p.P.acc_d[6 * i + c];
     }
-    for (int c = 0; c < 6; ++c) {
-        double v;
-        if (p.use_fixed) {
-            v = (double)p.P.acc_i[6 * i + c] * (1.0 / FIX_SCALE) + exact[c];
-            p.P.acc_i[6 * i + c] = 0;
-        } else {
-            v = p.P.acc_d[6 * i + c];
-            p.P.acc_d[6 * i + c] = 0.0;
-        }
-        const double old = p.first_step ? v : p.P.fp_old[6 * i + c];
-        p.P.fp[6 * i + c] = v;
-        p.P.fbar[6 * i + c] = p.averaging ? 0.5 * (v + old) : v;
-        p.P.fp_old[6 * i + c] = v;
+    const double old = p.first_step ? v : p.P.fp_old[6 * i + c];
+    p.P.fp[6 * i + c] = v;
+    p.P.fbar[6 * i + c] = p.averaging ? 0.5 * (v + old) : v;
+    p.P.fp_old[6 * i + c] = v;
+}
+
+// the accumulators cleared (after every component has been read)
+__device__ __forceinline__ void finalize_clear(const FinalizeParams& p, int i, int c) {
+    if (p.use_fixed) {
+        p.P.acc_i[6 * i + c] = 0;
+        if (c < 3) p.P.acc_k[3 * i + c] = 0;
+    } else {
+        p.P.acc_d[6 * i + c] = 0.0;
     }
+}
+
+__device__ __forceinline__ void finalize_body(const FinalizeParams& p, int bx) {
+    const int i = bx * blockDim.x + threadIdx.x;
+    if (i >= p.P.n) return;
+    for (int c = 0; c < 6; ++c) finalize_component(p, i, c);
+    for (int c = 0; c < 6; ++c) finalize_clear(p, i, c);
+}
+
+// lane s (0-5) of the particle's eight takes component s
+__device__ __forceinline__ void finalize_lane(const FinalizeParams& p, int i, int s) {
+    const bool on = i < p.P.n && s < 6;
+    if (on) finalize_component(p, i, s);
+    __syncwarp();
+    if (on) finalize_clear(p, i, s);
 }
 
 __global__ void finalize_kernel(const FinalizeParams p) { finalize_body(p, (int)blockIdx.x); }
@@ -220,6 +242,7 @@ __device__ __forceinline__ void neighbour_body(const DemParams& p, int bx) {
     static_assert(BIN_CAP == 32, "one lane per bin entry");
     const int i = (bx * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    if (bx == 0 && threadIdx.x == 0) *p.barrier = 0u;   // for the step's DEM launch
     if (i >= p.P.n) return;   // warp-uniform
     const unsigned FULL = 0xffffffffu;
     const float xi[3] = {p.P.xf[3 * i], p.P.xf[3 * i + 1], p.P.xf[3 * i + 2]};
@@ -381,7 +404,7 @@ __device__ void lubrication_on_i(const DemConsts<T>& k, int tangential, T Ri, T 
         const T i1 = T(1) / k1;
         const T i2 = i1 * i1;
         c_n = kr * kr * i2;
-        c_ftt = T(4) * kr * (T(2) + kr + T(2) * kr * kr) * (i2 * i1) * T(1.0 / 15.0);
+        c_ftt = T(4) * kr * mad(T(2) * kr, kr, T(2) + kr) * (i2 * i1) * T(1.0 / 15.0);
         c_ttt = kr * (T(4) + kr) * i2 * T(0.1);
         c_ftr = T(2) * kr * kr * i2 * T(1.0 / 15.0);
         c_ttr = T(2) * kr * i1 * T(0.2);
@@ -450,6 +473,44 @@ __device__ __forceinline__ double image_shift(float d, int n, int per) {
     return 0.0;
 }
 
+// Loads of particle state that other threads of the launch write between the
+// subcycles: CG from L2 (other multiprocessors' writes never reach this one's
+// L1), else plain.
+template <bool CG, typename U>
+__device__ __forceinline__ U ld_state(const U* p) {
+    if constexpr (CG) return __ldcg(p);
+    else return *p;
+}
+template <bool CG, typename U>
+__device__ __forceinline__ Vec3<U> ld3s(const U* p, int i) {
+    return {ld_state<CG>(p + 3 * i), ld_state<CG>(p + 3 * i + 1), ld_state<CG>(p + 3 * i + 2)};
+}
+
+// a neighbour's state and the own one as a pair law reads them
+template <typename T>
+struct PairState {
+    V3 xi, xj;
+    Vec3<float> xfi, xfj;
+    Vec3<T> ui, uj, omi, omj;
+};
+
+template <typename T, bool CG>
+__device__ __forceinline__ PairState<T> load_pair(const Particles& P, int cur, int i, int j) {
+    PairState<T> s;
+    s.xfi = ld3s<CG>(P.xfs[cur], i);
+    s.xfj = ld3s<CG>(P.xfs[cur], j);
+    s.xi = ld3s<CG>(P.xs[cur], i);
+    s.xj = ld3s<CG>(P.xs[cur], j);
+    if constexpr (sizeof(T) == 8) {
+        s.ui = ld3s<CG>(P.us[cur], i); s.omi = ld3s<CG>(P.oms[cur], i);
+        s.uj = ld3s<CG>(P.us[cur], j); s.omj = ld3s<CG>(P.oms[cur], j);
+    } else {
+        s.ui = ld3s<CG>(P.ufs[cur], i); s.omi = ld3s<CG>(P.omfs[cur], i);
+        s.uj = ld3s<CG>(P.ufs[cur], j); s.omj = ld3s<CG>(P.omfs[cur], j);
+    }
+    return s;
+}
+
 // Force and torque on particle i from its neighbour j (lubrication,
 // Eqs. (25)-(33), and contact, Eqs. (39)-(50)) at the subcycle's positions;
 // contact = the spring of the pair continues, dnew its new value. T = double:
@@ -457,33 +518,30 @@ __device__ __forceinline__ double image_shift(float d, int n, int per) {
 // float64 (the overlap delta = that / (|d| + Ri + Rj) keeps float32 relative
 // accuracy), the interaction laws in float32.
 template <typename T>
-__device__ __forceinline__ void pair_force(const DemParams& p, int cur, int hin, int i, int j, Vec3<T>& F,
+__device__ __forceinline__ void pair_force(const DemParams& p, const PairState<T>& s, int hin, int i, int j, Vec3<T>& F,
                                            Vec3<T>& Tq, bool& contact, Vec3<T>& dnew) {
     const Particles& P = p.P;
     const DemConsts<T>& k = consts<T>(p);
-    const double* X = P.xs[cur];
-    const V3 xi = ld3(X, i), xj = ld3(X, j);
     Vec3<T> d;
     T dist, delta, Ri, Rj;
     if constexpr (sizeof(T) == 8) {
-        d = mk(mimg(xi.x - xj.x, p.g.n[0], p.g.per[0]), mimg(xi.y - xj.y, p.g.n[1], p.g.per[1]),
-               mimg(xi.z - xj.z, p.g.n[2], p.g.per[2]));
+        d = mk(mimg(s.xi.x - s.xj.x, p.g.n[0], p.g.per[0]), mimg(s.xi.y - s.xj.y, p.g.n[1], p.g.per[1]),
+               mimg(s.xi.z - s.xj.z, p.g.n[2], p.g.per[2]));
         dist = sqrt(dot(d, d));
         Ri = P.R[i];
         Rj = P.R[j];
         delta = dist - (Ri + Rj);
     } else {
-        const float* Xf = P.xfs[cur];
-        V3 dd = xi - xj;
-        dd.x += image_shift(Xf[3 * i] - Xf[3 * j], p.g.n[0], p.g.per[0]);
-        dd.y += image_shift(Xf[3 * i + 1] - Xf[3 * j + 1], p.g.n[1], p.g.per[1]);
-        dd.z += image_shift(Xf[3 * i + 2] - Xf[3 * j + 2], p.g.n[2], p.g.per[2]);
-        const double S = P.R[i] + P.R[j];
+        V3 dd = s.xi - s.xj;
+        dd.x += image_shift(s.xfi.x - s.xfj.x, p.g.n[0], p.g.per[0]);
+        dd.y += image_shift(s.xfi.y - s.xfj.y, p.g.n[1], p.g.per[1]);
+        dd.z += image_shift(s.xfi.z - s.xfj.z, p.g.n[2], p.g.per[2]);
+        const double R1 = P.R[i], R2 = P.R[j], S = R1 + R2;
         const double e = fma(-S, S, dot(dd, dd));
         d = cvt3<float>(dd);
         dist = sqrtf(dot(d, d));
-        Ri = P.view[i].R;
-        Rj = P.view[j].R;
+        Ri = (float)R1;
+        Rj = (float)R2;
         delta = (float)e / (dist + (float)S);
     }
     F = zero3<T>();
@@ -492,21 +550,15 @@ __device__ __forceinline__ void pair_force(const DemParams& p, int cur, int hin,
     dnew = zero3<T>();
     if (delta >= k.cut_max && delta >= T(0)) return;
     const Vec3<T> n = (T(1) / dist) * d;
-    Vec3<T> ui, omi, uj, omj;
-    if constexpr (sizeof(T) == 8) {
-        ui = ld3(P.us[cur], i); omi = ld3(P.oms[cur], i); uj = ld3(P.us[cur], j); omj = ld3(P.oms[cur], j);
-    } else {
-        ui = ld3(P.ufs[cur], i); omi = ld3(P.omfs[cur], i); uj = ld3(P.ufs[cur], j); omj = ld3(P.omfs[cur], j);
-    }
-    const Vec3<T> uij = ui - uj;
+    const Vec3<T> uij = s.ui - s.uj;
     if (p.lubrication) {
         const T Rm = T(0.5) * (Ri + Rj);
-        const T dmin = (k.min_a + k.min_b * Rm) * Rm;
-        lubrication_on_i<T>(k, p.tangential, Ri, Rj, delta, n, uij, omi, omj, dmin, F, Tq);
+        const T dmin = mad(k.min_b, Rm, k.min_a) * Rm;
+        lubrication_on_i<T>(k, p.tangential, Ri, Rj, delta, n, uij, s.omi, s.omj, dmin, F, Tq);
     }
     if (delta < T(0)) {
         const Vec3<T> ri = T(-0.5) * d, rj = T(0.5) * d;
-        const Vec3<T> ucp = (ui + cross(omi, ri)) - (uj + cross(omj, rj));
+        const Vec3<T> ucp = (s.ui + cross(s.omi, ri)) - (s.uj + cross(s.omj, rj));
         const T mi = (T)P.m[i], mj = (T)P.m[j];
         const T m_eff = mi * mj / (mi + mj);
         const T Tc = collision_time<T>(Ri + Rj, k.Tc);
@@ -514,8 +566,8 @@ __device__ __forceinline__ void pair_force(const DemParams& p, int cur, int hin,
         const int nin = P.hist_n[hin][i];
         for (int h = 0; h < nin; ++h)
             if (P.hist_id[hin][i * NBR_CAP + h] == j) {
-                const double* s = P.hist_d[hin] + 3 * (i * NBR_CAP + h);
-                old = Vec3<T>{(T)s[0], (T)s[1], (T)s[2]};
+                const double* sp = P.hist_d[hin] + 3 * (i * NBR_CAP + h);
+                old = Vec3<T>{(T)sp[0], (T)sp[1], (T)sp[2]};
                 break;
             }
         Vec3<T> Fn, Ft;
@@ -526,387 +578,458 @@ __device__ __forceinline__ void pair_force(const DemParams& p, int cur, int hin,
     }
 }
 
-// One Velocity-Verlet subcycle (Algorithm 1, inner loop) for 32 particles per
-// block of 128 threads. Pass 1, four lanes per particle: a float32 prefilter
-// of the neighbour slots (float positions are within 1e-4 of the float64
-// ones, so a gap above cut_max + 1e-3 there is above cut_max exactly); the
-// surviving (particle, slot) pairs are queued in shared memory in particle
-// and slot order. Pass 2: all 128 threads evaluate the queued pairs in
-// float64 (lubrication, Eqs. (25)-(33); contact, Eqs. (39)-(50)), so the
-// slow float64 units see full warps; each particle then sums its pairs in
-// slot order (the result does not depend on scheduling). Pass 3, one thread
-// per particle: plane walls, the averaged fluid force and V (rho_p - rho_f) g,
-// then the velocities (Eq. (38)) and, unless it is the last subcycle, the
-// positions of the next subcycle (Eq. (37)) into buffer 1 - cur.
-// init = 1 evaluates the initial force F(t = 0) only (no state or history
-// update). Pair terms are evaluated by both partners with mirrored operands.
-constexpr int PPB = DEM_ONE_BLOCK_MAX;   // particles per block
-constexpr int PAIR_CHUNK = 128;  // queued pairs evaluated per pass of the block
+// ------------------------------------------------------------ subcycles
+//
+// Eight lanes per particle. Lane s holds neighbour slots s, s + 8, ... and, on
+// walled axes, face s (axis s / 2, side s % 2): it evaluates their pair and wall
+// laws; the sums of the eight lanes are formed by a butterfly that leaves
+// component s of (F, T) in lane s. Lanes 0-2 integrate the translation (Eqs.
+// (37)-(38)), lanes 3-5 the rotation, one component each, with the state in
+// registers: a float64 instruction occupies a scheduler's float64 unit for 64
+// cycles whatever its lanes do, and one lane per particle issued about a hundred
+// of them per subcycle where this takes about fifteen.
+//
+// Float64 pair laws cost some 250 float64 instructions, so there the pairs of
+// the block that pass the float32 prefilter are queued and evaluated by full
+// warps; float32 ones are evaluated where they are found.
+constexpr int DEM_LANES = 8;
+constexpr int DEM_THREADS = 128;                     // of a multi-block launch
+constexpr int DEM_PPB = DEM_THREADS / DEM_LANES;     // its particles per block
+constexpr int ONE_BLOCK_THREADS = DEM_ONE_BLOCK_MAX * DEM_LANES;
 
-// pass 3 of a subcycle for particle ip: plane walls, the averaged fluid force
-// and V (rho_p - rho_f) g, the velocities (Eq. (38)) and, unless it is the
-// last subcycle, the positions of the next subcycle (Eq. (37)) into buffer
-// 1 - cur; sum holds the particle's pair forces and torques
-template <typename T>
-__device__ void integrate_particle(const DemParams& p, int ip, const T (&sum)[6], int cur, int hin, int hout, int init,
-                                   int last) {
+template <int PPB>
+struct PairQueue {
+    int n;
+    unsigned short entry[PPB * NBR_CAP];   // particle of the block << 5 | slot
+    double res[DEM_LANES * PPB][6];
+};
+
+// one lane's registers over the subcycles of a step
+struct OctLane {
+    int i, s;            // particle, lane of its eight
+    bool on;             // the particle exists
+    int nn;              // its neighbour slots
+    int j[NBR_CAP / DEM_LANES];
+    float reach2[NBR_CAP / DEM_LANES];
+    double x, v, f_prev, f_const, coef;   // position (lanes 0-2), velocity component, force of the last subcycle,
+                                          // averaged fluid force + external force, dt / (2 m) or dt / (2 I)
+};
+
+template <bool CG>
+__device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, int s, int cur) {
     const Particles& P = p.P;
-    const double* X = P.xs[cur];
-    const double* Uv = P.us[cur];
-    const double* Om = P.oms[cur];
-    Vec3<T> F = {sum[0], sum[1], sum[2]};
-    Vec3<T> Tq = {sum[3], sum[4], sum[5]};
-    {
-        // plane walls on the faces of non-periodic axes
-        const DemConsts<T>& k = consts<T>(p);
-        const V3 xd = ld3(X, ip);
-        Vec3<T> ui, omi;
-        if constexpr (sizeof(T) == 8) {
-            ui = ld3(Uv, ip);
-            omi = ld3(Om, ip);
-        } else {
-            ui = ld3(P.ufs[cur], ip);
-            omi = ld3(P.omfs[cur], ip);
-        }
-        const double Rid = P.R[ip];
-        const T Ri = (T)Rid, mi = (T)P.m[ip];
-        const double xa[3] = {xd.x, xd.y, xd.z};
-        for (int a = 0; a < 3; ++a) {
-            if (p.g.per[a]) continue;
-            for (int side = 0; side < 2; ++side) {
-                const int face = 2 * a + side;
-                Vec3<T> nw = zero3<T>();
-                const T sgn = side == 0 ? T(1) : T(-1);
-                if (a == 0) nw.x = sgn; else if (a == 1) nw.y = sgn; else nw.z = sgn;
-                const double xw = side == 0 ? 0.0 : (double)p.g.n[a];
-                const T delta = (T)((xa[a] - xw) * (side == 0 ? 1.0 : -1.0) - Rid);
-                const double* uwp = p.g.wall_vel[side][a];
-                const Vec3<T> uw = {(T)uwp[0], (T)uwp[1], (T)uwp[2]};
-                const Vec3<T> uij = ui - uw;
-                if (p.lubrication) {
-                    const T dmin = (k.min_a + k.min_b * Ri) * Ri;
-                    lubrication_on_i<T>(k, p.tangential, Ri, T(-1), delta, nw, uij, omi, zero3<T>(), dmin, F, Tq);
-                }
-                if (!init) P.wact[hout][6 * ip + face] = 0;
-                if (delta < T(0)) {
-                    const Vec3<T> ri = (-(Ri + T(0.5) * delta)) * nw;
-                    const Vec3<T> ucp = (ui + cross(omi, ri)) - uw;
-                    const T Tc = collision_time<T>(T(2) * Ri, k.Tc);
-                    Vec3<T> old = zero3<T>();
-                    if (P.wact[hin][6 * ip + face]) {
-                        const double* sd = P.whist[hin] + 3 * (6 * ip + face);
-                        old = Vec3<T>{(T)sd[0], (T)sd[1], (T)sd[2]};
-                    }
-                    Vec3<T> Fn, Ft, dnew;
-                    contact_force<T>(k, nw, delta, ucp, uij, mi, Tc, old, Fn, Ft, dnew);
-                    F = F + (Fn + Ft);
-                    Tq = Tq + cross(ri, Ft);
-                    if (!init) {
-                        double* sd = P.whist[hout] + 3 * (6 * ip + face);
-                        sd[0] = (double)dnew.x; sd[1] = (double)dnew.y; sd[2] = (double)dnew.z;
-                        P.wact[hout][6 * ip + face] = 1;
-                    }
-                }
-            }
+    o.i = i;
+    o.s = s;
+    o.on = i < P.n;
+    o.nn = 0;
+    o.x = o.v = o.f_prev = o.f_const = o.coef = 0.0;
+    if (!o.on) return;
+    o.nn = P.nbr_count[i];
+    const float reach = (float)P.R[i] + ((float)p.cut_max + 1e-3f);
+#pragma unroll
+    for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
+        const int slot = s + DEM_LANES * k;
+        if (slot < o.nn) {
+            o.j[k] = P.nbr[i * NBR_CAP + slot];
+            const float r = reach + (float)P.R[o.j[k]];
+            o.reach2[k] = r * r;
         }
     }
-    const V3 Fd = cvt3<double>(F), Td = cvt3<double>(Tq);
-    const V3 Fs = mk(Fd.x + P.fbar[6 * ip] + P.ext[3 * ip], Fd.y + P.fbar[6 * ip + 1] + P.ext[3 * ip + 1],
-                     Fd.z + P.fbar[6 * ip + 2] + P.ext[3 * ip + 2]);
-    const V3 Ts = mk(Td.x + P.fbar[6 * ip + 3], Td.y + P.fbar[6 * ip + 4], Td.z + P.fbar[6 * ip + 5]);
-    if (init) {
-        st3(P.F_prev, ip, Fs);
-        st3(P.T_prev, ip, Ts);
-        return;
-    }
-    P.hist_n[hout][ip] = P.nbr_count[ip];
-    // Eq. (38) for u and its rotational analogue for omega (hm = 1/(2m), hI = 1/(2I))
-    const double cu = p.dt * P.hm[ip], co = p.dt * P.hI[ip];
-    const V3 Fp = ld3(P.F_prev, ip), Tp = ld3(P.T_prev, ip);
-    const V3 u = ld3(Uv, ip) + cu * (Fp + Fs);
-    const V3 om = ld3(Om, ip) + co * (Tp + Ts);
-    st3(P.F_prev, ip, Fs);
-    st3(P.T_prev, ip, Ts);
-    if (!(dot(u, u) < 0.25)) atomicOr(p.status, ST_FAST_PARTICLE);
-    const int nxt = 1 - cur;
-    st3(P.us[nxt], ip, u);
-    st3(P.oms[nxt], ip, om);
-    if constexpr (sizeof(T) == 4) {
-        for (int d = 0; d < 3; ++d) {
-            P.ufs[nxt][3 * ip + d] = (float)(d == 0 ? u.x : d == 1 ? u.y : u.z);
-            P.omfs[nxt][3 * ip + d] = (float)(d == 0 ? om.x : d == 1 ? om.y : om.z);
-        }
-    }
-    const double ua[3] = {u.x, u.y, u.z};
-    const double Fa[3] = {Fs.x, Fs.y, Fs.z};
-    const double c = p.dt * cu;
-    PartView v;
-    for (int d = 0; d < 3; ++d) {
-        // Eq. (37) for the next subcycle; the last subcycle keeps its positions
-        double x = X[3 * ip + d];
-        if (!last) x = wrap_pos(x + p.dt * ua[d] + c * Fa[d], p.g.n[d], p.g.per[d]);
-        P.xs[nxt][3 * ip + d] = x;
-        P.xfs[nxt][3 * ip + d] = (float)x;
-        if (last) {
-            const double b = floor(x);
-            v.base[d] = (int)b;
-            v.frac[d] = (float)(x - b);
-            v.u[d] = (float)ua[d];
-            v.om[d] = (float)(d == 0 ? om.x : d == 1 ? om.y : om.z);
-        }
-    }
-    if (last) {
-        v.R = (float)P.R[ip];
-        set_view_c(v, P.R[ip]);
-        P.view[ip] = v;
+    if (s < 3) {
+        o.x = P.xs[cur][3 * i + s];
+        o.v = P.us[cur][3 * i + s];
+        o.f_prev = P.F_prev[3 * i + s];
+        o.f_const = P.fbar[6 * i + s] + P.ext[3 * i + s];
+        o.coef = p.dt * P.hm[i];
+    } else if (s < 6) {
+        o.v = P.oms[cur][3 * i + s - 3];
+        o.f_prev = P.T_prev[3 * i + s - 3];
+        o.f_const = P.fbar[6 * i + s];
+        o.coef = p.dt * P.hI[i];
     }
 }
 
+// float positions are within 1e-4 of the float64 ones, so a gap above cut_max +
+// 1e-3 there is above cut_max exactly
+__device__ __forceinline__ bool may_touch(const DemParams& p, Vec3<float> a, Vec3<float> b, float reach2) {
+    const float dx = mimgf(a.x - b.x, p.g.n[0], p.g.per[0]), dy = mimgf(a.y - b.y, p.g.n[1], p.g.per[1]),
+                dz = mimgf(a.z - b.z, p.g.n[2], p.g.per[2]);
+    return dx * dx + dy * dy + dz * dz < reach2;
+}
 
+// wall law of face o.s of the particle into F, Tq; returns whether it acts
 template <typename T>
-__device__ __forceinline__ void subcycle_body(const DemParams& p, int cur, int hin, int hout, int init, int last, int pblock) {
+__device__ bool wall_force(const DemParams& p, const OctLane& o, V3 x, Vec3<T> ui, Vec3<T> omi, int hin, int hout,
+                           int init, Vec3<T>& F, Vec3<T>& Tq) {
     const Particles& P = p.P;
-    const int tid = threadIdx.x;
-    const int pl = tid >> 2, sub = tid & 3;   // pass 1: particle of the block, lane of its group
-    const int i = pblock * PPB + pl;
-    __shared__ unsigned short s_queue[PPB * NBR_CAP];   // pl << 5 | slot
-    __shared__ int s_off[PPB + 1];
-    __shared__ T s_res[PAIR_CHUNK][6];
-    __shared__ T s_sum[PPB][6];
-    const float* Xf = P.xfs[cur];
-    const unsigned FULL = 0xffffffffu;
+    const DemConsts<T>& k = consts<T>(p);
+    const int face = o.s, a = face >> 1, side = face & 1;
+    const double Rid = P.R[o.i];
+    const double xa = a == 0 ? x.x : (a == 1 ? x.y : x.z);
+    const T delta = (T)(side == 0 ? xa - Rid : ((double)p.g.n[a] - xa) - Rid);
+    if (!init) P.wact[hout][6 * o.i + face] = 0;
+    if (delta >= k.cut_max && delta >= T(0)) return false;
+    const T Ri = (T)Rid, mi = (T)P.m[o.i];
+    const T sgn = side == 0 ? T(1) : T(-1);
+    const Vec3<T> nw = {a == 0 ? sgn : T(0), a == 1 ? sgn : T(0), a == 2 ? sgn : T(0)};
+    const double* uwp = p.g.wall_vel[side][a];
+    const Vec3<T> uw = {(T)uwp[0], (T)uwp[1], (T)uwp[2]};
+    const Vec3<T> uij = ui - uw;
+    if (p.lubrication) {
+        const T dmin = mad(k.min_b, Ri, k.min_a) * Ri;
+        lubrication_on_i<T>(k, p.tangential, Ri, T(-1), delta, nw, uij, omi, zero3<T>(), dmin, F, Tq);
+    }
+    if (delta < T(0)) {
+        const Vec3<T> ri = (-(Ri + T(0.5) * delta)) * nw;
+        const Vec3<T> ucp = (ui + cross(omi, ri)) - uw;
+        const T Tc = collision_time<T>(T(2) * Ri, k.Tc);
+        Vec3<T> old = zero3<T>();
+        if (P.wact[hin][6 * o.i + face]) {
+            const double* sd = P.whist[hin] + 3 * (6 * o.i + face);
+            old = Vec3<T>{(T)sd[0], (T)sd[1], (T)sd[2]};
+        }
+        Vec3<T> Fn, Ft, dnew;
+        contact_force<T>(k, nw, delta, ucp, uij, mi, Tc, old, Fn, Ft, dnew);
+        F = F + (Fn + Ft);
+        Tq = Tq + cross(ri, Ft);
+        if (!init) {
+            double* sd = P.whist[hout] + 3 * (6 * o.i + face);
+            sd[0] = (double)dnew.x; sd[1] = (double)dnew.y; sd[2] = (double)dnew.z;
+            P.wact[hout][6 * o.i + face] = 1;
+        }
+    }
+    return true;
+}
 
-    // pass 1: candidate slots of particle pl (bit k = slot k)
-    unsigned mask = 0;
-    int nn = 0;
-    if (i < P.n) {
-        nn = P.nbr_count[i];
-        const float xif[3] = {Xf[3 * i], Xf[3 * i + 1], Xf[3 * i + 2]};
-        const float Rif = (float)P.R[i];
-        const float reach_pad = (float)p.cut_max + 1e-3f;
-        for (int k = sub; k < nn; k += 4) {
-            const int j = P.nbr[i * NBR_CAP + k];
-            float d2f = 0.f;
-            for (int d = 0; d < 3; ++d) {
-                const float dd = mimgf(xif[d] - Xf[3 * j + d], p.g.n[d], p.g.per[d]);
-                d2f += dd * dd;
-            }
-            const float reach = Rif + (float)P.R[j] + reach_pad;
-            if (d2f < reach * reach) mask |= 1u << k;
-            else if (!init) P.hist_id[hout][i * NBR_CAP + k] = -1;   // no spring on this slot
-        }
-    }
-    mask |= __shfl_xor_sync(FULL, mask, 1);
-    mask |= __shfl_xor_sync(FULL, mask, 2);
-    if (sub == 0) s_off[pl] = __popc(mask);
-    if (tid < 6 * PPB) reinterpret_cast<T*>(s_sum)[tid] = T(0);
-    if (tid + 128 < 6 * PPB) reinterpret_cast<T*>(s_sum)[tid + 128] = T(0);
-    __syncthreads();
-    if (tid < 32) {   // exclusive prefix over the 32 particles
-        const int c = s_off[tid];
-        int incl = c;
+// One subcycle of the particle of o (Algorithm 1, inner loop): pair and wall
+// laws at the state in buffer cur, the velocities (Eq. (38)) and, unless it is
+// the last subcycle, the positions of the next one (Eq. (37)), published in
+// buffer 1 - cur. init = 1 evaluates the initial force F(t = 0) only (no state
+// or history update). All threads of the block take part.
+template <typename T, bool CG, int PPB>
+__device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, PairQueue<PPB>* queue, int cur, int hin,
+                                             int hout, int init, int last) {
+    const Particles& P = p.P;
+    const unsigned FULL = 0xffffffffu;
+    T f[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    bool acts = false;
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, incl, o);
-            if (tid >= o) incl += v;
-        }
-        s_off[tid] = incl - c;
-        if (tid == 31) s_off[PPB] = incl;
-    }
-    __syncthreads();
-    {
-        // the group's lanes write the queue entries of their particle, in slot order
-        unsigned m = mask;
-        int r = 0;
-        const int base = s_off[pl];
-        while (m) {
-            const int k = __ffs(m) - 1;
-            m &= m - 1;
-            if ((r & 3) == sub) s_queue[base + r] = (unsigned short)((pl << 5) | k);
-            ++r;
-        }
-    }
-    __syncthreads();
-    // pass 2: the queued pairs in chunks of 128, one per thread
-    const int total = s_off[PPB];
-    for (int c0 = 0; c0 < total; c0 += PAIR_CHUNK) {
-        const int e = c0 + tid;
-        if (e < total) {
-            const int q = s_queue[e];
-            const int ep = q >> 5, k = q & 31;
-            const int ei = pblock * PPB + ep;
-            const int j = P.nbr[ei * NBR_CAP + k];
-            Vec3<T> F, Tq, dnew;
-            bool contact;
-            pair_force<T>(p, cur, hin, ei, j, F, Tq, contact, dnew);
-            s_res[tid][0] = F.x; s_res[tid][1] = F.y; s_res[tid][2] = F.z;
-            s_res[tid][3] = Tq.x; s_res[tid][4] = Tq.y; s_res[tid][5] = Tq.z;
-            if (!init) {
-                // tangential spring of this neighbour slot for the next subcycle
-                P.hist_id[hout][ei * NBR_CAP + k] = contact ? j : -1;
-                if (contact) {
-                    double* sd = P.hist_d[hout] + 3 * (ei * NBR_CAP + k);
+        for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
+            const int slot = o.s + DEM_LANES * k;
+            if (slot >= o.nn) continue;
+            const PairState<T> st = load_pair<T, CG>(P, cur, o.i, o.j[k]);
+            bool contact = false;
+            if (may_touch(p, st.xfi, st.xfj, o.reach2[k])) {
+                Vec3<T> F, Tq, dnew;
+                pair_force<T>(p, st, hin, o.i, o.j[k], F, Tq, contact, dnew);
+                f[0] += F.x; f[1] += F.y; f[2] += F.z;
+                f[3] += Tq.x; f[4] += Tq.y; f[5] += Tq.z;
+                acts = true;
+                if (contact && !init) {
+                    double* sd = P.hist_d[hout] + 3 * (o.i * NBR_CAP + slot);
                     sd[0] = (double)dnew.x; sd[1] = (double)dnew.y; sd[2] = (double)dnew.z;
                 }
             }
+            if (!init) P.hist_id[hout][o.i * NBR_CAP + slot] = contact ? o.j[k] : -1;
         }
+    } else {
+        // pairs that pass the prefilter into the block's queue, evaluated by
+        // whichever thread comes first; each lane then collects its slots'
+        const int pl = threadIdx.x / DEM_LANES;
         __syncthreads();
-        if (tid < PPB) {   // particle tid adds its pairs of this chunk in slot order
-            const int lo = max(s_off[tid], c0), hi = min(s_off[tid + 1], c0 + PAIR_CHUNK);
-            for (int e2 = lo; e2 < hi; ++e2)
-                for (int c = 0; c < 6; ++c) s_sum[tid][c] += s_res[e2 - c0][c];
-        }
+        if (threadIdx.x == 0) queue->n = 0;
         __syncthreads();
-    }
-    // pass 3: one thread per particle, lanes 0-7 of each warp (the float64
-    // work of the block spread over the four schedulers)
-    if ((tid & 31) < PPB / 4) {
-        const int pl3 = (tid >> 5) * (PPB / 4) + (tid & 31);
-        const int ip = pblock * PPB + pl3;
-        if (ip < P.n) {
-            T sum[6];
+        int place[NBR_CAP / DEM_LANES];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) sum[c] = s_sum[pl3][c];
-            integrate_particle<T>(p, ip, sum, cur, hin, hout, init, last);
+        for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
+            const int slot = o.s + DEM_LANES * k;
+            place[k] = -1;
+            if (slot >= o.nn) continue;
+            if (may_touch(p, ld3s<CG>(P.xfs[cur], o.i), ld3s<CG>(P.xfs[cur], o.j[k]), o.reach2[k])) {
+                place[k] = atomicAdd(&queue->n, 1);
+                queue->entry[place[k]] = (unsigned short)((pl << 5) | slot);
+            } else if (!init) {
+                P.hist_id[hout][o.i * NBR_CAP + slot] = -1;
+            }
         }
+        __syncthreads();
+        const int total = queue->n, threads = (int)blockDim.x;
+        for (int c0 = 0; c0 < total; c0 += threads) {
+            const int e = c0 + (int)threadIdx.x;
+            if (e < total) {
+                const int q = queue->entry[e], slot = q & 31;
+                const int i = o.i - pl + (q >> 5), j = P.nbr[i * NBR_CAP + slot];
+                Vec3<T> F, Tq, dnew;
+                bool contact;
+                pair_force<T>(p, load_pair<T, CG>(P, cur, i, j), hin, i, j, F, Tq, contact, dnew);
+                double* r = queue->res[threadIdx.x];
+                r[0] = F.x; r[1] = F.y; r[2] = F.z; r[3] = Tq.x; r[4] = Tq.y; r[5] = Tq.z;
+                if (!init) {
+                    P.hist_id[hout][i * NBR_CAP + slot] = contact ? j : -1;
+                    if (contact) {
+                        double* sd = P.hist_d[hout] + 3 * (i * NBR_CAP + slot);
+                        sd[0] = dnew.x; sd[1] = dnew.y; sd[2] = dnew.z;
+                    }
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < NBR_CAP / DEM_LANES; ++k)
+                if (place[k] >= c0 && place[k] < c0 + threads) {
+                    const double* r = queue->res[place[k] - c0];
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) f[c] += (T)r[c];
+                    acts = true;
+                }
+            __syncthreads();
+        }
+    }
+    if (!(p.g.per[0] && p.g.per[1] && p.g.per[2])) {
+        // the particle's position and velocities from its lanes
+        const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
+        V3 x;
+        Vec3<T> ui, omi;
+        x.x = __shfl_sync(FULL, o.x, base);
+        x.y = __shfl_sync(FULL, o.x, base + 1);
+        x.z = __shfl_sync(FULL, o.x, base + 2);
+        const T v = (T)o.v;
+        ui.x = __shfl_sync(FULL, v, base);
+        ui.y = __shfl_sync(FULL, v, base + 1);
+        ui.z = __shfl_sync(FULL, v, base + 2);
+        omi.x = __shfl_sync(FULL, v, base + 3);
+        omi.y = __shfl_sync(FULL, v, base + 4);
+        omi.z = __shfl_sync(FULL, v, base + 5);
+        if (o.on && o.s < 6 && !p.g.per[o.s >> 1]) {
+            Vec3<T> F = zero3<T>(), Tq = zero3<T>();
+            if (wall_force<T>(p, o, x, ui, omi, hin, hout, init, F, Tq)) {
+                f[0] += F.x; f[1] += F.y; f[2] += F.z;
+                f[3] += Tq.x; f[4] += Tq.y; f[5] += Tq.z;
+                acts = true;
+            }
+        }
+    }
+    T sum = T(0);   // component s of the particle's pair and wall sums
+    if (__any_sync(FULL, acts)) {
+        const bool b4 = o.s & 4, b2 = o.s & 2, b1 = o.s & 1;
+        T g[4], h[2];
+        g[0] = (b4 ? f[4] : f[0]) + __shfl_xor_sync(FULL, b4 ? f[0] : f[4], 4);
+        g[1] = (b4 ? f[5] : f[1]) + __shfl_xor_sync(FULL, b4 ? f[1] : f[5], 4);
+        g[2] = (b4 ? T(0) : f[2]) + __shfl_xor_sync(FULL, b4 ? f[2] : T(0), 4);
+        g[3] = (b4 ? T(0) : f[3]) + __shfl_xor_sync(FULL, b4 ? f[3] : T(0), 4);
+        h[0] = (b2 ? g[2] : g[0]) + __shfl_xor_sync(FULL, b2 ? g[0] : g[2], 2);
+        h[1] = (b2 ? g[3] : g[1]) + __shfl_xor_sync(FULL, b2 ? g[1] : g[3], 2);
+        sum = (b1 ? h[1] : h[0]) + __shfl_xor_sync(FULL, b1 ? h[0] : h[1], 1);
+    }
+    if (!o.on) return;
+    const double fs = (double)sum + o.f_const;
+    if (init) {
+        if (o.s < 3) P.F_prev[3 * o.i + o.s] = fs;
+        else if (o.s < 6) P.T_prev[3 * o.i + o.s - 3] = fs;
+        return;
+    }
+    if (o.s == 6) P.hist_n[hout][o.i] = o.nn;
+    // Eq. (38) for u and its rotational analogue for omega
+    o.v = fma(o.coef, o.f_prev + fs, o.v);
+    o.f_prev = fs;
+    const int nxt = 1 - cur;
+    if (o.s < 3) {
+        if (!last) {
+            // Eq. (37) for the next subcycle; the last subcycle keeps its positions
+            o.x = wrap_pos(fma(p.dt * o.coef, fs, fma(p.dt, o.v, o.x)), p.g.n[o.s], p.g.per[o.s]);
+            P.xs[nxt][3 * o.i + o.s] = o.x;
+            P.xfs[nxt][3 * o.i + o.s] = (float)o.x;
+        }
+        if (sizeof(T) == 8) P.us[nxt][3 * o.i + o.s] = o.v;
+        else P.ufs[nxt][3 * o.i + o.s] = (float)o.v;
+    } else if (o.s < 6) {
+        if (sizeof(T) == 8) P.oms[nxt][3 * o.i + o.s - 3] = o.v;
+        else P.omfs[nxt][3 * o.i + o.s - 3] = (float)o.v;
     }
 }
 
-// one DEM subcycle of Algorithm 1: lubrication (Eqs. (25)-(34)) and contact
-// (Eqs. (39)-(52)) for every pair and wall, then the Velocity-Verlet velocity
-// update (Eq. (38)) and the next position update (Eq. (37))
+// The particle's speed stays below 0.5 cells per step (checked per subcycle on
+// the squared components of lanes 0-2).
+__device__ __forceinline__ void oct_check_speed(const DemParams& p, const OctLane& o) {
+    const unsigned FULL = 0xffffffffu;
+    const double sq = o.on && o.s < 3 ? o.v * o.v : 0.0;
+    // the float32 sum decides unless it is near the limit
+    float q = (float)sq;
+    q += __shfl_down_sync(FULL, q, 2, DEM_LANES) + __shfl_down_sync(FULL, q, 1, DEM_LANES);
+    const bool near = o.on && o.s == 0 && !(q < 0.2499f);
+    if (!__any_sync(FULL, near)) return;
+    const double q1 = __shfl_down_sync(FULL, sq, 1, DEM_LANES), q2 = __shfl_down_sync(FULL, sq, 2, DEM_LANES);
+    if (near && !((sq + q1) + q2 < 0.25)) atomicOr(p.status, ST_FAST_PARTICLE);
+}
+
+// the state after the last subcycle into buffer 0 of the particle arrays and
+// the float32 view
 template <typename T>
-__global__ void __launch_bounds__(128) subcycle_kernel(const DemParams p, int cur, int init, int last) {
+__device__ __forceinline__ void oct_store(const DemParams& p, const OctLane& o) {
+    const Particles& P = p.P;
+    if (!o.on || o.s >= 6) return;
+    if (o.s < 3) {
+        P.x[3 * o.i + o.s] = o.x;
+        P.xf[3 * o.i + o.s] = (float)o.x;
+        P.u[3 * o.i + o.s] = o.v;
+        P.F_prev[3 * o.i + o.s] = o.f_prev;
+    } else {
+        P.om[3 * o.i + o.s - 3] = o.v;
+        P.T_prev[3 * o.i + o.s - 3] = o.f_prev;
+    }
+}
+// the view of the particle by its first lane, from the stored state's registers
+__device__ __forceinline__ void oct_store_view(const DemParams& p, const OctLane& o) {
+    const unsigned FULL = 0xffffffffu;
+    const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
+    const double fl = floor(o.x);
+    const int b = (int)fl;
+    const float fr = (float)(o.x - fl), v = (float)o.v;
+    PartView w;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        w.base[d] = __shfl_sync(FULL, b, base + d);
+        w.frac[d] = __shfl_sync(FULL, fr, base + d);
+        w.u[d] = __shfl_sync(FULL, v, base + d);
+        w.om[d] = __shfl_sync(FULL, v, base + 3 + d);
+    }
+    if (o.on && o.s == 0) {
+        w.R = (float)p.P.R[o.i];
+        set_view_c(w, p.P.R[o.i]);
+        p.P.view[o.i] = w;
+    }
+}
+
+// the first Velocity-Verlet position update of a step (Eq. (37))
+__device__ __forceinline__ void oct_first_position(const DemParams& p, OctLane& o) {
+    const Particles& P = p.P;
+    if (!o.on || o.s >= 3) return;
+    o.x = wrap_pos(fma(p.dt * o.coef, o.f_prev, fma(p.dt, o.v, o.x)), p.g.n[o.s], p.g.per[o.s]);
+    P.xs[0][3 * o.i + o.s] = o.x;
+    P.xfs[0][3 * o.i + o.s] = (float)o.x;
+}
+
+// one DEM subcycle of Algorithm 1 as a launch of its own (the initial force,
+// and more particles than fit one cooperative launch)
+template <typename T>
+__device__ __forceinline__ void subcycle_body(const DemParams& p, int cur, int hin, int hout, int init, int last,
+                                              int pblock) {
+    __shared__ PairQueue<sizeof(T) == 8 ? DEM_PPB : 1> queue;
+    OctLane o;
+    oct_load<false>(p, o, pblock * DEM_PPB + (int)threadIdx.x / DEM_LANES, threadIdx.x % DEM_LANES, cur);
+    oct_subcycle<T, false, sizeof(T) == 8 ? DEM_PPB : 1>(p, o, &queue, cur, hin, hout, init, last);
+    if (init) return;
+    oct_check_speed(p, o);
+    const Particles& P = p.P;
+    const int nxt = 1 - cur;
+    if (o.on && o.s < 3) {
+        P.xs[nxt][3 * o.i + o.s] = o.x;
+        P.xfs[nxt][3 * o.i + o.s] = (float)o.x;
+        P.us[nxt][3 * o.i + o.s] = o.v;
+        P.F_prev[3 * o.i + o.s] = o.f_prev;
+    } else if (o.on && o.s < 6) {
+        P.oms[nxt][3 * o.i + o.s - 3] = o.v;
+        P.T_prev[3 * o.i + o.s - 3] = o.f_prev;
+    }
+    if (last) oct_store_view(p, o);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(DEM_THREADS) subcycle_kernel(const __grid_constant__ DemParams p, int cur, int init,
+                                                               int last) {
     subcycle_body<T>(p, cur, p.hin, p.hout, init, last, blockIdx.x);
 }
 
-// All subcycles of a step in one block when the particles fit in it (at most
-// PPB): the first position update, n_sub subcycles separated by block
-// barriers (each reads the positions and velocities the previous one wrote),
-// and the copy back into buffer 0 after an odd count. The particles' state
-// stays in shared memory for the whole step: the block loads it once, points
-// the particle arrays of its (shared) parameter copy at the staged arrays, runs
-// the subcycles there -- the code of the multi-block path, reaching shared
-// memory through generic pointers -- and writes back what the step changed.
-// The neighbour counts are staged too (read every subcycle); the neighbour
-// lists, pair springs and the particle views stay in global memory.
-// Latency, not arithmetic, sets the time of a few-particle DEM step, so each
-// dependent global round trip saved per subcycle counts.
-struct DemStage {
-    double x[2][3 * PPB], u[2][3 * PPB], om[2][3 * PPB];
-    float xf[2][3 * PPB], uf[2][3 * PPB], omf[2][3 * PPB];
-    double F_prev[3 * PPB], T_prev[3 * PPB], ext[3 * PPB], fbar[6 * PPB];
-    double hm[PPB], hI[PPB], R[PPB], m[PPB];
-    double whist[2][18 * PPB];
-    unsigned char wact[2][6 * PPB];
-    int nbr_count[PPB];
-};
-
-// sp: the step's parameters in shared memory (n <= PPB particles); g receives
-// the global particle arrays
-template <typename T>
-__device__ void dem_step_block(DemParams& sp, Particles& g, DemStage& st, int hcur, int n_sub) {
-    const int tid = threadIdx.x;
-    const int n = sp.P.n;
-    if (tid == 0) g = sp.P;
+// A barrier of all blocks of a cooperative launch: *count rises by one per block
+// and barrier (0 at the launch). Gives up after a second with ST_TIMEOUT.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int* status) {
+    __shared__ int ok;
     __syncthreads();
-    for (int k = tid; k < 3 * n; k += blockDim.x) {
-        st.x[0][k] = g.x[k];
-        st.u[0][k] = g.u[k];
-        st.om[0][k] = g.om[k];
-        st.xf[0][k] = g.xf[k];
-        st.uf[0][k] = g.ufs[0][k];
-        st.omf[0][k] = g.omfs[0][k];
-        st.F_prev[k] = g.F_prev[k];
-        st.T_prev[k] = g.T_prev[k];
-        st.ext[k] = g.ext[k];
-    }
-    for (int k = tid; k < 6 * n; k += blockDim.x) {
-        st.fbar[k] = g.fbar[k];
-        st.wact[0][k] = g.wact[0][k];
-        st.wact[1][k] = g.wact[1][k];
-    }
-    for (int k = tid; k < 18 * n; k += blockDim.x) {
-        st.whist[0][k] = g.whist[0][k];
-        st.whist[1][k] = g.whist[1][k];
-    }
-    for (int k = tid; k < n; k += blockDim.x) {
-        st.hm[k] = g.hm[k];
-        st.hI[k] = g.hI[k];
-        st.R[k] = g.R[k];
-        st.m[k] = g.m[k];
-        st.nbr_count[k] = g.nbr_count[k];
-    }
-    if (tid == 0) {
-        Particles& P = sp.P;
-        P.x = P.xs[0] = st.x[0];
-        P.xs[1] = st.x[1];
-        P.u = P.us[0] = st.u[0];
-        P.us[1] = st.u[1];
-        P.om = P.oms[0] = st.om[0];
-        P.oms[1] = st.om[1];
-        P.xf = P.xfs[0] = st.xf[0];
-        P.xfs[1] = st.xf[1];
-        for (int h = 0; h < 2; ++h) {
-            P.ufs[h] = st.uf[h];
-            P.omfs[h] = st.omf[h];
-            P.whist[h] = st.whist[h];
-            P.wact[h] = st.wact[h];
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1u);
+        unsigned long long t0, t1;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+        unsigned now;
+        ok = 1;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(count) : "memory");
+            if (now >= target) break;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+            if (t1 - t0 > 1000000000ull) {
+                atomicOr(status, ST_TIMEOUT);
+                ok = 0;
+                break;
+            }
         }
-        P.F_prev = st.F_prev;
-        P.T_prev = st.T_prev;
-        P.ext = st.ext;
-        P.fbar = st.fbar;
-        P.hm = st.hm;
-        P.hI = st.hI;
-        P.R = st.R;
-        P.m = st.m;
-        P.nbr_count = st.nbr_count;
+        __threadfence();
     }
     __syncthreads();
-    if (tid < n) position_update(sp, tid);
-    __syncthreads();
-    int cur = 0;
-    for (int s = 0; s < n_sub; ++s) {
-        subcycle_body<T>(sp, cur, hcur, 1 - hcur, 0, s == n_sub - 1, 0);
-        __syncthreads();
+    return ok != 0;
+}
+
+// All subcycles of a step in one launch: the particles' state stays in
+// registers, buffers 0 and 1 only carry what partners read. One block
+// (barriers of the block) or a cooperative launch (GRID). With fin, the force
+// finalisation of the step comes first, with sc the counters' reset and the
+// tile scatter of the mapping last: a step of Algorithm 1 between the dense
+// kernel and the mapping is this one launch.
+template <typename T, bool GRID, int PPB>
+__device__ __forceinline__ void dem_step_body(const DemParams& p, const FinalizeParams* fin, const MapParams* sc,
+                                              PairQueue<PPB>* queue, int hcur, int n_sub, int first_particle) {
+    const int s = threadIdx.x % DEM_LANES, i = first_particle + (int)threadIdx.x / DEM_LANES;
+    if (fin) {
+        finalize_lane(*fin, i, s);
+        __syncwarp();
+    }
+    OctLane o;
+    oct_load<GRID>(p, o, i, s, 0);
+    oct_first_position(p, o);
+    unsigned target = 0;
+    bool ok = true;
+    auto barrier = [&]() {
+        if constexpr (GRID) {
+            target += gridDim.x;
+            ok = grid_barrier(p.barrier, target, p.status);
+        } else {
+            __syncthreads();
+        }
+    };
+    for (int k = 0; k < n_sub && ok; ++k) {
+        barrier();
+        if (!ok) break;
+        oct_subcycle<T, GRID, PPB>(p, o, queue, k & 1, hcur, 1 - hcur, 0, k == n_sub - 1);
+        oct_check_speed(p, o);
         hcur = 1 - hcur;
-        cur = 1 - cur;
     }
-    // the state after the last subcycle is in buffer cur; buffer 0 of the
-    // global arrays receives it
-    for (int k = tid; k < 3 * n; k += blockDim.x) {
-        g.x[k] = st.x[cur][k];
-        g.u[k] = st.u[cur][k];
-        g.om[k] = st.om[cur][k];
-        g.xf[k] = st.xf[cur][k];
-        g.ufs[0][k] = st.uf[cur][k];
-        g.omfs[0][k] = st.omf[cur][k];
-        g.F_prev[k] = st.F_prev[k];
-        g.T_prev[k] = st.T_prev[k];
-    }
-    for (int k = tid; k < 6 * n; k += blockDim.x) {
-        g.wact[0][k] = st.wact[0][k];
-        g.wact[1][k] = st.wact[1][k];
-    }
-    for (int k = tid; k < 18 * n; k += blockDim.x) {
-        g.whist[0][k] = st.whist[0][k];
-        g.whist[1][k] = st.whist[1][k];
+    // float64 laws read u, omega of buffer 0 in the last of an odd number of subcycles
+    if (sizeof(T) == 8 && (n_sub & 1)) barrier();
+    oct_store<T>(p, o);
+    oct_store_view(p, o);
+    if (sc) {
+        if (first_particle == 0 && threadIdx.x < 4) reinterpret_cast<int*>(sc->n_solid)[threadIdx.x] = 0;
+        const unsigned FULL = 0xffffffffu;
+        const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
+        const double x[3] = {__shfl_sync(FULL, o.x, base), __shfl_sync(FULL, o.x, base + 1),
+                             __shfl_sync(FULL, o.x, base + 2)};
+        if (o.on) tile_scatter_particle(*sc, o.i, x, s, DEM_LANES);
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) dem_step_one_block_kernel(const DemParams p, int hcur, int n_sub) {
-    __shared__ __align__(16) DemParams sp;
-    __shared__ __align__(16) Particles g;
-    __shared__ __align__(16) DemStage st;
-    constexpr int WORDS = (int)(sizeof(DemParams) / 4);
-    static_assert(sizeof(DemParams) % 4 == 0, "parameters copied in words");
-    const int* src = reinterpret_cast<const int*>(&p);
-    int* dst = reinterpret_cast<int*>(&sp);
-    for (int w = threadIdx.x; w < WORDS; w += blockDim.x) dst[w] = src[w];
-    __syncthreads();
-    dem_step_block<T>(sp, g, st, hcur, n_sub);
+__global__ void __launch_bounds__(ONE_BLOCK_THREADS)
+    dem_step_one_block_kernel(const __grid_constant__ DemParams p, const __grid_constant__ FinalizeParams fin,
+                              const __grid_constant__ MapParams sc, int hcur, int n_sub) {
+    __shared__ PairQueue<sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1> queue;
+    dem_step_body<T, false, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(p, &fin, &sc, &queue, hcur, n_sub, 0);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(DEM_THREADS, 5)
+    dem_step_grid_kernel(const __grid_constant__ DemParams p, const __grid_constant__ FinalizeParams fin,
+                         const __grid_constant__ MapParams sc, int hcur, int n_sub) {
+    __shared__ PairQueue<sizeof(T) == 8 ? DEM_PPB : 1> queue;
+    dem_step_body<T, true, sizeof(T) == 8 ? DEM_PPB : 1>(p, &fin, &sc, &queue, hcur, n_sub, (int)blockIdx.x * DEM_PPB);
 }
 
 // The one-block DEM steps of many instances in one launch: block b runs the
@@ -918,17 +1041,16 @@ struct DemBatchEntry {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(128) dem_step_batch_kernel(const DemBatchEntry* __restrict__ table) {
+__global__ void __launch_bounds__(ONE_BLOCK_THREADS) dem_step_batch_kernel(const DemBatchEntry* __restrict__ table) {
     __shared__ __align__(16) DemBatchEntry e;
-    __shared__ __align__(16) Particles g;
-    __shared__ __align__(16) DemStage st;
+    __shared__ PairQueue<sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1> queue;
     constexpr int WORDS = (int)(sizeof(DemBatchEntry) / 4);
     static_assert(sizeof(DemBatchEntry) % 4 == 0, "entry copied in words");
     const int* src = reinterpret_cast<const int*>(table + blockIdx.x);
     int* dst = reinterpret_cast<int*>(&e);
     for (int w = threadIdx.x; w < WORDS; w += blockDim.x) dst[w] = src[w];
     __syncthreads();
-    dem_step_block<T>(e.p, g, st, e.hcur, e.n_sub);
+    dem_step_body<T, false, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(e.p, nullptr, nullptr, &queue, e.hcur, e.n_sub, 0);
 }
 
 size_t dem_batch_entry_bytes() { return sizeof(DemBatchEntry); }
@@ -945,20 +1067,39 @@ void fill_dem_batch_entry(const DemParams& p, int hcur, int n_sub, void* out) {
 void launch_dem_step_batch(const void* d_table, int count, int pair_f32, cudaStream_t st) {
     if (count <= 0) return;
     const DemBatchEntry* t = static_cast<const DemBatchEntry*>(d_table);
-    if (pair_f32) dem_step_batch_kernel<float><<<count, 128, 0, st>>>(t);
-    else dem_step_batch_kernel<double><<<count, 128, 0, st>>>(t);
+    if (pair_f32) dem_step_batch_kernel<float><<<count, ONE_BLOCK_THREADS, 0, st>>>(t);
+    else dem_step_batch_kernel<double><<<count, ONE_BLOCK_THREADS, 0, st>>>(t);
 }
 
-void launch_dem_step_one_block(const DemParams& p, int hcur, int n_sub, cudaStream_t st) {
-    if (p.P.n == 0) return;
-    if (p.pair_f32) dem_step_one_block_kernel<float><<<1, 128, 0, st>>>(p, hcur, n_sub);
-    else dem_step_one_block_kernel<double><<<1, 128, 0, st>>>(p, hcur, n_sub);
+cudaError_t dem_grid_capacity(int storage_f64, int num_sms, int* particles) {
+    int blocks = 0;
+    const cudaError_t e = storage_f64
+        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, dem_step_grid_kernel<double>, DEM_THREADS, 0)
+        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, dem_step_grid_kernel<float>, DEM_THREADS, 0);
+    *particles = e == cudaSuccess ? blocks * num_sms * DEM_PPB : 0;
+    return e;
+}
+
+cudaError_t launch_dem_step(const DemParams& p, const FinalizeParams& fin, const MapParams& sc, int hcur, int n_sub,
+                            cudaStream_t st) {
+    if (p.P.n <= DEM_ONE_BLOCK_MAX) {
+        // no idle warps: a block of as many as the particles need
+        const int threads = (p.P.n * DEM_LANES + 31) / 32 * 32;
+        if (p.pair_f32) dem_step_one_block_kernel<float><<<1, threads, 0, st>>>(p, fin, sc, hcur, n_sub);
+        else dem_step_one_block_kernel<double><<<1, threads, 0, st>>>(p, fin, sc, hcur, n_sub);
+        return cudaGetLastError();
+    }
+    void* args[] = {const_cast<DemParams*>(&p), const_cast<FinalizeParams*>(&fin), const_cast<MapParams*>(&sc), &hcur,
+                    &n_sub};
+    const void* k = p.pair_f32 ? (const void*)dem_step_grid_kernel<float> : (const void*)dem_step_grid_kernel<double>;
+    return cudaLaunchCooperativeKernel(k, dim3((p.P.n + DEM_PPB - 1) / DEM_PPB), dim3(DEM_THREADS), args, 0, st);
 }
 
 void launch_dem_subcycle(const DemParams& p, int cur, int init, int last, cudaStream_t st) {
     if (p.P.n == 0) return;
-    if (p.pair_f32) subcycle_kernel<float><<<(p.P.n + PPB - 1) / PPB, 128, 0, st>>>(p, cur, init, last);
-    else subcycle_kernel<double><<<(p.P.n + PPB - 1) / PPB, 128, 0, st>>>(p, cur, init, last);
+    const int blocks = (p.P.n + DEM_PPB - 1) / DEM_PPB;
+    if (p.pair_f32) subcycle_kernel<float><<<blocks, DEM_THREADS, 0, st>>>(p, cur, init, last);
+    else subcycle_kernel<double><<<blocks, DEM_THREADS, 0, st>>>(p, cur, init, last);
 }
 
 // copy state buffer 1 into buffer 0 (after an odd number of subcycles)

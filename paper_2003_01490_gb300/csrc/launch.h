@@ -152,6 +152,7 @@ struct DemParams {
     DemConsts<double> kd;
     DemConsts<float> kf;
     int* status;
+    unsigned* barrier;      // arrivals at the barriers of the step's cooperative launch
 };
 // the one-block DEM steps of many instances in one launch (batches)
 size_t dem_batch_entry_bytes();
@@ -161,10 +162,15 @@ void launch_bins(const DemParams& p, cudaStream_t st);
 void launch_neighbours(const DemParams& p, cudaStream_t st);
 void launch_dem_position(const DemParams& p, cudaStream_t st);
 void launch_dem_subcycle(const DemParams& p, int cur, int init, int last, cudaStream_t st);
-// at most this many particles: the position update, all subcycles and the
-// state copy of a step in one single-block launch
+// The force finalisation, the position update, all subcycles, the counters'
+// reset and the tile scatter of a step in one launch: one block for at most
+// DEM_ONE_BLOCK_MAX particles, else a cooperative launch, for at most the
+// particles of dem_grid_capacity().
 constexpr int DEM_ONE_BLOCK_MAX = 32;
-void launch_dem_step_one_block(const DemParams& p, int hcur, int n_sub, cudaStream_t st);
+constexpr int DEM_BLOCK_PARTICLES = 16;   // particles per block of a multi-block launch
+cudaError_t dem_grid_capacity(int storage_f64, int num_sms, int* particles);
+cudaError_t launch_dem_step(const DemParams& p, const FinalizeParams& fin, const MapParams& sc, int hcur, int n_sub,
+                            cudaStream_t st);
 void launch_state_copy(const Particles& P, cudaStream_t st);
 void launch_fp_split(const double* fp, double* out, int n, cudaStream_t st);
 
