@@ -464,13 +464,13 @@ __device__ __forceinline__ T collision_time(T diameter, T Tc) {
 
 // periodic shift (0 or -+n) that takes the separation of a close pair to its
 // minimum image, decided on the float32 copy of the separation
-__device__ __forceinline__ double image_shift(float d, int n, int per) {
+__device__ __forceinline__ int image_shift(float d, int n, int per) {
     if (per) {
         const float half = 0.5f * (float)n;
-        if (d > half) return -(double)n;
-        if (d < -half) return (double)n;
+        if (d > half) return -n;
+        if (d < -half) return n;
     }
-    return 0.0;
+    return 0;
 }
 
 // Loads of particle state that other threads of the launch write between the
@@ -533,9 +533,14 @@ __device__ __forceinline__ void pair_force(const DemParams& p, const PairState<T
         delta = dist - (Ri + Rj);
     } else {
         V3 dd = s.xi - s.xj;
-        dd.x += image_shift(s.xfi.x - s.xfj.x, p.g.n[0], p.g.per[0]);
-        dd.y += image_shift(s.xfi.y - s.xfj.y, p.g.n[1], p.g.per[1]);
-        dd.z += image_shift(s.xfi.z - s.xfj.z, p.g.n[2], p.g.per[2]);
+        const int sx = image_shift(s.xfi.x - s.xfj.x, p.g.n[0], p.g.per[0]),
+                  sy = image_shift(s.xfi.y - s.xfj.y, p.g.n[1], p.g.per[1]),
+                  sz = image_shift(s.xfi.z - s.xfj.z, p.g.n[2], p.g.per[2]);
+        if (sx | sy | sz) {
+            dd.x += (double)sx;
+            dd.y += (double)sy;
+            dd.z += (double)sz;
+        }
         const double R1 = P.R[i], R2 = P.R[j], S = R1 + R2;
         const double e = fma(-S, S, dot(dd, dd));
         d = cvt3<float>(dd);
@@ -611,8 +616,10 @@ struct OctLane {
     int nn;              // its neighbour slots
     int j[NBR_CAP / DEM_LANES];
     float reach2[NBR_CAP / DEM_LANES];
-    double x, v, f_prev, f_const, coef;   // position (lanes 0-2), velocity component, force of the last subcycle,
-                                          // averaged fluid force + external force, dt / (2 m) or dt / (2 I)
+    double x, v, f_prev, f_const;   // position (lanes 0-2), velocity component, force of the last subcycle,
+                                    // averaged fluid force + external force
+    double coef, dcoef;             // dt / (2 m) or dt / (2 I), dt times it
+    float xf, vf, R;                // float32 copies for the tests that decide most cases
 };
 
 template <bool CG>
@@ -622,10 +629,12 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
     o.s = s;
     o.on = i < P.n;
     o.nn = 0;
-    o.x = o.v = o.f_prev = o.f_const = o.coef = 0.0;
+    o.x = o.v = o.f_prev = o.f_const = o.coef = o.dcoef = 0.0;
+    o.xf = o.vf = o.R = 0.f;
     if (!o.on) return;
     o.nn = P.nbr_count[i];
-    const float reach = (float)P.R[i] + ((float)p.cut_max + 1e-3f);
+    o.R = (float)P.R[i];
+    const float reach = o.R + ((float)p.cut_max + 1e-3f);
 #pragma unroll
     for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
         const int slot = s + DEM_LANES * k;
@@ -646,6 +655,21 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
         o.f_prev = P.T_prev[3 * i + s - 3];
         o.f_const = P.fbar[6 * i + s];
         o.coef = p.dt * P.hI[i];
+    }
+    o.dcoef = p.dt * o.coef;
+    o.xf = (float)o.x;
+    o.vf = (float)o.v;
+}
+
+// Eq. (37) for lanes 0-2; the periodic wrap is decided in float64 only for
+// positions within half a cell of a face
+__device__ __forceinline__ void oct_move(const DemParams& p, OctLane& o) {
+    o.x = fma(o.dcoef, o.f_prev, fma(p.dt, o.v, o.x));
+    o.xf = (float)o.x;
+    const int n = p.g.n[o.s];
+    if (!(o.xf > 0.5f && o.xf < (float)n - 0.5f)) {
+        o.x = wrap_pos(o.x, n, p.g.per[o.s]);
+        o.xf = (float)o.x;
     }
 }
 
@@ -785,7 +809,18 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
             __syncthreads();
         }
     }
-    if (!(p.g.per[0] && p.g.per[1] && p.g.per[2])) {
+    // faces within reach, by the float32 position (within 1e-4 of the float64
+    // one for boxes of up to 2^11 cells; the exact gap decides below)
+    bool face = false;
+    const bool walled = o.on && o.s < 6 && !p.g.per[o.s >> 1];
+    {
+        const float xa = __shfl_sync(FULL, o.xf, o.s >> 1, DEM_LANES);
+        const float gap = (o.s & 1 ? (float)p.g.n[(o.s >> 1) % 3] - xa : xa) - o.R;
+        const float slack = 1e-3f + 1e-6f * (float)p.g.n[(o.s >> 1) % 3];
+        face = walled && !(gap > (float)p.cut_max + slack);
+        if (walled && !face && !init) P.wact[hout][6 * o.i + o.s] = 0;
+    }
+    if (__any_sync(FULL, face)) {
         // the particle's position and velocities from its lanes
         const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
         V3 x;
@@ -800,7 +835,7 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
         omi.x = __shfl_sync(FULL, v, base + 3);
         omi.y = __shfl_sync(FULL, v, base + 4);
         omi.z = __shfl_sync(FULL, v, base + 5);
-        if (o.on && o.s < 6 && !p.g.per[o.s >> 1]) {
+        if (face) {
             Vec3<T> F = zero3<T>(), Tq = zero3<T>();
             if (wall_force<T>(p, o, x, ui, omi, hin, hout, init, F, Tq)) {
                 f[0] += F.x; f[1] += F.y; f[2] += F.z;
@@ -809,8 +844,9 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
             }
         }
     }
-    T sum = T(0);   // component s of the particle's pair and wall sums
+    double fs = o.f_const;
     if (__any_sync(FULL, acts)) {
+        // component s of the particle's pair and wall sums
         const bool b4 = o.s & 4, b2 = o.s & 2, b1 = o.s & 1;
         T g[4], h[2];
         g[0] = (b4 ? f[4] : f[0]) + __shfl_xor_sync(FULL, b4 ? f[0] : f[4], 4);
@@ -819,10 +855,9 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
         g[3] = (b4 ? T(0) : f[3]) + __shfl_xor_sync(FULL, b4 ? f[3] : T(0), 4);
         h[0] = (b2 ? g[2] : g[0]) + __shfl_xor_sync(FULL, b2 ? g[0] : g[2], 2);
         h[1] = (b2 ? g[3] : g[1]) + __shfl_xor_sync(FULL, b2 ? g[1] : g[3], 2);
-        sum = (b1 ? h[1] : h[0]) + __shfl_xor_sync(FULL, b1 ? h[0] : h[1], 1);
+        fs += (double)((b1 ? h[1] : h[0]) + __shfl_xor_sync(FULL, b1 ? h[0] : h[1], 1));
     }
     if (!o.on) return;
-    const double fs = (double)sum + o.f_const;
     if (init) {
         if (o.s < 3) P.F_prev[3 * o.i + o.s] = fs;
         else if (o.s < 6) P.T_prev[3 * o.i + o.s - 3] = fs;
@@ -832,19 +867,20 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
     // Eq. (38) for u and its rotational analogue for omega
     o.v = fma(o.coef, o.f_prev + fs, o.v);
     o.f_prev = fs;
+    o.vf = (float)o.v;
     const int nxt = 1 - cur;
     if (o.s < 3) {
         if (!last) {
-            // Eq. (37) for the next subcycle; the last subcycle keeps its positions
-            o.x = wrap_pos(fma(p.dt * o.coef, fs, fma(p.dt, o.v, o.x)), p.g.n[o.s], p.g.per[o.s]);
+            // the next subcycle's positions; the last subcycle keeps its own
+            oct_move(p, o);
             P.xs[nxt][3 * o.i + o.s] = o.x;
-            P.xfs[nxt][3 * o.i + o.s] = (float)o.x;
+            P.xfs[nxt][3 * o.i + o.s] = o.xf;
         }
         if (sizeof(T) == 8) P.us[nxt][3 * o.i + o.s] = o.v;
-        else P.ufs[nxt][3 * o.i + o.s] = (float)o.v;
+        else P.ufs[nxt][3 * o.i + o.s] = o.vf;
     } else if (o.s < 6) {
         if (sizeof(T) == 8) P.oms[nxt][3 * o.i + o.s - 3] = o.v;
-        else P.omfs[nxt][3 * o.i + o.s - 3] = (float)o.v;
+        else P.omfs[nxt][3 * o.i + o.s - 3] = o.vf;
     }
 }
 
@@ -852,12 +888,12 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Pai
 // the squared components of lanes 0-2).
 __device__ __forceinline__ void oct_check_speed(const DemParams& p, const OctLane& o) {
     const unsigned FULL = 0xffffffffu;
-    const double sq = o.on && o.s < 3 ? o.v * o.v : 0.0;
     // the float32 sum decides unless it is near the limit
-    float q = (float)sq;
+    float q = o.on && o.s < 3 ? o.vf * o.vf : 0.f;
     q += __shfl_down_sync(FULL, q, 2, DEM_LANES) + __shfl_down_sync(FULL, q, 1, DEM_LANES);
     const bool near = o.on && o.s == 0 && !(q < 0.2499f);
     if (!__any_sync(FULL, near)) return;
+    const double sq = o.v * o.v;
     const double q1 = __shfl_down_sync(FULL, sq, 1, DEM_LANES), q2 = __shfl_down_sync(FULL, sq, 2, DEM_LANES);
     if (near && !((sq + q1) + q2 < 0.25)) atomicOr(p.status, ST_FAST_PARTICLE);
 }
@@ -870,7 +906,7 @@ __device__ __forceinline__ void oct_store(const DemParams& p, const OctLane& o) 
     if (!o.on || o.s >= 6) return;
     if (o.s < 3) {
         P.x[3 * o.i + o.s] = o.x;
-        P.xf[3 * o.i + o.s] = (float)o.x;
+        P.xf[3 * o.i + o.s] = o.xf;
         P.u[3 * o.i + o.s] = o.v;
         P.F_prev[3 * o.i + o.s] = o.f_prev;
     } else {
@@ -884,7 +920,7 @@ __device__ __forceinline__ void oct_store_view(const DemParams& p, const OctLane
     const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
     const double fl = floor(o.x);
     const int b = (int)fl;
-    const float fr = (float)(o.x - fl), v = (float)o.v;
+    const float fr = (float)(o.x - fl), v = o.vf;
     PartView w;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -904,9 +940,9 @@ __device__ __forceinline__ void oct_store_view(const DemParams& p, const OctLane
 __device__ __forceinline__ void oct_first_position(const DemParams& p, OctLane& o) {
     const Particles& P = p.P;
     if (!o.on || o.s >= 3) return;
-    o.x = wrap_pos(fma(p.dt * o.coef, o.f_prev, fma(p.dt, o.v, o.x)), p.g.n[o.s], p.g.per[o.s]);
+    oct_move(p, o);
     P.xs[0][3 * o.i + o.s] = o.x;
-    P.xfs[0][3 * o.i + o.s] = (float)o.x;
+    P.xfs[0][3 * o.i + o.s] = o.xf;
 }
 
 // one DEM subcycle of Algorithm 1 as a launch of its own (the initial force,
@@ -924,7 +960,7 @@ __device__ __forceinline__ void subcycle_body(const DemParams& p, int cur, int h
     const int nxt = 1 - cur;
     if (o.on && o.s < 3) {
         P.xs[nxt][3 * o.i + o.s] = o.x;
-        P.xfs[nxt][3 * o.i + o.s] = (float)o.x;
+        P.xfs[nxt][3 * o.i + o.s] = o.xf;
         P.us[nxt][3 * o.i + o.s] = o.v;
         P.F_prev[3 * o.i + o.s] = o.f_prev;
     } else if (o.on && o.s < 6) {
