@@ -471,10 +471,6 @@ double s_b_of(double s_nu, double lb) { return 1.0 / (0.5 + lb * (1.0 / s_nu - 0
 
 MapParams map_params(lbm_ctx* ctx) {
     MapParams mp{};
-    const int ts[3] = {TILE_X, TILE_Y, TILE_Z};
-    const double reach = ctx->r_max + std::fmax(ctx->relax.shell_width, 1.4142135623730951) + 0.02;
-    for (int a = 0; a < 3; ++a)
-        mp.small[a] = ctx->g.per[a] && ctx->g.n[a] <= 2.0 * reach + ts[a] + 2.0;
     mp.g = ctx->g; mp.P = ctx->P; mp.flags = ctx->flags; mp.owner = ctx->owner;
     mp.solid = ctx->solid; mp.shell = ctx->shell;
     for (int a = 0; a < 3; ++a) mp.ntile[a] = ctx->ntile[a];
@@ -1672,7 +1668,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
             zc.add(&z, 1);
             const MapParams mp = map_params(c);
             scat.add(&mp, (32 * np + 127) / 128);
-            map.add(&mp, (int)c->ntiles);
+            map.add(&mp, map_blocks(c->ntile));
             RefillParams rp{};
             rp.storage = c->storage;
             rp.f = c->f[1 - c->cur];

@@ -55,7 +55,7 @@ struct MapParams {
     Particles P;
     uint8_t* flags;
     int* owner;
-    uint32_t* solid;        // one bit per cell: solid, in the shell (both or neither NULL)
+    uint32_t* solid;        // one bit per cell: solid, in the shell (both NULL: a mapping without history)
     uint32_t* shell;
     int ntile[3];
     int* tile_count;
@@ -69,11 +69,11 @@ struct MapParams {
     unsigned int* miss_list;
     int* miss_count;
     int miss_cap;
-    int small[3];           // periodic axis too short for one image per tile
     int* status;
 };
 void launch_tile_scatter(const MapParams& p, cudaStream_t st);
 void launch_map(const MapParams& p, cudaStream_t st);
+int map_blocks(const int* ntile);   // blocks of a box in a gang launch of the mapping
 // the bits per cell from the flags (after a restore)
 void launch_cell_bits(const MapParams& p, cudaStream_t st);
 

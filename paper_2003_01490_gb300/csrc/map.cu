@@ -3,8 +3,8 @@
 //
 // Mapping: every particle registers itself in the candidate list of each
 // 32x4x4 tile that its influence sphere (R + max(delta_aB, sqrt 2)) touches;
-// then one thread per (x, y) column of the tile tests the tile's candidates
-// against its four cells. The solid test |x_c - x_p|^2 <= R^2 and the shell
+// then the tile's cells are tested against its candidates, eight cells a
+// thread. The solid test |x_c - x_p|^2 <= R^2 and the shell
 // test R^2 < |x_c - x_p|^2 <= (R + delta_aB)^2 are decided in float32 when the
 // margin is clear and re-evaluated in float64 with round-to-nearest and no
 // contraction, ((dx dx + dy dy) + dz dz), when a value lies within 1e-5
@@ -17,19 +17,25 @@
 // next step reads. The solid and shell cells are also written as one bit per
 // cell (a tile row of 32 cells is one word), from which the dense kernel finds
 // the particle links.
-#include <type_traits>
+#include <cstddef>
 
 #include "common.cuh"
 #include "gang.cuh"
 #include "launch.h"
+#include "sc_common.cuh"
 #include "scatter.cuh"
 
 // minimum resident mapping blocks per SM (a register cap)
 #ifndef LBM_MAP_MIN_BLOCKS
 #define LBM_MAP_MIN_BLOCKS 16
 #endif
+#ifndef LBM_MAP_DEPTH_MAX
+#define LBM_MAP_DEPTH_MAX 4
+#endif
 
 namespace lbmdem {
+
+constexpr int MAP_BLOCKS_WANTED = 152 * LBM_MAP_MIN_BLOCKS, MAP_DEPTH_MAX = LBM_MAP_DEPTH_MAX;
 
 __device__ __forceinline__ double min_image_dd(double d, int n, int per) {
     if (per) {
@@ -90,276 +96,425 @@ __device__ __forceinline__ float short_axis_image(float n, float g, int L) {
     return tw > fl ? n - fl : (tw < -fl ? n + fl : n);
 }
 
-// One block per 32x4x4 tile, 128 threads; warp w takes the 8x4x4 brick of
-// x in [8w, 8w + 8) (a compact brick meets fewer spheres than a 32-cell row),
-// lane l the column x = 8w + (l & 7), y = l >> 3 of its four z cells. Per
-// candidate the shared arrays hold the integer offset n0 of the tile's first
-// cell from the particle's base cell (as an exact float; on long periodic
-// axes already moved to the image nearest to the tile), the common fractional
-// offset g = 1/2 - frac, R^2 and the thresholds of the shell and near tests
-// with their float32 tolerances. A cell's offset is (n0 + l) + g with the
-// integer part formed first, so no float32 intermediate is larger than the
-// offset itself. Each warp first drops the candidates that cannot reach its
-// brick.
-// (tile bx, by, bz of the box)
-__device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int bz) {
-    static_assert(TILE_X == 32 && TILE_Y == 4, "four 8x4 column bricks per tile");
-    __shared__ float4 cn[TILE_CAP];
-    __shared__ float4 ca[TILE_CAP];
-    __shared__ float4 cb[TILE_CAP];
-    __shared__ unsigned int s_cnt[4];          // per warp: missing-link cells
-    __shared__ unsigned int s_solid[4];
-    __shared__ unsigned int s_base;
-    __shared__ unsigned char s_bits[2][TILE_Z * TILE_Y * 4];   // solid, shell: byte w of row (z, y) from warp w
-    const long long t = ((long long)bz * p.ntile[1] + by) * p.ntile[0] + bx;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int lx = 8 * warp + (lane & 7), ly = lane >> 3;
-    const int org[3] = {bx * TILE_X, by * TILE_Y, bz * TILE_Z};
-    const int x = org[0] + lx, y = org[1] + ly;
-    const int nx = p.g.n[0], ny = p.g.n[1], nz = p.g.n[2];
-    const long long plane = (long long)nx * ny;
-    const bool valid_xy = x < nx && y < ny;
-    const long long idx0 = (long long)org[2] * plane + (long long)y * nx + x;
-    // previous flags of the column, loaded before the candidate tests
-    static_assert(TILE_Z <= 8, "previous flags of a column packed in one word");
-    using ZWord = typename std::conditional<(TILE_Z > 4), unsigned long long, unsigned>::type;
-    ZWord old4 = 0;
+constexpr int MAP_THREADS = 64;
+constexpr int MISS_HELD = 256;     // missing-link cells a block holds back before it appends them
+static_assert(TILE_X == 32 && TILE_Y == 4 && TILE_Z == 4 && MAP_THREADS * 8 == TILE_X * TILE_Y * TILE_Z,
+              "a thread takes four cells of a tile row in two planes");
+static_assert(MAP_THREADS >= TILE_CAP, "one thread stages one candidate");
+
+// candidate k of a tile: the integer offset n of the tile's first cell from the
+// particle's base cell (an exact float; on long periodic axes already moved to
+// the image nearest to the tile), the common fractional offset g = 1/2 - frac,
+// R^2, (R + shell)^2, the near threshold and the tolerance of the float32 tests
+struct MapShared {
+    float4 cn[2][TILE_CAP];   // n, particle
+    float4 ca[2][TILE_CAP];   // g, R^2
+    float4 cb[2][TILE_CAP];   // (R + shell)^2, near, tolerance, axes (bits) without one image per tile
+    unsigned miss[MISS_HELD + TILE_X * TILE_Y * TILE_Z];
+    unsigned n_miss, base, n_solid[MAP_THREADS / 32];
+};
+
+// the first 36 bytes of a view: base, frac, R (as two 16-byte words and one of 4)
+struct MapView {
+    int4 a;
+    float4 b;
+};
+__device__ __forceinline__ MapView load_map_view(const PartView* v) {
+    static_assert(offsetof(PartView, frac) == 12 && offsetof(PartView, R) == 24, "two words hold base, frac and R");
+    const int4* q = reinterpret_cast<const int4*>(v);
+    MapView m;
+    m.a = q[0];
+    m.b = reinterpret_cast<const float4*>(q)[1];
+    return m;
+}
+
+__device__ __forceinline__ void stage_candidate(const MapParams& p, MapShared& sh, int buf, int k, int i,
+                                                const MapView& v, int ox, int oy, int oz) {
+    const int org[3] = {ox, oy, oz}, base[3] = {v.a.x, v.a.y, v.a.z};
+    const float frac[3] = {__int_as_float(v.a.w), v.b.x, v.b.y};
+    const int ts[3] = {TILE_X, TILE_Y, TILE_Z};
+    const float R = v.b.z;
+    const float sw = (float)p.shell_width;
+    const float reach = R + fmaxf(sw, 1.4142136f) + 0.02f;
+    float n0[3], g[3];
+    unsigned small = 0;
 #pragma unroll
-    for (int j = 0; j < TILE_Z; ++j)
-        if (valid_xy && org[2] + j < nz) old4 |= (ZWord)p.flags[idx0 + j * plane] << (8 * j);
-    const int c = p.tile_count[t];
-    const int ncand = c < TILE_CAP ? c : TILE_CAP;
-    if (tid < ncand) {
-        const int i = p.tile_list[t * TILE_CAP + tid];
-        const PartView v = p.P.view[i];
-        const int ts[3] = {TILE_X, TILE_Y, TILE_Z};
-        float n0[3], g[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            int n = org[d] - v.base[d];
-            g[d] = 0.5f - v.frac[d];
-            if (p.g.per[d] && !p.small[d]) {
+    for (int d = 0; d < 3; ++d) {
+        int n = org[d] - base[d];
+        g[d] = 0.5f - frac[d];
+        if (p.g.per[d]) {
+            const int L = p.g.n[d];
+            if ((float)L <= 2.0f * reach + (float)(ts[d] + 2)) {
+                small |= 1u << d;   // some cells of the tile may be nearer to another image
+            } else {
                 // image nearest to the tile centre
-                const int L = p.g.n[d];
                 const float cc = (float)(2 * n + ts[d] - 1) + 2.0f * g[d];   // twice the centre offset
                 if (cc > (float)L) n -= L;
                 else if (cc < -(float)L) n += L;
             }
-            n0[d] = (float)n;
         }
-        const float R = v.R;
-        const float Rs = R + (float)p.shell_width;
-        const float Rn = R + 1.4142135f + 0.02f;
-        const float R2 = R * R, Rs2 = Rs * Rs;
-        cn[tid] = make_float4(n0[0], n0[1], n0[2], __int_as_float(i));
-        ca[tid] = make_float4(g[0], g[1], g[2], R2);
-        cb[tid] = make_float4(Rs2, Rn * Rn, 1e-5f * (R2 + 1.0f), 1e-5f * (Rs2 + 1.0f));
+        n0[d] = (float)n;
     }
-    __syncthreads();
-    // the tile's candidate count is consumed: reset it for the next scatter
-    if (tid == 0) p.tile_count[t] = 0;
+    const float Rs = R + sw;
+    const float Rn = R + 1.4142135f + 0.02f;
+    const float R2 = R * R, Rs2 = Rs * Rs;
+    // d2 <= Rn^2 as d2 < the next float
+    const float near = __int_as_float(__float_as_int(Rn * Rn) + 1);
+    sh.cn[buf][k] = make_float4(n0[0], n0[1], n0[2], __int_as_float(i));
+    sh.ca[buf][k] = make_float4(g[0], g[1], g[2], R2);
+    sh.cb[buf][k] = make_float4(Rs2, near, 1e-5f * (Rs2 + 1.0f), __uint_as_float(small));
+}
 
-    const bool any_small = p.small[0] | p.small[1] | p.small[2];
-    const float flx = (float)lx, fly = (float)ly;
-    const float bx0 = (float)(8 * warp);
-    // candidates that may reach this warp's brick (conservative float bound)
-    unsigned relm[2];
+__device__ __forceinline__ float lo_of(F2 a) {
+    float lo, hi;
+    split(a, lo, hi);
+    return lo;
+}
+__device__ __forceinline__ float hi_of(F2 a) {
+    float lo, hi;
+    split(a, lo, hi);
+    return hi;
+}
+// bit j of the result: the sign of t[j]
+__device__ __forceinline__ unsigned signs(const F2 (&t)[4]) {
+    unsigned m = __float_as_uint(hi_of(t[3])) >> 31;
+    m = __funnelshift_l(__float_as_uint(lo_of(t[3])), m, 1);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int k = lane + 32 * h;
-        bool rel = false;
-        if (k < ncand) {
-            if (any_small) {
-                rel = true;
-            } else {
-                const float4 Nn = cn[k], A = ca[k], B = cb[k];
-                const float xlo = (Nn.x + bx0) + A.x, xhi = (Nn.x + (bx0 + 7.0f)) + A.x;
-                const float ylo = Nn.y + A.y, yhi = (Nn.y + (float)(TILE_Y - 1)) + A.y;
-                const float zlo = Nn.z + A.z, zhi = (Nn.z + (float)(TILE_Z - 1)) + A.z;
-                const float dx = xlo > 0.f ? xlo : (xhi < 0.f ? -xhi : 0.f);
-                const float dy = ylo > 0.f ? ylo : (yhi < 0.f ? -yhi : 0.f);
-                const float dz = zlo > 0.f ? zlo : (zhi < 0.f ? -zhi : 0.f);
-                const float reach = fmaxf(B.y, B.x + B.w) * 1.0001f + 0.01f;
-                rel = dx * dx + dy * dy + dz * dz <= reach;
-            }
-        }
-        relm[h] = __ballot_sync(0xffffffffu, rel);
+    for (int k = 2; k >= 0; --k) {
+        m = __funnelshift_l(__float_as_uint(hi_of(t[k])), m, 1);
+        m = __funnelshift_l(__float_as_uint(lo_of(t[k])), m, 1);
     }
+    return m;
+}
+// bit j of m to bit 0 of byte j
+__device__ __forceinline__ unsigned bytes_of(unsigned m) { return (m * 0x00204081u) & 0x01010101u; }
 
-    int own[TILE_Z];
-    unsigned shell4 = 0;               // per z: shell bit
-    unsigned near1 = 0, near2 = 0;     // per z: near one / two particles
-    unsigned multi4 = 0;               // per z: inside a second sphere
-#pragma unroll
-    for (int j = 0; j < TILE_Z; ++j) own[j] = 0x7fffffff;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        unsigned mm = relm[h];
-        while (mm) {
-            const int k = __ffs(mm) - 1 + 32 * h;
-            mm &= mm - 1;
-            const float4 Nn = cn[k], A = ca[k], B = cb[k];
-            const int id = __float_as_int(Nn.w);
-            float fx = Nn.x + flx, fy = Nn.y + fly;
-            if (any_small) {
-                if (p.small[0]) fx = short_axis_image(fx, A.x, nx);
-                if (p.small[1]) fy = short_axis_image(fy, A.y, ny);
-            }
-            const float dx = fx + A.x, dy = fy + A.y;
-            const float sxy = dx * dx + dy * dy;
-            const float far2 = B.x + B.w;
-#pragma unroll
-            for (int j = 0; j < TILE_Z; ++j) {
-                float fz = Nn.z + (float)j;
-                if (any_small && p.small[2]) fz = short_axis_image(fz, A.z, nz);
-                const float dz = fz + A.z;
-                const float d2f = sxy + dz * dz;
-                if (d2f <= B.y) {
-                    near2 |= near1 & (1u << j);
-                    near1 |= 1u << j;
-                }
-                if (d2f > far2) continue;
-                const bool exact_needed = fabsf(d2f - A.w) <= B.z || fabsf(d2f - B.x) <= B.w;
-                bool inside, in_shell;
-                if (!exact_needed) {
-                    inside = d2f < A.w;
-                    in_shell = !inside && d2f < B.x;
-                } else {
-                    const int r = exact_tests(p, id, x, y, org[2] + j);
-                    inside = r & 1;
-                    in_shell = (r & 2) != 0;
-                }
-                if (inside) {
-                    if (own[j] != 0x7fffffff) multi4 |= 1u << j;
-                    if (id < own[j]) own[j] = id;
-                }
-                else if (in_shell) shell4 |= 1u << j;
-            }
-        }
-    }
-
-    bool wall_xy = false;
-    if (!p.g.per[0] && (x == 0 || x == nx - 1)) wall_xy = true;
-    if (!p.g.per[1] && (y == 0 || y == ny - 1)) wall_xy = true;
-    unsigned miss_bits = 0, solid_bits = 0, shell_bits = 0;
-#pragma unroll
-    for (int j = 0; j < TILE_Z; ++j) {
-        const int z = org[2] + j;
-        if (!valid_xy || z >= nz) continue;
-        const long long idx = idx0 + j * plane;
-        const bool wall_adj = wall_xy || (!p.g.per[2] && (z == 0 || z == nz - 1));
-        const unsigned nn = ((near1 >> j) & 1u) + ((near2 >> j) & 1u);
-        const uint8_t old = (uint8_t)(old4 >> (8 * j));
-        uint8_t nf = 0;
-        if (own[j] != 0x7fffffff) {
-            nf = FL_SOLID;
-            solid_bits |= 1u << j;
-            if (nn >= 2u || wall_adj) {
-                nf |= FL_MISS;
-                miss_bits |= 1u << j;
-            }
-            if ((multi4 >> j) & 1u) nf |= FL_MULTI;
-            p.owner[idx] = own[j];
-        } else {
-            if (shell4 & (1u << j)) {
-                nf |= FL_SHELL;
-                shell_bits |= 1u << j;
-            }
-            if (nn >= 1u) nf |= FL_NEAR;
-            if (old & FL_SOLID) {
-                // uncovered this step: refill with the former particle's velocity
-                nf |= FL_NEWFLUID;
-                const int prev = p.owner[idx];
-                p.owner[idx] = -1;
-                const int slot = atomicAdd(p.refill_count, 1);
-                if (slot < p.refill_cap) {
-                    p.refill_list[slot] = (unsigned int)idx;
-                    p.refill_owner[slot] = prev;
-                } else {
-                    atomicOr(p.status, ST_REFILL_OVERFLOW);
-                }
-            }
-        }
-        p.flags[idx] = nf;
-    }
-
-    // block-aggregated append to the missing-link list and solid count
+// Mapping of the tiles (bx, by, z0) .. (bx, by, z1 - 1) by one block. A warp takes
+// half a tile, the 16x4x4 brick at x in 16 warp .. (a compact brick meets fewer
+// spheres than rows of 32 cells), lane l eight cells: x from 4 (l & 3), y = (l >> 2)
+// & 3, z = 2 (l >> 4) and the next; bit 4 h + j of its masks is cell x + j of plane
+// z + h. Offsets are (n + l) + g with the integer part formed first, so no float32
+// intermediate is larger than the offset itself. Each warp first drops the
+// candidates that cannot reach its brick. While a tile is tested the candidates of
+// the next one are on their way.
+//
+// Bound by instruction issue and, in small boxes, by the chain from the tile's
+// count to its list, the views and the tests. A thread per (x, y) column with a
+// test per cell and byte-wide flags issued 787 warp instructions per 128 cells
+// at 76 % of the slots: 204 us for 256x256x512 cells and 10,000 spheres, 35 us for
+// 128x128x256 and 1,250, and without history 312 us plus 50 us for clearing the
+// outputs. Here the distances of eight cells are packed float32 arithmetic, every
+// decision is a mask of eight bits from the signs of the differences, flags are
+// written as words and owners as vectors (bytes and single words where a side is
+// no multiple of four), and a block appends to the shared counters once: 725
+// instructions per 256 cells at 59 %, 113 us, 25 us and 87 us without clearing.
+// (Four cells a thread: 137 us. 12 resident blocks 119 us, 20 136 us; walks of 8
+// tiles 115 us, 16 123 us.)
+//
+// FRESH: the outputs of a box without history (flags and owner only: the owner
+// of every cell is written, nothing is read, no list is kept).
+template <bool FRESH>
+__device__ __forceinline__ void map_body(const MapParams& p, int bx, int by, int z0, int z1) {
+    __shared__ MapShared sh;
     const unsigned FULL = 0xffffffffu;
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned mb[TILE_Z];
-    unsigned wm = 0, ws = 0;
-#pragma unroll
-    for (int j = 0; j < TILE_Z; ++j) {
-        mb[j] = __ballot_sync(FULL, (miss_bits >> j) & 1u);
-        wm += __popc(mb[j]);
-        const unsigned sb = __ballot_sync(FULL, (solid_bits >> j) & 1u);
-        const unsigned hb = __ballot_sync(FULL, (shell_bits >> j) & 1u);
-        ws += __popc(sb);
-        // lane l is column x = 8 warp + (l & 7), y = l >> 3: byte y of a ballot
-        if (lane < TILE_Y) {
-            s_bits[0][(j * TILE_Y + lane) * 4 + warp] = (unsigned char)(sb >> (8 * lane));
-            s_bits[1][(j * TILE_Y + lane) * 4 + warp] = (unsigned char)(hb >> (8 * lane));
-        }
+    int tid;   // opaque, or the compiler reads the special register again and again
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    const int warp = tid >> 5, lane = tid & 31;
+    const int lx = 16 * warp + 4 * (lane & 3), ly = (lane >> 2) & 3, lz = 2 * (lane >> 4);
+    const int nx = p.g.n[0], ny = p.g.n[1], nz = p.g.n[2];
+    const int ox = bx * TILE_X, oy = by * TILE_Y;
+    const int x = ox + lx, y = oy + ly;
+    const int plane = nx * ny;   // cells and words of a box are counted in 31 bits
+    const int nt = p.ntile[0] * p.ntile[1], words = p.ntile[0] * ny;
+    const bool vec = ((nx & 3) | ((unsigned)(uintptr_t)p.flags & 3) | ((unsigned)(uintptr_t)p.owner & 15)) == 0;
+    const unsigned valid_xy = y < ny ? (x + 4 <= nx ? 15u : (x < nx ? (1u << (nx - x)) - 1u : 0u)) : 0u;
+    // cells of the quad next to a wall in x or y
+    unsigned wall_xy = 0;
+    if (!p.g.per[0]) {
+        if (x == 0) wall_xy |= 1u;
+        if (nx - 1 >= x && nx - 1 < x + 4) wall_xy |= 1u << (nx - 1 - x);
     }
-    if (lane == 0) {
-        s_cnt[warp] = wm;
-        s_solid[warp] = ws;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        unsigned tm = 0;
-        unsigned long long tsol = 0;
-        for (int w = 0; w < 4; ++w) {
-            const unsigned c = s_cnt[w];
-            s_cnt[w] = tm;
-            tm += c;
-            tsol += s_solid[w];
-        }
-        s_base = tm ? (unsigned)atomicAdd(p.miss_count, (int)tm) : 0u;
-        if (tsol) atomicAdd(p.n_solid, tsol);
-    }
-    if (p.solid && tid >= 32 && tid < 32 + 2 * TILE_Z * TILE_Y) {
-        const int k = tid - 32, kind = k / (TILE_Z * TILE_Y), row = k % (TILE_Z * TILE_Y);
-        const int yy = org[1] + row % TILE_Y, zz = org[2] + row / TILE_Y;
-        if (yy < ny && zz < nz) {
-            const unsigned char* b = s_bits[kind] + 4 * row;
-            const uint32_t word = b[0] | (uint32_t)b[1] << 8 | (uint32_t)b[2] << 16 | (uint32_t)b[3] << 24;
-            (kind ? p.shell : p.solid)[((long long)zz * ny + yy) * p.ntile[0] + bx] = word;
-        }
+    if (!p.g.per[1] && (y == 0 || y == ny - 1)) wall_xy = 15u;
+    wall_xy *= 0x11u;
+    const float flx = (float)lx, fly = (float)ly, flz = (float)lz;
+
+    int t = (z0 * p.ntile[1] + by) * p.ntile[0] + bx;
+    int c_cur = min(p.tile_count[t], TILE_CAP);
+    int c_nxt = z0 + 1 < z1 ? min(p.tile_count[t + nt], TILE_CAP) : 0;
+    if (tid == 0) sh.n_miss = 0;
+    if (tid < c_cur) {
+        const int i = p.tile_list[(long long)t * TILE_CAP + tid];
+        stage_candidate(p, sh, 0, tid, i, load_map_view(p.P.view + i), ox, oy, z0 * TILE_Z);
     }
     __syncthreads();
-    if (miss_bits) {
-        int sm = (int)(s_base + s_cnt[warp]);
+
+    unsigned solid_count = 0;
+    int z = z0 * TILE_Z + lz;
+    int idx = z * plane + y * nx + x;
+    int half = 2 * (z * words + y * p.ntile[0] + bx) + warp;   // the row's 16 cells in the bits
+    for (int bz = z0; bz < z1; ++bz, t += nt, z += TILE_Z, idx += TILE_Z * plane, half += 2 * TILE_Z * words) {
+        const int buf = (bz - z0) & 1;
+        const unsigned valid = (z < nz ? valid_xy : 0u) | (z + 1 < nz ? valid_xy << 4 : 0u);
+        // the next tile's list entry, the count after it, the cells solid before
+        int next_i = 0;
+        const bool stage = tid < c_nxt;
+        if (stage) next_i = p.tile_list[(long long)(t + nt) * TILE_CAP + tid];
+        const int c_after = bz + 2 < z1 ? min(p.tile_count[t + 2 * nt], TILE_CAP) : 0;
+        unsigned old0 = 0, old1 = 0;
+        if (!FRESH && (valid & 15u)) old0 = reinterpret_cast<const unsigned short*>(p.solid)[half];
+        if (!FRESH && (valid >> 4)) old1 = reinterpret_cast<const unsigned short*>(p.solid)[half + 2 * words];
+
+        int own[8];
 #pragma unroll
-        for (int j = 0; j < TILE_Z; ++j) {
-            if ((miss_bits >> j) & 1u) {
-                const int slot = sm + __popc(mb[j] & lt);
-                if (slot < p.miss_cap) p.miss_list[slot] = (unsigned)(idx0 + j * plane);
+        for (int j = 0; j < 8; ++j) own[j] = 0x7fffffff;
+        unsigned near1 = 0, near2 = 0;     // cells near one / two particles
+        unsigned solid = 0, multi = 0, shell = 0;
+        for (int k0 = 0; k0 < c_cur; k0 += 32) {
+            // candidates that may reach this warp's brick (conservative float bound)
+            bool rel = false;
+            if (k0 + lane < c_cur) {
+                const float4 N = sh.cn[buf][k0 + lane], A = sh.ca[buf][k0 + lane], B = sh.cb[buf][k0 + lane];
+                const float xlo = (N.x + (float)(16 * warp)) + A.x, xhi = xlo + 15.0f;
+                const float ylo = N.y + A.y, yhi = ylo + 3.0f;
+                const float zlo = N.z + A.z, zhi = zlo + 3.0f;
+                const float dx = fmaxf(fmaxf(xlo, -xhi), 0.f), dy = fmaxf(fmaxf(ylo, -yhi), 0.f),
+                            dz = fmaxf(fmaxf(zlo, -zhi), 0.f);
+                const float far = fmaxf(B.y, B.x + B.z) * 1.0001f + 0.01f;
+                rel = dx * dx + dy * dy + dz * dz <= far || __float_as_uint(B.w) != 0u;
+            }
+            unsigned mm = __ballot_sync(FULL, rel);
+            while (mm) {
+                const int k = __ffs(mm) - 1 + k0;
+                mm &= mm - 1;
+                const float4 N = sh.cn[buf][k], A = sh.ca[buf][k], B = sh.cb[buf][k];
+                const int id = __float_as_int(N.w);
+                const float fx = N.x + flx;
+                float fy = N.y + fly, fz0 = N.z + flz, fz1 = fz0 + 1.0f;
+                F2 x01 = f2(fx, fx + 1.0f), x23 = f2(fx + 2.0f, fx + 3.0f);
+                const unsigned small = __float_as_uint(B.w);
+                if (small) {
+                    if (small & 1u) {
+                        x01 = f2(short_axis_image(fx, A.x, nx), short_axis_image(fx + 1.0f, A.x, nx));
+                        x23 = f2(short_axis_image(fx + 2.0f, A.x, nx), short_axis_image(fx + 3.0f, A.x, nx));
+                    }
+                    if (small & 2u) fy = short_axis_image(fy, A.y, ny);
+                    if (small & 4u) {
+                        fz0 = short_axis_image(fz0, A.z, nz);
+                        fz1 = short_axis_image(fz1, A.z, nz);
+                    }
+                }
+                const float dy = fy + A.y, dz0 = fz0 + A.z, dz1 = fz1 + A.z;
+                const float dy2 = __fmul_rn(dy, dy);
+                const F2 gx = f2(A.x, A.x), vy = f2(dy2, dy2), va = f2(dz0, dz0), vb = f2(dz1, dz1);
+                const F2 dx01 = x01 + gx, dx23 = x23 + gx;
+                const F2 p01 = mad(dx01, dx01, vy), p23 = mad(dx23, dx23, vy);
+                const F2 d[4] = {mad(va, va, p01), mad(va, va, p23), mad(vb, vb, p01), mad(vb, vb, p23)};
+                const F2 r2 = f2(A.w, A.w), s2 = f2(B.x, B.x), n2 = f2(B.y, B.y);
+                const F2 di[4] = {d[0] - r2, d[1] - r2, d[2] - r2, d[3] - r2};
+                const F2 dh[4] = {d[0] - s2, d[1] - s2, d[2] - s2, d[3] - s2};
+                const F2 dn[4] = {d[0] - n2, d[1] - n2, d[2] - n2, d[3] - n2};
+                const unsigned near = signs(dn);
+                unsigned in = signs(di), within = signs(dh);
+                float least = fabsf(lo_of(di[0]));
+#pragma unroll
+                for (int k2 = 0; k2 < 4; ++k2) {
+                    least = fminf(fminf(least, fabsf(lo_of(di[k2]))), fabsf(hi_of(di[k2])));
+                    least = fminf(fminf(least, fabsf(lo_of(dh[k2]))), fabsf(hi_of(dh[k2])));
+                }
+                if (least <= B.z) {
+                    // within the tolerance of a threshold: the float64 decision
+                    unsigned close = 0;
+#pragma unroll
+                    for (int k2 = 0; k2 < 4; ++k2) {
+                        if (fabsf(lo_of(di[k2])) <= B.z || fabsf(lo_of(dh[k2])) <= B.z) close |= 1u << (2 * k2);
+                        if (fabsf(hi_of(di[k2])) <= B.z || fabsf(hi_of(dh[k2])) <= B.z) close |= 2u << (2 * k2);
+                    }
+                    close &= valid;
+                    while (close) {
+                        const int j = __ffs(close) - 1;
+                        close &= close - 1;
+                        const int r = exact_tests(p, id, x + (j & 3), y, z + (j >> 2));
+                        in = (in & ~(1u << j)) | (unsigned)(r & 1) << j;
+                        within = (within & ~(1u << j)) | (unsigned)(r != 0) << j;
+                    }
+                }
+                near2 |= near1 & near;
+                near1 |= near;
+                shell |= within & ~in;
+                if (in) {
+                    multi |= solid & in;
+                    solid |= in;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (in & (1u << j)) own[j] = min(own[j], id);
+                }
+            }
+        }
+
+        // the next tile's views
+        MapView nv{};
+        if (stage) nv = load_map_view(p.P.view + next_i);
+
+        solid &= valid;
+        const unsigned fluid = valid & ~solid;
+        shell &= fluid;
+        unsigned wall = wall_xy;
+        if (!p.g.per[2]) {
+            if (z == 0 || z == nz - 1) wall |= 0x0fu;
+            if (z + 1 == nz - 1) wall |= 0xf0u;
+        }
+        const unsigned miss = solid & (near2 | wall);
+        unsigned fresh = 0;   // uncovered now
+        if (!FRESH) fresh = (((old0 >> (4 * (lane & 3))) & 15u) | ((old1 >> (4 * (lane & 3))) & 15u) << 4) & fluid;
+        near1 &= fluid;
+        multi &= solid;
+        // refill with the former particle's velocity
+        for (unsigned m = fresh; m; m &= m - 1) {
+            const int j = __ffs(m) - 1, c = idx + (j & 3) + (j >> 2) * plane;
+            const int prev = p.owner[c];
+            p.owner[c] = -1;
+            const int slot = atomicAdd(p.refill_count, 1);
+            if (slot < p.refill_cap) {
+                p.refill_list[slot] = (unsigned int)c;
+                p.refill_owner[slot] = prev;
+            } else {
+                atomicOr(p.status, ST_REFILL_OVERFLOW);
+            }
+        }
+        const unsigned write_own = FRESH ? valid : solid;
+        if (FRESH) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (own[j] == 0x7fffffff) own[j] = -1;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            auto quad = [&](unsigned m) { return bytes_of((m >> (4 * h)) & 15u); };
+            unsigned word = quad(solid) * FL_SOLID + quad(shell) * FL_SHELL + quad(near1) * FL_NEAR;
+            if (miss | multi | fresh) word += quad(miss) * FL_MISS + quad(multi) * FL_MULTI + quad(fresh) * FL_NEWFLUID;
+            const unsigned v = (valid >> (4 * h)) & 15u, wo = (write_own >> (4 * h)) & 15u;
+            uint8_t* const fl = p.flags + (idx + h * plane);
+            int* const ow = p.owner + (idx + h * plane);
+            if (vec) {
+                if (v) *reinterpret_cast<unsigned*>(fl) = word;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (v & (1u << j)) fl[j] = (uint8_t)(word >> (8 * j));
+            }
+            if (vec && wo == 15u) {
+                *reinterpret_cast<int4*>(ow) = make_int4(own[4 * h], own[4 * h + 1], own[4 * h + 2], own[4 * h + 3]);
+            } else if (wo) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (wo & (1u << j)) ow[j] = own[4 * h + j];
+            }
+        }
+        bool flush_it = false;
+        if (!FRESH) {
+            // solid and shell bits of the rows' 16 cells, from their four lanes
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                unsigned bits = (((solid >> (4 * h)) & 15u) | ((shell >> (4 * h)) & 15u) << 16) << (4 * (lane & 3));
+                bits |= __shfl_xor_sync(FULL, bits, 1);
+                bits |= __shfl_xor_sync(FULL, bits, 2);
+                if ((lane & 3) == 0 && y < ny && z + h < nz) {
+                    reinterpret_cast<unsigned short*>(p.solid)[half + 2 * h * words] = (unsigned short)bits;
+                    reinterpret_cast<unsigned short*>(p.shell)[half + 2 * h * words] = (unsigned short)(bits >> 16);
+                }
+            }
+            solid_count += __popc(solid);
+            if (__any_sync(FULL, miss != 0u)) {
+                const int n = __popc(miss);
+                int at = n;   // inclusive sum over the lanes
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, at, o);
+                    if (lane >= o) at += v;
+                }
+                unsigned base = 0;
+                if (lane == 31) base = atomicAdd(&sh.n_miss, (unsigned)at);
+                base = __shfl_sync(FULL, base, 31);
+                const unsigned end = base + (unsigned)__shfl_sync(FULL, at, 31);
+                flush_it = end > (unsigned)MISS_HELD;
+                unsigned slot = base + (unsigned)(at - n);
+                for (unsigned m = miss; m; m &= m - 1) {
+                    const int j = __ffs(m) - 1;
+                    sh.miss[slot++] = (unsigned)(idx + (j & 3) + (j >> 2) * plane);
+                }
+            }
+        }
+        if (stage) stage_candidate(p, sh, buf ^ 1, tid, next_i, nv, ox, oy, (bz + 1) * TILE_Z);
+        if (tid == 0) p.tile_count[t] = 0;   // consumed: zero for the next scatter
+        c_cur = c_nxt;
+        c_nxt = c_after;
+        if (FRESH) {
+            __syncthreads();
+        } else if (__syncthreads_or(flush_it || bz + 1 == z1)) {
+            // append the cells held back to the list
+            const unsigned n = sh.n_miss;
+            if (tid == 0 && n) sh.base = (unsigned)atomicAdd(p.miss_count, (int)n);
+            __syncthreads();
+            for (unsigned k = tid; k < n; k += MAP_THREADS) {
+                const unsigned slot = sh.base + k;
+                if (slot < (unsigned)p.miss_cap) p.miss_list[slot] = sh.miss[k];
                 else atomicOr(p.status, ST_REFILL_OVERFLOW);
             }
-            sm += __popc(mb[j]);
+            if (tid == 0) sh.n_miss = 0;
+            __syncthreads();
+        }
+    }
+    if (!FRESH) {
+        const unsigned ws = __reduce_add_sync(FULL, solid_count);
+        if (lane == 0) sh.n_solid[warp] = ws;
+        __syncthreads();
+        if (tid == 0) {
+            unsigned n = 0;
+#pragma unroll
+            for (int w = 0; w < MAP_THREADS / 32; ++w) n += sh.n_solid[w];
+            if (n) atomicAdd(p.n_solid, (unsigned long long)n);
         }
     }
 }
 
-__global__ void __launch_bounds__(128, LBM_MAP_MIN_BLOCKS) map_kernel(const __grid_constant__ MapParams p) {
-    map_body(p, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
+template <bool FRESH>
+__global__ void __launch_bounds__(MAP_THREADS, LBM_MAP_MIN_BLOCKS)
+    map_kernel(const __grid_constant__ MapParams p, int depth) {
+    const int z0 = (int)blockIdx.z * depth;
+    map_body<FRESH>(p, (int)blockIdx.x, (int)blockIdx.y, z0, min(z0 + depth, p.ntile[2]));
 }
 
-// instance i's tiles are its blocks off[i] .. off[i + 1] - 1, x fastest
-__global__ void __launch_bounds__(128, LBM_MAP_MIN_BLOCKS / 2)
+// Tiles in z that a block walks: as many as keep the blocks resident at once,
+// at most four (a longer walk hides more of the loads but leaves an emptier end)
+int map_depth(const int* ntile) {
+    const long long columns = (long long)ntile[0] * ntile[1];
+    const long long d = (columns * ntile[2] + MAP_BLOCKS_WANTED - 1) / MAP_BLOCKS_WANTED;
+    return (int)(d < 1 ? 1 : (d > MAP_DEPTH_MAX ? MAP_DEPTH_MAX : d));
+}
+
+int map_blocks(const int* ntile) {
+    const int d = map_depth(ntile);
+    return ntile[0] * ntile[1] * ((ntile[2] + d - 1) / d);
+}
+
+// instance i's tiles are walked by its blocks off[i] .. off[i + 1] - 1, x fastest
+__global__ void __launch_bounds__(MAP_THREADS, LBM_MAP_MIN_BLOCKS)
     map_gang_kernel(const MapParams* __restrict__ table, const int* __restrict__ off, int n) {
     __shared__ __align__(16) MapParams sp;
     const int i = gang_instance(off, n, (int)blockIdx.x);
     gang_load(table, i, sp);
     const int b = (int)blockIdx.x - off[i];
-    const int t0 = sp.ntile[0], t1 = sp.ntile[1];
-    map_body(sp, b % t0, (b / t0) % t1, b / (t0 * t1));
+    const int t0 = sp.ntile[0], t1 = sp.ntile[1], layers = (off[i + 1] - off[i]) / (t0 * t1);
+    const int depth = (sp.ntile[2] + layers - 1) / layers;
+    const int z0 = b / (t0 * t1) * depth;
+    map_body<false>(sp, b % t0, (b / t0) % t1, z0, min(z0 + depth, sp.ntile[2]));
 }
 
 void launch_map(const MapParams& p, cudaStream_t st) {
-    dim3 grid(p.ntile[0], p.ntile[1], p.ntile[2]);
-    map_kernel<<<grid, TILE_X * TILE_Y, 0, st>>>(p);
+    const int d = map_depth(p.ntile);
+    const dim3 grid(p.ntile[0], p.ntile[1], (p.ntile[2] + d - 1) / d);
+    if (p.solid) map_kernel<false><<<grid, MAP_THREADS, 0, st>>>(p, d);
+    else map_kernel<true><<<grid, MAP_THREADS, 0, st>>>(p, d);
 }
 
 // one thread per word of 32 cells
@@ -527,7 +682,7 @@ void launch_map_gang(int kind, int storage, const void* table, const int* off, i
     if (kind == GANG_SCATTER) {
         tile_scatter_gang_kernel<<<blocks, 128, 0, st>>>(static_cast<const MapParams*>(table), off, n);
     } else if (kind == GANG_MAP) {
-        map_gang_kernel<<<blocks, TILE_X * TILE_Y, 0, st>>>(static_cast<const MapParams*>(table), off, n);
+        map_gang_kernel<<<blocks, MAP_THREADS, 0, st>>>(static_cast<const MapParams*>(table), off, n);
     } else {
         const RefillParams* t = static_cast<const RefillParams*>(table);
         switch (storage) {

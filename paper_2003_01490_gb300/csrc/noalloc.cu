@@ -13,6 +13,7 @@
 #include "../../include/lbmdem.h"
 #include "common.cuh"
 #include "launch.h"
+#include "scatter.cuh"
 
 namespace lbmdem {
 
@@ -21,38 +22,32 @@ constexpr int NOALLOC_MAX_TILES = 98304;      // boxes up to 50,331,648 cells
 constexpr int NOALLOC_MAX_SPHERES = 65536;
 
 struct NoallocScratch {
+    int status[4];            // one word used; cleared together with the counts
     int tile_count[NOALLOC_MAX_TILES];
     int tile_list[NOALLOC_MAX_TILES * TILE_CAP];
     PartView view[NOALLOC_MAX_SPHERES];
-    float xf[3 * NOALLOC_MAX_SPHERES];
-    unsigned long long n_solid;
-    int counters[4];          // refill and missing-link counts (the lists are disabled)
-    int status;
-    unsigned int dummy_list[4];
 };
 
 // about 29 MB; shared by every call on a device
 static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 
-// float views (base cell + fraction, radius) of the spheres for the mapping
-__global__ void noalloc_view_kernel(int n, const double* __restrict__ pos, const double* __restrict__ radius,
-                                    NoallocScratch* s) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    PartView v;
-    for (int d = 0; d < 3; ++d) {
-        const double x = pos[3 * i + d];
-        const double b = floor(x);
-        v.base[d] = (int)b;
-        v.frac[d] = (float)(x - b);
-        v.u[d] = 0.f;
-        v.om[d] = 0.f;
-        s->xf[3 * i + d] = (float)x;
+// one warp per sphere: its float view (base cell + fraction, radius) for the
+// mapping and its entries in the tile lists
+__global__ void __launch_bounds__(128) noalloc_scatter_kernel(const __grid_constant__ MapParams p) {
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (i >= p.P.n) return;   // warp-uniform
+    const double x[3] = {p.P.x[3 * i], p.P.x[3 * i + 1], p.P.x[3 * i + 2]};
+    if (lane == 0) {
+        PartView v{};   // the rest is unused by the mapping
+        for (int d = 0; d < 3; ++d) {
+            const double b = floor(x[d]);
+            v.base[d] = (int)b;
+            v.frac[d] = (float)(x[d] - b);
+        }
+        v.R = (float)p.P.R[i];
+        p.P.view[i] = v;
     }
-    v.R = (float)radius[i];
-    v.C = 0.f;   // unused by the mapping
-    v.C_lo = 0.f;
-    s->view[i] = v;
+    tile_scatter_particle(p, i, x, lane, 32);
 }
 
 namespace {
@@ -133,27 +128,18 @@ extern "C" lbm_status lbm_map_spheres_noalloc(const lbm_grid* grid, double shell
             }
         }
     } sync_on_exit{st};
-    // outputs start as a box without particles; shared counters start at zero
-    if ((e = cudaMemsetAsync(d_flags, 0, (size_t)ncells, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(d_owner, 0xff, 4 * (size_t)ncells, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s->tile_count, 0, sizeof(int) * (size_t)ntiles, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(&s->n_solid, 0, sizeof(unsigned long long), st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s->counters, 0, sizeof(s->counters), st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(&s->status, 0, sizeof(int), st)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(s->status, 0, sizeof(s->status) + sizeof(int) * (size_t)ntiles, st)) != cudaSuccess)
         return noalloc_fail(LBM_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
     Particles P{};
     P.n = n;
     P.x = const_cast<double*>(d_pos);
     P.R = const_cast<double*>(d_radius);
     P.view = s->view;
-    P.xf = s->xf;
-    if (n > 0) noalloc_view_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, d_pos, d_radius, s);
-    MapParams mp{};
+    MapParams mp{};   // no bits per cell: the mapping writes flags and owners only, all of them
     mp.g.n[0] = grid->nx; mp.g.n[1] = grid->ny; mp.g.n[2] = grid->nz;
     for (int a = 0; a < 3; ++a) {
         mp.g.per[a] = grid->periodic[a] ? 1 : 0;
         mp.ntile[a] = nt[a];
-        mp.small[a] = mp.g.per[a];   // per-cell minimum image on every periodic axis
     }
     mp.g.ncells = ncells;
     mp.P = P;
@@ -162,18 +148,13 @@ extern "C" lbm_status lbm_map_spheres_noalloc(const lbm_grid* grid, double shell
     mp.tile_count = s->tile_count;
     mp.tile_list = s->tile_list;
     mp.shell_width = shell_width;
-    // the refill and missing-link lists of the time stepper are not produced here
-    mp.refill_list = s->dummy_list; mp.refill_owner = reinterpret_cast<int*>(s->dummy_list);
-    mp.refill_count = &s->counters[0]; mp.refill_cap = 0;
-    mp.miss_list = s->dummy_list; mp.miss_count = &s->counters[1]; mp.miss_cap = 0;
-    mp.n_solid = &s->n_solid;
-    mp.status = &s->status;
-    launch_tile_scatter(mp, st);
+    mp.status = s->status;
+    if (n > 0) noalloc_scatter_kernel<<<(n + 3) / 4, 128, 0, st>>>(mp);
     launch_map(mp, st);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return noalloc_fail(LBM_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     int status = 0;
-    if ((e = cudaMemcpyAsync(&status, &s->status, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+    if ((e = cudaMemcpyAsync(&status, s->status, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return noalloc_fail(LBM_ERR_CUDA, std::string("status read: ") + cudaGetErrorString(e));
     sync_on_exit.armed = false;   // the stream was synchronised just above

@@ -20,7 +20,14 @@ __device__ __forceinline__ int axis_pieces(double xc, double r, int n, int per, 
         return 1;
     }
     if (hi - lo + 1 >= n) { a[0] = 0; b[0] = n - 1; return 1; }
-    long long lw = ((lo % n) + n) % n, hw = ((hi % n) + n) % n;
+    long long lw, hw;
+    if (lo >= -n && hi < 2LL * n) {   // a centre in the box: no 64-bit remainders
+        lw = lo < 0 ? lo + n : (lo >= n ? lo - n : lo);
+        hw = hi < 0 ? hi + n : (hi >= n ? hi - n : hi);
+    } else {
+        lw = ((lo % n) + n) % n;
+        hw = ((hi % n) + n) % n;
+    }
     if (lw <= hw) { a[0] = (int)lw; b[0] = (int)hw; return 1; }
     a[0] = (int)lw; b[0] = n - 1; a[1] = 0; b[1] = (int)hw;
     return 2;
