@@ -256,16 +256,14 @@ void build_layout(const lbm_grid* g, lbm_storage st, int np, Layout& L, const Si
     L.add(8 * n);                                // 55 hI
     L.add(8 * 3 * n);                            // 56 ext
     L.add(4 * (size_t)s.refill_cap);             // 57 refill_owner
-    for (int h = 0; h < 2; ++h) {
-        L.add(4 * 3 * n);                        // 58/60 float32 u
-        L.add(4 * 3 * n);                        // 59/61 float32 omega
-    }
+    for (int k = 0; k < 4; ++k) L.add(4 * 3 * n);  // 58 .. 61 (unused)
     L.state = L.total;
     // derived data, rebuilt after a restore: one bit per cell
     const size_t words = (size_t)((g->nx + 31) / 32) * g->ny * g->nz;
     L.add(4 * words);                            // 62 solid
     L.add(4 * words);                            // 63 shell
     L.add(4);                                    // 64 barrier
+    for (int h = 0; h < 2; ++h) L.add(sizeof(DemRec) * n);  // 65/66 records of the float32 laws
 }
 
 lbm_status validate(const lbm_grid* g, const lbm_relax* r, const lbm_dem* d, lbm_storage st,
@@ -396,10 +394,7 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
     ctx->P.hm = (double*)at(54);
     ctx->P.hI = (double*)at(55);
     ctx->P.ext = (double*)at(56);
-    for (int h = 0; h < 2; ++h) {
-        ctx->P.ufs[h] = (float*)at(58 + 2 * h);
-        ctx->P.omfs[h] = (float*)at(59 + 2 * h);
-    }
+    for (int h = 0; h < 2; ++h) ctx->P.rec[h] = (DemRec*)at(65 + h);
     ctx->scratch = (double*)at(11);
     ctx->scratch_cells = s.scratch_cells;
     ctx->bin_cap = s.bin_cap;

@@ -136,6 +136,15 @@ __device__ __forceinline__ void set_view_c(PartView& v, double R) {
     v.C_lo = (float)(C - (double)v.C);
 }
 
+// What the float32 interaction laws read of a partner, one 64-byte line.
+// Positions and radii are sums of two floats (48 bits).
+struct __align__(64) DemRec {
+    float4 a;    // leading part of the position, of the radius
+    float4 b;    // trailing parts
+    float4 c;    // velocity, mass
+    float4 d;    // angular velocity
+};
+
 struct Particles {
     int n;                 // particle count
     double* x;             // [3n] centre positions
@@ -165,8 +174,7 @@ struct Particles {
     double* us[2];
     double* oms[2];
     float* xfs[2];
-    float* ufs[2];         // float32 copies of us, oms for the float32 pair laws
-    float* omfs[2];
+    DemRec* rec[2];        // the same state for the float32 laws
     // DEM neighbour structure and contact history
     int* bin_count;        // [nbins]
     int* bin_list;         // [nbins * BIN_CAP]

@@ -4,8 +4,8 @@
 // Coulomb-limited tangential spring (Eqs. (39)-(52)) and the Velocity-Verlet
 // subcycles (Eqs. (37)-(38)); the prescribed-motion update. Particle state
 // and integration are float64; the pair and wall laws run in float64 for
-// float64 PDF storage and in float32 (separations and overlaps from float64
-// positions) for the other formats.
+// float64 PDF storage and in float32 (gaps of pairs from positions held as sums
+// of two floats, of walls from float64 positions) for the other formats.
 //
 // Each particle gathers every interaction of its own with eight lanes, so no
 // force atomics are needed; a pair is evaluated by both partners with mirrored
@@ -102,6 +102,27 @@ __device__ __forceinline__ void write_view(const Particles& P, int i) {
     v.R = (float)P.R[i];
     set_view_c(v, P.R[i]);
     P.view[i] = v;
+}
+
+// x as a sum of two floats
+__device__ __forceinline__ float trailing(double x) { return (float)(x - (double)(float)x); }
+
+// the record of particle i in buffer 0, for the float32 laws
+__device__ __forceinline__ void write_record(const Particles& P, int i) {
+    DemRec r;
+    float* w = reinterpret_cast<float*>(&r);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        w[d] = (float)P.x[3 * i + d];
+        w[4 + d] = trailing(P.x[3 * i + d]);
+        w[8 + d] = (float)P.u[3 * i + d];
+        w[12 + d] = (float)P.om[3 * i + d];
+    }
+    r.a.w = (float)P.R[i];
+    r.b.w = trailing(P.R[i]);
+    r.c.w = (float)P.m[i];
+    r.d.w = 0.f;
+    P.rec[0][i] = r;
 }
 
 // rebuild the float view of every particle (after insertion or a velocity
@@ -211,12 +232,7 @@ __device__ __forceinline__ void bin_fill_body(const DemParams& p, int bx) {
     int b[3];
     for (int d = 0; d < 3; ++d) b[d] = bin_coord(p.P.xf[3 * i + d], (float)p.binsize[d], p.nbins[d]);
     const long long bi = ((long long)b[2] * p.nbins[1] + b[1]) * p.nbins[0] + b[0];
-    if (p.pair_f32) {   // float32 copies of the subcycle state read by the float32 pair laws
-        for (int d = 0; d < 3; ++d) {
-            p.P.ufs[0][3 * i + d] = (float)p.P.us[0][3 * i + d];
-            p.P.omfs[0][3 * i + d] = (float)p.P.oms[0][3 * i + d];
-        }
-    }
+    if (p.pair_f32) write_record(p.P, i);
     const int slot = atomicAdd(p.P.bin_count + bi, 1);
     if (slot < BIN_CAP) p.P.bin_list[bi * BIN_CAP + slot] = i;
     else atomicOr(p.status, ST_BIN_OVERFLOW);
@@ -342,6 +358,7 @@ __device__ __forceinline__ void position_update(const DemParams& p, int i) {
         p.P.x[3 * i + d] = x;
         p.P.xf[3 * i + d] = (float)x;
     }
+    if (p.pair_f32) write_record(p.P, i);
 }
 
 // the first Velocity-Verlet position update of a step (Eq. (37)); later
@@ -482,85 +499,57 @@ __device__ __forceinline__ Vec3<U> ld3s(const U* p, int i) {
     return {ld_state<CG>(p + 3 * i), ld_state<CG>(p + 3 * i + 1), ld_state<CG>(p + 3 * i + 2)};
 }
 
-// a neighbour's state and the own one as a pair law reads them
-template <typename T>
+// a float64 pair's state
 struct PairState {
-    V3 xi, xj;
-    Vec3<float> xfi, xfj;
-    Vec3<T> ui, uj, omi, omj;
+    V3 xi, xj, ui, uj, omi, omj;
 };
 
-template <typename T, bool CG>
-__device__ __forceinline__ PairState<T> load_pair(const Particles& P, int cur, int i, int j) {
-    PairState<T> s;
-    s.xfi = ld3s<CG>(P.xfs[cur], i);
-    s.xfj = ld3s<CG>(P.xfs[cur], j);
+template <bool CG>
+__device__ __forceinline__ PairState load_pair(const Particles& P, int cur, int i, int j) {
+    PairState s;
     s.xi = ld3s<CG>(P.xs[cur], i);
     s.xj = ld3s<CG>(P.xs[cur], j);
-    if constexpr (sizeof(T) == 8) {
-        s.ui = ld3s<CG>(P.us[cur], i); s.omi = ld3s<CG>(P.oms[cur], i);
-        s.uj = ld3s<CG>(P.us[cur], j); s.omj = ld3s<CG>(P.oms[cur], j);
-    } else {
-        s.ui = ld3s<CG>(P.ufs[cur], i); s.omi = ld3s<CG>(P.omfs[cur], i);
-        s.uj = ld3s<CG>(P.ufs[cur], j); s.omj = ld3s<CG>(P.omfs[cur], j);
-    }
+    s.ui = ld3s<CG>(P.us[cur], i); s.omi = ld3s<CG>(P.oms[cur], i);
+    s.uj = ld3s<CG>(P.us[cur], j); s.omj = ld3s<CG>(P.oms[cur], j);
     return s;
 }
 
+template <bool CG>
+__device__ __forceinline__ DemRec load_record(const DemRec* r) {
+    DemRec v;
+    const float4* q = reinterpret_cast<const float4*>(r);
+    v.a = ld_state<CG>(q);
+    v.b = ld_state<CG>(q + 1);
+    v.c = ld_state<CG>(q + 2);
+    v.d = ld_state<CG>(q + 3);
+    return v;
+}
+
 // Force and torque on particle i from its neighbour j (lubrication,
-// Eqs. (25)-(33), and contact, Eqs. (39)-(50)) at the subcycle's positions;
-// contact = the spring of the pair continues, dnew its new value. T = double:
-// all in float64. T = float: the separation and |d|^2 - (Ri + Rj)^2 in
-// float64 (the overlap delta = that / (|d| + Ri + Rj) keeps float32 relative
-// accuracy), the interaction laws in float32.
+// Eqs. (25)-(33), and contact, Eqs. (39)-(50)) at separation d = x_i - x_j
+// (nearest image) of length dist and gap delta; contact = the spring of the
+// pair continues, dnew its new value.
 template <typename T>
-__device__ __forceinline__ void pair_force(const DemParams& p, const PairState<T>& s, int hin, int i, int j, Vec3<T>& F,
-                                           Vec3<T>& Tq, bool& contact, Vec3<T>& dnew) {
+__device__ __forceinline__ void pair_law(const DemParams& p, Vec3<T> d, T dist, T delta, T Ri, T Rj, T mi, T mj,
+                                         Vec3<T> ui, Vec3<T> uj, Vec3<T> omi, Vec3<T> omj, int hin, int i, int j,
+                                         Vec3<T>& F, Vec3<T>& Tq, bool& contact, Vec3<T>& dnew) {
     const Particles& P = p.P;
     const DemConsts<T>& k = consts<T>(p);
-    Vec3<T> d;
-    T dist, delta, Ri, Rj;
-    if constexpr (sizeof(T) == 8) {
-        d = mk(mimg(s.xi.x - s.xj.x, p.g.n[0], p.g.per[0]), mimg(s.xi.y - s.xj.y, p.g.n[1], p.g.per[1]),
-               mimg(s.xi.z - s.xj.z, p.g.n[2], p.g.per[2]));
-        dist = sqrt(dot(d, d));
-        Ri = P.R[i];
-        Rj = P.R[j];
-        delta = dist - (Ri + Rj);
-    } else {
-        V3 dd = s.xi - s.xj;
-        const int sx = image_shift(s.xfi.x - s.xfj.x, p.g.n[0], p.g.per[0]),
-                  sy = image_shift(s.xfi.y - s.xfj.y, p.g.n[1], p.g.per[1]),
-                  sz = image_shift(s.xfi.z - s.xfj.z, p.g.n[2], p.g.per[2]);
-        if (sx | sy | sz) {
-            dd.x += (double)sx;
-            dd.y += (double)sy;
-            dd.z += (double)sz;
-        }
-        const double R1 = P.R[i], R2 = P.R[j], S = R1 + R2;
-        const double e = fma(-S, S, dot(dd, dd));
-        d = cvt3<float>(dd);
-        dist = sqrtf(dot(d, d));
-        Ri = (float)R1;
-        Rj = (float)R2;
-        delta = (float)e / (dist + (float)S);
-    }
     F = zero3<T>();
     Tq = zero3<T>();
     contact = false;
     dnew = zero3<T>();
     if (delta >= k.cut_max && delta >= T(0)) return;
     const Vec3<T> n = (T(1) / dist) * d;
-    const Vec3<T> uij = s.ui - s.uj;
+    const Vec3<T> uij = ui - uj;
     if (p.lubrication) {
         const T Rm = T(0.5) * (Ri + Rj);
         const T dmin = mad(k.min_b, Rm, k.min_a) * Rm;
-        lubrication_on_i<T>(k, p.tangential, Ri, Rj, delta, n, uij, s.omi, s.omj, dmin, F, Tq);
+        lubrication_on_i<T>(k, p.tangential, Ri, Rj, delta, n, uij, omi, omj, dmin, F, Tq);
     }
     if (delta < T(0)) {
         const Vec3<T> ri = T(-0.5) * d, rj = T(0.5) * d;
-        const Vec3<T> ucp = (s.ui + cross(s.omi, ri)) - (s.uj + cross(s.omj, rj));
-        const T mi = (T)P.m[i], mj = (T)P.m[j];
+        const Vec3<T> ucp = (ui + cross(omi, ri)) - (uj + cross(omj, rj));
         const T m_eff = mi * mj / (mi + mj);
         const T Tc = collision_time<T>(Ri + Rj, k.Tc);
         Vec3<T> old = zero3<T>();
@@ -577,6 +566,72 @@ __device__ __forceinline__ void pair_force(const DemParams& p, const PairState<T
         Tq = Tq + cross(ri, Ft);
         contact = true;
     }
+}
+
+// all in float64
+__device__ __forceinline__ void pair_force(const DemParams& p, const PairState& s, int hin, int i, int j, V3& F, V3& Tq,
+                                           bool& contact, V3& dnew) {
+    const Particles& P = p.P;
+    const V3 d = mk(mimg(s.xi.x - s.xj.x, p.g.n[0], p.g.per[0]), mimg(s.xi.y - s.xj.y, p.g.n[1], p.g.per[1]),
+                    mimg(s.xi.z - s.xj.z, p.g.n[2], p.g.per[2]));
+    const double dist = sqrt(dot(d, d)), Ri = P.R[i], Rj = P.R[j];
+    pair_law<double>(p, d, dist, dist - (Ri + Rj), Ri, Rj, P.m[i], P.m[j], s.ui, s.uj, s.omi, s.omj, hin, i, j, F, Tq,
+                     contact, dnew);
+}
+
+// Sums of two floats: h the leading part, l what it leaves. Every operation is
+// rounded on its own, so that h + l is exact where the formulas say so (Knuth's
+// two-sum, Dekker's products by a fused multiply-add).
+struct Two {
+    float h, l;
+};
+__device__ __forceinline__ Two two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Two two_square(float a) {
+    const float p = __fmul_rn(a, a);
+    return {p, fmaf(a, a, -p)};
+}
+// (ah + al) - (bh + bl) + shift
+__device__ __forceinline__ Two two_diff(float ah, float al, float bh, float bl, int shift) {
+    Two s = two_sum(ah, -bh);
+    if (shift) {
+        const Two t = two_sum(s.h, (float)shift);
+        s.h = t.h;
+        s.l = __fadd_rn(s.l, t.l);
+    }
+    const float l = __fadd_rn(s.l, __fsub_rn(al, bl));
+    const float h = __fadd_rn(s.h, l);
+    return {h, __fsub_rn(l, __fsub_rn(h, s.h))};
+}
+
+// In float32: the separation and e = |d|^2 - (Ri + Rj)^2 as sums of two floats
+// (the gap delta = e / (|d| + Ri + Rj) keeps float32 relative accuracy: e is
+// known to 2e-11 in boxes of 512 cells, a thousandth of its float32 spacing at
+// the smallest gap the lubrication resolves), the laws in float32. In float64
+// the separation issued 17 instructions of 64 cycles per pair and warp, and the
+// partner's state was 18 loads: the DEM of a step took 115 us with 10,000
+// particles, 66 us with 1,250 and 61 us with 150, this way 91, 59 and 54 us.
+__device__ __forceinline__ void pair_force(const DemParams& p, const DemRec& ri, const DemRec& rj, int hin, int i, int j,
+                                           Vec3<float>& F, Vec3<float>& Tq, bool& contact, Vec3<float>& dnew) {
+    const Two x = two_diff(ri.a.x, ri.b.x, rj.a.x, rj.b.x, image_shift(ri.a.x - rj.a.x, p.g.n[0], p.g.per[0])),
+              y = two_diff(ri.a.y, ri.b.y, rj.a.y, rj.b.y, image_shift(ri.a.y - rj.a.y, p.g.n[1], p.g.per[1])),
+              z = two_diff(ri.a.z, ri.b.z, rj.a.z, rj.b.z, image_shift(ri.a.z - rj.a.z, p.g.n[2], p.g.per[2]));
+    Two S = two_sum(ri.a.w, rj.a.w);
+    S.l = __fadd_rn(S.l, __fadd_rn(ri.b.w, rj.b.w));
+    // |d|^2 - S^2: the leading squares exactly, then everything small
+    const Two xx = two_square(x.h), yy = two_square(y.h), zz = two_square(z.h), SS = two_square(S.h);
+    const Two t1 = two_sum(xx.h, yy.h), t2 = two_sum(t1.h, zz.h), t3 = two_sum(t2.h, -SS.h);
+    float low = mad(x.h, x.l, mad(y.h, y.l, mad(z.h, z.l, -mul_rn(S.h, S.l))));
+    low = __fadd_rn(__fadd_rn(low, low), __fadd_rn(__fadd_rn(xx.l, yy.l), __fsub_rn(zz.l, SS.l)));
+    low = __fadd_rn(low, __fadd_rn(__fadd_rn(t1.l, t2.l), t3.l));
+    const float e = __fadd_rn(t3.h, low);
+    const Vec3<float> d = {x.h, y.h, z.h};
+    const float dist = sqrtf(dot(d, d));
+    pair_law<float>(p, d, dist, e / __fadd_rn(dist, S.h), ri.a.w, rj.a.w, ri.c.w, rj.c.w, {ri.c.x, ri.c.y, ri.c.z},
+                    {rj.c.x, rj.c.y, rj.c.z}, {ri.d.x, ri.d.y, ri.d.z}, {rj.d.x, rj.d.y, rj.d.z}, hin, i, j, F, Tq,
+                    contact, dnew);
 }
 
 // ------------------------------------------------------------ subcycles
@@ -616,7 +671,25 @@ struct OctLane {
                                     // averaged fluid force + external force
     double coef, dcoef;             // dt / (2 m) or dt / (2 I), dt times it
     float xf, vf, R;                // float32 copies for the tests that decide most cases
+    float xl, Rl, m;                // trailing parts of position and radius, the mass, for the float32 laws
 };
+
+// lane s's share of the particle's record
+__device__ __forceinline__ void oct_publish(const DemParams& p, const OctLane& o, int buf) {
+    float* r = reinterpret_cast<float*>(p.P.rec[buf] + o.i);
+    if (o.s < 3) {
+        r[o.s] = o.xf;
+        r[4 + o.s] = o.xl;
+        r[8 + o.s] = o.vf;
+    } else if (o.s < 6) {
+        r[9 + o.s] = o.vf;
+    } else if (o.s == 6) {
+        r[3] = o.R;
+        r[7] = o.Rl;
+    } else {
+        r[11] = o.m;
+    }
+}
 
 template <bool CG>
 __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, int s, int cur) {
@@ -626,10 +699,12 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
     o.on = i < P.n;
     o.nn = 0;
     o.x = o.v = o.f_prev = o.f_const = o.coef = o.dcoef = 0.0;
-    o.xf = o.vf = o.R = 0.f;
+    o.xf = o.vf = o.R = o.xl = o.Rl = o.m = 0.f;
     if (!o.on) return;
     o.nn = P.nbr_count[i];
     o.R = (float)P.R[i];
+    o.Rl = trailing(P.R[i]);
+    o.m = (float)P.m[i];
     const float reach = o.R + ((float)p.cut_max + 1e-3f);
 #pragma unroll
     for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
@@ -654,6 +729,7 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
     }
     o.dcoef = p.dt * o.coef;
     o.xf = (float)o.x;
+    o.xl = trailing(o.x);
     o.vf = (float)o.v;
 }
 
@@ -667,6 +743,7 @@ __device__ __forceinline__ void oct_move(const DemParams& p, OctLane& o) {
         o.x = wrap_pos(o.x, n, p.g.per[o.s]);
         o.xf = (float)o.x;
     }
+    o.xl = trailing(o.x);
 }
 
 // float positions are within 1e-4 of the float64 ones, so a gap above cut_max +
@@ -827,24 +904,37 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
     T f[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
     bool acts = false;
     if constexpr (sizeof(T) == 4) {
+        if (__any_sync(FULL, o.nn > 0)) {
+            // the own record from the particle's lanes
+            const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
+            DemRec me;
+            me.a = make_float4(__shfl_sync(FULL, o.xf, base), __shfl_sync(FULL, o.xf, base + 1),
+                               __shfl_sync(FULL, o.xf, base + 2), o.R);
+            me.b = make_float4(__shfl_sync(FULL, o.xl, base), __shfl_sync(FULL, o.xl, base + 1),
+                               __shfl_sync(FULL, o.xl, base + 2), o.Rl);
+            me.c = make_float4(__shfl_sync(FULL, o.vf, base), __shfl_sync(FULL, o.vf, base + 1),
+                               __shfl_sync(FULL, o.vf, base + 2), o.m);
+            me.d = make_float4(__shfl_sync(FULL, o.vf, base + 3), __shfl_sync(FULL, o.vf, base + 4),
+                               __shfl_sync(FULL, o.vf, base + 5), 0.f);
 #pragma unroll
-        for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
-            const int slot = o.s + DEM_LANES * k;
-            if (slot >= o.nn) continue;
-            const PairState<T> st = load_pair<T, CG>(P, cur, o.i, o.j[k]);
-            bool contact = false;
-            if (may_touch(p, st.xfi, st.xfj, o.reach2[k])) {
-                Vec3<T> F, Tq, dnew;
-                pair_force<T>(p, st, hin, o.i, o.j[k], F, Tq, contact, dnew);
-                f[0] += F.x; f[1] += F.y; f[2] += F.z;
-                f[3] += Tq.x; f[4] += Tq.y; f[5] += Tq.z;
-                acts = true;
-                if (contact && !init) {
-                    double* sd = P.hist_d[hout] + 3 * (o.i * NBR_CAP + slot);
-                    sd[0] = (double)dnew.x; sd[1] = (double)dnew.y; sd[2] = (double)dnew.z;
+            for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
+                const int slot = o.s + DEM_LANES * k;
+                if (slot >= o.nn) continue;
+                const DemRec you = load_record<CG>(P.rec[cur] + o.j[k]);
+                bool contact = false;
+                if (may_touch(p, {me.a.x, me.a.y, me.a.z}, {you.a.x, you.a.y, you.a.z}, o.reach2[k])) {
+                    Vec3<T> F, Tq, dnew;
+                    pair_force(p, me, you, hin, o.i, o.j[k], F, Tq, contact, dnew);
+                    f[0] += F.x; f[1] += F.y; f[2] += F.z;
+                    f[3] += Tq.x; f[4] += Tq.y; f[5] += Tq.z;
+                    acts = true;
+                    if (contact && !init) {
+                        double* sd = P.hist_d[hout] + 3 * (o.i * NBR_CAP + slot);
+                        sd[0] = (double)dnew.x; sd[1] = (double)dnew.y; sd[2] = (double)dnew.z;
+                    }
                 }
+                if (!init) P.hist_id[hout][o.i * NBR_CAP + slot] = contact ? o.j[k] : -1;
             }
-            if (!init) P.hist_id[hout][o.i * NBR_CAP + slot] = contact ? o.j[k] : -1;
         }
     } else {
         // pairs that pass the prefilter into the block's queue, evaluated by
@@ -875,7 +965,7 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
                 const int i = o.i - pl + (q >> 5), j = P.nbr[i * NBR_CAP + slot];
                 Vec3<T> F, Tq, dnew;
                 bool contact;
-                pair_force<T>(p, load_pair<T, CG>(P, cur, i, j), hin, i, j, F, Tq, contact, dnew);
+                pair_force(p, load_pair<CG>(P, cur, i, j), hin, i, j, F, Tq, contact, dnew);
                 double* r = queue->res[threadIdx.x];
                 r[0] = F.x; r[1] = F.y; r[2] = F.z; r[3] = Tq.x; r[4] = Tq.y; r[5] = Tq.z;
                 if (!init) {
@@ -954,18 +1044,18 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
     o.f_prev = fs;
     o.vf = (float)o.v;
     const int nxt = 1 - cur;
-    if (o.s < 3) {
+    // the next subcycle's positions; the last subcycle keeps its own
+    if (o.s < 3 && !last) oct_move(p, o);
+    if constexpr (sizeof(T) == 4) {
+        if (!last) oct_publish(p, o, nxt);
+    } else if (o.s < 3) {
         if (!last) {
-            // the next subcycle's positions; the last subcycle keeps its own
-            oct_move(p, o);
             P.xs[nxt][3 * o.i + o.s] = o.x;
             P.xfs[nxt][3 * o.i + o.s] = o.xf;
         }
-        if (sizeof(T) == 8) P.us[nxt][3 * o.i + o.s] = o.v;
-        else P.ufs[nxt][3 * o.i + o.s] = o.vf;
+        P.us[nxt][3 * o.i + o.s] = o.v;
     } else if (o.s < 6) {
-        if (sizeof(T) == 8) P.oms[nxt][3 * o.i + o.s - 3] = o.v;
-        else P.omfs[nxt][3 * o.i + o.s - 3] = o.vf;
+        P.oms[nxt][3 * o.i + o.s - 3] = o.v;
     }
 }
 
@@ -1022,12 +1112,17 @@ __device__ __forceinline__ void oct_store_view(const DemParams& p, const OctLane
 }
 
 // the first Velocity-Verlet position update of a step (Eq. (37))
+template <typename T>
 __device__ __forceinline__ void oct_first_position(const DemParams& p, OctLane& o) {
     const Particles& P = p.P;
-    if (!o.on || o.s >= 3) return;
-    oct_move(p, o);
-    P.xs[0][3 * o.i + o.s] = o.x;
-    P.xfs[0][3 * o.i + o.s] = o.xf;
+    if (!o.on) return;
+    if (o.s < 3) oct_move(p, o);
+    if constexpr (sizeof(T) == 4) {
+        oct_publish(p, o, 0);
+    } else if (o.s < 3) {
+        P.xs[0][3 * o.i + o.s] = o.x;
+        P.xfs[0][3 * o.i + o.s] = o.xf;
+    }
 }
 
 // one DEM subcycle of Algorithm 1 as a launch of its own (the initial force,
@@ -1110,7 +1205,7 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
     oct_load<GRID>(p, o, i, s, 0);
     WallSpring<T> w;
     wall_load<T>(p, o, w, hcur);
-    oct_first_position(p, o);
+    oct_first_position<T>(p, o);
     unsigned target = 0;
     bool ok = true;
     auto barrier = [&]() {
