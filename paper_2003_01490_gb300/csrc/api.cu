@@ -53,6 +53,7 @@ struct lbm_ctx {
     float* accel_f = nullptr;
     unsigned* barrier = nullptr;   // of the cooperative DEM launch
     int grid_particles = 0;        // particles a cooperative DEM launch holds
+    int cluster_particles = 0;     // particles a DEM launch of one cluster holds
     uint32_t* solid = nullptr;     // one bit per cell (see launch.h)
     uint32_t* shell = nullptr;
     unsigned int* miss_list = nullptr;
@@ -313,6 +314,7 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
             ctx->num_sms = sms;
         cudaError_t pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
+        ctx->cluster_particles = dem_cluster_capacity();
         if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
@@ -942,7 +944,7 @@ lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepStat
     if (move) {
         if (ss.one_launch) {
             // Algorithm 1, lines 4-10, in one launch
-            CK(launch_dem_step(dp, fpp, map_params(ctx), ctx->hcur, d.n_sub, sm));
+            CK(launch_dem_step(dp, fpp, map_params(ctx), ctx->hcur, d.n_sub, ctx->cluster_particles, sm));
             ctx->launches += 1;
             if (d.n_sub & 1) ctx->hcur = 1 - ctx->hcur;
         } else if (dem) {

@@ -12,7 +12,8 @@
 // operands (n_ji = -n_ij, u_ji = -u_ij, ...). Each particle keeps its own copy of
 // the tangential spring of every active contact (double buffered per
 // subcycle). All subcycles of a step run in one launch: one block for up to 32
-// particles, a cooperative launch as long as its blocks fit the GPU at once.
+// particles, one cluster for up to 512 with float32 laws, a cooperative launch as
+// long as its blocks fit the GPU at once.
 #include <cstring>
 
 #include "common.cuh"
@@ -1187,13 +1188,21 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, i
     return ok != 0;
 }
 
+// A barrier of all threads of a cluster, with the memory order of a release and
+// an acquire at cluster scope.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+enum DemSpan { SPAN_BLOCK, SPAN_CLUSTER, SPAN_GRID };
+
 // All subcycles of a step in one launch: the particles' state stays in
-// registers, buffers 0 and 1 only carry what partners read. One block
-// (barriers of the block) or a cooperative launch (GRID). With fin, the force
+// registers, buffers 0 and 1 only carry what partners read. One block, one
+// cluster or a cooperative launch, with the barrier of each. With fin, the force
 // finalisation of the step comes first, with sc the counters' reset and the
 // tile scatter of the mapping last: a step of Algorithm 1 between the dense
 // kernel and the mapping is this one launch.
-template <typename T, bool GRID, int PPB>
+template <typename T, DemSpan SPAN, int PPB>
 __device__ __forceinline__ void dem_step_body(const DemParams& p, const FinalizeParams* fin, const MapParams* sc,
                                               PairQueue<PPB>* queue, int hcur, int n_sub, int first_particle) {
     const int s = threadIdx.x % DEM_LANES, i = first_particle + (int)threadIdx.x / DEM_LANES;
@@ -1202,14 +1211,17 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
         __syncwarp();
     }
     OctLane o;
-    oct_load<GRID>(p, o, i, s, 0);
+    constexpr bool CG = SPAN != SPAN_BLOCK;   // partners' state is written by other multiprocessors
+    oct_load<CG>(p, o, i, s, 0);
     WallSpring<T> w;
     wall_load<T>(p, o, w, hcur);
     oct_first_position<T>(p, o);
     unsigned target = 0;
     bool ok = true;
     auto barrier = [&]() {
-        if constexpr (GRID) {
+        if constexpr (SPAN == SPAN_CLUSTER) {
+            cluster_barrier();
+        } else if constexpr (SPAN == SPAN_GRID) {
             target += gridDim.x;
             ok = grid_barrier(p.barrier, target, p.status);
         } else {
@@ -1219,7 +1231,7 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
     for (int k = 0; k < n_sub && ok; ++k) {
         barrier();
         if (!ok) break;
-        oct_subcycle<T, GRID, PPB>(p, o, w, queue, k & 1, hcur, 1 - hcur, 0, k == n_sub - 1);
+        oct_subcycle<T, CG, PPB>(p, o, w, queue, k & 1, hcur, 1 - hcur, 0, k == n_sub - 1);
         oct_check_speed(p, o);
         hcur = 1 - hcur;
     }
@@ -1243,7 +1255,7 @@ __global__ void __launch_bounds__(ONE_BLOCK_THREADS)
     dem_step_one_block_kernel(const __grid_constant__ DemParams p, const __grid_constant__ FinalizeParams fin,
                               const __grid_constant__ MapParams sc, int hcur, int n_sub) {
     __shared__ PairQueue<sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1> queue;
-    dem_step_body<T, false, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(p, &fin, &sc, &queue, hcur, n_sub, 0);
+    dem_step_body<T, SPAN_BLOCK, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(p, &fin, &sc, &queue, hcur, n_sub, 0);
 }
 
 template <typename T>
@@ -1251,7 +1263,24 @@ __global__ void __launch_bounds__(DEM_THREADS, 5)
     dem_step_grid_kernel(const __grid_constant__ DemParams p, const __grid_constant__ FinalizeParams fin,
                          const __grid_constant__ MapParams sc, int hcur, int n_sub) {
     __shared__ PairQueue<sizeof(T) == 8 ? DEM_PPB : 1> queue;
-    dem_step_body<T, true, sizeof(T) == 8 ? DEM_PPB : 1>(p, &fin, &sc, &queue, hcur, n_sub, (int)blockIdx.x * DEM_PPB);
+    dem_step_body<T, SPAN_GRID, sizeof(T) == 8 ? DEM_PPB : 1>(p, &fin, &sc, &queue, hcur, n_sub,
+                                                            (int)blockIdx.x * DEM_PPB);
+}
+
+// Float32 laws, one cluster of CLUSTER_BLOCKS blocks: the cluster's hardware
+// barrier takes the place of the counter in memory, which costs a subcycle of few
+// particles a fifth of its time. 150 particles 54 -> 45 us per step of ten
+// subcycles, 500 particles 65 -> 61 us; with 1,250 the particles crowd 16
+// multiprocessors (20 warps each on their float64 units): 59 -> 77 us, so the
+// cluster ends at two warps per scheduler.
+constexpr int CLUSTER_BLOCKS = 16, CLUSTER_THREADS = 256;   // at most, in steps of a warp
+static_assert(DEM_CLUSTER_MAX == CLUSTER_BLOCKS * CLUSTER_THREADS / DEM_LANES, "particles of a cluster");
+
+__global__ void __launch_bounds__(CLUSTER_THREADS)
+    dem_step_cluster_kernel(const __grid_constant__ DemParams p, const __grid_constant__ FinalizeParams fin,
+                            const __grid_constant__ MapParams sc, int hcur, int n_sub) {
+    dem_step_body<float, SPAN_CLUSTER, 1>(p, &fin, &sc, nullptr, hcur, n_sub,
+                                          (int)(blockIdx.x * blockDim.x) / DEM_LANES);
 }
 
 // The one-block DEM steps of many instances in one launch: block b runs the
@@ -1272,7 +1301,8 @@ __global__ void __launch_bounds__(ONE_BLOCK_THREADS) dem_step_batch_kernel(const
     int* dst = reinterpret_cast<int*>(&e);
     for (int w = threadIdx.x; w < WORDS; w += blockDim.x) dst[w] = src[w];
     __syncthreads();
-    dem_step_body<T, false, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(e.p, nullptr, nullptr, &queue, e.hcur, e.n_sub, 0);
+    dem_step_body<T, SPAN_BLOCK, sizeof(T) == 8 ? DEM_ONE_BLOCK_MAX : 1>(e.p, nullptr, nullptr, &queue, e.hcur, e.n_sub,
+                                                                       0);
 }
 
 size_t dem_batch_entry_bytes() { return sizeof(DemBatchEntry); }
@@ -1302,14 +1332,45 @@ cudaError_t dem_grid_capacity(int storage_f64, int num_sms, int* particles) {
     return e;
 }
 
+static cudaLaunchConfig_t cluster_config(int threads, cudaLaunchAttribute* attr, cudaStream_t st) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = CLUSTER_BLOCKS;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(CLUSTER_BLOCKS);
+    c.blockDim = dim3(threads);
+    c.stream = st;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return c;
+}
+
+int dem_cluster_capacity() {
+    int clusters = 0;
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t c = cluster_config(CLUSTER_THREADS, &attr, nullptr);
+    if (cudaFuncSetAttribute(dem_step_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, dem_step_cluster_kernel, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return clusters > 0 ? DEM_CLUSTER_MAX : 0;
+}
+
 cudaError_t launch_dem_step(const DemParams& p, const FinalizeParams& fin, const MapParams& sc, int hcur, int n_sub,
-                            cudaStream_t st) {
+                            int cluster_particles, cudaStream_t st) {
     if (p.P.n <= DEM_ONE_BLOCK_MAX) {
         // no idle warps: a block of as many as the particles need
         const int threads = (p.P.n * DEM_LANES + 31) / 32 * 32;
         if (p.pair_f32) dem_step_one_block_kernel<float><<<1, threads, 0, st>>>(p, fin, sc, hcur, n_sub);
         else dem_step_one_block_kernel<double><<<1, threads, 0, st>>>(p, fin, sc, hcur, n_sub);
         return cudaGetLastError();
+    }
+    if (p.pair_f32 && p.P.n <= cluster_particles) {
+        const int warps = (p.P.n * DEM_LANES + 32 * CLUSTER_BLOCKS - 1) / (32 * CLUSTER_BLOCKS);   // per block
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t c = cluster_config(32 * warps, &attr, st);
+        return cudaLaunchKernelEx(&c, dem_step_cluster_kernel, p, fin, sc, hcur, n_sub);
     }
     void* args[] = {const_cast<DemParams*>(&p), const_cast<FinalizeParams*>(&fin), const_cast<MapParams*>(&sc), &hcur,
                     &n_sub};

@@ -164,13 +164,15 @@ void launch_dem_position(const DemParams& p, cudaStream_t st);
 void launch_dem_subcycle(const DemParams& p, int cur, int init, int last, cudaStream_t st);
 // The force finalisation, the position update, all subcycles, the counters'
 // reset and the tile scatter of a step in one launch: one block for at most
-// DEM_ONE_BLOCK_MAX particles, else a cooperative launch, for at most the
-// particles of dem_grid_capacity().
-constexpr int DEM_ONE_BLOCK_MAX = 32;
+// DEM_ONE_BLOCK_MAX particles, one cluster for at most cluster_particles with
+// float32 laws, else a cooperative launch, for at most the particles of
+// dem_grid_capacity().
+constexpr int DEM_ONE_BLOCK_MAX = 32, DEM_CLUSTER_MAX = 512;
 constexpr int DEM_BLOCK_PARTICLES = 16;   // particles per block of a multi-block launch
 cudaError_t dem_grid_capacity(int storage_f64, int num_sms, int* particles);
+int dem_cluster_capacity();               // DEM_CLUSTER_MAX, or 0 where no such cluster fits the device
 cudaError_t launch_dem_step(const DemParams& p, const FinalizeParams& fin, const MapParams& sc, int hcur, int n_sub,
-                            cudaStream_t st);
+                            int cluster_particles, cudaStream_t st);
 void launch_state_copy(const Particles& P, cudaStream_t st);
 void launch_fp_split(const double* fp, double* out, int n, cudaStream_t st);
 

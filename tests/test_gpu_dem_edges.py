@@ -1,7 +1,8 @@
 """The particle step at the sizes where its launch changes shape, between six
-walls, against the oracle: one block up to 32 particles, several above; odd and
-even numbers of subcycles; contacts with walls of either side of every axis,
-all of them moving, close partners, unequal radii."""
+walls, against the oracle: one block up to 32 particles, with float32 laws one
+cluster up to 512, a grid above; odd and even numbers of subcycles; contacts with
+walls of either side of every axis, all of them moving, close partners, unequal
+radii."""
 import numpy as np
 import pytest
 
@@ -11,13 +12,14 @@ pytestmark = pytest.mark.gpu
 
 
 def packed_case(n, n_sub, storage):
-    """n spheres on a jittered 4x4x3 lattice; the outer ones run into the six walls."""
+    """n spheres on a jittered lattice; the outer ones run into the six walls."""
     rng = np.random.default_rng(n)
     pitch, radius = 5.0, 2.35 + 0.1 * rng.random(n)     # small gaps, no overlap at the start
-    cells = np.array([(i, j, k) for k in range(3) for j in range(4) for i in range(4)])
+    sites = (4, 4, 3) if n <= 48 else (9, 9, 7)
+    cells = np.array([(i, j, k) for k in range(sites[2]) for j in range(sites[1]) for i in range(sites[0])])
     # few spheres sit in opposite corners
     pick = np.arange(n) if n > 2 else np.array([0, 47])[:n]
-    side = np.array([20.0, 20.0, 15.0])
+    side = pitch * np.array(sites)
     pos = (cells[pick] + 0.5) * pitch + rng.uniform(-0.045, 0.045, (n, 3))
     # the outer ones close to their walls and on their way into them
     reach = radius[:, None] + 0.004
@@ -26,7 +28,7 @@ def packed_case(n, n_sub, storage):
     toward = 0.03 * high - 0.03 * low
     lo = [[0.0, 0.004, -0.002], [0.003, 0.0, 0.0], [0.0, -0.005, 0.0]]
     hi = [[0.0, 0.0, 0.003], [0.0, 0.0, -0.004], [0.006, 0.0, 0.0]]
-    return dict(shape=(20, 20, 15), periodic=(0, 0, 0), tau=0.7, storage=storage, wall_vel_lo=lo, wall_vel_hi=hi,
+    return dict(shape=tuple(int(v) for v in side), periodic=(0, 0, 0), tau=0.7, storage=storage, wall_vel_lo=lo, wall_vel_hi=hi,
                 spheres=spheres(pos, radius, density=rng.uniform(20.0, 40.0, n), vel=toward + rng.normal(0.0, 0.005, (n, 3)),
                                 omega=rng.normal(0.0, 0.003, (n, 3))),
                 dem=dict(gravity=(1e-4, -5e-5, -2e-4), Tc=8.0, n_sub=n_sub))
@@ -39,8 +41,16 @@ def packed_case(n, n_sub, storage):
 @pytest.mark.parametrize('storage,tol', [('f64', 1e-11), ('f32', 1e-4)])
 @pytest.mark.parametrize('n,n_sub', [(1, 10), (2, 7), (32, 7), (33, 10), (48, 7)])
 def test_packed_box_between_walls(n, n_sub, storage, tol):
+    check(packed_case(n, n_sub, storage), tol)
+
+
+@pytest.mark.parametrize('n,n_sub', [(512, 10), (513, 7)])
+def test_cluster_and_grid(n, n_sub):
+    check(packed_case(n, n_sub, 'f32'), 1e-4)
+
+
+def check(case, tol):
     from paper_2003_01490_gb300 import lbmdem as L
-    case = packed_case(n, n_sub, storage)
     ora = build_oracle(case)
     ctx = build_gpu(case)
     ora.step(5)
