@@ -51,6 +51,7 @@ struct lbm_ctx {
     int* status = nullptr;
     double* accel = nullptr;
     float* accel_f = nullptr;
+    bool accel_set = true;         // they hold the body force of a box without counterforce
     unsigned* barrier = nullptr;   // of the cooperative DEM launch
     int grid_particles = 0;        // particles a cooperative DEM launch holds
     int cluster_particles = 0;     // particles a DEM launch of one cluster holds
@@ -882,7 +883,12 @@ lbm_status enqueue_pre(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepState& 
     CK(prof_mark(ctx));
     LbmStepParams& lp = ss.lp;
     fill_step_params(ctx, lp);
-    launch_boundary(lp, sm, BC_ACCEL);
+    // without a counterforce the body force is the one set at creation: a launch
+    // of 3 us less in front of every dense kernel
+    if (lp.counterforce) {
+        launch_boundary(lp, sm, BC_ACCEL);
+        ctx->launches += 1;
+    }
     // beside the dense kernel, on the side stream: the missing links (their
     // sums commute with the dense kernel's) and the DEM's neighbour lists,
     // which read only the positions the dense kernel reads too; finalize
@@ -935,7 +941,7 @@ lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepStat
     // the DEM step takes the finalisation and the mapping's tile scatter with
     // it where its particles fit one launch
     ss.one_launch = dem && (ctx->P.n <= DEM_ONE_BLOCK_MAX || ctx->P.n <= ctx->grid_particles);
-    ctx->launches += 2;
+    ctx->launches += 1;
     if (!ss.one_launch) {
         launch_finalize(fpp, sm);
         ctx->launches += ctx->P.n > 0 ? 1 : 0;
@@ -994,7 +1000,7 @@ lbm_status enqueue_post_b(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, const St
         rp.list = ctx->refill_list;
         rp.count = ctx->refill_count;
         rp.cap = ctx->refill_cap;
-        rp.s_nu = s_nu;
+        rp.cs2_over_s_nu = 1.0 / (3.0 * s_nu);
         rp.accel = ctx->accel;
         launch_refill(rp, sm);
         ctx->launches += 1;
@@ -1070,6 +1076,13 @@ lbm_status lbm_step(lbm_ctx* ctx, int n_steps) {
     if (!ctx) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
     if (n_steps < 0) return fail(ctx, LBM_ERR_INVALID, "n_steps must be >= 0");
     DemParams dp = dem_params(ctx);
+    if (!ctx->accel_set && n_steps > 0) {
+        LbmStepParams lp;
+        fill_step_params(ctx, lp);
+        launch_boundary(lp, ctx->stream, BC_ACCEL);
+        ctx->launches += 1;
+        ctx->accel_set = true;
+    }
     for (int step = 0; step < n_steps; ++step) {
         if (ctx->stepped && !ctx->profiling && !ctx->dem_restart) {
             bool done = false;
@@ -1270,6 +1283,7 @@ lbm_status lbm_restore(lbm_ctx* ctx, const void* buf, size_t bytes) {
     ctx->hR.assign(hd + 3 * mp, hd + 3 * mp + (size_t)h.np);
     reset_graphs(ctx);
     launch_cell_bits(map_params(ctx), ctx->stream);
+    ctx->accel_set = false;   // the body force is the saved one's until the next step
     ctx->launches += 1;
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1676,7 +1690,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
             rp.list = c->refill_list;
             rp.count = c->refill_count;
             rp.cap = c->refill_cap;
-            rp.s_nu = 1.0 / c->relax.tau;
+            rp.cs2_over_s_nu = 1.0 / (3.0 * (1.0 / c->relax.tau));
             rp.accel = c->accel;
             ref.add(&rp, list_blocks);
         }

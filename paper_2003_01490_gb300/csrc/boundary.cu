@@ -139,6 +139,61 @@ __device__ __forceinline__ void missing_links(const BcArgs<S>& a, long long idx,
     }
 }
 
+// The same in float64 with one warp per cell, lane q for direction q: a link is
+// some 60 float64 instructions of 64 cycles, and with a thread per cell and loop
+// over its links a sphere on a wall, whose cells fill one block, kept one
+// multiprocessor busy for longer than the dense kernel beside it.
+template <typename S>
+__device__ __forceinline__ void missing_links_of_cell(const BcArgs<S>& a, int idx, int q, const Sinks& sk) {
+    const int nx = a.g.n[0], ny = a.g.n[1];
+    const int x = idx % nx, yz = idx / nx, y = yz % ny, z = yz / ny;
+    const int cpos[3] = {x, y, z};
+    const int i = a.owner[idx];
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    bool missing = false;
+    if (q >= 1 && q < Q) {
+        const int c[3] = {k_c[q][0], k_c[q][1], k_c[q][2]};
+        int u[3];
+        bool outside = false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            u[d] = cpos[d] - c[d];
+            if (!a.g.per[d] && (u[d] < 0 || u[d] >= a.g.n[d])) outside = true;
+            u[d] = wrap_idx(u[d], a.g.n[d]);
+        }
+        missing = outside;
+        if (!outside) {
+            const int j = (u[2] * ny + u[1]) * nx + u[0];
+            missing = (a.flags[j] & FL_SOLID) && a.owner[j] != i;
+        }
+        if (missing) {
+            // exact float64 inside test, in the operation order of the mapping
+            double dd[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                dd[d] = min_image_d(((double)(cpos[d] - c[d]) + 0.5) - a.px[3 * i + d], a.g.n[d], a.g.per[d]);
+            const double Ri = a.pR[i];
+            const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dd[0], dd[0]), __dmul_rn(dd[1], dd[1])), __dmul_rn(dd[2], dd[2]));
+            missing = d2 > __dmul_rn(Ri, Ri);
+        }
+        if (missing) {
+            double r[3], R, up[3], om[3];
+            int n[3];
+            PartOps<double>::load(a, i, x - c[0], y - c[1], z - c[2], r, n, R, up, om);
+            const int cc2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
+            const double cf0 = c[0], cf1 = c[1], cf2 = c[2];
+            const double t = link_fraction<double>(r, cf0, cf1, cf2, (double)cc2, R);
+            const double rb[3] = {r[0] + t * cf0, r[1] + t * cf1, r[2] + t * cf2};
+            const double w2 = cc2 == 1 ? 2.0 / 18.0 : 2.0 / 36.0;
+            v[0] = w2 * cf0; v[1] = w2 * cf1; v[2] = w2 * cf2;
+            v[3] = rb[1] * v[2] - rb[2] * v[1];
+            v[4] = rb[2] * v[0] - rb[0] * v[2];
+            v[5] = rb[0] * v[1] - rb[1] * v[0];
+        }
+    }
+    if (__any_sync(0xffffffffu, missing)) commit_warp<double>(i, v, sk, q);
+}
+
 // mode BC_ACCEL: one thread forms the fluid body force of the step; mode
 // BC_LINKS: the missing-link terms 2 w_q c_q of Sec. 2.2 and their torques, one
 // thread per listed solid cell, committed per warp
@@ -160,6 +215,15 @@ __device__ __forceinline__ void boundary_body(const BcArgs<S>& a, int mode, int 
     if (!(mode & BC_LINKS) || !a.other_links) return;
     const Sinks sk{a.acc_d, a.acc_i, a.acc_k, a.status};
     const int mcount = min(*a.miss_count, a.miss_cap);
+    if constexpr (sizeof(T) == 8) {
+        // one warp per cell as long as every warp has one at most (a thread per
+        // cell issues a third of the instructions)
+        if (a.missing_links && mcount <= gx * (int)(blockDim.x >> 5)) {
+            const int w = (int)(bx * blockDim.x + threadIdx.x) >> 5;
+            if (w < mcount) missing_links_of_cell<S>(a, (int)a.miss[w], (int)(threadIdx.x & 31), sk);
+            return;
+        }
+    }
     const int stride = (int)(gx * blockDim.x);
     for (int base = (int)(bx * blockDim.x); base < mcount; base += stride) {
         const int k = base + threadIdx.x;
@@ -216,7 +280,15 @@ template <typename S>
 void launch_boundary_t(const LbmStepParams& p, cudaStream_t st, int mode) {
     BcArgs<S> b;
     fill_bc_args_t<S>(p, b);
-    const int blocks = (mode & BC_LINKS) && p.other_links ? 8 * (p.num_sms > 0 ? p.num_sms : 1) : 1;
+    // a thread, in float64 a warp, per surface cell of the particles, of which the
+    // listed cells are a part: with few particles no crowd of idle blocks beside the
+    // dense kernel's (margin is the largest radius and three cells)
+    int blocks = 1;
+    if ((mode & BC_LINKS) && p.other_links) {
+        const double cells = 13.0 * p.P.n * (p.margin - 2) * (double)(p.margin - 2), each = sizeof(S) == 8 ? 4.0 : 128.0;
+        const int most = 8 * (p.num_sms > 0 ? p.num_sms : 1);
+        blocks = cells < each * most ? 1 + (int)(cells / each) : most;
+    }
     boundary_kernel<S><<<blocks, 128, 0, st>>>(b, mode);
 }
 

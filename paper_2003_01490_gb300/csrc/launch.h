@@ -87,7 +87,7 @@ struct RefillParams {
     const unsigned int* list;
     const int* count;
     int cap;
-    double s_nu;
+    double cs2_over_s_nu;  // 1 / (3 s_nu)
     const double* accel;   // fluid body force of the step [3]
 };
 void launch_refill(const RefillParams& p, cudaStream_t st);

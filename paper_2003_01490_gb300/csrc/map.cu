@@ -561,10 +561,12 @@ __device__ __forceinline__ void refill_body(const RefillParams& p, int bx, int g
     constexpr unsigned long long PX = pack_dirs(0), PY = pack_dirs(1), PZ = pack_dirs(2);
     const int warps = gx * (blockDim.x >> 5);
     for (int k = bx * (blockDim.x >> 5) + (threadIdx.x >> 5); k < count; k += warps) {   // warp-uniform
-        const long long idx = p.list[k];
-        const int x = (int)(idx % nx);
-        const int y = (int)((idx / nx) % ny);
-        const int z = (int)(idx / ((long long)nx * ny));
+        const unsigned cell = p.list[k];
+        const long long idx = cell;
+        const unsigned yz = cell / (unsigned)nx;
+        const int x = (int)(cell % (unsigned)nx);
+        const int y = (int)(yz % (unsigned)ny);
+        const int z = (int)(yz / (unsigned)ny);
         const int cpos[3] = {x, y, z};
         const int i = p.list_owner[k];
         const int q = lane < Q ? lane : 0;
@@ -588,9 +590,9 @@ __device__ __forceinline__ void refill_body(const RefillParams& p, int bx, int g
                     for (int r = 0; r < Q; ++r) {
                         const T v = Store<S>::load(f + (long long)r * N + j);
                         dr += v;
-                        jx += (T)cx(r) * v;
-                        jy += (T)cy(r) * v;
-                        jz += (T)cz(r) * v;
+                        if (cx(r)) jx += cx(r) > 0 ? v : -v;
+                        if (cy(r)) jy += cy(r) > 0 ? v : -v;
+                        if (cz(r)) jz += cz(r) > 0 ? v : -v;
                     }
                 }
             }
@@ -643,7 +645,7 @@ __device__ __forceinline__ void refill_body(const RefillParams& p, int bx, int g
             }
         }
         if (lane < Q) {
-            const T coef = T(1) / (T(3) * (T)p.s_nu);   // c_s^2 / s_nu
+            const T coef = (T)p.cs2_over_s_nu;
             const T cf[3] = {(T)c[0], (T)c[1], (T)c[2]};
             T second = T(0);
 #pragma unroll
@@ -695,7 +697,8 @@ void launch_map_gang(int kind, int storage, const void* table, const int* off, i
 }
 
 void launch_refill(const RefillParams& p, cudaStream_t st) {
-    const int blocks = 152 * 8, threads = 128;   // 4 warps (cells) per block
+    // 4 warps (cells) per block; some 32 cells a particle at once, more take turns
+    const int blocks = p.P.n < 152 ? 8 * p.P.n : 152 * 8, threads = 128;
     switch (p.storage) {
         case 0: refill_kernel<double><<<blocks, threads, 0, st>>>(p); break;
         case 1: refill_kernel<float><<<blocks, threads, 0, st>>>(p); break;
