@@ -23,6 +23,8 @@ using namespace lbmdem;
 // mapping, refill
 constexpr int LBM_PHASES = 6;
 
+constexpr size_t IO_WORDS = 8192;   // of a context's page-locked memory (64 KB)
+
 struct lbm_ctx {
     Geom g{};
     lbm_relax relax{};
@@ -51,6 +53,9 @@ struct lbm_ctx {
     int* status = nullptr;
     double* accel = nullptr;
     float* accel_f = nullptr;
+    // page-locked memory for small transfers (NULL: none could be had): kernels read
+    // and write it themselves, so a call waits once; word 0 takes the status
+    double* io = nullptr;
     bool accel_set = true;         // they hold the body force of a box without counterforce
     unsigned* barrier = nullptr;   // of the cooperative DEM launch
     int grid_particles = 0;        // particles a cooperative DEM launch holds
@@ -97,6 +102,8 @@ struct lbm_ctx {
 
 // streams, events and graphs a context holds (device memory is separate)
 void destroy_handles(lbm_ctx* ctx) {
+    if (ctx->io) cudaFreeHost(ctx->io);
+    ctx->io = nullptr;
     for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
     ctx->events.clear();
     for (int a = 0; a < 2; ++a)
@@ -316,6 +323,10 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
             ctx->num_sms = sms;
         cudaError_t pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
         ctx->cluster_particles = dem_cluster_capacity();
+        if (cudaHostAlloc(&ctx->io, sizeof(double) * IO_WORDS, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->io = nullptr;
+        }
         if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
@@ -570,10 +581,7 @@ cudaError_t prof_mark(lbm_ctx* ctx) {
     return cudaEventRecord(ctx->events[ctx->ev_used++], ctx->stream);
 }
 
-lbm_status check_status(lbm_ctx* ctx) {
-    int st = 0;
-    CK(cudaMemcpyAsync(&st, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+lbm_status status_result(lbm_ctx* ctx, int st) {
     if (st & ST_UNSTABLE) return fail(ctx, LBM_ERR_UNSTABLE, "density left (0.5, 1.5) or became NaN");
     if (st & (ST_TILE_OVERFLOW | ST_NBR_OVERFLOW | ST_BIN_OVERFLOW | ST_REFILL_OVERFLOW | ST_HIST_OVERFLOW |
               ST_FIXED_OVERFLOW)) {
@@ -584,6 +592,15 @@ lbm_status check_status(lbm_ctx* ctx) {
     if (st & ST_TIMEOUT) return fail(ctx, LBM_ERR_TIMEOUT, "a barrier of the DEM launch ran out");
     if (st & ST_FAST_PARTICLE) return fail(ctx, LBM_ERR_UNSTABLE, "particle speed above 0.5 cells per step");
     return LBM_OK;
+}
+
+// waits for the stream
+lbm_status check_status(lbm_ctx* ctx) {
+    int own = 0;
+    int* const st = ctx->io ? reinterpret_cast<int*>(ctx->io) : &own;
+    CK(cudaMemcpyAsync(st, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    return status_result(ctx, *st);
 }
 
 }  // namespace
@@ -1107,7 +1124,6 @@ lbm_status lbm_set_stream(lbm_ctx* ctx, void* cuda_stream) {
 
 lbm_status lbm_sync(lbm_ctx* ctx) {
     if (!ctx) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
-    CK(cudaStreamSynchronize(ctx->stream));
     if (ctx->readout_stream) CK(cudaStreamSynchronize(ctx->readout_stream));
     return check_status(ctx);
 }
@@ -1120,6 +1136,17 @@ lbm_status lbm_get_particle_state(lbm_ctx* ctx, int n_cap, double* pos, double* 
     if (n_cap < n && (pos || vel || omega || force_hyd || torque_hyd))
         return fail(ctx, LBM_ERR_INVALID, "n_cap smaller than the particle count");
     cudaStream_t sm = ctx->stream;
+    if (n > 0 && ctx->io && 15 * (size_t)n < IO_WORDS && (pos || vel || omega || force_hyd || torque_hyd)) {
+        double* const src = ctx->io + 1;
+        launch_read_state(ctx->P, src, ctx->status, reinterpret_cast<int*>(ctx->io), sm);
+        ctx->launches += 1;
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(sm));
+        double* const dst[5] = {pos, vel, omega, force_hyd, torque_hyd};
+        for (int k = 0; k < 5; ++k)
+            if (dst[k]) std::memcpy(dst[k], src + 3 * (size_t)n * k, 24 * (size_t)n);
+        return status_result(ctx, *reinterpret_cast<int*>(ctx->io));
+    }
     if (n > 0) {
         if (pos) CK(cudaMemcpyAsync(pos, ctx->P.x, 24 * (size_t)n, cudaMemcpyDeviceToHost, sm));
         if (vel) CK(cudaMemcpyAsync(vel, ctx->P.u, 24 * (size_t)n, cudaMemcpyDeviceToHost, sm));
@@ -1308,13 +1335,23 @@ lbm_status lbm_set_particle_velocity(lbm_ctx* ctx, int n, const double* vel, con
     if (n < 0 || n > ctx->P.n) return fail(ctx, LBM_ERR_INVALID, "n outside [0, particle count]");
     if (n == 0) return LBM_OK;
     cudaStream_t sm = ctx->stream;
+    if (ctx->io && 6 * (size_t)n < IO_WORDS) {
+        double* const src = ctx->io + 1;
+        if (vel) std::memcpy(src, vel, 24 * (size_t)n);
+        if (omega) std::memcpy(src + 3 * (size_t)n, omega, 24 * (size_t)n);
+        launch_set_velocity(ctx->P, n, vel ? src : nullptr, omega ? src + 3 * (size_t)n : nullptr, ctx->status,
+                            reinterpret_cast<int*>(ctx->io), sm);
+        ctx->launches += 1;
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(sm));
+        return status_result(ctx, *reinterpret_cast<int*>(ctx->io));
+    }
     if (vel) CK(cudaMemcpyAsync(ctx->P.u, vel, 24 * (size_t)n, cudaMemcpyHostToDevice, sm));
     if (omega) CK(cudaMemcpyAsync(ctx->P.om, omega, 24 * (size_t)n, cudaMemcpyHostToDevice, sm));
     // the float32 view carries the velocities into the link arithmetic
     launch_view_update(ctx->P, sm);
     ctx->launches += 1;
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(sm));
     return check_status(ctx);
 }
 
@@ -1324,7 +1361,7 @@ lbm_status lbm_get_fields(lbm_ctx* ctx, double* rho, double* u, unsigned char* f
     const long long N = ctx->g.ncells;
     if (flags) CK(cudaMemcpyAsync(flags, ctx->flags, (size_t)N, cudaMemcpyDeviceToHost, sm));
     if (rho || u) {
-        std::vector<double> buf(4 * (size_t)ctx->scratch_cells);
+        // straight into the caller's arrays, a slab of cells at a time
         for (long long first = 0; first < N; first += ctx->scratch_cells) {
             const long long cnt = (N - first) < ctx->scratch_cells ? (N - first) : ctx->scratch_cells;
             FieldsParams fp{};
@@ -1339,15 +1376,12 @@ lbm_status lbm_get_fields(lbm_ctx* ctx, double* rho, double* u, unsigned char* f
             launch_fields(fp, sm);
             ctx->launches += 1;
             CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(buf.data(), ctx->scratch, 32 * (size_t)cnt, cudaMemcpyDeviceToHost, sm));
-            CK(cudaStreamSynchronize(sm));
-            if (rho) std::memcpy(rho + first, buf.data(), 8 * (size_t)cnt);
-            if (u)
-                for (int c = 0; c < 3; ++c)
-                    std::memcpy(u + (size_t)c * N + first, buf.data() + (size_t)(c + 1) * cnt, 8 * (size_t)cnt);
+            if (rho) CK(cudaMemcpyAsync(rho + first, ctx->scratch, 8 * (size_t)cnt, cudaMemcpyDeviceToHost, sm));
+            for (int c = 0; c < 3 && u; ++c)
+                CK(cudaMemcpyAsync(u + (size_t)c * N + first, ctx->scratch + (size_t)(c + 1) * cnt, 8 * (size_t)cnt,
+                                   cudaMemcpyDeviceToHost, sm));
         }
     }
-    CK(cudaStreamSynchronize(sm));
     return check_status(ctx);
 }
 
@@ -1356,21 +1390,34 @@ lbm_status lbm_sample_density(lbm_ctx* ctx, int n, const double* pos, double* rh
     if (n < 0 || (long long)n > ctx->scratch_cells) return fail(ctx, LBM_ERR_INVALID, "n outside [0, scratch size]");
     if (n == 0) return LBM_OK;
     cudaStream_t sm = ctx->stream;
-    // points and results in the scratch buffer (4 doubles per scratch cell)
-    CK(cudaMemcpyAsync(ctx->scratch, pos, 24 * (size_t)n, cudaMemcpyHostToDevice, sm));
     SampleParams sp{};
+    const bool small = ctx->io && 4 * (size_t)n < IO_WORDS;
+    // points and results in page-locked memory, many of them in the scratch buffer
+    // (4 doubles per scratch cell)
+    double* const io = small ? ctx->io + 1 : ctx->scratch;
+    if (small) {
+        std::memcpy(io, pos, 24 * (size_t)n);
+        sp.status = ctx->status;
+        sp.status_out = reinterpret_cast<int*>(ctx->io);
+    } else {
+        CK(cudaMemcpyAsync(io, pos, 24 * (size_t)n, cudaMemcpyHostToDevice, sm));
+    }
     sp.storage = ctx->storage;
     sp.f = ctx->f[ctx->cur];
     sp.flags = ctx->flags;
     sp.g = ctx->g;
     sp.n = n;
-    sp.pos = ctx->scratch;
-    sp.out = ctx->scratch + 3 * (size_t)n;
+    sp.pos = io;
+    sp.out = io + 3 * (size_t)n;
     launch_sample_density(sp, sm);
     ctx->launches += 1;
     CK(cudaGetLastError());
+    if (small) {
+        CK(cudaStreamSynchronize(sm));
+        std::memcpy(rho, sp.out, 8 * (size_t)n);
+        return status_result(ctx, *sp.status_out);
+    }
     CK(cudaMemcpyAsync(rho, sp.out, 8 * (size_t)n, cudaMemcpyDeviceToHost, sm));
-    CK(cudaStreamSynchronize(sm));
     return check_status(ctx);
 }
 

@@ -134,6 +134,41 @@ __global__ void view_kernel(const Particles P) {
     write_view(P, i);
 }
 
+__global__ void read_state_kernel(const Particles P, double* __restrict__ out, const int* __restrict__ status,
+                                  int* __restrict__ status_out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, n3 = 3 * P.n;
+    if (k == 0) *status_out = *status;
+    if (k >= n3) return;
+    out[k] = P.x[k];
+    out[n3 + k] = P.u[k];
+    out[2 * n3 + k] = P.om[k];
+    const int i = k / 3, d = k % 3;
+    out[3 * n3 + k] = P.fp[6 * i + d];
+    out[4 * n3 + k] = P.fp[6 * i + 3 + d];
+}
+
+void launch_read_state(const Particles& P, double* out, const int* status, int* status_out, cudaStream_t st) {
+    read_state_kernel<<<(3 * P.n + 127) / 128, 128, 0, st>>>(P, out, status, status_out);
+}
+
+__global__ void set_velocity_kernel(const Particles P, int n, const double* __restrict__ vel,
+                                    const double* __restrict__ omega, const int* __restrict__ status,
+                                    int* __restrict__ status_out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *status_out = *status;
+    if (i >= P.n) return;
+    for (int d = 0; d < 3 && i < n; ++d) {
+        if (vel) P.u[3 * i + d] = vel[3 * i + d];
+        if (omega) P.om[3 * i + d] = omega[3 * i + d];
+    }
+    write_view(P, i);
+}
+
+void launch_set_velocity(const Particles& P, int n, const double* vel, const double* omega, const int* status,
+                         int* status_out, cudaStream_t st) {
+    set_velocity_kernel<<<(P.n + 127) / 128, 128, 0, st>>>(P, n, vel, omega, status, status_out);
+}
+
 void launch_view_update(const Particles& P, cudaStream_t st) {
     if (P.n == 0) return;
     view_kernel<<<(P.n + 127) / 128, 128, 0, st>>>(P);

@@ -112,6 +112,8 @@ struct SampleParams {
     int n;
     const double* pos;      // [3n] sample points
     double* out;            // [n] density at each point
+    const int* status;      // copied to status_out (or status_out NULL)
+    int* status_out;
 };
 void launch_sample_density(const SampleParams& p, cudaStream_t st);
 
@@ -174,6 +176,13 @@ int dem_cluster_capacity();               // DEM_CLUSTER_MAX, or 0 where no such
 cudaError_t launch_dem_step(const DemParams& p, const FinalizeParams& fin, const MapParams& sc, int hcur, int n_sub,
                             int cluster_particles, cudaStream_t st);
 void launch_state_copy(const Particles& P, cudaStream_t st);
+// state of n particles (positions, velocities, angular velocities, F^fp, T^fp,
+// 3n values each) to out and the status to status_out, in page-locked host memory
+void launch_read_state(const Particles& P, double* out, const int* status, int* status_out, cudaStream_t st);
+// velocities of particles 0 .. n - 1 from page-locked host memory (either NULL:
+// kept), the views of all particles, the status to status_out
+void launch_set_velocity(const Particles& P, int n, const double* vel, const double* omega, const int* status,
+                         int* status_out, cudaStream_t st);
 void launch_fp_split(const double* fp, double* out, int n, cudaStream_t st);
 
 // Gang launches (gang.cuh): one launch of a per-step kernel for many

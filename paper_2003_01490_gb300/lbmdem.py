@@ -289,7 +289,8 @@ def lbm_get_particle_state(ctx, out=None):
     ``out`` may hold preallocated (pinned) float64 arrays under the same keys."""
     lib = load_library()
     n = c_int(0)
-    _check(lib.lbm_get_particle_state(ctx.handle, 0, None, None, None, None, None, ctypes.byref(n)),
+    # the count alone, without a wait
+    _check(lib.lbm_get_particle_state_async(ctx.handle, 0, None, None, None, None, None, ctypes.byref(n)),
            ctx.handle)
     n = n.value
     keys = ('pos', 'vel', 'omega', 'force_hyd', 'torque_hyd')
