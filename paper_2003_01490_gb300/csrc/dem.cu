@@ -708,6 +708,9 @@ struct OctLane {
     double coef, dcoef;             // dt / (2 m) or dt / (2 I), dt times it
     float xf, vf, R;                // float32 copies for the tests that decide most cases
     float xl, Rl, m;                // trailing parts of position and radius, the mass, for the float32 laws
+    float side;                     // of the box on the lane's axis (lanes 0-2)
+    float face;                     // face o.s is in reach where the position (negated for the upper face) is at most
+                                    // this, minus infinity without a wall
 };
 
 // lane s's share of the particle's record
@@ -735,13 +738,21 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
     o.on = i < P.n;
     o.nn = 0;
     o.x = o.v = o.f_prev = o.f_const = o.coef = o.dcoef = 0.0;
-    o.xf = o.vf = o.R = o.xl = o.Rl = o.m = 0.f;
+    o.xf = o.vf = o.R = o.xl = o.Rl = o.m = o.side = 0.f;
+    o.face = -INFINITY;
     if (!o.on) return;
     o.nn = P.nbr_count[i];
     o.R = (float)P.R[i];
     o.Rl = trailing(P.R[i]);
     o.m = (float)P.m[i];
     const float reach = o.R + ((float)p.cut_max + 1e-3f);
+    if (s < 3) o.side = (float)p.g.n[s];
+    if (s < 6 && !p.g.per[s >> 1]) {
+        // the float32 position is within 1e-4 of the float64 one for boxes of up to
+        // 2^11 cells; the exact gap decides where the face is in reach
+        const float n = (float)p.g.n[s >> 1];
+        o.face = reach + 1e-6f * n - (s & 1 ? n : 0.f);
+    }
 #pragma unroll
     for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
         const int slot = s + DEM_LANES * k;
@@ -769,14 +780,20 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
     o.vf = (float)o.v;
 }
 
+// whether the warp (float32 laws) or the block has a neighbour slot
+template <typename T>
+__device__ __forceinline__ bool oct_pairs(const OctLane& o) {
+    if constexpr (sizeof(T) == 4) return __any_sync(0xffffffffu, o.nn > 0);
+    else return __syncthreads_or(o.nn > 0);
+}
+
 // Eq. (37) for lanes 0-2; the periodic wrap is decided in float64 only for
 // positions within half a cell of a face
 __device__ __forceinline__ void oct_move(const DemParams& p, OctLane& o) {
     o.x = fma(o.dcoef, o.f_prev, fma(p.dt, o.v, o.x));
     o.xf = (float)o.x;
-    const int n = p.g.n[o.s];
-    if (!(o.xf > 0.5f && o.xf < (float)n - 0.5f)) {
-        o.x = wrap_pos(o.x, n, p.g.per[o.s]);
+    if (!(o.xf > 0.5f && o.xf < o.side - 0.5f)) {
+        o.x = wrap_pos(o.x, p.g.n[o.s], p.g.per[o.s]);
         o.xf = (float)o.x;
     }
     o.xl = trailing(o.x);
@@ -930,17 +947,19 @@ __device__ bool wall_force(const DemParams& p, const OctLane& o, WallSpring<T>& 
 // One subcycle of the particle of o (Algorithm 1, inner loop): pair and wall
 // laws at the state in buffer cur, the velocities (Eq. (38)) and, unless it is
 // the last subcycle, the positions of the next one (Eq. (37)), published in
-// buffer 1 - cur. init = 1 evaluates the initial force F(t = 0) only (no state
-// or history update). All threads of the block take part.
+// buffer 1 - cur, where the particle has neighbours (which then have it as
+// theirs). init = 1 evaluates the initial force F(t = 0) only (no state or history
+// update). All threads of the block take part; pairs: the block (float32: the
+// warp) has a neighbour slot; put_n: hist_n is to be written.
 template <typename T, bool CG, int PPB>
 __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, WallSpring<T>& w, PairQueue<PPB>* queue,
-                                             int cur, int hin, int hout, int init, int last) {
+                                             bool pairs, int cur, int hin, int hout, bool put_n, int init, int last) {
     const Particles& P = p.P;
     const unsigned FULL = 0xffffffffu;
     T f[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
     bool acts = false;
     if constexpr (sizeof(T) == 4) {
-        if (__any_sync(FULL, o.nn > 0)) {
+        if (pairs) {
             // the own record from the particle's lanes
             const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
             DemRec me;
@@ -972,7 +991,7 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
                 if (!init) P.hist_id[hout][o.i * NBR_CAP + slot] = contact ? o.j[k] : -1;
             }
         }
-    } else {
+    } else if (pairs) {
         // pairs that pass the prefilter into the block's queue, evaluated by
         // whichever thread comes first; each lane then collects its slots'
         const int pl = threadIdx.x / DEM_LANES;
@@ -1024,15 +1043,10 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
             __syncthreads();
         }
     }
-    // faces within reach, by the float32 position (within 1e-4 of the float64
-    // one for boxes of up to 2^11 cells; the exact gap decides below)
     bool face = false;
-    const bool walled = o.on && o.s < 6 && !p.g.per[o.s >> 1];
-    {
+    if (!(p.g.per[0] && p.g.per[1] && p.g.per[2])) {
         const float xa = __shfl_sync(FULL, o.xf, o.s >> 1, DEM_LANES);
-        const float gap = (o.s & 1 ? (float)p.g.n[(o.s >> 1) % 3] - xa : xa) - o.R;
-        const float slack = 1e-3f + 1e-6f * (float)p.g.n[(o.s >> 1) % 3];
-        face = walled && !(gap > (float)p.cut_max + slack);
+        face = (o.s & 1 ? -xa : xa) <= o.face;
         if (!face && !init) w.on = false;
     }
     if (__any_sync(FULL, face)) {
@@ -1074,7 +1088,7 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
         else if (o.s < 6) P.T_prev[3 * o.i + o.s - 3] = fs;
         return;
     }
-    if (o.s == 6) P.hist_n[hout][o.i] = o.nn;
+    if (put_n && o.s == 6) P.hist_n[hout][o.i] = o.nn;
     // Eq. (38) for u and its rotational analogue for omega
     o.v = fma(o.coef, o.f_prev + fs, o.v);
     o.f_prev = fs;
@@ -1083,14 +1097,14 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
     // the next subcycle's positions; the last subcycle keeps its own
     if (o.s < 3 && !last) oct_move(p, o);
     if constexpr (sizeof(T) == 4) {
-        if (!last) oct_publish(p, o, nxt);
-    } else if (o.s < 3) {
+        if (!last && o.nn > 0) oct_publish(p, o, nxt);
+    } else if (o.nn > 0 && o.s < 3) {
         if (!last) {
             P.xs[nxt][3 * o.i + o.s] = o.x;
             P.xfs[nxt][3 * o.i + o.s] = o.xf;
         }
         P.us[nxt][3 * o.i + o.s] = o.v;
-    } else if (o.s < 6) {
+    } else if (o.nn > 0 && o.s < 6) {
         P.oms[nxt][3 * o.i + o.s - 3] = o.v;
     }
 }
@@ -1099,14 +1113,11 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
 // the squared components of lanes 0-2).
 __device__ __forceinline__ void oct_check_speed(const DemParams& p, const OctLane& o) {
     const unsigned FULL = 0xffffffffu;
-    // the float32 sum decides unless it is near the limit
-    float q = o.on && o.s < 3 ? o.vf * o.vf : 0.f;
-    q += __shfl_down_sync(FULL, q, 2, DEM_LANES) + __shfl_down_sync(FULL, q, 1, DEM_LANES);
-    const bool near = o.on && o.s == 0 && !(q < 0.2499f);
-    if (!__any_sync(FULL, near)) return;
+    // three components below 0.288 are below the limit together
+    if (!__any_sync(FULL, o.on && o.s < 3 && !(fabsf(o.vf) < 0.288f))) return;
     const double sq = o.v * o.v;
     const double q1 = __shfl_down_sync(FULL, sq, 1, DEM_LANES), q2 = __shfl_down_sync(FULL, sq, 2, DEM_LANES);
-    if (near && !((sq + q1) + q2 < 0.25)) atomicOr(p.status, ST_FAST_PARTICLE);
+    if (o.on && o.s == 0 && !((sq + q1) + q2 < 0.25)) atomicOr(p.status, ST_FAST_PARTICLE);
 }
 
 // the state after the last subcycle into buffer 0 of the particle arrays and
@@ -1171,7 +1182,8 @@ __device__ __forceinline__ void subcycle_body(const DemParams& p, int cur, int h
     oct_load<false>(p, o, pblock * DEM_PPB + (int)threadIdx.x / DEM_LANES, threadIdx.x % DEM_LANES, cur);
     WallSpring<T> w;
     wall_load<T>(p, o, w, hin);
-    oct_subcycle<T, false, sizeof(T) == 8 ? DEM_PPB : 1>(p, o, w, &queue, cur, hin, hout, init, last);
+    oct_subcycle<T, false, sizeof(T) == 8 ? DEM_PPB : 1>(p, o, w, &queue, oct_pairs<T>(o), cur, hin, hout, true, init,
+                                                        last);
     if (init) return;
     wall_store<T>(p, o, w, hout);
     oct_check_speed(p, o);
@@ -1251,6 +1263,7 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
     WallSpring<T> w;
     wall_load<T>(p, o, w, hcur);
     oct_first_position<T>(p, o);
+    const bool pairs = oct_pairs<T>(o);
     unsigned target = 0;
     bool ok = true;
     auto barrier = [&]() {
@@ -1266,7 +1279,7 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
     for (int k = 0; k < n_sub && ok; ++k) {
         barrier();
         if (!ok) break;
-        oct_subcycle<T, CG, PPB>(p, o, w, queue, k & 1, hcur, 1 - hcur, 0, k == n_sub - 1);
+        oct_subcycle<T, CG, PPB>(p, o, w, queue, pairs, k & 1, hcur, 1 - hcur, k < 2, 0, k == n_sub - 1);
         oct_check_speed(p, o);
         hcur = 1 - hcur;
     }
