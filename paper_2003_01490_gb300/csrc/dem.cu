@@ -1290,11 +1290,7 @@ __device__ __forceinline__ void dem_step_body(const DemParams& p, const Finalize
     oct_store_view(p, o);
     if (sc) {
         if (first_particle == 0 && threadIdx.x < 4) reinterpret_cast<int*>(sc->n_solid)[threadIdx.x] = 0;
-        const unsigned FULL = 0xffffffffu;
-        const int base = (threadIdx.x & 31) & ~(DEM_LANES - 1);
-        const double x[3] = {__shfl_sync(FULL, o.x, base), __shfl_sync(FULL, o.x, base + 1),
-                             __shfl_sync(FULL, o.x, base + 2)};
-        if (o.on) tile_scatter_particle(*sc, o.i, x, s, DEM_LANES);
+        tile_scatter_particle<DEM_LANES>(*sc, o.i, o.on, o.x, s);
     }
 }
 

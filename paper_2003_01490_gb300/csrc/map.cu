@@ -51,8 +51,8 @@ __device__ __forceinline__ double min_image_dd(double d, int n, int per) {
 __device__ __forceinline__ void tile_scatter_body(const MapParams& p, int bx) {
     const int i = (bx * blockDim.x + threadIdx.x) >> 5;
     if (i >= p.P.n) return;   // warp-uniform
-    const double xc[3] = {p.P.x[3 * i], p.P.x[3 * i + 1], p.P.x[3 * i + 2]};
-    tile_scatter_particle(p, i, xc, threadIdx.x & 31, 32);
+    const int lane = threadIdx.x & 31;
+    tile_scatter_particle<32>(p, i, true, lane < 3 ? p.P.x[3 * i + lane] : 0.0, lane);
 }
 
 __global__ void tile_scatter_kernel(const MapParams p) { tile_scatter_body(p, (int)blockIdx.x); }

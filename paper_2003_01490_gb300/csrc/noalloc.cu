@@ -36,18 +36,15 @@ static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 __global__ void __launch_bounds__(128) noalloc_scatter_kernel(const __grid_constant__ MapParams p) {
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (i >= p.P.n) return;   // warp-uniform
-    const double x[3] = {p.P.x[3 * i], p.P.x[3 * i + 1], p.P.x[3 * i + 2]};
-    if (lane == 0) {
-        PartView v{};   // the rest is unused by the mapping
-        for (int d = 0; d < 3; ++d) {
-            const double b = floor(x[d]);
-            v.base[d] = (int)b;
-            v.frac[d] = (float)(x[d] - b);
-        }
-        v.R = (float)p.P.R[i];
-        p.P.view[i] = v;
+    const double x = lane < 3 ? p.P.x[3 * i + lane] : 0.0;
+    if (lane < 3) {   // the rest of the view is unused by the mapping
+        const double b = floor(x);
+        p.P.view[i].base[lane] = (int)b;
+        p.P.view[i].frac[lane] = (float)(x - b);
+    } else if (lane == 3) {
+        p.P.view[i].R = (float)p.P.R[i];
     }
-    tile_scatter_particle(p, i, x, lane, 32);
+    tile_scatter_particle<32>(p, i, true, x, lane);
 }
 
 namespace {
