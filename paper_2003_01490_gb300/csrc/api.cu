@@ -1686,7 +1686,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
             fp.use_fixed = c->storage != LBM_STORE_F64;
             fp.first_step = 0;
             fp.averaging = d.force_averaging;
-            fin.add(&fp, (np + 127) / 128);
+            fin.add(&fp, (8 * np + 127) / 128);
         }
         if (dem && np <= DEM_ONE_BLOCK_MAX) {
             fill_dem_batch_entry(dp, c->hcur, d.n_sub, &host_dem[db * G.n_dem]);

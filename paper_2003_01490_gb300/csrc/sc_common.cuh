@@ -258,8 +258,9 @@ __host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? 
 //   s_nu X + (1 - s_nu/2) 2 Y / 2 = s_nu [drho - 3/2 u^2 - 3/2 k u.a + 9/2 (c.u)(c.v)],  v = u + k a, k = (2 - s_nu)/s_nu
 //   s_nu^- 3 c.u + (1 - s_nu^-/2) 3 c.a = s_nu^- 3 c.t,                                  t = u + (k^-/2) a, k^- = (2 - s_nu^-)/s_nu^-
 // (ke = k, ko = k^-/2)
-// so a pair costs the same few multiply-adds with and without a body force.
-template <typename T>
+// so a pair costs the same few multiply-adds with and without a body force; FORCE =
+// false is the form for a = 0 (the same values), which leaves out the sums with a.
+template <typename T, bool FORCE>
 __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V (&f)[Q],
                                                             const bool (&shell)[Pack<T>::ROWS], T ax, T ay, T az, T sp,
                                                             T sm, T ke, T ko, T s_b_shell, T s_b_bulk,
@@ -280,11 +281,15 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         if (cy(q)) jy = cy(q) * sg > 0 ? jy + d : jy - d;
         if (cz(q)) jz = cz(q) * sg > 0 ? jz + d : jz - d;
     }
-    const V ux = jx + P::all(T(0.5) * ax), uy = jy + P::all(T(0.5) * ay), uz = jz + P::all(T(0.5) * az);
+    const V ux = FORCE ? jx + P::all(T(0.5) * ax) : jx, uy = FORCE ? jy + P::all(T(0.5) * ay) : jy,
+            uz = FORCE ? jz + P::all(T(0.5) * az) : jz;
     const V usq = mad(uz, uz, mad(ux, ux, uy * uy));
-    const V ua = mad(ux, P::all(ax), mad(uy, P::all(ay), uz * P::all(az)));
-    const V vx = ux + P::all(ke * ax), vy = uy + P::all(ke * ay), vz = uz + P::all(ke * az);
-    const V tx = ux + P::all(ko * ax), ty = uy + P::all(ko * ay), tz = uz + P::all(ko * az);
+    V ua = P::all(T(0)), vx = ux, vy = uy, vz = uz, tx = ux, ty = uy, tz = uz;
+    if constexpr (FORCE) {
+        ua = mad(ux, P::all(ax), mad(uy, P::all(ay), uz * P::all(az)));
+        vx = ux + P::all(ke * ax); vy = uy + P::all(ke * ay); vz = uz + P::all(ke * az);
+        tx = ux + P::all(ko * ax); ty = uy + P::all(ko * ay); tz = uz + P::all(ko * az);
+    }
     // bulk moments m4 = sum (c^2 - 1) f and m5 (row 6 of M) of the streamed
     // PDFs relax with s_b in shell cells (and everywhere when Lambda_b,bulk != 1)
     bool bulk = bulk_corr != 0;
@@ -305,11 +310,11 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         const V m4 = sdiag - f[0];
         const V m5 = mad(P::all(T(-2)), saxis, f[0]) + sdiag;
         // M^-1 e_k = w_q M_kq / (sum_q w_q M_kq^2): norms 2/3 (row 4) and 2 (row 5)
-        k4 = P::all(T(1.5)) * (ds * ((usq - m4) - ua));
+        k4 = P::all(T(1.5)) * (ds * (FORCE ? (usq - m4) - ua : usq - m4));
         k5 = P::all(T(-0.5)) * (ds * m5);
     }
     // equilibrium part common to all directions, with the u.a term of the source
-    const V X0 = mad(P::all(T(-1.5)), mad(P::all(ke), ua, usq), drho);
+    const V X0 = mad(P::all(T(-1.5)), FORCE ? mad(P::all(ke), ua, usq) : usq, drho);
     // Weights of the update: w2 = 2 w (even parts), w6 = 6 w (odd parts) per
     // class (axis, diagonal) and w0. In float32 they are chosen within 1.2e-7
     // of the exact fractions such that w0 + 3 w2_axis + 6 w2_diag = 1 and
@@ -340,10 +345,14 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         const bool y_plus = cy(q) * sg > 0, z_plus = cz(q) * sg > 0;
         V cu = cx(q) ? ux : (cy(q) ? uy : uz), cv = cx(q) ? vx : (cy(q) ? vy : vz), ct = cx(q) ? tx : (cy(q) ? ty : tz);
         if (cx(q) && cy(q)) {
-            cu = y_plus ? cu + uy : cu - uy; cv = y_plus ? cv + vy : cv - vy; ct = y_plus ? ct + ty : ct - ty;
+            cu = y_plus ? cu + uy : cu - uy;
+            cv = FORCE ? (y_plus ? cv + vy : cv - vy) : cu;
+            ct = FORCE ? (y_plus ? ct + ty : ct - ty) : cu;
         }
         if ((cx(q) || cy(q)) && cz(q)) {
-            cu = z_plus ? cu + uz : cu - uz; cv = z_plus ? cv + vz : cv - vz; ct = z_plus ? ct + tz : ct - tz;
+            cu = z_plus ? cu + uz : cu - uz;
+            cv = FORCE ? (z_plus ? cv + vz : cv - vz) : cu;
+            ct = FORCE ? (z_plus ? ct + tz : ct - tz) : cu;
         }
         const V X = mad(c45 * cu, cv, X0);
         const V dp = mad(hsp, mad(mw2[k], X, mad(one, f[q], f[qb])), corr[k]);

@@ -51,8 +51,7 @@ __device__ __forceinline__ int axis_tiles(int np, const int (&a)[2], const int (
 // lanes 0-2 find the tiles of one axis each (with all three axes in every lane the
 // 27 float64 instructions of 64 cycles took most of the scatter: 10,000 particles
 // mapped without history 144 us per call, this way 131), then all lanes share out
-// the tiles of the box. All lanes of the warp take
-// part.
+// the tiles of the box. All lanes of the warp take part.
 template <int LANES>
 __device__ __forceinline__ void tile_scatter_particle(const MapParams& p, int i, bool on, double x, int lane) {
     const unsigned FULL = 0xffffffffu;
