@@ -319,8 +319,7 @@ lbm_status lbm_fp64_fma_rate(int iters, double *tflops_out);
 /* ------------------------------------------------------------------ batches
  * A batch advances many independent contexts (instances: boxes of any size,
  * their own relaxation and particle parameters) in lock step, one CUDA graph
- * per step: each instance's boundary, finalisation and mapping kernels stay
- * per instance (on parallel branches of the graph); the DEM steps of all
+ * per step: each per-step kernel runs once for all instances; the DEM steps of all
  * instances with at most 32 particles run as one launch (a block each), and the
  * dense kernels of all active instances run as ONE persistent launch over a
  * table of work items (instance, tile, chunk of z planes), whose tile width and
