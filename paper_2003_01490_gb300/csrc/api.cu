@@ -211,7 +211,7 @@ void build_layout(const lbm_grid* g, lbm_storage st, int np, Layout& L, const Si
     const size_t n = (size_t)np;
     L.add(19 * N * es);                 // 0 f[0]
     L.add(19 * N * es);                 // 1 f[1]
-    L.add(N + 256);                     // 2 flags (+ padding: the staged dense kernel copies whole 16-byte units)
+    L.add(N + 256);                     // 2 flags (the padding keeps the layout of saved states)
     L.add(4 * N);                       // 3 owner
     L.add(4 * s.ntiles);                // 4 tile_count
     L.add(4 * s.ntiles * TILE_CAP);     // 5 tile_list
@@ -1041,7 +1041,7 @@ lbm_status enqueue_step(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm) {
 }
 
 // Steady-state steps (after the first, profiling off) run as CUDA graphs: the
-// step's ~20 launches are captured once per (PDF buffer, history buffer)
+// step's launches are captured once per (PDF buffer, history buffer)
 // parity on a private stream and replayed on the context stream, which
 // removes the launch overhead that dominates small boxes.
 lbm_status graph_step(lbm_ctx* ctx, DemParams& dp, bool& done) {
