@@ -44,9 +44,10 @@ def test_packed_box_between_walls(n, n_sub, storage, tol):
     check(packed_case(n, n_sub, storage), tol)
 
 
-@pytest.mark.parametrize('n,n_sub', [(512, 10), (513, 7)])
-def test_cluster_and_grid(n, n_sub):
-    check(packed_case(n, n_sub, 'f32'), 1e-4)
+# the float64 one has more missing-link cells than warps that walk them
+@pytest.mark.parametrize('n,n_sub,storage,tol', [(512, 10, 'f32', 1e-4), (513, 7, 'f32', 1e-4), (513, 7, 'f64', 1e-11)])
+def test_cluster_and_grid(n, n_sub, storage, tol):
+    check(packed_case(n, n_sub, storage), tol)
 
 
 def check(case, tol):
