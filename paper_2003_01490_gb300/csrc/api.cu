@@ -321,8 +321,12 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
             ctx->num_sms = sms;
-        cudaError_t pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
-        ctx->cluster_particles = dem_cluster_capacity();
+        // what more particles than one block holds would run in
+        cudaError_t pe = cudaSuccess;
+        if (max_particles > DEM_ONE_BLOCK_MAX) {
+            pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
+            if (st != LBM_STORE_F64) ctx->cluster_particles = dem_cluster_capacity();
+        }
         if (cudaHostAlloc(&ctx->io, sizeof(double) * IO_WORDS, cudaHostAllocPortable) != cudaSuccess) {
             cudaGetLastError();
             ctx->io = nullptr;
