@@ -44,15 +44,6 @@ __device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
 }
-// a product that is rounded before it is added (the packed form is merged with
-// a following addition, which changes the collision's rounding)
-__device__ __forceinline__ F2 mul_rn(F2 a, F2 b) {
-    float a0, a1, b0, b1;
-    split(a, a0, a1);
-    split(b, b0, b1);
-    return f2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
-}
-__device__ __forceinline__ double mul_rn(double a, double b) { return a * b; }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 
 // the cells a thread collides together: V holds ROWS values of type T
@@ -72,6 +63,53 @@ template <> struct Pack<double> {
     __device__ static void get(V v, double (&a)[1]) { a[0] = v; }
 };
 
+// sign of the first non-zero component of c_q
+__host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? cy(q) : cz(q)); }
+
+// Weights w2 = 2 w (even parts), w6 = 6 w (odd parts) per class (axis,
+// diagonal) and w0. In float32 they are chosen within 1.2e-7 of the exact
+// fractions such that w0 + 3 w2_axis + 6 w2_diag = 1 and w6_axis + 4 w6_diag = 1
+// hold exactly: the relaxation towards the equilibrium then keeps the mass and
+// momentum of every cell, where the plain roundings of 1/18, 1/36 and 1/3 would
+// leave a steady source of relative size 3e-8 per step that builds up over a
+// long run.
+template <typename T>
+struct Weights {
+    static constexpr T w2d = sizeof(T) == 4 ? T(0.0555555522441864) : T(1) / T(18);
+    static constexpr T w2a = T(2) * w2d;
+    static constexpr T w0 = T(1) - T(12) * w2d;
+    static constexpr T w6d = T(1) / T(6);
+    static constexpr T w6a = T(1) - T(4) * w6d;
+};
+
+// What the collision reads of the body force a per pair of directions (q, qbar),
+// the same for every cell, once per packed cell: even = 2 lead(q) c_q.a, in
+// float64 times (1 - s_plus / 2) w_q already (a multiply-add less per pair), and
+// odd = (1 - s_minus / 2) (6 w_q / 2) lead(q) c_q.a.
+template <typename T>
+struct __align__(16) ForceTerms {
+    T even[Pack<T>::ROWS], odd[Pack<T>::ROWS];
+};
+template <typename T>
+__device__ __forceinline__ ForceTerms<T> force_terms(int qi, T ax, T ay, T az, T gp, T gm) {
+    const int c0 = (qi & 3) - 1, c1 = ((qi >> 2) & 3) - 1, c2_ = ((qi >> 4) & 3) - 1;
+    const int sg = c0 ? c0 : (c1 ? c1 : c2_);
+    T ca = T(0);
+    if (c0) ca += c0 * sg > 0 ? ax : -ax;
+    if (c1) ca += c1 * sg > 0 ? ay : -ay;
+    if (c2_) ca += c2_ * sg > 0 ? az : -az;
+    const bool axis = c0 * c0 + c1 * c1 + c2_ * c2_ == 1;
+    const T g = T(0.5) * gm * (axis ? Weights<T>::w6a : Weights<T>::w6d);
+    const T e = sizeof(T) == 8 ? T(0.5) * gp * (axis ? Weights<T>::w2a : Weights<T>::w2d) : T(1);
+    ForceTerms<T> t;
+#pragma unroll
+    for (int r = 0; r < Pack<T>::ROWS; ++r) {
+        t.even[r] = e * (ca + ca);
+        t.odd[r] = g * ca;
+    }
+    return t;
+}
+
 template <typename S, typename T>
 struct SCArgs {
     // the arrays of each direction: their addresses come from the argument
@@ -84,7 +122,7 @@ struct SCArgs {
     const uint32_t* __restrict__ shell;
     int words;                       // 32-bit words per row
     T s_plus, s_minus, s_b_shell, s_b_bulk;
-    T ke, ko;                        // weights of the body force in the equilibrium (collide_core)
+    T gp, gm;                        // weights of the body force, 1 - s_plus / 2 and 1 - s_minus / 2
     T uw[2][3][3];                   // wall velocities [side][axis][component]
     int bulk_corr;
     const T* __restrict__ accel;     // [3]
@@ -119,8 +157,8 @@ void fill_sc_args(const LbmStepParams& p, SCArgs<S, T>& a) {
     a.s_minus = (T)p.s_minus;
     a.s_b_shell = (T)p.s_b_shell;
     a.s_b_bulk = (T)p.s_b_bulk;
-    a.ke = (T)((2.0 - p.s_plus) / p.s_plus);
-    a.ko = (T)((1.0 - 0.5 * p.s_minus) / p.s_minus);
+    a.gp = T(1) - T(0.5) * a.s_plus;
+    a.gm = T(1) - T(0.5) * a.s_minus;
     for (int s = 0; s < 2; ++s)
         for (int ax = 0; ax < 3; ++ax)
             for (int c = 0; c < 3; ++c) a.uw[s][ax][c] = (T)p.g.wall_vel[s][ax][c];
@@ -153,6 +191,7 @@ struct DirTable {
     const S* src[Q];
     int qi[Q];
     int dq[Q];   // cell index offset of c_q
+    ForceTerms<typename Store<S>::T> force[Q];   // of the body force, for the first of each pair of directions
 };
 
 // One particle link: cell (x, y, z) pulls direction q (velocity c) from a solid
@@ -241,11 +280,8 @@ __device__ __forceinline__ float link_value(const SCArgs<S, float>& a, int, cons
     return val;
 }
 
-// sign of the first non-zero component of c_q
-__host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? cy(q) : cz(q)); }
-
 // TRT+aB collision of the cells packed in f, in place, with the body force
-// (ax, ay, az); shell[r]: cell r lies in the shell. Returns the density
+// a = (ax, ay, az); shell[r]: cell r lies in the shell. Returns the density
 // deviations. The arithmetic is that of the moment-space update with S of
 // Eq. (12) written per pair of opposite directions (q, qbar): with
 // s = f_q + f_qbar and d = f_q - f_qbar the even part relaxes with s_nu and
@@ -254,19 +290,21 @@ __host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? 
 //   dm = -s_nu^- (d/2 - 3 w c.u) + (1 - s_nu^-/2) 3 w c.a, Y = -3 u.a + 9 (c.u)(c.a)
 //   f_q += dp + dm,  f_qbar += dp - dm,
 // the Guo source in Y and 3 w c.a; corr is the rank-2 bulk correction of the
-// shell cells. The source is taken into the equilibrium's velocities:
-//   s_nu X + (1 - s_nu/2) 2 Y / 2 = s_nu [drho - 3/2 u^2 - 3/2 k u.a + 9/2 (c.u)(c.v)],  v = u + k a, k = (2 - s_nu)/s_nu
-//   s_nu^- 3 c.u + (1 - s_nu^-/2) 3 c.a = s_nu^- 3 c.t,                                  t = u + (k^-/2) a, k^- = (2 - s_nu^-)/s_nu^-
-// (ke = k, ko = k^-/2)
-// so a pair costs the same few multiply-adds with and without a body force; FORCE =
-// false is the form for a = 0 (the same values), which leaves out the sums with a.
+// shell cells. Each pair costs one chain of fused multiply-adds. The source
+// is added at the size of the pair's correction: taken into the equilibrium's
+// velocities (u + k a in place of u) a body force some hundred times smaller
+// than u is rounded to the last bit of u in every step, which made the float32
+// velocities 1.3 to 1.9 times less exact over 50 steps. FORCE = false is the
+// form for a = 0 (the same values), which leaves out the sums with a; force: the
+// parts of the source that are the same for every cell (force_terms).
 template <typename T, bool FORCE>
 __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V (&f)[Q],
-                                                            const bool (&shell)[Pack<T>::ROWS], T ax, T ay, T az, T sp,
-                                                            T sm, T ke, T ko, T s_b_shell, T s_b_bulk,
-                                                            int bulk_corr) {
+                                                            const bool (&shell)[Pack<T>::ROWS], T ax, T ay, T az,
+                                                            const ForceTerms<T>* force, T sp, T sm, T gp, T s_b_shell,
+                                                            T s_b_bulk, int bulk_corr) {
     using P = Pack<T>;
     using V = typename P::V;
+    using K = Weights<T>;
     // pair sums and differences are formed twice (here and in the update):
     // keeping them takes 36 registers more than the cell's PDFs
     V drho = f[0], jx = P::all(T(0)), jy = jx, jz = jx;
@@ -284,11 +322,10 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
     const V ux = FORCE ? jx + P::all(T(0.5) * ax) : jx, uy = FORCE ? jy + P::all(T(0.5) * ay) : jy,
             uz = FORCE ? jz + P::all(T(0.5) * az) : jz;
     const V usq = mad(uz, uz, mad(ux, ux, uy * uy));
-    V ua = P::all(T(0)), vx = ux, vy = uy, vz = uz, tx = ux, ty = uy, tz = uz;
+    V ua = P::all(T(0)), m3ua = ua;
     if constexpr (FORCE) {
-        ua = mad(ux, P::all(ax), mad(uy, P::all(ay), uz * P::all(az)));
-        vx = ux + P::all(ke * ax); vy = uy + P::all(ke * ay); vz = uz + P::all(ke * az);
-        tx = ux + P::all(ko * ax); ty = uy + P::all(ko * ay); tz = uz + P::all(ko * az);
+        ua = mad(uz, P::all(az), mad(ux, P::all(ax), uy * P::all(ay)));
+        m3ua = P::all(T(-3)) * ua;
     }
     // bulk moments m4 = sum (c^2 - 1) f and m5 (row 6 of M) of the streamed
     // PDFs relax with s_b in shell cells (and everywhere when Lambda_b,bulk != 1)
@@ -313,23 +350,18 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         k4 = P::all(T(1.5)) * (ds * (FORCE ? (usq - m4) - ua : usq - m4));
         k5 = P::all(T(-0.5)) * (ds * m5);
     }
-    // equilibrium part common to all directions, with the u.a term of the source
-    const V X0 = mad(P::all(T(-1.5)), FORCE ? mad(P::all(ke), ua, usq) : usq, drho);
-    // Weights of the update: w2 = 2 w (even parts), w6 = 6 w (odd parts) per
-    // class (axis, diagonal) and w0. In float32 they are chosen within 1.2e-7
-    // of the exact fractions such that w0 + 3 w2_axis + 6 w2_diag = 1 and
-    // w6_axis + 4 w6_diag = 1 hold exactly: the relaxation towards the
-    // equilibrium then keeps the mass and momentum of every cell, where the
-    // plain roundings of 1/18, 1/36 and 1/3 would leave a steady source of
-    // relative size 3e-8 per step that builds up over a long run.
-    const T w2d = sizeof(T) == 4 ? T(0.0555555522441864) : T(1) / T(18);
-    const T w2a = T(2) * w2d;
-    const T w0 = T(1) - T(12) * w2d;
-    const T w6d = T(1) / T(6);
-    const T w6a = T(1) - T(4) * w6d;
-    const V mw2[2] = {P::all(-w2a), P::all(-w2d)}, mw6[2] = {P::all(-w6a), P::all(-w6d)};
-    const V corr[2] = {mw2[0] * k5, P::all(T(0.5) * w2d) * (k4 + k5)};
-    f[0] = mad(P::all(w0), k5 - k4, mad(P::all(sp), mad(P::all(w0), X0, P::all(T(0)) - f[0]), f[0]));
+    // equilibrium part common to all directions
+    const V drp = mad(P::all(T(-1.5)), usq, drho);
+    const V mw2[2] = {P::all(-K::w2a), P::all(-K::w2d)}, mw6[2] = {P::all(-K::w6a), P::all(-K::w6d)};
+    const V gpw[2] = {P::all(T(0.5) * gp * K::w2a), P::all(T(0.5) * gp * K::w2d)};
+    V corr[2] = {mw2[0] * k5, P::all(T(0.5) * K::w2d) * (k4 + k5)};
+    if constexpr (FORCE && sizeof(T) == 8) {
+        corr[0] = mad(gpw[0], m3ua, corr[0]);
+        corr[1] = mad(gpw[1], m3ua, corr[1]);
+    }
+    V f0 = mad(P::all(sp), mad(P::all(K::w0), drp, P::all(T(0)) - f[0]), f[0]);
+    if constexpr (FORCE) f0 = mad(P::all(gp), P::all(K::w0) * m3ua, f0);
+    f[0] = mad(P::all(K::w0), k5 - k4, f0);
     const V hsp = P::all(T(-0.5) * sp), hsm = P::all(T(-0.5) * sm), c45 = P::all(T(4.5));
     // each part relaxes as rate x (value - its equilibrium). The pair sums and
     // differences as (exact) multiply-adds, which the compiler does not merge
@@ -341,23 +373,23 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         if (qb < q) continue;
         const int k = c2(q) == 1 ? 0 : 1;
         const int sg = lead(q);
-        // c.u, c.v, c.t times lead(q), which their product and e share
-        const bool y_plus = cy(q) * sg > 0, z_plus = cz(q) * sg > 0;
-        V cu = cx(q) ? ux : (cy(q) ? uy : uz), cv = cx(q) ? vx : (cy(q) ? vy : vz), ct = cx(q) ? tx : (cy(q) ? ty : tz);
-        if (cx(q) && cy(q)) {
-            cu = y_plus ? cu + uy : cu - uy;
-            cv = FORCE ? (y_plus ? cv + vy : cv - vy) : cu;
-            ct = FORCE ? (y_plus ? ct + ty : ct - ty) : cu;
+        // c.u times lead(q), which its products with itself, c.a and the odd part share
+        V cu = cx(q) ? ux : (cy(q) ? uy : uz);
+        if (cx(q) && cy(q)) cu = cy(q) * sg > 0 ? cu + uy : cu - uy;
+        if ((cx(q) || cy(q)) && cz(q)) cu = cz(q) * sg > 0 ? cu + uz : cu - uz;
+        const V cu45 = c45 * cu;
+        const V X = mad(cu45, cu, drp);
+        // the zero is read from memory: the compiler merges a packed product with the
+        // sum that follows, which rounds once less than with a body force
+        V src = corr[k], odd = P::all(ax);
+        if constexpr (FORCE) {
+            const V even = P::make(force[q].even);
+            src = sizeof(T) == 8 ? mad(cu45, even, corr[k]) : mad(gpw[k], mad(cu45, even, m3ua), corr[k]);
+            odd = P::make(force[q].odd);
         }
-        if ((cx(q) || cy(q)) && cz(q)) {
-            cu = z_plus ? cu + uz : cu - uz;
-            cv = FORCE ? (z_plus ? cv + vz : cv - vz) : cu;
-            ct = FORCE ? (z_plus ? ct + tz : ct - tz) : cu;
-        }
-        const V X = mad(c45 * cu, cv, X0);
-        const V dp = mad(hsp, mad(mw2[k], X, mad(one, f[q], f[qb])), corr[k]);
+        const V dp = mad(hsp, mad(mw2[k], X, mad(one, f[q], f[qb])), src);
         // lead(q) dm
-        const V dm = mul_rn(hsm, mad(mw6[k], ct, sg > 0 ? mad(mone, f[qb], f[q]) : mad(mone, f[q], f[qb])));
+        const V dm = mad(hsm, mad(mw6[k], cu, sg > 0 ? mad(mone, f[qb], f[q]) : mad(mone, f[q], f[qb])), odd);
         f[q] = f[q] + (sg > 0 ? dp + dm : dp - dm);
         f[qb] = f[qb] + (sg > 0 ? dp - dm : dp + dm);
     }
