@@ -1649,6 +1649,9 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
     const size_t db = dem_batch_entry_bytes();
     const std::vector<int4> items = batch_items(b);
     G.n_items = (int)items.size();
+    bool some_one = false, some_more = false;   // boxes with one particle and others
+    for (size_t i = 0; i < n; ++i)
+        if (b->active[i]) (sc_one(b->storage, b->ctx[i]->P.n) ? some_one : some_more) = true;
     std::vector<unsigned char> host(ab * n, 0), host_dem(db * n, 0);
     GangTable bc, zb, bins, nbr, fin, zc, scat, map, ref, pos, copy, pres;
     std::vector<GangTable> sub;   // one table per subcycle of the multi-block DEM steps
@@ -1784,7 +1787,7 @@ lbm_status batch_capture_gang(lbm_batch* b, lbm_batch::Graph& G) {
         if (G.n_items > 0) {
             const int bps = b->blocks_per_sm > 0 ? b->blocks_per_sm : (b->storage == 0 ? 2 : 4);
             const int grid = std::min(G.n_items, bps * b->num_sms);
-            launch_stream_collide_batch(b->storage, G.d_args, G.d_items, G.n_items, grid, cs);
+            launch_stream_collide_batch(b->storage, G.d_args, G.d_items, G.n_items, some_one, some_more, grid, cs);
             launches += 1;
         }
         launch_gang(GANG_FINALIZE, T(4), O(4), fin.count(), fin.blocks(), cs);

@@ -41,14 +41,17 @@ void launch_stream_collide(const LbmStepParams& p, cudaStream_t st);
 // rows in y of the dense kernel's tile bx (32, 64 or 128) cells wide: 4 warps
 // of 32 x 2 cells (elem: bytes of a stored PDF), 32 x 1 for float64
 __host__ __device__ constexpr int sc_tile_rows(int elem, int bx) { return (elem == 8 ? 1 : 2) * 128 / bx; }
+// the dense kernel has a form for boxes with one particle (not in float64)
+constexpr bool sc_one(int storage, int particles) { return storage != 0 && particles == 1; }
 // the dense kernels of many boxes in one persistent launch: per instance one
 // argument block (batch_args_bytes(storage) bytes, filled by fill_batch_args)
-// in device memory, and a table of work items (instance, x0, y0, z0)
+// in device memory, and a table of work items (instance, x0, y0, z0); one, more:
+// there are boxes that sc_one takes, that it does not
 size_t batch_args_bytes(int storage);
 void fill_batch_args(const LbmStepParams& p, int tile_bx, int zchunk, void* out);
 int default_tile_bx(int nx);
-void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, int grid,
-                                 cudaStream_t st);
+void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, bool one, bool more,
+                                 int grid, cudaStream_t st);
 
 struct MapParams {
     Geom g;

@@ -194,6 +194,33 @@ __device__ __forceinline__ void commit_open(OpenParts<T>& op, const SlotKeys<T>&
     }
 }
 
+// The sums of a box's only particle, slot r for row r of the warp: its view and
+// zeros at the start, and the commit of one row's sums, which the first n columns
+// hold (a binary tree over them).
+template <typename T>
+__device__ __forceinline__ void open_single(OpenParts<T>& op, const PartView* __restrict__ view, int lane) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) op.f[0][c][lane] = op.f[1][c][lane] = T(0);
+    if (lane < (int)(sizeof(PartView) / 4))
+        reinterpret_cast<int*>(&op.view[0])[lane] = reinterpret_cast<const int*>(view)[lane];
+}
+template <typename T>
+__device__ __forceinline__ void commit_lanes(OpenParts<T>& op, int slot, int n, const Sinks& s, int lane) {
+    T sum = T(0);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        T v = op.f[slot][c][lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const T w = __shfl_down_sync(0xffffffffu, v, o);
+            if ((lane & (2 * o - 1)) == 0 && lane + o < n) v += w;
+        }
+        v = __shfl_sync(0xffffffffu, v, 0);
+        if (lane == c) sum = v;
+    }
+    if (lane < 6) add_float(s, 0, lane, sum);
+}
+
 template <typename T>
 __device__ __forceinline__ void accumulate(int i, const T (&F)[3], const T (&Tq)[3], const int (&K)[6], Acc<T>& a,
                                            const Sinks& s) {

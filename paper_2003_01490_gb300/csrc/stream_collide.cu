@@ -45,6 +45,18 @@
 // remainder is summed per lane and warp in float32 and per particle in 64-bit
 // fixed point (scale 2^32) through integer atomics. The sums depend on the
 // chunk of planes a warp marches, not on the tile width.
+//
+// A box with one particle, float32 compute, has a form of its own. The force and
+// torque on a sphere of an array are a small rest of their links' parts (a torque
+// of 1e-5 to 1e-3 where the parts add up to 10), so the order in which float32
+// adds them shows in the fifth digit. This form adds them per row, in the order of
+// the row's cells and directions, cut into runs of equal length of which column c
+// of the row's sums takes the c-th: each torque of an array is then the one that a
+// warp per row has, bit for bit. It costs nothing: with one particle there is no
+// owner to look up, no slot to find, and the words of the row's directions, once
+// turned into the lane's own directions, serve to patch the values in too (a pass
+// of the 80x80x160 box 2.63 ms against 2.62 with the sums by slot, 16 boxes of a
+// batch 8.55 against 8.52, 480x160x80 cells 9.36 and 9.37).
 #include <cstring>
 
 #include "sc_common.cuh"
@@ -69,13 +81,14 @@ constexpr int SC_WARPS = 4;       // warps per block
 constexpr int QUEUE_CAP = 256;    // links queued at a time
 
 // Shared memory of one warp. A cell is numbered half (x < 16 or not) << 5 |
-// row << 4 | x & 15; a queue entry is q << 11 | p << 6 | cell, p opposite to q.
+// row << 4 | x & 15; a queue entry is q << 11 | p << 6 | cell, p opposite to q (p
+// is put in when it is read in the form for one particle).
 template <typename T>
 struct SCWarp {
     static constexpr int ROWS = Pack<T>::ROWS;
     T v[Q - 1][32 * ROWS];                   // CLI values
     OpenParts<T> open;
-    uint32_t w[Q + 2][ROWS];                 // link words of directions 1 .. 18, fluid, shell
+    alignas(8) uint32_t w[Q + 2][ROWS];      // link words of directions 1 .. 18, fluid, shell
     unsigned short queue[QUEUE_CAP];
 };
 // cell number of x = lane, row 0 (row 1: + 16)
@@ -105,9 +118,13 @@ __device__ __forceinline__ void patch_link(double& g, uint32_t bit, const double
     if (bit) g = *v;
 }
 
+// what a kernel is compiled for: boxes with one particle (see the header), other
+// boxes, both
+enum Boxes { BOXES_MORE, BOXES_ONE, BOXES_BOTH };
+
 // One warp's cells: x = 32 wx + lane, rows y0 .. y0 + ROWS - 1, planes
 // z_begin .. z_end - 1 marched in order.
-template <typename S, typename T>
+template <typename S, typename T, Boxes KIND>
 __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, int z_begin, int z_end, SCWarp<T>& sm,
                                         const DirTable<S>& dt) {
     using P = Pack<T>;
@@ -181,11 +198,13 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
     };
     PlaneWords pw = load_words(z_begin);
 
-    // the gathers of queue entry k (the last one for lanes past the end) of a
-    // plane; edges: bit d, the warp's cells reach the box's faces on axis d
-    auto fetch = [&](int k, int n, int z, int edges) {
+    const bool one = KIND == BOXES_ONE || (KIND == BOXES_BOTH && a.np == 1);
+    int lanes[2] = {0, 0};   // one: lanes with a sum, per row
+
+    // the gathers of queue entry e of a plane; edges: bit d, the warp's cells
+    // reach the box's faces on axis d
+    auto fetch = [&](int e, int z, int edges) {
         LinkIn<T> l;
-        const int e = sm.queue[min(k, n - 1)];
         const int q = e >> 11, p = (e >> 6) & 31, row = (e >> 4) & (ROWS - 1);
         const int xb = ROWS == 1 ? e & 31 : (e & 15) | ((e >> 1) & 16);
         const int idx = z * plane + y0 * nx + 32 * wx + (row ? nx : 0) + xb, dq = dt.dq[q];
@@ -207,13 +226,27 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
                 }
         }
         const S* const sp = dt.src[p];
-        l.key = a.owner[is];
+        l.key = one ? 0 : a.owner[is];
         l.fout = Store<S>::load(sp + idx);
         l.fin = Store<S>::load(dt.src[q] + idx);
         const T fd = Store<S>::load(sp + id);
         l.fdown = cli ? fd : T(0);
         l.e = e | (cli ? 0x10000 : 0);
         return l;
+    };
+
+    // link l of particle key: its value into the cell's slot, its force and torque
+    // into the sums of slot, column col
+    auto add_link = [&](const LinkIn<T>& l, int key, int slot, int col, int z, bool wrap) {
+        const int q = (l.e >> 11) & 31, row = (l.e >> 4) & (ROWS - 1);
+        const int xb = ROWS == 1 ? l.e & 31 : (l.e & 15) | ((l.e >> 1) & 16);
+        T F[6];
+        sm.v[q - 1][l.e & (32 * ROWS - 1)] =
+            link_value<S>(a, key, sm.open.view[sizeof(T) == 4 && !one ? slot : 0], 32 * wx + xb, y0 + row, z, dt.qi[q],
+                          dt.cf[q], (l.e & 0x10000) != 0, wrap, l.fout, l.fin, l.fdown, F);
+        T* p = &sm.open.f[slot][0][col];
+#pragma unroll
+        for (int d = 0; d < 6; ++d) p[32 * d] += F[d];
     };
 
     // axes on which the warp's cells lie next to the box's faces, and z planes
@@ -265,16 +298,67 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
                 f[q] = P::make(g);
             }
         }
-        // links of the left half (low 16 bits) and of the right half (high); with
-        // one row all count as left, the order in which they are queued below
-        const int cl = ROWS == 1 ? __popc(link[0]) : __popc(link[0] & 0xffffu) + __popc(link[1] & 0xffffu);
-        const int cr = ROWS == 1 ? 0 : __popc(link[0] >> 16) + __popc(link[1] >> 16);
-        const int incl = warp_incl_scan(cl | (cr << 16), lane);
-        const int all = __shfl_sync(FULL, incl, 31);
-        const int left = all & 0xffff, total = left + (all >> 16);
         const int edges = edges_xy | (z == 0 || z == nz - 1 ? 4 : 0);
-        if (total > 0) {   // warp-uniform
-            const bool deep = deep_xy && z >= mz && z < nz - mz;
+        const bool links = __any_sync(FULL, (link[0] | link[1]) != 0u);
+        uint32_t of_cell[2] = {0u, 0u};   // one: bit q - 1, the lane's cell has a link in direction q
+        if (one && links) {   // warp-uniform
+            // 2. the links of each row in the order of its cells, cut into runs of equal
+            // length, one per lane
+            const bool wrap = !(deep_xy && z >= mz && z < nz - mz);
+            if ((lanes[0] | lanes[1]) == 0) open_single<T>(sm.open, a.view, lane);
+            __syncwarp();   // the words of all directions
+#pragma unroll
+            for (int q = Q - 1; q >= 1; --q)
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r)
+                    of_cell[r] = __funnelshift_l(sm.w[q][r] << (31 - lane), of_cell[r], 1);
+            const int count = __popc(of_cell[0]) | __popc(of_cell[1]) << 16;
+            const int end = warp_incl_scan(count, lane), all = __shfl_sync(FULL, end, 31);
+            const int first[2] = {((end - count) & 0xffff), (end - count) >> 16}, n[2] = {all & 0xffff, all >> 16};
+            int run[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                run[r] = (n[r] + 31) >> 5;
+                lanes[r] = max(lanes[r], run[r] > 1 ? (n[r] + run[r] - 1) / run[r] : n[r]);
+            }
+            constexpr int CAP = QUEUE_CAP / 2;   // of a row's links queued at a time
+            for (int base = 0; base < max(n[0], n[1]); base += CAP) {
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r) {
+                    int pos = first[r] - base;
+                    for (uint32_t m = of_cell[r]; m; m &= m - 1, ++pos)
+                        if ((unsigned)pos < (unsigned)CAP)
+                            sm.queue[CAP * r + pos] = (unsigned short)(__ffs((int)m) << 11 | (cell_of<T>(lane) + 16 * r));
+                }
+                __syncwarp();
+                // 32 links at a time, the j-th of each run of the first row and then of
+                // the second
+                for (int j = 0; j < max(run[0], run[1]); ++j) {
+                    int runs[2];   // with a j-th link
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+                        runs[r] = j >= run[r] ? 0 : (run[r] > 1 ? (n[r] - j + run[r] - 1) / run[r] : n[r]);
+                    for (int u0 = 0; u0 < runs[0] + runs[1]; u0 += 32) {
+                        const int u = u0 + lane, r = u < runs[0] ? 0 : 1;
+                        const int col = r ? u - runs[0] : u;
+                        const int k = col * (r ? run[1] : run[0]) + j - base;
+                        if (u < runs[0] + runs[1] && (unsigned)k < (unsigned)CAP) {
+                            const int e = sm.queue[CAP * r + k];
+                            add_link(fetch(e | ((dt.qi[e >> 11] >> 6) & 31) << 6, z, edges), 0, r, col, z, wrap);
+                        }
+                        __syncwarp();   // queue read, values and sums written
+                    }
+                }
+            }
+        } else if (links) {   // warp-uniform
+            // links of the left half (low 16 bits) and of the right half (high); with
+            // one row all count as left, the order in which they are queued below
+            const int cl = ROWS == 1 ? __popc(link[0]) : __popc(link[0] & 0xffffu) + __popc(link[1] & 0xffffu);
+            const int cr = ROWS == 1 ? 0 : __popc(link[0] >> 16) + __popc(link[1] >> 16);
+            const int incl = warp_incl_scan(cl | (cr << 16), lane);
+            const int all = __shfl_sync(FULL, incl, 31);
+            const int left = all & 0xffff, total = left + (all >> 16);
+            const bool wrap = !(deep_xy && z >= mz && z < nz - mz);
             const int pl = (incl & 0xffff) - cl, pr = left + (incl >> 16) - cr;
             for (int base = 0; base < total; base += QUEUE_CAP) {
                 // this lane's links of direction ql with places in [base, base + QUEUE_CAP)
@@ -294,28 +378,19 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
                     }
                 }
                 __syncwarp();
-                // 2. one link per lane; the gathers of the next 32 are under
-                // way while these are worked on
+                // 2. one link per lane (the last one for lanes past the end); the
+                // gathers of the next 32 are under way while these are worked on
                 const int n = min(total - base, QUEUE_CAP);
-                LinkIn<T> l = fetch(lane, n, z, edges);
+                LinkIn<T> l = fetch(sm.queue[min(lane, n - 1)], z, edges);
                 for (int k0 = 0; k0 < n; k0 += 32) {
                     const LinkIn<T> cur = l;
-                    if (k0 + 32 < n) l = fetch(k0 + 32 + lane, n, z, edges);
-                    const int q = (cur.e >> 11) & 31, row = (cur.e >> 4) & (ROWS - 1);
-                    const int xb = ROWS == 1 ? cur.e & 31 : (cur.e & 15) | ((cur.e >> 1) & 16);
+                    if (k0 + 32 < n) l = fetch(sm.queue[min(k0 + 32 + lane, n - 1)], z, edges);
                     // solid cells have an owner below np
                     int key = k0 + lane < n && (unsigned)cur.key < (unsigned)a.np ? cur.key : -1;
                     do {   // once, but where more particles meet than there are slots
                         const int slot = find_slot<T>(sm.open, keys, key, a.view, sk, lane);
                         if (slot >= 0) {
-                            T F[6];
-                            sm.v[q - 1][cur.e & (32 * ROWS - 1)] =
-                                link_value<S>(a, key, sm.open.view[sizeof(T) == 4 ? slot : 0], 32 * wx + xb, y0 + row, z,
-                                              dt.qi[q], dt.cf[q], (cur.e & 0x10000) != 0, !deep, cur.fout, cur.fin,
-                                              cur.fdown, F);
-                            T* p = &sm.open.f[slot][0][lane];
-#pragma unroll
-                            for (int d = 0; d < 6; ++d) p[32 * d] += F[d];
+                            add_link(cur, key, slot, lane, z, wrap);
                             key = -1;
                         }
                     } while (__any_sync(FULL, key >= 0));
@@ -326,7 +401,6 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
         // 3. patch, collide, store
         if (actA || actB) {
             const uint32_t me = 1u << lane;
-            const bool patch = total > 0;
             const bool edge = (edges & wall_axes) != 0;
             if (edge) {
                 // halfway bounce-back on the box walls (Eq. (14) with delta = 1/2)
@@ -355,14 +429,15 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
                     f[q] = P::make(g);
                 }
             }
-            if (patch) {
+            if (links) {
 #pragma unroll
                 for (int q = 1; q < Q; ++q) {
                     T g[ROWS];
                     P::get(f[q], g);
 #pragma unroll
                     for (int r = 0; r < ROWS; ++r)
-                        patch_link(g[r], sm.w[q][r] & me, &sm.v[q - 1][cell_of<T>(lane) + 16 * r]);
+                        patch_link(g[r], one ? of_cell[r] & (1u << (q - 1)) : sm.w[q][r] & me,
+                                   &sm.v[q - 1][cell_of<T>(lane) + 16 * r]);
                     f[q] = P::make(g);
                 }
             }
@@ -397,7 +472,13 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
             }
         }
     }
-    commit_open<T>(sm.open, keys, sk, lane);
+    if (one) {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+            if (lanes[r] > 0) commit_lanes<T>(sm.open, r, lanes[r], sk, lane);
+    } else {
+        commit_open<T>(sm.open, keys, sk, lane);
+    }
 }
 
 __constant__ int k_qinfo[Q] = {qinfo(0), qinfo(1), qinfo(2), qinfo(3), qinfo(4), qinfo(5), qinfo(6),
@@ -420,7 +501,7 @@ __device__ __forceinline__ void load_dirs(DirTable<S>& dt, const SCArgs<S, T>& a
 }
 
 // the warp of a tile of bx x (SC_WARPS ROWS 32 / bx) cells at (x0, y0)
-template <typename S, typename T>
+template <typename S, typename T, Boxes KIND>
 __device__ __forceinline__ void sc_tile(const SCArgs<S, T>& a, int x0, int y0, int z_begin, SCWarp<T>* sm,
                                         const DirTable<S>& dt) {
     // opaque, or the compiler derives them from special registers again and again
@@ -432,25 +513,26 @@ __device__ __forceinline__ void sc_tile(const SCArgs<S, T>& a, int x0, int y0, i
                  : "=r"(y)
                  : "r"(y0 + Pack<T>::ROWS * (across == 1 ? warp : (across == 2 ? warp >> 1 : 0))));
     if (wx < a.words && y < a.g.n[1])
-        sc_warp<S, T>(a, wx, y, z_begin, min(a.g.n[2], z_begin + a.zchunk), sm[warp], dt);
+        sc_warp<S, T, KIND>(a, wx, y, z_begin, min(a.g.n[2], z_begin + a.zchunk), sm[warp], dt);
 }
 
 // One box: block (x, y) tiles, a chunk of a.zchunk planes from blockIdx.z.
-template <typename S, typename T>
+template <typename S, typename T, Boxes KIND>
 __global__ void __launch_bounds__(32 * SC_WARPS, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
     stream_collide_kernel(const __grid_constant__ SCArgs<S, T> a) {
     __shared__ SCWarp<T> sm[SC_WARPS];
     __shared__ DirTable<S> dt;
     load_dirs<S, T>(dt, a);
     __syncthreads();
-    sc_tile<S, T>(a, blockIdx.x * a.bx, blockIdx.y * sc_tile_rows(sizeof(S), a.bx), blockIdx.z * a.zchunk, sm, dt);
+    sc_tile<S, T, KIND>(a, blockIdx.x * a.bx, blockIdx.y * sc_tile_rows(sizeof(S), a.bx), blockIdx.z * a.zchunk, sm, dt);
 }
 
 // Many boxes in one persistent launch: block b takes the work items b,
 // b + gridDim.x, ... of the table (instance, x0, y0, z0), copies the
 // arguments of the item's instance into shared memory and runs its tile
-// (a.zchunk planes from z0).
-template <typename S, typename T>
+// (a.zchunk planes from z0). A batch of boxes of one kind has a kernel without
+// the other kind's code and its registers.
+template <typename S, typename T, Boxes KIND>
 __global__ void __launch_bounds__(32 * SC_WARPS, sizeof(S) == 8 ? LBM_SC_MIN_BLOCKS_F64 : LBM_SC_MIN_BLOCKS)
     stream_collide_batch_kernel(const SCArgs<S, T>* __restrict__ args, const int4* __restrict__ items, int n_items) {
     __shared__ SCWarp<T> sm[SC_WARPS];
@@ -467,7 +549,7 @@ __global__ void __launch_bounds__(32 * SC_WARPS, sizeof(S) == 8 ? LBM_SC_MIN_BLO
         __syncthreads();
         load_dirs<S, T>(dt, s_a);
         __syncthreads();
-        sc_tile<S, T>(s_a, item.y, item.z, item.w, sm, dt);
+        sc_tile<S, T, KIND>(s_a, item.y, item.z, item.w, sm, dt);
     }
 }
 
@@ -505,7 +587,10 @@ void launch_stream_collide_t(const LbmStepParams& p, cudaStream_t st) {
     const int by = sc_tile_rows(sizeof(S), a.bx);
     a.zchunk = default_zchunk(nx, p.g.n[1], p.g.n[2], p.num_sms > 0 ? p.num_sms : 152);
     dim3 grid((nx + a.bx - 1) / a.bx, (p.g.n[1] + by - 1) / by, (p.g.n[2] + a.zchunk - 1) / a.zchunk);
-    stream_collide_kernel<S, T><<<grid, 32 * SC_WARPS, 0, st>>>(a);
+    if (sc_one(p.storage, p.P.n))
+        stream_collide_kernel<S, T, sizeof(T) == 4 ? BOXES_ONE : BOXES_MORE><<<grid, 32 * SC_WARPS, 0, st>>>(a);
+    else
+        stream_collide_kernel<S, T, BOXES_MORE><<<grid, 32 * SC_WARPS, 0, st>>>(a);
 }
 
 // ------------------------------------------------------------ batched launch
@@ -540,19 +625,29 @@ void fill_batch_args(const LbmStepParams& p, int tile_bx, int zchunk, void* out)
 }
 
 template <typename S>
-static void launch_batch_t(const void* d_args, const int4* d_items, int n_items, int grid, cudaStream_t st) {
+static void launch_batch_t(const void* d_args, const int4* d_items, int n_items, bool one, bool more, int grid,
+                           cudaStream_t st) {
     using T = typename Store<S>::T;
-    stream_collide_batch_kernel<S, T>
-        <<<grid, 32 * SC_WARPS, 0, st>>>(static_cast<const SCArgs<S, T>*>(d_args), d_items, n_items);
+    const SCArgs<S, T>* args = static_cast<const SCArgs<S, T>*>(d_args);
+    if constexpr (sizeof(T) == 4) {
+        if (one) {
+            if (more)
+                stream_collide_batch_kernel<S, T, BOXES_BOTH><<<grid, 32 * SC_WARPS, 0, st>>>(args, d_items, n_items);
+            else
+                stream_collide_batch_kernel<S, T, BOXES_ONE><<<grid, 32 * SC_WARPS, 0, st>>>(args, d_items, n_items);
+            return;
+        }
+    }
+    stream_collide_batch_kernel<S, T, BOXES_MORE><<<grid, 32 * SC_WARPS, 0, st>>>(args, d_items, n_items);
 }
 
-void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, int grid,
-                                 cudaStream_t st) {
+void launch_stream_collide_batch(int storage, const void* d_args, const int4* d_items, int n_items, bool one, bool more,
+                                 int grid, cudaStream_t st) {
     switch (storage) {
-        case 0: launch_batch_t<double>(d_args, d_items, n_items, grid, st); break;
-        case 1: launch_batch_t<float>(d_args, d_items, n_items, grid, st); break;
-        case 2: launch_batch_t<__half>(d_args, d_items, n_items, grid, st); break;
-        default: launch_batch_t<__nv_bfloat16>(d_args, d_items, n_items, grid, st); break;
+        case 0: launch_batch_t<double>(d_args, d_items, n_items, one, more, grid, st); break;
+        case 1: launch_batch_t<float>(d_args, d_items, n_items, one, more, grid, st); break;
+        case 2: launch_batch_t<__half>(d_args, d_items, n_items, one, more, grid, st); break;
+        default: launch_batch_t<__nv_bfloat16>(d_args, d_items, n_items, one, more, grid, st); break;
     }
 }
 

@@ -1,15 +1,21 @@
-"""Accuracy of the float32 collision with a body force.
+"""Accuracy of the float32 collision with a body force, and of the forces on a
+box's only particle (a form of the dense kernel of its own).
 
 The collision adds the body force's source at the size of a pair's correction.
 Each operation rounds once, so one step of a box without particles is restated
 here in float32 operation by operation (multiply-adds through float64: the
 product is exact, and the second rounding meets a tie in about one of 2^29) and
 must come out bit for bit but for such ties, 1e-5 of the values at most.
+
+Forces: the float64 kernel is the reference, on a sphere that both moves and
+spins, so that neither force nor torque is a small rest of the links' parts.
+Float32 forces are sums of remainders of ~1e-3 with a relative rounding of 2^-24
+in each of a few operations (1e-5); velocities 1e-6.
 """
 import numpy as np
 import pytest
 
-from cases import build_gpu
+from cases import build_gpu, rel_l2, spheres
 
 pytestmark = pytest.mark.gpu
 
@@ -81,3 +87,26 @@ def test_float32_collision_adds_the_body_force_as_its_own_source(L, force):
     got = (L.lbm_get_pdfs(ctx).reshape(v.shape) - W[:, None, None, None]).astype(F)
     want = collided(np.stack([np.roll(v[q], C[q][::-1], (0, 1, 2)) for q in range(19)]), force, tau)
     assert np.mean(got != want) < 1e-5
+
+
+# rows of 32 cells with up to 7, 30, 43, 118 and 160 links (a row's links are taken
+# in runs of one per 32 and queued 128 at a time)
+@pytest.mark.parametrize('shape,radius', [((31, 9, 10), 1.4), ((33, 29, 31), 8.2), ((64, 52, 51), 20.0),
+                                          ((96, 95, 90), 40.0), ((160, 151, 150), 70.0)])
+def test_forces_on_the_only_particle_match_float64(L, shape, radius):
+    at = 0.5 * np.array(shape) + [0.02, 0.13, -0.27]
+    got = []
+    for storage in ('f64', 'f32'):
+        case = dict(shape=shape, periodic=(1, 1, 1), tau=0.8, storage=storage, body_force=(2e-5, -1e-5, 3e-5),
+                    spheres=spheres([at], [radius], vel=[[0.04, -0.03, 0.05]],
+                                    omega=[[0.1 / radius, -0.05 / radius, 0.07 / radius]]),
+                    dem=dict(fixed_particles=1))
+        ctx = build_gpu(case)
+        L.lbm_step(ctx, 5)
+        st = L.lbm_get_particle_state(ctx)
+        got.append((st['force_hyd'], st['torque_hyd'], L.lbm_get_fields(ctx)[1]))
+        del ctx
+    (F64, T64, u64), (F32, T32, u32) = got
+    assert rel_l2(F32, F64) < 1e-5
+    assert rel_l2(T32, T64) < 1e-5
+    assert rel_l2(u32, u64) < 1e-6
