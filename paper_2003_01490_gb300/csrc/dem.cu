@@ -818,6 +818,13 @@ struct WallSpring {
     T kn, dn, kt, dtg, ikt;
 };
 
+// whether the particle touches the face: a contact that ends takes its spring with it
+template <typename T>
+__device__ __forceinline__ void wall_touch(WallSpring<T>& w, bool touch) {
+    w.on = touch;
+    if (!touch) w.b = w.c = T(0);
+}
+
 template <typename T>
 __device__ __forceinline__ void wall_load(const DemParams& p, const OctLane& o, WallSpring<T>& w, int hin) {
     const int a = o.s >> 1;
@@ -871,7 +878,7 @@ __device__ bool wall_force(const DemParams& p, const OctLane& o, WallSpring<T>& 
     const double Rid = P.R[o.i];
     const T delta = (T)(side == 0 ? xa - Rid : ((double)p.g.n[a] - xa) - Rid);
     const bool touch = negative(delta);
-    if (!init) w.on = touch;
+    if (!init) wall_touch(w, touch);
     if (!touch && !less_pos(delta, k.cut_max)) return false;
     const T Ri = (T)Rid;
     const T sg = side == 0 ? T(1) : T(-1);
@@ -1047,7 +1054,7 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
     if (!(p.g.per[0] && p.g.per[1] && p.g.per[2])) {
         const float xa = __shfl_sync(FULL, o.xf, o.s >> 1, DEM_LANES);
         face = (o.s & 1 ? -xa : xa) <= o.face;
-        if (!face && !init) w.on = false;
+        if (!face && !init) wall_touch(w, false);
     }
     if (__any_sync(FULL, face)) {
         // what face s needs of the particle's position and velocities, from its lanes
