@@ -385,12 +385,11 @@ __device__ __forceinline__ double wrap_pos(double x, int n, int per) {
 }
 
 __device__ __forceinline__ void position_update(const DemParams& p, int i) {
-    // Eq. (37): x += dt u + dt^2 / (2 m) F
-    const double dt = p.dt;
-    const double c = dt * dt * p.P.hm[i];
+    // Eq. (37): x += dt u + dt^2 / (2 m) F, every operation rounded as in oct_move
+    const double c = __dmul_rn(p.dt, __dmul_rn(p.dt, p.P.hm[i]));
     for (int d = 0; d < 3; ++d) {
-        const double x = wrap_pos(p.P.x[3 * i + d] + dt * p.P.u[3 * i + d] + c * p.P.F_prev[3 * i + d],
-                                  p.g.n[d], p.g.per[d]);
+        const double x = wrap_pos(fma(c, p.P.F_prev[3 * i + d], fma(p.dt, p.P.u[3 * i + d], p.P.x[3 * i + d])), p.g.n[d],
+                                  p.g.per[d]);
         p.P.x[3 * i + d] = x;
         p.P.xf[3 * i + d] = (float)x;
     }
@@ -767,14 +766,14 @@ __device__ __forceinline__ void oct_load(const DemParams& p, OctLane& o, int i, 
         o.v = P.us[cur][3 * i + s];
         o.f_prev = P.F_prev[3 * i + s];
         o.f_const = P.fbar[6 * i + s] + P.ext[3 * i + s];
-        o.coef = p.dt * P.hm[i];
+        o.coef = __dmul_rn(p.dt, P.hm[i]);
     } else if (s < 6) {
         o.v = P.oms[cur][3 * i + s - 3];
         o.f_prev = P.T_prev[3 * i + s - 3];
         o.f_const = P.fbar[6 * i + s];
-        o.coef = p.dt * P.hI[i];
+        o.coef = __dmul_rn(p.dt, P.hI[i]);
     }
-    o.dcoef = p.dt * o.coef;
+    o.dcoef = __dmul_rn(p.dt, o.coef);
     o.xf = (float)o.x;
     o.xl = trailing(o.x);
     o.vf = (float)o.v;
