@@ -379,9 +379,10 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
         if ((cx(q) || cy(q)) && cz(q)) cu = cz(q) * sg > 0 ? cu + uz : cu - uz;
         const V cu45 = c45 * cu;
         const V X = mad(cu45, cu, drp);
-        // the zero is read from memory: the compiler merges a packed product with the
-        // sum that follows, which rounds once less than with a body force
-        V src = corr[k], odd = P::all(ax);
+        // In float32 the zero is read from memory: the compiler merges a product with the
+        // sums that follow (rounded once less than with a body force). Float64 gains
+        // the nine instructions (32x32x64 cells 41.5 -> 39.8 us).
+        V src = corr[k], odd = P::all(sizeof(T) == 4 ? ax : T(-0.0));
         if constexpr (FORCE) {
             const V even = P::make(force[q].even);
             src = sizeof(T) == 8 ? mad(cu45, even, corr[k]) : mad(gpw[k], mad(cu45, even, m3ua), corr[k]);

@@ -301,9 +301,23 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
             }
         }
         const int edges = edges_xy | (z == 0 || z == nz - 1 ? 4 : 0);
-        const bool links = __any_sync(FULL, (link[0] | link[1]) != 0u);
+        bool links;   // warp-uniform
+        int cl = 0, cr = 0, incl = 0, left = 0, total = 0;
+        if (one) {
+            links = __any_sync(FULL, (link[0] | link[1]) != 0u);
+        } else {
+            // links of the left half (low 16 bits) and of the right half (high); with
+            // one row all count as left, the order in which they are queued below
+            cl = ROWS == 1 ? __popc(link[0]) : __popc(link[0] & 0xffffu) + __popc(link[1] & 0xffffu);
+            cr = ROWS == 1 ? 0 : __popc(link[0] >> 16) + __popc(link[1] >> 16);
+            incl = warp_incl_scan(cl | (cr << 16), lane);
+            const int all = __shfl_sync(FULL, incl, 31);
+            left = all & 0xffff;
+            total = left + (all >> 16);
+            links = total > 0;
+        }
         uint32_t of_cell[2] = {0u, 0u};   // one: bit q - 1, the lane's cell has a link in direction q
-        if (one && links) {   // warp-uniform
+        if (one && links) {
             // 2. the links of each row in the order of its cells, cut into runs of equal
             // length, one per lane
             const bool wrap = !(deep_xy && z >= mz && z < nz - mz);
@@ -352,14 +366,7 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
                     }
                 }
             }
-        } else if (links) {   // warp-uniform
-            // links of the left half (low 16 bits) and of the right half (high); with
-            // one row all count as left, the order in which they are queued below
-            const int cl = ROWS == 1 ? __popc(link[0]) : __popc(link[0] & 0xffffu) + __popc(link[1] & 0xffffu);
-            const int cr = ROWS == 1 ? 0 : __popc(link[0] >> 16) + __popc(link[1] >> 16);
-            const int incl = warp_incl_scan(cl | (cr << 16), lane);
-            const int all = __shfl_sync(FULL, incl, 31);
-            const int left = all & 0xffff, total = left + (all >> 16);
+        } else if (links) {
             const bool wrap = !(deep_xy && z >= mz && z < nz - mz);
             const int pl = (incl & 0xffff) - cl, pr = left + (incl >> 16) - cr;
             for (int base = 0; base < total; base += QUEUE_CAP) {
@@ -448,9 +455,11 @@ __device__ __forceinline__ void sc_warp(const SCArgs<S, T>& a, int wx, int y0, i
             for (int r = 0; r < ROWS; ++r) sh[r] = (sm.w[Q + 1][r] & me) != 0u;
             T dr[ROWS];
             // without a body force its sums are left out: float64, each instruction 64
-            // cycles of the unit, 32x32x64 cells 43.0 -> 39.4 us; float32, a pass of the
-            // 80x80x160 box 2.67 -> 2.63 ms
-            if (ax == T(0) && ay == T(0) && az == T(0))
+            // cycles of the unit, 32x32x64 cells 43.0 -> 39.4 us; boxes with one particle
+            // in float32, a pass of the 80x80x160 box 2.67 -> 2.63 ms. With many
+            // particles the second copy of the collision costs more than it gives
+            // (256 x 256 x 512 cells 1380 us without, 1411 with it).
+            if ((sizeof(T) == 8 || KIND == BOXES_ONE) && ax == T(0) && ay == T(0) && az == T(0))
                 P::get(collide_core<T, false>(f, sh, ax, ay, az, dt.force, a.s_plus, a.s_minus, a.gp, a.s_b_shell,
                                              a.s_b_bulk, a.bulk_corr),
                        dr);
