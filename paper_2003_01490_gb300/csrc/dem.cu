@@ -338,8 +338,8 @@ __device__ __forceinline__ void neighbour_body(const DemParams& p, int bx) {
                 cnt += __popc(m);
             }
     // ascending partner order (a bitonic sort over the warp), so that the
-    // subcycles' pair sums, taken in slot order, do not depend on the order
-    // in which atomics filled the bins
+    // subcycles' pair sums (each lane its slots in order, then the lanes in a
+    // fixed order) do not depend on the order in which atomics filled the bins
     const int m = cnt < NBR_CAP ? cnt : NBR_CAP;
     __syncwarp();
     int v = lane < m ? p.P.nbr[i * NBR_CAP + lane] : 0x7fffffff;
@@ -690,7 +690,7 @@ constexpr int ONE_BLOCK_THREADS = DEM_ONE_BLOCK_MAX * DEM_LANES;
 
 template <int PPB>
 struct PairQueue {
-    int n;
+    int count[(DEM_LANES * PPB + 31) / 32];   // pairs of each warp
     unsigned short entry[PPB * NBR_CAP];   // particle of the block << 5 | slot
     double res[DEM_LANES * PPB][6];
 };
@@ -998,27 +998,44 @@ __device__ __forceinline__ void oct_subcycle(const DemParams& p, OctLane& o, Wal
             }
         }
     } else if (pairs) {
-        // pairs that pass the prefilter into the block's queue, evaluated by
-        // whichever thread comes first; each lane then collects its slots'
-        const int pl = threadIdx.x / DEM_LANES;
-        __syncthreads();
-        if (threadIdx.x == 0) queue->n = 0;
-        __syncthreads();
-        int place[NBR_CAP / DEM_LANES];
+        // pairs that pass the prefilter into the block's queue, in the order of the
+        // threads and their slots, evaluated by full warps; each lane then collects its
+        // slots'. The places, and with them the order of every sum, are the same in
+        // every run (taken by an atomic counter 1 % faster: 150 particles 132.7 us a
+        // step, this way 134.3).
+        const int pl = threadIdx.x / DEM_LANES, lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
+        const int threads = (int)blockDim.x;
+        bool near[NBR_CAP / DEM_LANES];
+        int mine = 0;
 #pragma unroll
         for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
             const int slot = o.s + DEM_LANES * k;
-            place[k] = -1;
-            if (slot >= o.nn) continue;
-            if (may_touch(p, ld3s<CG>(P.xfs[cur], o.i), ld3s<CG>(P.xfs[cur], o.j[k]), o.reach2[k])) {
-                place[k] = atomicAdd(&queue->n, 1);
-                queue->entry[place[k]] = (unsigned short)((pl << 5) | slot);
-            } else if (!init) {
-                P.hist_id[hout][o.i * NBR_CAP + slot] = -1;
-            }
+            near[k] = slot < o.nn && may_touch(p, ld3s<CG>(P.xfs[cur], o.i), ld3s<CG>(P.xfs[cur], o.j[k]), o.reach2[k]);
+            mine += near[k];
+            if (slot < o.nn && !near[k] && !init) P.hist_id[hout][o.i * NBR_CAP + slot] = -1;
+        }
+        int at = mine;   // inclusive sum over the lanes
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(FULL, at, d);
+            if (lane >= d) at += v;
+        }
+        if (lane == 31) queue->count[warp] = at;
+        __syncthreads();
+        at -= mine;
+        int total = 0;
+        for (int w = 0; w < threads / 32; ++w) {
+            const int n = queue->count[w];
+            at += w < warp ? n : 0;
+            total += n;
+        }
+        int place[NBR_CAP / DEM_LANES];
+#pragma unroll
+        for (int k = 0; k < NBR_CAP / DEM_LANES; ++k) {
+            place[k] = near[k] ? at++ : -1;
+            if (near[k]) queue->entry[place[k]] = (unsigned short)((pl << 5) | (o.s + DEM_LANES * k));
         }
         __syncthreads();
-        const int total = queue->n, threads = (int)blockDim.x;
         for (int c0 = 0; c0 < total; c0 += threads) {
             const int e = c0 + (int)threadIdx.x;
             if (e < total) {
