@@ -937,6 +937,34 @@ lbm_status enqueue_pre(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepState& 
     return LBM_OK;
 }
 
+// a launch that the device, or the part of it that the stream may use, has no room for
+bool no_room(cudaError_t e) {
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+           e == cudaErrorInvalidClusterSize || e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
+}
+
+// the DEM step in one launch; where the one that its particle count asks for has no
+// room the next larger form is tried, and done is false (nothing ran) where none has
+lbm_status dem_step(lbm_ctx* ctx, const DemParams& dp, const FinalizeParams& fin, cudaStream_t sm, bool& done) {
+    const MapParams mp = map_params(ctx);
+    cudaError_t e = launch_dem_step(dp, fin, mp, ctx->hcur, ctx->dem.n_sub, ctx->cluster_particles, sm);
+    if (no_room(e) && ctx->P.n <= ctx->cluster_particles) {
+        cudaGetLastError();
+        ctx->cluster_particles = 0;
+        e = launch_dem_step(dp, fin, mp, ctx->hcur, ctx->dem.n_sub, 0, sm);
+    }
+    done = !(no_room(e) && ctx->P.n > DEM_ONE_BLOCK_MAX);
+    if (!done) {
+        cudaGetLastError();
+        ctx->grid_particles = 0;
+        return LBM_OK;
+    }
+    CK(e);
+    ctx->launches += 1;
+    if (ctx->dem.n_sub & 1) ctx->hcur = 1 - ctx->hcur;
+    return LBM_OK;
+}
+
 lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepState& ss);
 lbm_status enqueue_post_b(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, const StepState& ss);
 
@@ -971,10 +999,14 @@ lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepStat
     if (move) {
         if (ss.one_launch) {
             // Algorithm 1, lines 4-10, in one launch
-            CK(launch_dem_step(dp, fpp, map_params(ctx), ctx->hcur, d.n_sub, ctx->cluster_particles, sm));
-            ctx->launches += 1;
-            if (d.n_sub & 1) ctx->hcur = 1 - ctx->hcur;
-        } else if (dem) {
+            const lbm_status st = dem_step(ctx, dp, fpp, sm, ss.one_launch);
+            if (st != LBM_OK) return st;
+            if (!ss.one_launch) {
+                launch_finalize(fpp, sm);
+                ctx->launches += 1;
+            }
+        }
+        if (dem && !ss.one_launch) {
             // Algorithm 1, lines 4-10: DEM subcycles
             launch_dem_position(dp, sm);
             ctx->launches += 1;
@@ -991,7 +1023,7 @@ lbm_status enqueue_post_a(lbm_ctx* ctx, DemParams& dp, cudaStream_t sm, StepStat
                 launch_state_copy(ctx->P, sm);
                 ctx->launches += 1;
             }
-        } else {
+        } else if (!dem) {
             // prescribed motion: x += u over the step
             launch_prescribed_move(ctx->P, ctx->g, sm);
             ctx->launches += 1;
@@ -1505,6 +1537,14 @@ lbm_status lbm_profile_read(lbm_ctx* ctx, double* phase_ms, long long* steps) {
         }
     if (steps) *steps = ctx->prof_steps;
     return LBM_OK;
+}
+
+// particles up to which the context tries the DEM step in one cooperative launch or
+// one cluster (for tests of the launches that take its place; not in the header)
+void lbmdem_set_dem_capacity(lbm_ctx* ctx, int grid_particles, int cluster_particles) {
+    ctx->grid_particles = grid_particles;
+    ctx->cluster_particles = cluster_particles;
+    reset_graphs(ctx);
 }
 
 long long lbm_launch_count(const lbm_ctx* ctx) { return ctx ? ctx->launches : 0; }
