@@ -53,9 +53,11 @@ struct lbm_ctx {
     int* status = nullptr;
     double* accel = nullptr;
     float* accel_f = nullptr;
-    // page-locked memory for small transfers (NULL: none could be had): kernels read
-    // and write it themselves, so a call waits once; word 0 takes the status
+    // page-locked memory for small transfers (NULL: not asked for yet, or none could be
+    // had): kernels read and write it themselves, so a call waits once; word 0 takes the
+    // status
     double* io = nullptr;
+    bool io_asked = false;
     bool accel_set = true;         // they hold the body force of a box without counterforce
     unsigned* barrier = nullptr;   // of the cooperative DEM launch
     int grid_particles = 0;        // particles a cooperative DEM launch holds
@@ -327,10 +329,6 @@ lbm_status create_impl(const lbm_grid* g, const lbm_relax* r, const double* bf, 
             pe = dem_grid_capacity(st == LBM_STORE_F64, ctx->num_sms, &ctx->grid_particles);
             if (st != LBM_STORE_F64) ctx->cluster_particles = dem_cluster_capacity();
         }
-        if (cudaHostAlloc(&ctx->io, sizeof(double) * IO_WORDS, cudaHostAllocPortable) != cudaSuccess) {
-            cudaGetLastError();
-            ctx->io = nullptr;
-        }
         if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
@@ -596,6 +594,21 @@ lbm_status status_result(lbm_ctx* ctx, int st) {
     if (st & ST_TIMEOUT) return fail(ctx, LBM_ERR_TIMEOUT, "a barrier of the DEM launch ran out");
     if (st & ST_FAST_PARTICLE) return fail(ctx, LBM_ERR_UNSTABLE, "particle speed above 0.5 cells per step");
     return LBM_OK;
+}
+
+// whether a transfer of so many words goes through the context's page-locked memory,
+// which is had when the first one asks for it (20 us, which a context that is
+// created, stepped and read out asynchronously need not pay)
+bool fits_io(lbm_ctx* ctx, size_t words) {
+    if (words >= IO_WORDS) return false;
+    if (!ctx->io_asked) {
+        ctx->io_asked = true;
+        if (cudaHostAlloc(&ctx->io, sizeof(double) * IO_WORDS, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->io = nullptr;
+        }
+    }
+    return ctx->io != nullptr;
 }
 
 // waits for the stream
@@ -1172,7 +1185,7 @@ lbm_status lbm_get_particle_state(lbm_ctx* ctx, int n_cap, double* pos, double* 
     if (n_cap < n && (pos || vel || omega || force_hyd || torque_hyd))
         return fail(ctx, LBM_ERR_INVALID, "n_cap smaller than the particle count");
     cudaStream_t sm = ctx->stream;
-    if (n > 0 && ctx->io && 15 * (size_t)n < IO_WORDS && (pos || vel || omega || force_hyd || torque_hyd)) {
+    if (n > 0 && (pos || vel || omega || force_hyd || torque_hyd) && fits_io(ctx, 15 * (size_t)n)) {
         double* const src = ctx->io + 1;
         launch_read_state(ctx->P, src, ctx->status, reinterpret_cast<int*>(ctx->io), sm);
         ctx->launches += 1;
@@ -1371,7 +1384,7 @@ lbm_status lbm_set_particle_velocity(lbm_ctx* ctx, int n, const double* vel, con
     if (n < 0 || n > ctx->P.n) return fail(ctx, LBM_ERR_INVALID, "n outside [0, particle count]");
     if (n == 0) return LBM_OK;
     cudaStream_t sm = ctx->stream;
-    if (ctx->io && 6 * (size_t)n < IO_WORDS) {
+    if (fits_io(ctx, 6 * (size_t)n)) {
         double* const src = ctx->io + 1;
         if (vel) std::memcpy(src, vel, 24 * (size_t)n);
         if (omega) std::memcpy(src + 3 * (size_t)n, omega, 24 * (size_t)n);
@@ -1427,7 +1440,7 @@ lbm_status lbm_sample_density(lbm_ctx* ctx, int n, const double* pos, double* rh
     if (n == 0) return LBM_OK;
     cudaStream_t sm = ctx->stream;
     SampleParams sp{};
-    const bool small = ctx->io && 4 * (size_t)n < IO_WORDS;
+    const bool small = fits_io(ctx, 4 * (size_t)n);
     // points and results in page-locked memory, many of them in the scratch buffer
     // (4 doubles per scratch cell)
     double* const io = small ? ctx->io + 1 : ctx->scratch;
