@@ -343,10 +343,10 @@ lbm_status lbm_fp64_fma_rate(int iters, double *tflops_out);
  * lbm_batch_set_launch(b, instance, tile_bx, zchunk, blocks_per_sm): launch
  *   shape of the batched dense kernel for one instance (instance = -1: all):
  *   tile width tile_bx in x (0 automatic: the narrowest of 32, 64, 128 that
- *   covers the box width, else 32, 64 or 128; 256 / tile_bx rows),
- *   zchunk z planes per work item (0 automatic = 16), and blocks_per_sm
- *   resident blocks per multiprocessor for the whole launch (0 automatic:
- *   4, 2 for float64). Synchronises the stream and drops the captured graphs.
+ *   covers the box width, else 32, 64 or 128; 256 / tile_bx rows, 128 / tile_bx
+ *   for float64), zchunk z planes per work item (0 automatic = 16), and
+ *   blocks_per_sm resident blocks of 128 threads per multiprocessor for the
+ *   whole launch (0 automatic: 4). Synchronises the stream and drops the captured graphs.
  * lbm_batch_set_active(b, instance, active): whether the instance takes part
  *   in the following lbm_batch_step() calls (finished instances are
  *   deactivated; an inactive instance's state is not touched).
