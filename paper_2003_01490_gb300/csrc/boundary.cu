@@ -196,7 +196,8 @@ __device__ __forceinline__ void missing_links_of_cell(const BcArgs<S>& a, int id
 
 // mode BC_ACCEL: one thread forms the fluid body force of the step; mode
 // BC_LINKS: the missing-link terms 2 w_q c_q of Sec. 2.2 and their torques, one
-// thread per listed solid cell, committed per warp
+// thread per listed solid cell (float64: one warp, as long as the list has a cell
+// per warp at most), committed per warp
 // (block bx of a grid of gx blocks)
 template <typename S>
 __device__ __forceinline__ void boundary_body(const BcArgs<S>& a, int mode, int bx, int gx) {

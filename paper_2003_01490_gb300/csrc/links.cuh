@@ -264,38 +264,28 @@ template <> struct PartOps<double> {
     }
 };
 template <> struct PartOps<float> {
-    template <typename A>
-    __device__ static void load(const A& a, int i, int x, int y, int z, float (&r)[3], int (&n)[3], float& R,
-                                float (&u)[3], float (&om)[3]) {
-        float g[3], C[2];
-        load(a, i, x, y, z, r, n, g, C, R, u, om);
-    }
-    // also the fractional offset g and C = |g|^2 - R^2 of the particle. The
-    // image is chosen on the integer offset: a link cell lies within R + 2
+    // The image is chosen on the integer offset: a link cell lies within R + 2
     // cells of the centre on every axis and a periodic side is longer than
     // 2 R + 4, so exactly one image has |n_d| <= floor(n / 2)
     template <typename A>
-    __device__ static void load(const A& a, int i, int x, int y, int z, float (&r)[3], int (&n)[3], float (&g)[3],
-                                float (&C)[2], float& R, float (&u)[3], float (&om)[3]) {
+    __device__ static void load(const A& a, int i, int x, int y, int z, float (&r)[3], int (&n)[3], float& R,
+                                float (&u)[3], float (&om)[3]) {
         const PartView v = a.view[i];
         const int c[3] = {x, y, z};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             int nd = c[d] - v.base[d];
-            g[d] = 0.5f - v.frac[d];
             if (a.g.per[d]) {
                 const int L = a.g.n[d], half = L >> 1;
                 if (nd > half) nd -= L;
                 else if (nd < -half) nd += L;
             }
             n[d] = nd;
-            r[d] = (float)nd + g[d];
+            r[d] = (float)nd + (0.5f - v.frac[d]);
             u[d] = v.u[d];
             om[d] = v.om[d];
         }
         R = v.R;
-        C[0] = v.C;
-        C[1] = v.C_lo;
     }
 };
 
@@ -347,17 +337,6 @@ __device__ __forceinline__ T surface_cc(const T (&r)[3], T R) {
     return sum + (err + e);
 }
 
-// the same for r = n + g with integer n and the particle's common fractional
-// offset g: (|n|^2 + C) + (2 n.g + C_lo), with C + C_lo = |g|^2 - R^2
-// precomputed per particle to float64 accuracy. Near the surface |n|^2 and
-// -C agree to within a factor of two, so their sum is exact and only the
-// small terms round.
-__device__ __forceinline__ float surface_cc_split(const int (&n)[3], const float (&g)[3], const float (&C)[2]) {
-    const int nn = n[0] * n[0] + n[1] * n[1] + n[2] * n[2];
-    const float ng = fmaf((float)n[2], g[2], fmaf((float)n[1], g[1], (float)n[0] * g[0]));
-    return ((float)nn + C[0]) + fmaf(2.0f, ng, C[1]);
-}
-
 template <typename T>
 __device__ __forceinline__ T link_fraction(const T (&r)[3], T c0, T c1, T c2_, T cc2, T R) {
     return link_root<T>(r, surface_cc<T>(r, R), c0, c1, c2_, cc2);
@@ -368,7 +347,6 @@ static __constant__ signed char k_c[Q][3] = {{0, 0, 0},   {0, 1, 0},   {0, -1, 0
                                       {0, 0, 1},   {0, 0, -1},  {-1, 1, 0},  {1, 1, 0},   {-1, -1, 0},
                                       {1, -1, 0},  {0, 1, 1},   {0, -1, 1},  {-1, 0, 1},  {1, 0, 1},
                                       {0, 1, -1},  {0, -1, -1}, {-1, 0, -1}, {1, 0, -1}};
-static __constant__ signed char k_opp[Q] = {0, 2, 1, 4, 3, 6, 5, 10, 9, 8, 7, 16, 15, 18, 17, 12, 11, 14, 13};
 
 // inclusive prefix sum over the warp
 __device__ __forceinline__ int warp_incl_scan(int v, int lane) {

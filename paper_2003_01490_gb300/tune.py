@@ -3,13 +3,12 @@
 A batch (``lbm_batch_create``) runs the stream/collide kernels of all its
 instances as one persistent launch over a table of work items (instance,
 tile of tile_bx x 256/tile_bx cells, x 128/tile_bx in float64, chunk of zchunk
-planes). Which tile width,
-chunk depth and number of resident blocks per multiprocessor is fastest
-depends on the mix of box sizes and on the GPU, so this module measures it:
-every candidate is set with ``lbm_batch_set_launch``, warmed up (its graph is
-captured) and timed over a few batched steps with CUDA events on the batch's
-stream; the fastest is set on the batch and stored in a JSON cache keyed by
-the GPU, the storage format and the sorted box shapes, so a later batch of the
+planes). Which tile width, chunk depth and number of resident blocks per
+multiprocessor is fastest depends on the mix of box sizes and on the GPU, so
+this module measures it: every candidate is set with ``lbm_batch_set_launch``,
+warmed up (its graph is captured) and timed over a few batched steps with
+CUDA events on the batch's stream; the fastest is set on the batch and stored
+in a JSON cache keyed by the GPU, the storage format and the sorted box shapes, so a later batch of the
 same kind starts from it without timing again.
 
 Timing advances the instances by the steps it runs (as a warm-up would); pass
