@@ -75,11 +75,11 @@ __host__ __device__ constexpr int lead(int q) { return cx(q) ? cx(q) : (cy(q) ? 
 // long run.
 template <typename T>
 struct Weights {
-    static constexpr T w2d = sizeof(T) == 4 ? T(0.0555555522441864) : T(1) / T(18);
-    static constexpr T w2a = T(2) * w2d;
-    static constexpr T w0 = T(1) - T(12) * w2d;
-    static constexpr T w6d = T(1) / T(6);
-    static constexpr T w6a = T(1) - T(4) * w6d;
+    const T w2d = sizeof(T) == 4 ? T(0.0555555522441864) : T(1) / T(18);
+    const T w2a = T(2) * w2d;
+    const T w0 = T(1) - T(12) * w2d;
+    const T w6d = T(1) / T(6);
+    const T w6a = T(1) - T(4) * w6d;
 };
 
 // What the collision reads of the body force a per pair of directions (q, qbar),
@@ -98,9 +98,10 @@ __device__ __forceinline__ ForceTerms<T> force_terms(int qi, T ax, T ay, T az, T
     if (c0) ca += c0 * sg > 0 ? ax : -ax;
     if (c1) ca += c1 * sg > 0 ? ay : -ay;
     if (c2_) ca += c2_ * sg > 0 ? az : -az;
+    const Weights<T> w{};
     const bool axis = c0 * c0 + c1 * c1 + c2_ * c2_ == 1;
-    const T g = T(0.5) * gm * (axis ? Weights<T>::w6a : Weights<T>::w6d);
-    const T e = sizeof(T) == 8 ? T(0.5) * gp * (axis ? Weights<T>::w2a : Weights<T>::w2d) : T(1);
+    const T g = T(0.5) * gm * (axis ? w.w6a : w.w6d);
+    const T e = sizeof(T) == 8 ? T(0.5) * gp * (axis ? w.w2a : w.w2d) : T(1);
     ForceTerms<T> t;
 #pragma unroll
     for (int r = 0; r < Pack<T>::ROWS; ++r) {
@@ -304,7 +305,7 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
                                                             T s_b_bulk, int bulk_corr) {
     using P = Pack<T>;
     using V = typename P::V;
-    using K = Weights<T>;
+    const Weights<T> k_w{};
     // pair sums and differences are formed twice (here and in the update):
     // keeping them takes 36 registers more than the cell's PDFs
     V drho = f[0], jx = P::all(T(0)), jy = jx, jz = jx;
@@ -352,16 +353,16 @@ __device__ __forceinline__ typename Pack<T>::V collide_core(typename Pack<T>::V 
     }
     // equilibrium part common to all directions
     const V drp = mad(P::all(T(-1.5)), usq, drho);
-    const V mw2[2] = {P::all(-K::w2a), P::all(-K::w2d)}, mw6[2] = {P::all(-K::w6a), P::all(-K::w6d)};
-    const V gpw[2] = {P::all(T(0.5) * gp * K::w2a), P::all(T(0.5) * gp * K::w2d)};
-    V corr[2] = {mw2[0] * k5, P::all(T(0.5) * K::w2d) * (k4 + k5)};
+    const V mw2[2] = {P::all(-k_w.w2a), P::all(-k_w.w2d)}, mw6[2] = {P::all(-k_w.w6a), P::all(-k_w.w6d)};
+    const V gpw[2] = {P::all(T(0.5) * gp * k_w.w2a), P::all(T(0.5) * gp * k_w.w2d)};
+    V corr[2] = {mw2[0] * k5, P::all(T(0.5) * k_w.w2d) * (k4 + k5)};
     if constexpr (FORCE && sizeof(T) == 8) {
         corr[0] = mad(gpw[0], m3ua, corr[0]);
         corr[1] = mad(gpw[1], m3ua, corr[1]);
     }
-    V f0 = mad(P::all(sp), mad(P::all(K::w0), drp, P::all(T(0)) - f[0]), f[0]);
-    if constexpr (FORCE) f0 = mad(P::all(gp), P::all(K::w0) * m3ua, f0);
-    f[0] = mad(P::all(K::w0), k5 - k4, f0);
+    V f0 = mad(P::all(sp), mad(P::all(k_w.w0), drp, P::all(T(0)) - f[0]), f[0]);
+    if constexpr (FORCE) f0 = mad(P::all(gp), P::all(k_w.w0) * m3ua, f0);
+    f[0] = mad(P::all(k_w.w0), k5 - k4, f0);
     const V hsp = P::all(T(-0.5) * sp), hsm = P::all(T(-0.5) * sm), c45 = P::all(T(4.5));
     // each part relaxes as rate x (value - its equilibrium). The pair sums and
     // differences as (exact) multiply-adds, which the compiler does not merge
