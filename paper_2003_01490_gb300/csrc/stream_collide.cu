@@ -29,11 +29,11 @@
 // whatever the arithmetic gives), so DRAM never has to merge part of one.
 //
 // What bounds it (256 x 256 x 512 cells, 10,000 spheres, 27 % solids, float32):
-// instruction issue and latency together, 930 warp instructions per row of 32
+// instruction issue and latency together, 900 warp instructions per row of 32
 // cells (1,310 with a test of every pulled value for a marker, one row per warp
-// and force sums flushed when a lane's particle changed) at 54 % issue; 1.36 ms
-// against 1.58 ms that way, 128 x 128 x 256 cells 214 us against 284 us, float16
-// 192^3 with 2,000 spheres 328 us against 466 us. Streaming alone takes the
+// and force sums flushed when a lane's particle changed) at 51 % issue; 1.38 ms
+// against 1.58 ms that way, 128 x 128 x 256 cells 216 us against 284 us, float16
+// 192^3 with 2,000 spheres 334 us against 466 us. Streaming alone takes the
 // memory's time (95 us of the 128 x 128 x 256 case at 6.7 TB/s).
 //
 // Per-particle sums. Float64 storage: float64 sums per lane and warp, float64
